@@ -249,9 +249,10 @@ int monarch_dense(const void *L, const void *R, void *M, int32_t n, int32_t m, i
  * R[k][j][:] = sqrt(sigma_1) v_1.  The paper fixes only the product u v^T; the
  * sign of the pair is arbitrary, and where sigma_1 = sigma_2 the slice's
  * approximation itself is not unique.  A: [n][n] row-major; L, R: [m][m][m];
- * all in the storage dtype, arithmetic in fp32 (one-sided Jacobi per slice).
- * `rotation_count` is null or a device counter to which the number of plane
- * rotations performed is added (for FLOP accounting). */
+ * all in the storage dtype, arithmetic in fp32.  `rotation_count` is null (only
+ * the leading singular pair of each slice is iterated for) or a device counter:
+ * the slices are then decomposed by one-sided Jacobi iterations and the number
+ * of plane rotations performed is added to it (for FLOP accounting). */
 int monarch_project(const void *A, void *L, void *R, int32_t n, int32_t m, int dtype,
                     unsigned long long *rotation_count, void *stream);
 

@@ -56,10 +56,38 @@ template <> struct elem<__nv_bfloat16> {
     static __device__ __forceinline__ void store(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 };
 
+// Two fp32 values in a register pair; fma2 rounds each half like fmaf, in one instruction for both.
+typedef unsigned long long f32x2;
+static __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+static __device__ __forceinline__ f32x2 pack2(float x, float y)
+{
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
+static __device__ __forceinline__ float2 unpack2(f32x2 a)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+
 // erf form of GELU, evaluated in fp32.
 static __device__ __forceinline__ float gelu_erf(float a)
 {
     return 0.5f * a * (1.0f + erff(a * 0.70710678118654752440f));
+}
+
+// d/da of a/2 (1 + erf(a / sqrt 2)):  Phi(a) + a phi(a)
+static __device__ __forceinline__ float gelu_erf_grad(float a)
+{
+    const float cdf = 0.5f * (1.0f + erff(a * 0.70710678118654752440f));
+    return cdf + a * 0.39894228040143267794f * expf(-0.5f * a * a);
 }
 
 // GELU(a) = a/2 (1 + erf(a / sqrt 2)) evaluated as a * sigmoid(2 a (c0 + c1 a^2 + c2 a^4)): the logistic form

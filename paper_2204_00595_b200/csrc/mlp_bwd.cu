@@ -49,13 +49,6 @@ template <> struct vec16<__nv_bfloat16> {
     }
 };
 
-// d/da of a/2 (1 + erf(a / sqrt 2)):  Phi(a) + a phi(a)
-__device__ __forceinline__ float gelu_erf_grad(float a)
-{
-    const float cdf = 0.5f * (1.0f + erff(a * 0.70710678118654752440f));
-    return cdf + a * 0.39894228040143267794f * expf(-0.5f * a * a);
-}
-
 // fp32 tensors get the libm-grade forms; bf16 results are rounded to 8 bits of mantissa, so the cheaper forms
 // (error <= 5.1e-5) change nothing there and keep both kernels bound by memory rather than by erff / expf
 template <typename T> struct act_math;

@@ -3,26 +3,51 @@
 //   monarch_project  Algorithm 1:   view A as A~[l][j][k][i] = A[l*m+j][k*m+i]; for every (j, k) replace the m x m
 //                                   slice A~[:, j, k, :] by its best rank-1 approximation sigma u v^T and store
 //                                   L[j][:, k] = sqrt(sigma) u,  R[k][j][:] = sqrt(sigma) v.
-// The m*m slices are independent: one CTA per slice.  The leading singular triplet comes from a one-sided Jacobi
-// iteration in shared memory (columns are rotated in pairs until they are mutually orthogonal; their norms are then
-// the singular values and the normalised columns the left singular vectors), which converges at the same rate
-// whatever the gap between the first two singular values - a power iteration would not.  v = S^T u / sigma is one
-// more pass over the slice.  Arithmetic is fp32 whatever the storage dtype.
+// The m*m slices are independent: one CTA per slice.  Only the leading singular triplet is needed, so
+// leading_pair_kernel iterates for that one vector and never forms the rest of the decomposition; a caller that asks
+// for the number of plane rotations gets jacobi_kernel, the full one-sided Jacobi iteration that performs them.
+// Arithmetic is fp32 whatever the storage dtype.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace monarch {
 namespace {
 
+// Bound by the n*n elements written.  A CTA keeps a column range of R~_j (j fixed) in registers, 16 bytes per access,
+// and writes it scaled by L[j][l][k] for kDenseRows rows l, so that R is read m / kDenseRows times instead of m times
+// and every store is 16 bytes (n = 4096 fp32: 30.6 us with one scalar store per element and thread).
+constexpr int kDenseRows = 16, kDenseVecs = 4;
+
 template <typename T>
 __global__ void __launch_bounds__(256)
 dense_kernel(const T *__restrict__ L, const T *__restrict__ R, T *__restrict__ M, int m)
 {
-    // one CTA per output row (l, j); thread -> column k*m + i
-    const int row = blockIdx.x, l = row / m, j = row % m, n = m * m;
-    for (int col = threadIdx.x; col < n; col += 256) {
-        const int k = col / m, i = col % m;
-        const float v = elem<T>::load(L + ((size_t)j * m + l) * m + k) * elem<T>::load(R + ((size_t)k * m + j) * m + i);
-        elem<T>::store(M + (size_t)row * n + col, v);
+    constexpr int V = 16 / sizeof(T);
+    const int j = blockIdx.x, l0 = blockIdx.y * kDenseRows, n = m * m;
+    const int c0 = (blockIdx.z * kDenseVecs * 256 + threadIdx.x) * V;
+    float r[kDenseVecs][V];
+#pragma unroll
+    for (int q = 0; q < kDenseVecs; ++q) {
+        const int col = c0 + q * 256 * V;
+        if (col < n) {
+            const uint4 raw = *reinterpret_cast<const uint4 *>(R + ((size_t)(col / m) * m + j) * m + col % m);
+#pragma unroll
+            for (int e = 0; e < V; ++e) r[q][e] = elem<T>::load(reinterpret_cast<const T *>(&raw) + e);
+        }
+    }
+#pragma unroll 4
+    for (int l = l0; l < l0 + kDenseRows; ++l) {
+#pragma unroll
+        for (int q = 0; q < kDenseVecs; ++q) {
+            const int col = c0 + q * 256 * V;
+            if (col >= n) continue;
+            const float w = elem<T>::load(L + ((size_t)j * m + l) * m + col / m);
+            uint4 raw;
+#pragma unroll
+            for (int e = 0; e < V; ++e) elem<T>::store(reinterpret_cast<T *>(&raw) + e, w * r[q][e]);
+            *reinterpret_cast<uint4 *>(M + ((size_t)l * m + j) * n + col) = raw;
+        }
     }
 }
 
@@ -30,8 +55,9 @@ constexpr int kMaxSweeps = 30;
 // columns count as orthogonal below this cosine: a few times the rounding noise of an fp32 dot product of m terms
 constexpr float kOrthoTol = 2e-6f;
 
-// Rotation counter for the benchmark's FLOP count (optional, may be null).
-// A column pair is handled by G lanes (m/G rows each): G = 8 for m <= 64, so that a warp rotates four pairs at once
+// One-sided Jacobi in shared memory: columns are rotated in pairs until they are mutually orthogonal; their norms are
+// then the singular values and the normalised columns the left singular vectors; v = S^T u / sigma is one more pass
+// over the slice.  `rotations` counts the plane rotations.  A column pair is handled by G lanes (m/G rows each): G = 8 for m <= 64, so that a warp rotates four pairs at once
 // - with 64-element columns a whole warp per pair would spend most of its instructions on shuffle and scalar work
 // replicated over 32 lanes - and G = 32 for m = 128, where the strided rows of four different columns would
 // collide in the shared-memory banks.  Several CTAs share an SM.
@@ -44,7 +70,7 @@ template <int M> struct ProjectCfg {
 
 template <typename T, int M>
 __global__ void __launch_bounds__(ProjectCfg<M>::kWarps * 32)
-project_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ R, unsigned long long *rotations)
+jacobi_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ R, unsigned long long *rotations)
 {
     using C = ProjectCfg<M>;
     constexpr int N = M * M;
@@ -121,7 +147,7 @@ project_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ R, un
         }
         if (!__syncthreads_or(rotated)) break;
     }
-    if (rotations != nullptr && my_rot) atomicAdd(rotations, (unsigned long long)my_rot);
+    if (my_rot) atomicAdd(rotations, (unsigned long long)my_rot);
 
     // the column of largest norm carries sigma_1 u_1
     float best = -1.0f;
@@ -165,19 +191,405 @@ project_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ R, un
 }
 
 template <typename T, int M>
-int launch_project(const void *A, void *L, void *R, unsigned long long *rotations, cudaStream_t s)
+int launch_jacobi(const void *A, void *L, void *R, unsigned long long *rotations, cudaStream_t s)
 {
     constexpr int kWarps = ProjectCfg<M>::kWarps;
     constexpr int smem = M * (M + 1) * (int)sizeof(float);
     static bool attr = false;
     if (!attr && smem > 48 * 1024) {
-        MONARCH_CUDA_TRY(cudaFuncSetAttribute(project_kernel<T, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        MONARCH_CUDA_TRY(cudaFuncSetAttribute(jacobi_kernel<T, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         attr = true;
     }
-    project_kernel<T, M><<<M * M, kWarps * 32, smem, s>>>((const T *)A, (T *)L, (T *)R, rotations);
+    jacobi_kernel<T, M><<<M * M, kWarps * 32, smem, s>>>((const T *)A, (T *)L, (T *)R, rotations);
     note_launch();
     MONARCH_CUDA_TRY(cudaGetLastError());
     return MONARCH_OK;
+}
+
+// ---- leading singular pair of a slice ------------------------------------------------------------------------------
+//  1. Power iteration on S^T S from TWO fixed unrelated start vectors.  It has converged when the two agree and have
+//     stopped moving, to kPowerTol: neither alone would show a start vector that happens to be orthogonal to v_1.
+//     At most kPowerSteps steps are spent on it, enough for (sigma_2 / sigma_1)^2 up to about 0.7.
+//  2. Otherwise (a small gap) H = S^T S is squared and scaled to trace 1 until it has rank 1 - doubling the exponent
+//     each time, so the cost grows with the logarithm of 1 / gap and is bounded - and any column of H is v_1.
+// Both end in vectors accurate to rounding / gap.
+// One warp per slice (four for m = 128), a 4 x 8 grid of lanes, each lane holding an (m/4) x (m/8) patch of S in
+// registers for the whole iteration.  A product then needs m/8 (or m/4) values of the vector per lane from shared
+// memory and a reduce-scatter over 8 (or 4) lanes; with a whole row per lane every lane would read the whole vector,
+// and the 128 bytes per clock that shared memory returns were the limit (149 us for 4096 slices of 64 x 64).
+// Bound by fp32 issue: products are packed two to an instruction (fma.rn.f32x2), ten warps share an SM.
+// Measured, fp32, against the Jacobi iteration that ran before: 4096 slices of 64 x 64 with a clear leading value
+// 7714 -> 113 us, Gaussian 7690 -> 747 us; 128 x 128 Gaussian 165 -> 17.8 ms; largest error of a Gaussian slice's
+// rank-1 part 2.3e-4 -> 2e-6 (the Jacobi iteration stops at a cosine of 2e-6).  Where all singular values of a slice
+// are equal the squarings run to their bound: 0.57 -> 1.29 ms.
+constexpr int kPowerSteps = 40, kPolishSteps = 4, kMaxSquarings = 24;
+constexpr float kPowerTol = 1e-6f;
+
+template <int M> struct LeadCfg {
+    static constexpr int kWarps = M == 128 ? 4 : 1, kThreads = 32 * kWarps;
+    static constexpr int kRows = M / (4 * kWarps), kCols = M / 8;       // a lane's patch of S
+    static constexpr int kYC = kRows >= 8 ? kRows / 8 : 1;              // rows of S x a lane ends up with
+    static constexpr int kZC = kWarps > 1 || kCols < 4 ? 1 : kCols / 4; // columns of S^T y a thread ends up with
+    static constexpr int kPitch = M + 4;                                // of H, floats: rows stay 16-byte aligned
+    // the squaring step: kTR x kTC threads, each kRQ x kCQ patches of 4 x 4 of H
+    static constexpr int kTC = M <= 16 ? 4 : M == 128 ? 16 : 8, kTR = M == 128 ? 8 : 4;
+    static constexpr int kRQ = M / (4 * kTR), kCQ = M / (4 * kTC);
+    static constexpr int kSmem = (M * kPitch + 4 * M + (kWarps > 1 ? 2 * kWarps * M : 0)) * (int)sizeof(float);
+};
+
+template <int NT> __device__ __forceinline__ void slice_sync()
+{
+    if (NT == 32) __syncwarp();
+    else __syncthreads();
+}
+
+// sums over the CTA, the same bits in every thread; `red` has two halves used in turn, so one barrier is enough
+template <int NT, int K> __device__ __forceinline__ void slice_sum(float (&v)[K], float (*red)[NT / 32][4], int &phase)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (NT == 32) return;
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int k = 0; k < K; ++k) red[phase][threadIdx.x >> 5][k] = v[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        v[k] = red[phase][0][k];
+#pragma unroll
+        for (int w = 1; w < NT / 32; ++w) v[k] += red[phase][w][k];
+    }
+    phase ^= 1;
+}
+
+// Sum v over the lanes that differ in the bits [BIT, BIT_END) of the lane number; afterwards v[0 .. max(1, N >> bits))
+// hold this lane's share: the elements from scatter_base(lane) on.
+template <int BIT, int BIT_END, int N> __device__ __forceinline__ void reduce_scatter(float *v, int lane)
+{
+    if constexpr (BIT < BIT_END) {
+        if constexpr (N > 1) {
+            const bool up = lane >> BIT & 1;
+#pragma unroll
+            for (int i = 0; i < N / 2; ++i) {
+                const float send = up ? v[i] : v[i + N / 2];
+                const float keep = up ? v[i + N / 2] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 1 << BIT);
+            }
+            reduce_scatter<BIT + 1, BIT_END, N / 2>(v, lane);
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1 << BIT);
+            reduce_scatter<BIT + 1, BIT_END, 1>(v, lane);
+        }
+    }
+}
+template <int BIT, int BIT_END, int N> __device__ __forceinline__ int scatter_base(int lane)
+{
+    int base = 0, n = N;
+#pragma unroll
+    for (int b = BIT; b < BIT_END; ++b)
+        if (n > 1) {
+            n /= 2;
+            base += (lane >> b & 1) * n;
+        }
+    return base;
+}
+
+template <int N> __device__ __forceinline__ void load_vec(const float *from, float (&to)[N])
+{
+    if constexpr (N >= 4) {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) *reinterpret_cast<float4 *>(to + i) = *reinterpret_cast<const float4 *>(from + i);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) to[i] = from[i];
+    }
+}
+
+// acc = the calling thread's patches of A^T A, A in shared memory
+template <int M>
+__device__ __forceinline__ void gram_patches(const float *A, float (&acc)[LeadCfg<M>::kRQ * 4][LeadCfg<M>::kCQ * 4], int tr, int tc)
+{
+    using C = LeadCfg<M>;
+#pragma unroll
+    for (int r = 0; r < C::kRQ * 4; ++r)
+#pragma unroll
+        for (int c = 0; c < C::kCQ * 4; ++c) acc[r][c] = 0.0f;
+#pragma unroll 2
+    for (int k = 0; k < M; ++k) {
+        float a[C::kRQ * 4], b[C::kCQ * 4];
+#pragma unroll
+        for (int q = 0; q < C::kRQ; ++q)
+            *reinterpret_cast<float4 *>(a + 4 * q) = *reinterpret_cast<const float4 *>(A + k * C::kPitch + 4 * (tr + q * C::kTR));
+#pragma unroll
+        for (int q = 0; q < C::kCQ; ++q)
+            *reinterpret_cast<float4 *>(b + 4 * q) = *reinterpret_cast<const float4 *>(A + k * C::kPitch + 4 * (tc + q * C::kTC));
+#pragma unroll
+        for (int r = 0; r < C::kRQ * 4; ++r)
+#pragma unroll
+            for (int c = 0; c < C::kCQ * 4; ++c) acc[r][c] = fmaf(a[r], b[c], acc[r][c]);
+    }
+}
+
+template <typename T, int M>
+__global__ void __launch_bounds__(LeadCfg<M>::kThreads)
+leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ R)
+{
+    using C = LeadCfg<M>;
+    constexpr int N = M * M, NT = C::kThreads, W = C::kWarps, P = C::kPitch, RH = C::kRows, CW = C::kCols;
+    constexpr float kOnce = (float)M / (NT * C::kZC);     // columns are held 1 / kOnce times over the CTA
+    extern __shared__ __align__(16) float lead_smem[];
+    float *H = lead_smem, *x = H + M * P, *y = x + 2 * M; // x[2][M], y[2][M]: the two iterates
+    float *part = y + 2 * M;                              // W > 1: [2][W][M] partial sums of S^T y
+    __shared__ float red[2][W][4];
+    int phase = 0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int row0 = (warp * 4 + (lane >> 3)) * RH, col0 = (lane & 7) * CW;
+    const int my_row = row0 + scatter_base<0, 3, RH>(lane);
+    const int my_col = W > 1 ? tid : col0 + scatter_base<3, 5, CW>(lane);
+    const int j = blockIdx.x / M, k = blockIdx.x % M;
+    const T *slice = A + (size_t)j * N + (size_t)k * M;   // element (l, i) at slice[l * M * N + i]
+
+    f32x2 S[RH][CW / 2];
+    auto load_patch = [&](float scale) {
+        constexpr int kBytes = CW * (int)sizeof(T), kVec = kBytes < 16 ? kBytes : 16;
+        using Vec = typename std::conditional<kVec == 16, uint4, typename std::conditional<kVec == 8, uint2, unsigned>::type>::type;
+#pragma unroll
+        for (int q = 0; q < RH; ++q) {
+            Vec raw[kBytes / kVec];
+#pragma unroll
+            for (int v = 0; v < kBytes / kVec; ++v)
+                raw[v] = reinterpret_cast<const Vec *>(slice + (size_t)(row0 + q) * M * N + col0)[v];
+            const T *e = reinterpret_cast<const T *>(raw);
+#pragma unroll
+            for (int c = 0; c < CW / 2; ++c)
+                S[q][c] = pack2(elem<T>::load(e + 2 * c) * scale, elem<T>::load(e + 2 * c + 1) * scale);
+        }
+    };
+    // out = this lane's kYC elements of S v from row my_row on
+    auto times_S = [&](const float *v, float (&out)[C::kYC]) {
+        float vv[CW], p[RH];
+        load_vec(v + col0, vv);
+#pragma unroll
+        for (int q = 0; q < RH; ++q) {
+            f32x2 acc = 0;
+#pragma unroll
+            for (int c = 0; c < CW / 2; ++c) acc = fma2(S[q][c], pack2(vv[2 * c], vv[2 * c + 1]), acc);
+            const float2 t = unpack2(acc);
+            p[q] = t.x + t.y;
+        }
+        reduce_scatter<0, 3, RH>(p, lane);
+#pragma unroll
+        for (int i = 0; i < C::kYC; ++i) out[i] = p[i];
+    };
+    // out = this lane's share of S^T v over the rows of its warp
+    auto times_St = [&](const float *v, float (&out)[CW]) {
+        float vv[RH];
+        load_vec(v + row0, vv);
+        f32x2 acc[CW / 2];
+#pragma unroll
+        for (int c = 0; c < CW / 2; ++c) acc[c] = 0;
+#pragma unroll
+        for (int q = 0; q < RH; ++q)
+#pragma unroll
+            for (int c = 0; c < CW / 2; ++c) acc[c] = fma2(S[q][c], pack2(vv[q], vv[q]), acc[c]);
+#pragma unroll
+        for (int c = 0; c < CW / 2; ++c) {
+            const float2 t = unpack2(acc[c]);
+            out[2 * c] = t.x;
+            out[2 * c + 1] = t.y;
+        }
+        reduce_scatter<3, 5, CW>(out, lane);
+    };
+    // (za, zb) = elements my_col .. of S^T ya and S^T yb
+    auto back = [&](const float *ya, const float *yb, float (&za)[C::kZC], float (&zb)[C::kZC]) {
+        float a[CW], b[CW];
+        times_St(ya, a);
+        times_St(yb, b);
+        if constexpr (W > 1) {
+            const int at = warp * M + col0 + scatter_base<3, 5, CW>(lane);
+#pragma unroll
+            for (int i = 0; i < CW / 4; ++i) {
+                part[at + i] = a[i];
+                part[W * M + at + i] = b[i];
+            }
+            __syncthreads();
+            za[0] = zb[0] = 0.0f;
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                za[0] += part[w * M + tid];
+                zb[0] += part[(W + w) * M + tid];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < C::kZC; ++i) {
+                za[i] = a[i];
+                zb[i] = b[i];
+            }
+        }
+    };
+
+    load_patch(1.0f);
+    float fro2[1] = {0.0f};
+#pragma unroll
+    for (int q = 0; q < RH; ++q)
+#pragma unroll
+        for (int c = 0; c < CW / 2; ++c) {
+            const float2 t = unpack2(S[q][c]);
+            fro2[0] = fmaf(t.x, t.x, fmaf(t.y, t.y, fro2[0]));
+        }
+    slice_sum<NT>(fro2, red, phase);
+    const float fro = sqrtf(fro2[0]);
+    if (fro == 0.0f) {                                    // the same value in every thread
+        for (int i = tid; i < M; i += NT) {
+            elem<T>::store(L + ((size_t)j * M + i) * M + k, 0.0f);
+            elem<T>::store(R + ((size_t)k * M + j) * M + i, 0.0f);
+        }
+        return;
+    }
+    // scaled to Frobenius norm 1: sigma_1 is then in [1 / sqrt(m), 1] and a few steps need no normalisation
+    const float inv_fro = 1.0f / fro;
+#pragma unroll
+    for (int q = 0; q < RH; ++q)
+#pragma unroll
+        for (int c = 0; c < CW / 2; ++c) S[q][c] = fma2(S[q][c], pack2(inv_fro, inv_fro), 0);
+    for (int i = tid; i < 2 * M; i += NT) {
+        unsigned h = (unsigned)(i + 1) * 0x9E3779B1u;     // an integer hash: values in [-1, 1) without structure
+        h ^= h >> 15; h *= 0x85EBCA77u; h ^= h >> 13; h *= 0xC2B2AE3Du; h ^= h >> 16;
+        x[i] = (float)(int)h * 4.656612873e-10f;
+    }
+    slice_sync<NT>();
+
+    for (int round = 0; round < 2; ++round) {
+        bool done = round == 1;
+        float before[C::kZC] = {};
+        const int steps = round == 0 ? kPowerSteps : kPolishSteps;
+#pragma unroll 1
+        for (int step = 0; step < steps; ++step) {
+            float ya[C::kYC], yb[C::kYC], a[C::kZC], b[C::kZC];
+            times_S(x, ya);
+            times_S(x + M, yb);
+#pragma unroll
+            for (int i = 0; i < C::kYC; ++i) {
+                y[my_row + i] = ya[i];
+                y[M + my_row + i] = yb[i];
+            }
+            slice_sync<NT>();
+            back(y, y + M, a, b);
+            if ((step & 3) == 3) {
+                float v[3] = {0.0f, 0.0f, 0.0f}, d[2] = {0.0f, 0.0f};
+#pragma unroll
+                for (int i = 0; i < C::kZC; ++i) {
+                    v[0] = fmaf(a[i], a[i], v[0]);
+                    v[1] = fmaf(b[i], b[i], v[1]);
+                    v[2] = fmaf(a[i], b[i], v[2]);
+                }
+                slice_sum<NT>(v, red, phase);
+                const float na = rsqrtf(v[0] * kOnce), nb = copysignf(rsqrtf(v[1] * kOnce), v[2]);
+#pragma unroll
+                for (int i = 0; i < C::kZC; ++i) {
+                    a[i] *= na;
+                    b[i] *= nb;
+                    d[0] = fmaf(a[i] - b[i], a[i] - b[i], d[0]);
+                    d[1] = fmaf(a[i] - before[i], a[i] - before[i], d[1]);
+                    before[i] = a[i];
+                }
+                slice_sum<NT>(d, red, phase);
+                if (fmaxf(d[0], d[1]) * kOnce < kPowerTol * kPowerTol) done = true;
+            }
+#pragma unroll
+            for (int i = 0; i < C::kZC; ++i) {
+                x[my_col + i] = a[i];
+                x[M + my_col + i] = b[i];
+            }
+            slice_sync<NT>();
+            if (done && (step & 3) == 3) break;
+        }
+        if (done) break;
+
+#pragma unroll
+        for (int q = 0; q < RH; ++q)
+#pragma unroll
+            for (int c = 0; c < CW / 2; ++c) *reinterpret_cast<f32x2 *>(H + (row0 + q) * P + col0 + 2 * c) = S[q][c];
+        slice_sync<NT>();
+        const int tr = tid / C::kTC, tc = tid % C::kTC;
+        const bool on = tr < C::kTR;
+        float acc[C::kRQ * 4][C::kCQ * 4];
+        bool last = false;
+#pragma unroll 1
+        for (int sq = 0; sq <= kMaxSquarings; ++sq) {     // pass 0 forms S^T S, the others square it
+            gram_patches<M>(H, acc, on ? tr : 0, tc);
+            float trace[1] = {0.0f};
+            if (on)
+#pragma unroll
+                for (int r = 0; r < C::kRQ * 4; ++r)
+#pragma unroll
+                    for (int c = 0; c < C::kCQ * 4; ++c)
+                        if (4 * (tr + r / 4 * C::kTR) + r % 4 == 4 * (tc + c / 4 * C::kTC) + c % 4) trace[0] += acc[r][c];
+            slice_sum<NT>(trace, red, phase);
+            slice_sync<NT>();                             // the reads of H are over
+            const float scale = 1.0f / trace[0];
+            if (on)
+#pragma unroll
+                for (int r = 0; r < C::kRQ * 4; ++r)
+#pragma unroll
+                    for (int c = 0; c < C::kCQ * 4; c += 4)
+                        *reinterpret_cast<float4 *>(H + (4 * (tr + r / 4 * C::kTR) + r % 4) * P + 4 * (tc + c / 4 * C::kTC)) =
+                            make_float4(acc[r][c] * scale, acc[r][c + 1] * scale, acc[r][c + 2] * scale, acc[r][c + 3] * scale);
+            slice_sync<NT>();
+            if (last) break;
+            // trace 1 before squaring: 1 - trace(H^2) is about 2 (lambda_2 / lambda_1)^(2^sq); the next squaring squares it
+            last = sq > 0 && 1.0f - trace[0] < 1e-3f;
+        }
+        float best = -1.0f;
+        int at = 0;
+        for (int i = 0; i < M; ++i) {
+            const float d = H[i * P + i];
+            if (d > best) { best = d; at = i; }
+        }
+        for (int i = tid; i < M; i += NT) x[i] = x[M + i] = H[at * P + i];
+        load_patch(inv_fro);
+        slice_sync<NT>();
+    }
+
+    float u[C::kYC], z[C::kZC], unused[C::kZC];
+    times_S(x, u);
+    float s2[1] = {0.0f};
+#pragma unroll
+    for (int i = 0; i < C::kYC; ++i) s2[0] = fmaf(u[i], u[i], s2[0]);
+    slice_sum<NT>(s2, red, phase);
+    s2[0] *= (float)M / (NT * C::kYC);
+    const float inv_sigma = rsqrtf(s2[0]), root = sqrtf(fro * sqrtf(s2[0]));
+#pragma unroll
+    for (int i = 0; i < C::kYC; ++i) {
+        u[i] *= inv_sigma;
+        y[my_row + i] = y[M + my_row + i] = u[i];
+        elem<T>::store(L + ((size_t)j * M + my_row + i) * M + k, root * u[i]);
+    }
+    slice_sync<NT>();
+    back(y, y + M, z, unused);                            // sigma_1 v_1 of the scaled slice
+#pragma unroll
+    for (int i = 0; i < C::kZC; ++i)
+        elem<T>::store(R + ((size_t)k * M + j) * M + my_col + i, fro / root * z[i]);
+}
+
+template <typename T, int M>
+int launch_leading_pair(const void *A, void *L, void *R, cudaStream_t s)
+{
+    auto kern = leading_pair_kernel<T, M>;
+    constexpr int smem = LeadCfg<M>::kSmem;
+    if (smem > 48 * 1024) MONARCH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    kern<<<M * M, LeadCfg<M>::kThreads, smem, s>>>((const T *)A, (T *)L, (T *)R);
+    note_launch();
+    MONARCH_CUDA_TRY(cudaGetLastError());
+    return MONARCH_OK;
+}
+
+template <typename T, int M>
+int launch_project(const void *A, void *L, void *R, unsigned long long *rotations, cudaStream_t s)
+{
+    return rotations != nullptr ? launch_jacobi<T, M>(A, L, R, rotations, s) : launch_leading_pair<T, M>(A, L, R, s);
 }
 
 template <typename T>
@@ -196,11 +608,13 @@ int project_t(const void *A, void *L, void *R, int m, unsigned long long *rotati
 
 int dense_from_factors(const void *L, const void *R, void *M, int m, int dtype, cudaStream_t s)
 {
+    const int n = m * m, per = kDenseVecs * 256 * (dtype == MONARCH_F32 ? 4 : 8);
+    const dim3 grid((unsigned)m, (unsigned)(m / kDenseRows), (unsigned)((n + per - 1) / per));
     if (dtype == MONARCH_F32)
-        dense_kernel<float><<<m * m, 256, 0, s>>>((const float *)L, (const float *)R, (float *)M, m);
+        dense_kernel<float><<<grid, 256, 0, s>>>((const float *)L, (const float *)R, (float *)M, m);
     else
-        dense_kernel<__nv_bfloat16><<<m * m, 256, 0, s>>>((const __nv_bfloat16 *)L, (const __nv_bfloat16 *)R,
-                                                          (__nv_bfloat16 *)M, m);
+        dense_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>((const __nv_bfloat16 *)L, (const __nv_bfloat16 *)R,
+                                                         (__nv_bfloat16 *)M, m);
     note_launch();
     MONARCH_CUDA_TRY(cudaGetLastError());
     return MONARCH_OK;

@@ -896,6 +896,41 @@ def test_project_m128_sampled_slices(P):
         assert tail * (1 - 1e-9) <= res <= tail * (1 + 1e-5)
 
 
+@pytest.mark.parametrize("m,dtype", [(16, "f32"), (32, "f32"), (64, "f32"), (128, "f32"), (16, "bf16"), (64, "bf16")])
+@pytest.mark.parametrize("kind", ["planted", "gauss", "near", "equal", "zero"])
+def test_project_leading_pair(P, m, dtype, kind):
+    """The projection without a rotation count (power iteration, then repeated squaring where the gap is small): every
+    slice's residual is the discarded spectrum to fp32 (bf16: rounding of both factors, 2 * 2^-9 of the slice) -
+    independent of the gap, from a clear one (planted) through sigma_2 = 0.999 sigma_1 (near) to none (equal)."""
+    import torch
+    n, rng = m * m, np.random.default_rng(760 + m)
+    if kind in ("near", "equal"):
+        A4 = np.zeros((m, m, m, m), np.float32)
+        A4[np.arange(m), :, :, np.arange(m)] = 1.0                     # every slice the identity
+        if kind == "near":
+            A4[m // 2, :, :, m // 2] = 1.001 if dtype == "f32" else 1.0078125
+    else:
+        A4 = rng.standard_normal((m, m, m, m), dtype=np.float32) * np.float32({"planted": 0.5, "gauss": 1.0, "zero": 0.0}[kind])
+        if kind == "planted":
+            l, r = (rng.standard_normal((m, m, m), dtype=np.float32) for _ in range(2))
+            A4 += np.einsum("jlk,kji->ljki", l, r)
+    A32 = round_to_storage(A4.reshape(n, n), dtype)
+    A = to_device(A32, dtype)
+    Lf, L = _guarded((m, m, m), _tdtype(dtype))
+    Rf, R = _guarded((m, m, m), _tdtype(dtype))
+    P.monarch_project(A, L, R, n, m)
+    torch.cuda.synchronize()
+    _check_guard(Lf, "project L")
+    _check_guard(Rf, "project R")
+    Lg, Rg, A4 = to_host64(L), to_host64(R), A32.reshape(m, m, m, m).astype(np.float64)
+    for j, k in {(0, 0), (m - 1, m - 1), *(tuple(v) for v in rng.integers(0, m, (40, 2)))}:
+        S = A4[:, j, k, :]
+        sv = np.linalg.svd(S, compute_uv=False)
+        res, tail = float(np.sum((S - np.outer(Lg[j, :, k], Rg[k, j, :])) ** 2)), float(np.sum(sv[1:] ** 2))
+        rounding = (2 * 2.0 ** -9 * sv[0]) ** 2 if dtype == "bf16" else 0.0
+        assert tail * (1 - 1e-9) <= res <= tail * (1 + 1e-5) + rounding + (1e-6 * sv[0]) ** 2
+
+
 # ----------------------------------------------------------------- the five workloads
 
 def _sample_tokens(T, count, seed):
