@@ -1,0 +1,790 @@
+// Whole calls as one cooperative launch over "units" of block products (block_units.cu): the device code shared by the
+// calls.  A call is a list of operations in phases; a phase's operations are cut into units that depend on nothing in
+// the same phase, every CTA runs its share, and a grid barrier separates the phases.
+//
+// A unit of a stage is TT tokens x 8 neighbouring blocks x ES outputs of each block, one warp per block.  Eight blocks
+// because the permutation P turns "block b, output e" into column e*m + b: eight blocks make 16 bytes (bf16) or 32
+// bytes (fp32) of consecutive columns, so the permuted side is read and written in such pieces and re-ordered in
+// shared memory.  The intermediates u, du between two stages are private to the library and are kept as
+// mid[j/8][t][k][j%8], which both sides read and write in full lines.
+//
+// What bounds them: at a few tokens the chain of latencies of a phase (barrier, input from L2, product, result: 4 us
+// per phase with the cold instruction fetches), which is why a phase's weights are fetched before its barrier; at many
+// tokens the warps' issue of shared-memory accesses and legacy-shaped MMAs (ncu at 4096 tokens, m = 64: LSU data pipe
+// 52 %, issue 29 %), which is why the tcgen05 kernels take over there.  One CTA of 16 warps with a two-deep pipeline was
+// no faster at any size than two CTAs of 8 warps whose loads overlap the other's work (23 against 27 us at 1000 tokens),
+// and starting the permuted loads early cost spills (31 us).
+#pragma once
+
+#include <type_traits>
+
+#include "common.cuh"
+
+namespace monarch {
+namespace units {
+
+typedef __nv_bfloat16 bf16;
+
+// What an operation does.  Roles of a tensor: kNat - block b is the major index of the row (columns b*m + c);
+// kPerm - block b is the minor index (columns c*m + b).
+enum Kind : int { kStage = 0, kWgrad = 1, kReduce = 2, kColsum = 3 };
+enum Act : int { kNone = 0, kGelu = 1, kGeluGrad = 2 };
+
+// How the pieces of 8 elements of a tensor are addressed, in pieces (32 bits: at most 2^20 tokens of 16384 elements):
+// kNat: t * t_stride + b * b_stride + (c / 8) * c_stride;  kPerm: t * t_stride + (b / 8) * b_stride + c * c_stride.
+struct View {
+    void *p;
+    unsigned t_stride, b_stride, c_stride;
+    int mid;                 // the intermediate layout (decides which pieces are neighbours in memory)
+};
+
+struct Op {
+    int kind, phase;
+    int perm;                // role of the blocks in this operation's tensors
+    int trans;               // stage: multiply by the transposed blocks
+    int act, accumulate;
+    int splits;              // wgrad: token ranges; > 1 leaves partial sums; reduce: number of parts
+    View in, out;            // stage: input, output; wgrad: operand whose columns index the rows of the result; colsum: in
+    View in2;                // wgrad: the other operand; stage: kGelu - where to leave the pre-activation (p may be
+                             // null); kGeluGrad - the pre-activation
+    const void *w;           // stage: weights [block][out][in]
+    const void *bias;        // stage: bias by column or null
+    float *sums;             // wgrad / reduce / colsum: result; stage with kGeluGrad: column sums per token tile
+    const float *parts;      // reduce: parts, `count` apart
+    long long count;         // reduce: elements
+};
+
+constexpr int kMaxOps = 18;
+struct Params {
+    Op op[kMaxOps];
+    int n_ops, n_phases;
+    int tokens;
+    unsigned *status;        // [0] status word, [1] wait limit, [8] grid barrier, [9] CTAs done
+};
+
+constexpr int kBarrierWord = 8, kDoneWord = 9;
+constexpr unsigned kErrGridWait = 0x301;
+
+template <typename T_, int M_, int TT_, int ES_, int LS_, int KS_> struct Cfg {
+    typedef T_ T;
+    static constexpr int M = M_, TT = TT_, ES = ES_, LS = LS_, KS = KS_, G = 8;
+    static constexpr bool kBf = std::is_same<T, bf16>::value;
+    static constexpr int kWpb = 1, kThreads = 32 * G * kWpb;
+    static constexpr int EW = ES / kWpb, KW = KS / kWpb;      // outputs / gradient columns of one warp
+    static constexpr int kPad = kBf ? 8 : 4;                  // rows 16 bytes longer: conflict-free ldmatrix / 16-byte reads
+    static constexpr int PA = M + kPad, PE = ES + kPad, PL = LS + kPad, PK = KS + kPad;
+    static constexpr int TW = 32;                             // tokens per step of a weight gradient
+    static constexpr int cmax(int a, int b) { return a > b ? a : b; }
+    // staging of results: permuted role - one plane of words per pair of bf16 blocks (per fp32 block), pitch 8 mod 32;
+    // natural role - rows of ES outputs and rows of 8 blocks, each 16 bytes longer
+    static constexpr int PS = ES + (40 - ES % 32) % 32, kPlanes = kBf ? G / 2 : G;
+    static constexpr int kNatB = ES * (int)sizeof(T) + 16, kNatT = G * kNatB + 16;
+    static constexpr int kStageBytes = cmax(kPlanes * TT * PS * 4, TT * kNatT);
+    static constexpr int kTileBytes = G * TT * PA * (int)sizeof(T);
+    static constexpr int kWBytes = cmax(G * ES * PA, kBf ? G * M * PE : 0) * (int)sizeof(T);
+    static constexpr int kStepBytes = G * TW * (PL + PK) * (int)sizeof(T);
+    // Two CTAs per SM work on different units while each waits for its own loads.  Within that share of shared memory: two
+    // tiles (the next unit's input is on its way during this one's work), or one, or one that the results are staged over.
+    static constexpr int kHalf = 113 * 1024 - 512;
+    static constexpr int kBufs = 2 * kTileBytes + kWBytes + kStageBytes <= kHalf ? 2 : 1;
+    static constexpr bool kAlias = kTileBytes + kWBytes + kStageBytes > kHalf;
+    static constexpr int kWAt = kAlias ? cmax(kTileBytes, kStageBytes) : kBufs * kTileBytes, kStageAt = kAlias ? 0 : kWAt + kWBytes;
+    static constexpr int kStageSmem = kAlias ? kWAt + kWBytes : kStageAt + kStageBytes;
+    static constexpr int kSteps = 2 * kStepBytes <= cmax(kStageSmem, kHalf) ? 2 : 1;   // buffers of a weight gradient
+    static constexpr int kSmem = cmax(kStageSmem, kSteps * kStepBytes);
+    static constexpr int kCtas = kSmem <= kHalf ? 2 : 1;
+};
+
+// ---------------------------------------------------------------- small device helpers
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool valid)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void *p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm4_trans(uint32_t (&r)[4], const void *p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)) : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t pack2bf(float lo, float hi)
+{
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+template <typename T> struct Math;
+template <> struct Math<bf16> {
+    static __device__ __forceinline__ float gelu(float a) { return gelu_fast(a); }
+    static __device__ __forceinline__ float grad(float a) { return gelu_fast_grad(a); }
+};
+template <> struct Math<float> {
+    static __device__ __forceinline__ float gelu(float a) { return gelu_erf(a); }
+    static __device__ __forceinline__ float grad(float a) { return gelu_erf_grad(a); }
+};
+
+// ---------------------------------------------------------------- loads into shared memory
+// tile[b][t][c - 8 c8]: 8 blocks from b0 on, R tokens from t0 on (zeros past the last), NC columns from 8*c8 on.  begin()
+// starts the transfer; end() finishes what goes through registers (the permuted role, which has to be re-ordered);
+// afterwards cp_async_wait() and a barrier.
+template <typename C, int R, int NC, int PITCH> struct TileLoad {
+    typedef typename C::T T;
+    static constexpr int kThreads = C::kThreads, H = (int)sizeof(T) / 2;         // 16-byte accesses per piece
+    static constexpr int kTasks = R * NC / 2, U = (kTasks + kThreads - 1) / kThreads;
+    uint4 lo[U][H], hi[U][H];
+
+    // `left`: tokens from t0 on
+    __device__ __forceinline__ void begin(T *tile, const View &v, int perm, int b0, int c8, int t0, int left)
+    {
+        const uint4 *src = static_cast<const uint4 *>(v.p);
+        if (!perm) {
+            constexpr int kPieces = R * NC;            // per token: 8 blocks x NC / 8
+            const unsigned first = t0 * v.t_stride + b0 * v.b_stride + c8 * v.c_stride;
+#pragma unroll 4
+            for (int i = threadIdx.x; i < kPieces; i += kThreads) {
+                int b, c;
+                if (v.mid) { b = i % 8; c = i / 8 % (NC / 8); }
+                else       { c = i % (NC / 8); b = i / (NC / 8) % 8; }
+                const int t = i / NC;
+                const bool ok = t < left;
+                const uint4 *g = src + (size_t)(first + (ok ? t : 0) * v.t_stride + b * v.b_stride + c * v.c_stride) * H;
+                T *d = tile + (b * R + t) * PITCH + c * 8;
+                cp_async16(d, g, ok);
+                if (H == 2) cp_async16(d + 4, g + 1, ok);
+            }
+            return;
+        }
+        // pieces of 8 blocks: two columns per thread and task, so that bf16 is stored as pairs (a word of shared memory)
+        const unsigned first = t0 * v.t_stride + b0 / 8 * v.b_stride + c8 * 8 * v.c_stride;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = u * kThreads + threadIdx.x, c = i % (NC / 2) * 2, t = i / (NC / 2);
+            const bool ok = t < R && t < left;
+            const unsigned g = first + (ok ? t : 0) * v.t_stride + c * v.c_stride;
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                lo[u][h] = ok ? src[(size_t)g * H + h] : make_uint4(0, 0, 0, 0);
+                hi[u][h] = ok ? src[(size_t)(g + v.c_stride) * H + h] : make_uint4(0, 0, 0, 0);
+            }
+        }
+    }
+    __device__ __forceinline__ void end(T *tile, int perm)
+    {
+        if (!perm) return;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = u * kThreads + threadIdx.x, c = i % (NC / 2) * 2, t = i / (NC / 2);
+            if (t >= R) break;
+            T *d = tile + t * PITCH + c;
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const uint32_t a[4] = {lo[u][h].x, lo[u][h].y, lo[u][h].z, lo[u][h].w};
+                const uint32_t b[4] = {hi[u][h].x, hi[u][h].y, hi[u][h].z, hi[u][h].w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if constexpr (H == 1) {
+                        *reinterpret_cast<uint32_t *>(d + (2 * q) * R * PITCH) = __byte_perm(a[q], b[q], 0x5410);
+                        *reinterpret_cast<uint32_t *>(d + (2 * q + 1) * R * PITCH) = __byte_perm(a[q], b[q], 0x7632);
+                    } else {
+                        *reinterpret_cast<uint2 *>(d + (4 * h + q) * R * PITCH) = make_uint2(a[q], b[q]);
+                    }
+                }
+            }
+        }
+    }
+};
+
+// rows e0 .. e0 + ES of the result of 8 blocks: bf16 keeps the storage order (ldmatrix transposes), fp32 is stored
+// [b][e][c] either way
+template <typename C>
+__device__ __forceinline__ void load_weights(typename C::T *wt, const void *w, int trans, int b0, int e0)
+{
+    typedef typename C::T T;
+    constexpr int M = C::M, ES = C::ES, V = 16 / (int)sizeof(T);
+    const T *src = static_cast<const T *>(w) + (size_t)b0 * M * M;
+    if (!trans) {
+        constexpr int kVecs = 8 * ES * (M / V);
+#pragma unroll 4
+        for (int i = threadIdx.x; i < kVecs; i += C::kThreads) {
+            const int c = i % (M / V) * V, e = i / (M / V) % ES, b = i / (M / V * ES);
+            cp_async16(wt + (b * ES + e) * C::PA + c, src + ((size_t)b * M + e0 + e) * M + c, true);
+        }
+    } else if constexpr (C::kBf) {
+        constexpr int kVecs = 8 * M * (ES / V);
+#pragma unroll 4
+        for (int i = threadIdx.x; i < kVecs; i += C::kThreads) {
+            const int e = i % (ES / V) * V, c = i / (ES / V) % M, b = i / (ES / V * M);
+            cp_async16(wt + (b * M + c) * C::PE + e, src + ((size_t)b * M + c) * M + e0 + e, true);
+        }
+    } else {
+        constexpr int kVecs = 8 * M * (ES / V);
+#pragma unroll 4
+        for (int i = threadIdx.x; i < kVecs; i += C::kThreads) {
+            const int c = i % M, e = i / M % (ES / V) * V, b = i / (ES / V * M);
+            const float4 f = *reinterpret_cast<const float4 *>(src + ((size_t)b * M + c) * M + e0 + e);
+            float *d = reinterpret_cast<float *>(wt) + (b * ES + e) * C::PA + c;
+            d[0] = f.x; d[C::PA] = f.y; d[2 * C::PA] = f.z; d[3 * C::PA] = f.w;
+        }
+    }
+}
+
+// ---------------------------------------------------------------- results of a stage unit
+// Accumulators of one warp (TT tokens, EW outputs of its block), visited with their token and output numbers.
+template <typename C, bool BF = C::kBf> struct Acc;
+template <typename C> struct Acc<C, true> {
+    float v[C::TT / 16][C::EW / 8][4];
+    template <typename F> __device__ __forceinline__ void each(F f)
+    {
+        const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
+#pragma unroll
+        for (int mt = 0; mt < C::TT / 16; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < C::EW / 8; ++nt)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) f(v[mt][nt][r], mt * 16 + g + (r >> 1) * 8, nt * 8 + 2 * q + (r & 1));
+    }
+    // f(sum over the tile's tokens, output) in one lane per output
+    template <typename F> __device__ __forceinline__ void column_sums(F f)
+    {
+        const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
+#pragma unroll
+        for (int nt = 0; nt < C::EW / 8; ++nt)
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                float s = 0.0f;
+#pragma unroll
+                for (int mt = 0; mt < C::TT / 16; ++mt) s += v[mt][nt][p] + v[mt][nt][p + 2];
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (g == 0) f(s, nt * 8 + 2 * q + p);
+            }
+    }
+};
+template <typename C> struct Acc<C, false> {
+    float v[C::TT / 4][C::EW / 8];
+    template <typename F> __device__ __forceinline__ void each(F f)
+    {
+        const int tl = (threadIdx.x & 31) >> 3, el = threadIdx.x & 7;
+#pragma unroll
+        for (int i = 0; i < C::TT / 4; ++i)
+#pragma unroll
+            for (int q = 0; q < C::EW / 8; ++q) f(v[i][q], tl + 4 * i, el + 8 * q);
+    }
+    template <typename F> __device__ __forceinline__ void column_sums(F f)
+    {
+        const int tl = (threadIdx.x & 31) >> 3, el = threadIdx.x & 7;
+#pragma unroll
+        for (int q = 0; q < C::EW / 8; ++q) {
+            float s = 0.0f;
+#pragma unroll
+            for (int i = 0; i < C::TT / 4; ++i) s += v[i][q];
+            s += __shfl_xor_sync(0xffffffffu, s, 8);
+            s += __shfl_xor_sync(0xffffffffu, s, 16);
+            if (tl == 0) f(s, el + 8 * q);
+        }
+    }
+};
+
+__device__ __forceinline__ uint32_t f2w(float x) { return __float_as_uint(x); }
+
+// Accumulators -> storage type -> staging in shared memory (stage_results), then, after a barrier, staging -> global
+// memory in pieces of 8 elements (copy_out).  The permuted role needs the 8 blocks of one (token, output) side by side,
+// one value from each warp: hence the planes, whose pitch keeps both sides free of bank conflicts.
+template <typename C> __device__ __forceinline__ void stage_results(Acc<C> &acc, unsigned char *stage, int perm)
+{
+    const int w = threadIdx.x >> 5, b = w / C::kWpb, e0 = w % C::kWpb * C::EW;
+    if (!perm) {
+        if constexpr (C::kBf) {
+            const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
+#pragma unroll
+            for (int mt = 0; mt < C::TT / 16; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < C::EW / 8; ++nt)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        *reinterpret_cast<uint32_t *>(stage + (mt * 16 + g + 8 * h) * C::kNatT + b * C::kNatB + (e0 + nt * 8 + 2 * q) * 2) =
+                            pack2bf(acc.v[mt][nt][2 * h], acc.v[mt][nt][2 * h + 1]);
+        } else {
+            acc.each([&](float v, int t, int e) { *reinterpret_cast<float *>(stage + t * C::kNatT + b * C::kNatB + (e0 + e) * 4) = v; });
+        }
+    } else if constexpr (C::kBf) {
+        acc.each([&](float v, int t, int e) {
+            reinterpret_cast<bf16 *>(stage)[(((b >> 1) * C::TT + t) * C::PS + e0 + e) * 2 + (b & 1)] = __float2bfloat16_rn(v);
+        });
+    } else {
+        acc.each([&](float v, int t, int e) { reinterpret_cast<float *>(stage)[(b * C::TT + t) * C::PS + e0 + e] = v; });
+    }
+}
+
+template <typename C>
+__device__ __forceinline__ void copy_out(const unsigned char *stage, const View &out, int perm, int b0, int e0, int t0, int left)
+{
+    typedef typename C::T T;
+    constexpr int H = (int)sizeof(T) / 2;
+    uint4 *dst = static_cast<uint4 *>(out.p);
+    constexpr int kPieces = C::TT * C::ES;             // natural: per token 8 blocks x ES / 8; permuted: ES
+    if (!perm) {
+        const unsigned first = t0 * out.t_stride + b0 * out.b_stride + e0 / 8 * out.c_stride;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < kPieces; i += C::kThreads) {
+            int b, c;
+            if (out.mid) { b = i % 8; c = i / 8 % (C::ES / 8); }
+            else         { c = i % (C::ES / 8); b = i / (C::ES / 8) % 8; }
+            const int t = i / C::ES;
+            if (t >= left) break;
+            const uint4 *s = reinterpret_cast<const uint4 *>(stage + t * C::kNatT + b * C::kNatB + c * 8 * sizeof(T));
+            uint4 *d = dst + (size_t)(first + t * out.t_stride + b * out.b_stride + c * out.c_stride) * H;
+            d[0] = s[0];
+            if (H == 2) d[1] = s[1];
+        }
+        return;
+    }
+    const unsigned first = t0 * out.t_stride + b0 / 8 * out.b_stride + e0 * out.c_stride;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < kPieces; i += C::kThreads) {
+        const int e = i % C::ES, t = i / C::ES;
+        if (t >= left) break;
+        const uint32_t *s = reinterpret_cast<const uint32_t *>(stage) + t * C::PS + e;
+        uint4 *d = dst + (size_t)(first + t * out.t_stride + e * out.c_stride) * H;
+        constexpr int kPlane = C::TT * C::PS;
+        d[0] = make_uint4(s[0], s[kPlane], s[2 * kPlane], s[3 * kPlane]);
+        if constexpr (!C::kBf) d[1] = make_uint4(s[4 * kPlane], s[5 * kPlane], s[6 * kPlane], s[7 * kPlane]);
+    }
+}
+
+// ---------------------------------------------------------------- a stage unit
+template <typename C>
+__device__ __forceinline__ void multiply(Acc<C> &acc, const typename C::T *tile, const typename C::T *wt, int trans)
+{
+    constexpr int M = C::M, TT = C::TT, ES = C::ES, EW = C::EW;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, b = w / C::kWpb, e0 = w % C::kWpb * EW;
+    if constexpr (C::kBf) {
+#pragma unroll
+        for (int mt = 0; mt < TT / 16; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < EW / 8; ++nt)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) acc.v[mt][nt][r] = 0.0f;
+        const bf16 *a = tile + (b * TT + (lane & 15)) * C::PA + (lane >> 4) * 8;
+        // with 8 outputs per warp one ldmatrix brings two steps of the contraction, otherwise two groups of 8 outputs
+        constexpr bool kPair = EW >= 16;
+        const bf16 *bn = wt + (b * ES + e0 + (lane & 7) + (kPair ? (lane >> 4) * 8 : 0)) * C::PA + (kPair ? lane >> 3 & 1 : lane >> 3) * 8;
+        const bf16 *bt = wt + (b * M + (kPair ? lane & 15 : lane)) * C::PE + e0 + (kPair ? (lane >> 4) * 8 : 0);
+        uint32_t keep[2];
+#pragma unroll
+        for (int ks = 0; ks < M / 16; ++ks) {
+            uint32_t fa[TT / 16][4];
+#pragma unroll
+            for (int mt = 0; mt < TT / 16; ++mt) ldsm4(fa[mt], a + mt * 16 * C::PA + ks * 16);
+            if constexpr (kPair) {
+#pragma unroll
+                for (int np = 0; np < EW / 16; ++np) {
+                    uint32_t fb[4];
+                    if (trans) ldsm4_trans(fb, bt + ks * 16 * C::PE + np * 16);
+                    else       ldsm4(fb, bn + np * 16 * C::PA + ks * 16);
+#pragma unroll
+                    for (int mt = 0; mt < TT / 16; ++mt) {
+                        mma16816(acc.v[mt][2 * np], fa[mt], fb[0], fb[1]);
+                        mma16816(acc.v[mt][2 * np + 1], fa[mt], fb[2], fb[3]);
+                    }
+                }
+            } else if constexpr (M == 16) {            // a single step: both halves of the lanes fetch the same 16 columns
+                uint32_t fb[4];
+                if (trans) ldsm4_trans(fb, wt + (b * M + (lane & 15)) * C::PE + e0);
+                else       ldsm4(fb, wt + (b * ES + e0 + (lane & 7)) * C::PA + (lane >> 3 & 1) * 8);
+#pragma unroll
+                for (int mt = 0; mt < TT / 16; ++mt) mma16816(acc.v[mt][0], fa[mt], fb[0], fb[1]);
+            } else {
+                uint32_t b0 = keep[0], b1 = keep[1];
+                if (ks % 2 == 0) {
+                    uint32_t fb[4];
+                    if (trans) ldsm4_trans(fb, bt + ks * 16 * C::PE);
+                    else       ldsm4(fb, bn + ks * 16);
+                    b0 = fb[0];
+                    b1 = fb[1];
+                    keep[0] = fb[2];
+                    keep[1] = fb[3];
+                }
+#pragma unroll
+                for (int mt = 0; mt < TT / 16; ++mt) mma16816(acc.v[mt][0], fa[mt], b0, b1);
+            }
+        }
+    } else {
+        // two partial sums per result (even and odd columns), packed for fma.rn.f32x2
+        const float *a = tile + (b * TT + (lane >> 3)) * C::PA, *bw = wt + (b * ES + e0 + (lane & 7)) * C::PA;
+        f32x2 s[TT / 4][EW / 8];
+#pragma unroll
+        for (int i = 0; i < TT / 4; ++i)
+#pragma unroll
+            for (int q = 0; q < EW / 8; ++q) s[i][q] = 0;
+#pragma unroll 2
+        for (int c = 0; c < M; c += 4) {
+            ulonglong2 fb[EW / 8];
+#pragma unroll
+            for (int q = 0; q < EW / 8; ++q) fb[q] = *reinterpret_cast<const ulonglong2 *>(bw + 8 * q * C::PA + c);
+#pragma unroll
+            for (int i = 0; i < TT / 4; ++i) {
+                const ulonglong2 fa = *reinterpret_cast<const ulonglong2 *>(a + 4 * i * C::PA + c);
+#pragma unroll
+                for (int q = 0; q < EW / 8; ++q) s[i][q] = fma2(fa.y, fb[q].y, fma2(fa.x, fb[q].x, s[i][q]));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < TT / 4; ++i)
+#pragma unroll
+            for (int q = 0; q < EW / 8; ++q) {
+                const float2 t = unpack2(s[i][q]);
+                acc.v[i][q] = t.x + t.y;
+            }
+    }
+}
+
+// Units i0 .. i1 of a stage, in order: (8 blocks, ES outputs) major, token tile minor.  `held`: whose weights are in
+// shared memory.
+template <typename C>
+__device__ __forceinline__ void stage_units(const Op &op, int i0, int i1, int tiles, int tokens, unsigned char *smem, int &held)
+{
+    typedef typename C::T T;
+    constexpr int M = C::M, N = M * M, kSlices = M / C::ES;
+    T *wt = reinterpret_cast<T *>(smem + C::kWAt);
+    unsigned char *stage = smem + C::kStageAt;
+    const int w = threadIdx.x >> 5;
+    TileLoad<C, C::TT, M, C::PA> load;
+    int at = i0 / tiles, tile_no = i0 % tiles, buf = 0;
+    __syncthreads();                                   // what ran before has left shared memory
+    if (held != at) {
+        load_weights<C>(wt, op.w, op.trans, at / kSlices * 8, at % kSlices * C::ES);
+        held = at;
+    }
+    load.begin(reinterpret_cast<T *>(smem), op.in, op.perm, at / kSlices * 8, 0, tile_no * C::TT, tokens - tile_no * C::TT);
+    load.end(reinterpret_cast<T *>(smem), op.perm);
+    for (int i = i0; i < i1; ++i) {
+        const int b0 = at / kSlices * 8, e0 = at % kSlices * C::ES;
+        const int t0 = tile_no * C::TT, left = tokens - t0, this_tile = tile_no;
+        T *tile = reinterpret_cast<T *>(smem + buf * C::kTileBytes);
+        const bool more = i + 1 < i1;
+        if (++tile_no == tiles) { tile_no = 0; ++at; }
+        if (C::kBufs == 2) buf ^= 1;
+        T *next = reinterpret_cast<T *>(smem + buf * C::kTileBytes);
+        cp_async_wait();
+        __syncthreads();                               // tile and weights are here; the last results have been copied out
+        // (what goes through registers starts late: held across the product it would cost more than it hides)
+        const bool early = more && C::kBufs == 2 && !op.perm;
+        if (early) load.begin(next, op.in, op.perm, at / kSlices * 8, 0, tile_no * C::TT, tokens - tile_no * C::TT);
+        Acc<C> acc;
+        multiply<C>(acc, tile, wt, op.trans);
+        const int b = b0 + w / C::kWpb, ew = e0 + w % C::kWpb * C::EW;
+        if (op.bias != nullptr) {
+            const T *bias = static_cast<const T *>(op.bias);
+            acc.each([&](float &v, int, int e) { v += elem<T>::load(bias + (op.perm ? (ew + e) * M + b : b * M + ew + e)); });
+        }
+        if (C::kAlias) __syncthreads();                // every warp is done with the tile
+        if (op.act == kGelu) {
+            if (op.in2.p != nullptr) {
+                stage_results<C>(acc, stage, op.perm);
+                __syncthreads();
+                copy_out<C>(stage, op.in2, op.perm, b0, e0, t0, left);
+                __syncthreads();
+            }
+            acc.each([&](float &v, int, int) { v = Math<T>::gelu(v); });
+        } else if (op.act == kGeluGrad) {
+            const T *a = static_cast<const T *>(op.in2.p);
+            acc.each([&](float &v, int t, int e) {
+                if (t < left) v *= Math<T>::grad(elem<T>::load(a + (size_t)(t0 + t) * N + b * M + ew + e));
+            });
+            acc.column_sums([&](float s, int e) { op.sums[(size_t)this_tile * N + b * M + ew + e] = s; });
+        }
+        stage_results<C>(acc, stage, op.perm);
+        __syncthreads();                               // results staged; nobody reads the tile or the weights any more
+        if (more) {
+            if (held != at) {
+                load_weights<C>(wt, op.w, op.trans, at / kSlices * 8, at % kSlices * C::ES);
+                held = at;
+            }
+            if (!early && !C::kAlias) load.begin(next, op.in, op.perm, at / kSlices * 8, 0, tile_no * C::TT, tokens - tile_no * C::TT);
+        }
+        copy_out<C>(stage, op.out, op.perm, b0, e0, t0, left);
+        if (C::kAlias && more) {
+            __syncthreads();                           // the staged results have been read
+            if (!early) load.begin(next, op.in, op.perm, at / kSlices * 8, 0, tile_no * C::TT, tokens - tile_no * C::TT);
+        }
+        if (more) load.end(next, op.perm);
+    }
+}
+
+// ---------------------------------------------------------------- a weight-gradient unit
+// sums[b][l][k] = sum over a range of tokens of in[t](b, l) in2[t](b, k), for 8 blocks, LS rows and KS columns
+template <typename C>
+__device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0, int split, int tokens, unsigned char *smem)
+{
+    typedef typename C::T T;
+    constexpr int M = C::M, LS = C::LS, KS = C::KS, KW = C::KW, TW = C::TW;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, bw = w / C::kWpb, kw = w % C::kWpb * KW;
+    const int steps = (tokens + TW - 1) / TW, per = (steps + op.splits - 1) / op.splits;
+    const int s0 = split * per, s1 = s0 + per < steps ? s0 + per : steps;
+    float *dst = op.sums + (op.splits > 1 ? (size_t)split * M * M * M : 0) + (size_t)(b0 + bw) * M * M + (size_t)l0 * M + k0 + kw;
+    const bool add = op.splits == 1 && op.accumulate;
+    constexpr int kMask = C::kSteps - 1;
+    TileLoad<C, TW, LS, C::PL> load_a;
+    TileLoad<C, TW, KS, C::PK> load_b;
+    auto tile_a = [&](int buf) { return reinterpret_cast<T *>(smem + buf * C::kStepBytes); };
+    auto tile_b = [&](int buf) { return tile_a(buf) + C::G * TW * C::PL; };
+    // the operand of the natural role is asynchronous; the other goes through registers, one operand after the other
+    auto load = [&](int s) {
+        load_a.begin(tile_a(s & kMask), op.in, op.perm, b0, l0 / 8, s * TW, tokens - s * TW);
+        load_a.end(tile_a(s & kMask), op.perm);
+        load_b.begin(tile_b(s & kMask), op.in2, op.perm, b0, k0 / 8, s * TW, tokens - s * TW);
+        load_b.end(tile_b(s & kMask), op.perm);
+    };
+    constexpr int RL = LS / 4, RK = KW / 8;            // fp32: rows and columns of a lane
+    float acc[C::kBf ? LS / 16 : RL][C::kBf ? KW / 8 : RK][C::kBf ? 4 : 1] = {};
+
+    __syncthreads();                                   // what ran before has left shared memory
+    if (s0 < s1) load(s0);
+#pragma unroll 1
+    for (int s = s0; s < s1; ++s) {
+        cp_async_wait();
+        __syncthreads();                               // the operands of s are here, those of s - 1 have been read
+        const bool early = C::kSteps == 2 && !op.perm;
+        if (early && s + 1 < s1) load(s + 1);
+        if constexpr (C::kBf) {
+            const bf16 *a = tile_a(s & kMask) + (bw * TW + (lane & 7) + (lane >> 4) * 8) * C::PL + (lane >> 3 & 1) * 8;
+            // with 8 columns per warp one ldmatrix brings both 16-token steps
+            constexpr bool kPair = KW >= 16;
+            const bf16 *b = tile_b(s & kMask) + (bw * TW + (kPair ? lane & 15 : lane)) * C::PK + kw + (kPair ? (lane >> 4) * 8 : 0);
+            uint32_t fb[4];
+            if (!kPair) ldsm4_trans(fb, b);
+#pragma unroll
+            for (int ks = 0; ks < TW / 16; ++ks) {
+                uint32_t fa[LS / 16][4];
+#pragma unroll
+                for (int mt = 0; mt < LS / 16; ++mt) ldsm4_trans(fa[mt], a + ks * 16 * C::PL + mt * 16);
+                if constexpr (kPair) {
+#pragma unroll
+                    for (int np = 0; np < KW / 16; ++np) {
+                        ldsm4_trans(fb, b + ks * 16 * C::PK + np * 16);
+#pragma unroll
+                        for (int mt = 0; mt < LS / 16; ++mt) {
+                            mma16816(acc[mt][2 * np], fa[mt], fb[0], fb[1]);
+                            mma16816(acc[mt][2 * np + 1], fa[mt], fb[2], fb[3]);
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int mt = 0; mt < LS / 16; ++mt) mma16816(acc[mt][0], fa[mt], fb[2 * ks], fb[2 * ks + 1]);
+                }
+            }
+        } else {
+            const float *a = tile_a(s & kMask) + bw * TW * C::PL + (lane >> 3) * RL, *b = tile_b(s & kMask) + bw * TW * C::PK + (lane & 7) * RK;
+#pragma unroll 4
+            for (int t = 0; t < TW; ++t) {
+                float fa[RL], fb[RK];
+#pragma unroll
+                for (int i = 0; i < RL; i += 4) *reinterpret_cast<float4 *>(fa + i) = *reinterpret_cast<const float4 *>(a + t * C::PL + i);
+#pragma unroll
+                for (int i = 0; i < RK; i += 2) *reinterpret_cast<float2 *>(fb + i) = *reinterpret_cast<const float2 *>(b + t * C::PK + i);
+#pragma unroll
+                for (int i = 0; i < RL; ++i)
+#pragma unroll
+                    for (int k = 0; k < RK; ++k) acc[i][k][0] = fmaf(fa[i], fb[k], acc[i][k][0]);
+            }
+        }
+        if (!early && s + 1 < s1) {
+            if (C::kSteps == 1) __syncthreads();
+            load(s + 1);
+        }
+    }
+    if constexpr (C::kBf) {
+        const int g = lane >> 2, q = lane & 3;
+#pragma unroll
+        for (int mt = 0; mt < LS / 16; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < KW / 8; ++nt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float2 *d = reinterpret_cast<float2 *>(dst + (mt * 16 + g + 8 * h) * M + nt * 8 + 2 * q);
+                    float2 r = make_float2(acc[mt][nt][2 * h], acc[mt][nt][2 * h + 1]);
+                    if (add) { const float2 o = *d; r.x += o.x; r.y += o.y; }
+                    *d = r;
+                }
+    } else {
+#pragma unroll
+        for (int i = 0; i < RL; ++i)
+#pragma unroll
+            for (int k = 0; k < RK; ++k) {
+                float *d = dst + ((lane >> 3) * RL + i) * M + (lane & 7) * RK + k;
+                *d = add ? *d + acc[i][k][0] : acc[i][k][0];
+            }
+    }
+}
+
+// ---------------------------------------------------------------- sums
+constexpr int kReducePer = 1024;                       // elements of a reduce unit
+__device__ __forceinline__ void reduce_unit(const Op &op, int unit)
+{
+    const long long i = (long long)unit * kReducePer + threadIdx.x * 4;
+    if (threadIdx.x * 4 >= kReducePer || i >= op.count) return;
+    float4 s = op.accumulate ? *reinterpret_cast<const float4 *>(op.sums + i) : make_float4(0, 0, 0, 0);
+#pragma unroll 4
+    for (int p = 0; p < op.splits; ++p) {
+        const float4 v = *reinterpret_cast<const float4 *>(op.parts + p * op.count + i);
+        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    *reinterpret_cast<float4 *>(op.sums + i) = s;
+}
+
+constexpr int kColsumCols = 64;                        // columns of a column-sum unit
+template <typename C> __device__ __forceinline__ void colsum_unit(const Op &op, int unit, int tokens, unsigned char *smem)
+{
+    typedef typename C::T T;
+    constexpr int N = C::M * C::M, V = 16 / (int)sizeof(T), kLanes = kColsumCols / V, kRows = C::kThreads / kLanes;
+    const int cl = threadIdx.x % kLanes, r = threadIdx.x / kLanes;
+    const T *src = static_cast<const T *>(op.in.p) + unit * kColsumCols + cl * V;
+    float s[V] = {};
+#pragma unroll 4
+    for (int t = r; t < tokens; t += kRows) {
+        const uint4 raw = *reinterpret_cast<const uint4 *>(src + (size_t)t * N);
+#pragma unroll
+        for (int e = 0; e < V; ++e) s[e] += elem<T>::load(reinterpret_cast<const T *>(&raw) + e);
+    }
+    float *red = reinterpret_cast<float *>(smem);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < V; ++e) red[r * kColsumCols + cl * V + e] = s[e];
+    __syncthreads();
+    if (threadIdx.x < kColsumCols) {
+        float v = 0.0f;
+        for (int q = 0; q < kRows; ++q) v += red[q * kColsumCols + threadIdx.x];
+        float *d = op.sums + unit * kColsumCols + threadIdx.x;
+        *d = op.accumulate ? *d + v : v;
+    }
+}
+
+// ---------------------------------------------------------------- the launch
+struct Plan {                                          // shares of the CTAs, worked out on the host
+    int units[kMaxOps], shift[kMaxOps];                // of an operation: units, and log2 of the weight of one
+    long long share[kMaxOps], rest[kMaxOps];           // of a phase: total weight / and mod the number of CTAs
+};
+
+// Every CTA of the grid has arrived: all are resident (cooperative launch).  Bounded like every wait of the library.
+__device__ __forceinline__ bool grid_barrier(unsigned *status, unsigned target, volatile int *dead)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(status + kBarrierWord, 1u);
+        unsigned long long t0 = 0;
+        for (unsigned spin = 0;; ++spin) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(status + kBarrierWord) : "memory");
+            if (v >= target) break;
+            if ((spin & 1023) == 1023) {
+                unsigned long long now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                if (t0 == 0) t0 = now;
+                const unsigned us = reinterpret_cast<volatile unsigned *>(status)[1];
+                if (now - t0 > (us ? us * 1000ull : 1000000000ull)) {
+                    *dead = 1;
+                    atomicCAS(status, 0u, kErrGridWait);
+                    break;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    return *dead == 0;
+}
+
+template <typename C>
+__global__ void __launch_bounds__(C::kThreads, C::kCtas) units_kernel(const __grid_constant__ Params p, const __grid_constant__ Plan plan)
+{
+    constexpr int M = C::M;
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ int dead;
+    if (threadIdx.x == 0) dead = 0;
+    const int tiles = (int)((p.tokens + C::TT - 1) / C::TT);
+    const int bid = blockIdx.x;
+    int held_op = -1, held_at = -1;                    // whose weights are in shared memory
+
+    // calls f(op, first unit, end) for this CTA's share of the operations of a phase, until f returns false
+    auto share = [&](int phase, auto f) {
+        const long long lo = bid * plan.share[phase] + min((long long)bid, plan.rest[phase]);
+        const long long hi = lo + plan.share[phase] + (bid < plan.rest[phase]);
+        long long base = 0;
+        for (int o = 0; o < p.n_ops; ++o) {
+            if (p.op[o].phase != phase) continue;
+            const int sh = plan.shift[o];
+            const long long w = 1ll << sh, n = plan.units[o];
+            long long i0 = lo > base ? (lo - base + w - 1) >> sh : 0, i1 = hi > base ? (hi - base + w - 1) >> sh : 0;
+            if (i0 > n) i0 = n;
+            if (i1 > n) i1 = n;
+            base += n << sh;
+            if (i0 < i1 && !f(o, (int)i0, (int)i1)) return;
+        }
+    };
+
+    for (int phase = 0; phase < p.n_phases; ++phase) {
+        share(phase, [&](int o, int i0, int i1) {
+            const Op &op = p.op[o];
+            if (op.kind == kStage) {
+                if (held_op != o) held_at = -1;
+                stage_units<C>(op, i0, i1, tiles, p.tokens, smem, held_at);
+                held_op = o;
+                return true;
+            }
+            for (int i = i0; i < i1; ++i) {
+                if (op.kind == kWgrad) {
+                    constexpr int kL = M / C::LS, kK = M / C::KS;
+                    wgrad_unit<C>(op, i / (kL * kK) % (M / 8) * 8, i / kK % kL * C::LS, i % kK * C::KS, i / (kL * kK * (M / 8)), p.tokens, smem);
+                    held_op = -1;
+                } else if (op.kind == kReduce) {
+                    reduce_unit(op, i);
+                } else {
+                    colsum_unit<C>(op, i, p.tokens, smem);
+                    held_op = -1;
+                }
+            }
+            return true;
+        });
+        if (phase + 1 == p.n_phases) break;
+        // the weights of the next phase do not depend on this one: fetched while the barrier is waited for
+        share(phase + 1, [&](int o, int i0, int) {
+            if (p.op[o].kind == kStage) {
+                const int at = i0 / tiles;
+                if (held_op != o || held_at != at) {
+                    __syncthreads();
+                    load_weights<C>(reinterpret_cast<typename C::T *>(smem + C::kWAt), p.op[o].w, p.op[o].trans, at / (M / C::ES) * 8,
+                                    at % (M / C::ES) * C::ES);
+                    held_op = o;
+                    held_at = at;
+                }
+            }
+            return false;
+        });
+        if (!grid_barrier(p.status, (unsigned)(phase + 1) * gridDim.x, &dead)) break;
+    }
+    cp_async_wait();                                   // nothing in flight when the CTA exits, also after a timeout
+    if (threadIdx.x == 0 && p.n_phases > 1 && dead == 0) {
+        if (atomicAdd(p.status + kDoneWord, 1u) == gridDim.x - 1) {     // the last to leave puts the counters back to zero
+            p.status[kBarrierWord] = 0;
+            p.status[kDoneWord] = 0;
+        }
+    }
+}
+
+}  // namespace units
+}  // namespace monarch

@@ -1068,6 +1068,7 @@ size_t planes_bytes(int64_t tokens) { return (size_t)((tokens + 127) / 128) * 12
 }  // namespace tc
 
 void debug_skip_next_plane_load(long long item) { tc::g_skip_load.store(item); }
+bool chain_fwd_m128_split() { return !tc::chain_fused_enabled() || tc::g_skip_load.load(std::memory_order_relaxed) >= 0; }
 
 // Forward workspace: [status][tile counters 64 KB][u' planes][w' planes]; the backward call reads u' from it.
 constexpr size_t kChainCounterBytes = 65536;

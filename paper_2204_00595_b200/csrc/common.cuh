@@ -154,6 +154,8 @@ int chain_bwd_m128(const void *x, const void *dy, const void *L, const void *R, 
 const void *chain_fwd_m128_saved_u(const void *fwd_ws, int64_t tokens);
 // test aid: the next plane-transpose launch (last step of the m = 128 forward) leaves out the load of this item
 void debug_skip_next_plane_load(long long item);
+// true when the next forward call has to run as three launches: the switch for comparison runs, or a load to leave out
+bool chain_fwd_m128_split();
 
 // ---- backward as a chain of tensor-core launches (bf16; dx for m >= 32, dL/dR for m = 128), tc_bwd.cu ----
 // fixed_order (m = 32, 64): kTcPartialBytes more; the token slices of the weight-gradient launches store their sums there and a
@@ -262,6 +264,24 @@ int rectw_fwd(const void *x, const void *Lw, const void *R, void *y, int64_t tok
               int dtype, bool fast, void *ws, cudaStream_t s);
 int rectw_bwd(const void *x, const void *dy, const void *Lw, const void *R, void *dx, float *dLw, float *dR, int accumulate,
               int64_t tokens, int q, int b1, int b2, int b3, int r, int dtype, bool fast, void *ws, cudaStream_t s);
+
+// ---- whole calls as one cooperative launch over units of block products, both dtypes, any m (block_units.cu) ----
+// u, u_saved: the intermediate of the forward call in this family's own layout
+namespace units {
+// where a forward call leaves u in its workspace: after the status area and the counters of the other kernels, which
+// have to stay zero
+void *saved_u(const void *fwd_ws);
+size_t workspace_bytes(int op, int64_t tokens, int m, int dtype);
+int fwd(const void *x, const void *L, const void *R, void *y, int64_t tokens, int m, int dtype, void *u, void *ws, cudaStream_t s);
+// dx null: weight gradients only; dL null: dx only; u_saved null: recomputed
+int bwd(const void *x, const void *dy, const void *L, const void *R, const void *u_saved, void *dx, float *dL, float *dR,
+        int accumulate, int64_t tokens, int m, int dtype, void *ws, cudaStream_t s);
+int mlp_fwd(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2, void *y,
+            int64_t tokens, int m, int dtype, void *ws, cudaStream_t s);
+int mlp_bwd(const void *x, const void *dy, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, void *dx,
+            float *dL1, float *dR1, float *db1, float *dL2, float *dR2, float *db2, int accumulate, int64_t tokens, int m, int dtype,
+            void *ws, cudaStream_t s);
+}  // namespace units
 
 // ---- dense <-> Monarch factors (project.cu): Eq. (2) and Algorithm 1 ----
 int dense_from_factors(const void *L, const void *R, void *M, int m, int dtype, cudaStream_t s);

@@ -123,6 +123,43 @@ int pick(int op, int m, int dtype)
     return tc_staged_available(op, m, dtype) ? kTcStaged : kSimt;
 }
 
+// Largest batch that runs as one launch over block-product units (block_units.cu); beyond it the kernels above are
+// faster.  Measured per pass, back to back (us, units / the others):
+//   bf16 m = 16   forward 27 / 213 at 32768 tokens, forward + backward 148 / 484: every batch
+//   bf16 m = 32   forward 12.4 / 14.5 at 1000, 20.6 / 14.5 at 4000; forward + backward 66 / 105 at 4000; feed-forward
+//                 block 41 / 84 at 4000, 122 / 167 at 16384, with its backward 96 / 277 at 1000
+//   bf16 m = 64   forward 14.5 / 16.5 at 256, 19.8 / 16.5 at 512; forward + backward 32 / 45 at 128, 45 / 46 at 256;
+//                 block 29 / 35 at 256, 41 / 35 at 512, with its backward 113 / 147 at 256, 172 / 163 at 512
+//   bf16 m = 128  forward 10.7 / 12.1 at 16; block 54 / 115 at 128, 147 / 116 at 512, with its backward 148 / 183 at 64
+//   fp32          the other family (one launch per stage) is slower at every size
+int64_t units_limit(int op, int m, int dtype)
+{
+    const int64_t all = 1 << 20;                          // what the 32-bit addressing of the units allows
+    if (dtype == MONARCH_F32 || m == 16) return all;
+    const bool fwd = op == MONARCH_OP_FWD, mlp = op == MONARCH_OP_MLP_FWD, mlp_bwd = op == MONARCH_OP_MLP_BWD;
+    if (m == 32) return fwd ? 1500 : all;
+    if (m == 64) return fwd ? 320 : mlp ? 384 : mlp_bwd ? 448 : 256;
+    return fwd ? 16 : mlp ? 320 : mlp_bwd ? 96 : 0;
+}
+
+// (the switches that ask for a particular form of the other kernels keep their meaning at every size)
+bool use_units(int op, int m, int dtype, int64_t tokens)
+{
+    // the smallest m = 16 forwards: both stages of a few tokens fit one CTA, which needs no barrier (fused_m16.cu)
+    if (m == 16 && op == MONARCH_OP_FWD && tokens <= 256) return false;
+    return g_impl.load(std::memory_order_relaxed) == MONARCH_IMPL_AUTO && tokens > 0 && tokens <= units_limit(op, m, dtype) &&
+           !(m == 64 && fused_fwd_m64_on_clusters()) && !(m == 128 && chain_fwd_m128_split());
+}
+
+// grows with the tokens: a workspace sized for a batch serves every smaller one, whichever kernels run it
+size_t with_units(size_t bytes, int op, int64_t tokens, int m, int dtype)
+{
+    if (bytes == 0 || g_impl.load(std::memory_order_relaxed) != MONARCH_IMPL_AUTO) return bytes;
+    const int64_t limit = units_limit(op, m, dtype);
+    const size_t u = units::workspace_bytes(op, tokens < limit ? tokens : limit, m, dtype);
+    return u > bytes ? u : bytes;
+}
+
 // Workspace of monarch_mlp_bwd: [backward workspace (status word first)][forward workspace][a][h][dh]
 struct MlpBwdLayout {
     size_t ws_b, ws_f, act, off_f, off_a, off_h, off_dh, total;
@@ -151,10 +188,10 @@ using namespace monarch;
 
 extern "C" {
 
-size_t monarch_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int dtype)
+namespace {
+// what the kernels for large batches need
+size_t large_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int dtype, bool fixed_order)
 {
-    if (op < MONARCH_OP_FWD || op > MONARCH_OP_CPLX) return 0;
-    if (check_shape(tokens, n, m, dtype) != MONARCH_OK) return 0;
     if (op == MONARCH_OP_CPLX) {
         // [inner workspace for 2 * tokens rows][four results of 2 * tokens rows]
         const size_t f = monarch_workspace_bytes(MONARCH_OP_FWD, 2 * tokens, n, m, dtype);
@@ -172,10 +209,10 @@ size_t monarch_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int
     // refuse, and so does this query (shard the tokens)
     if (which == kFused && m == 64 && tokens > ((int64_t)1 << 20)) return 0;
     if (which == kTcStaged && op != MONARCH_OP_FWD && op != MONARCH_OP_MLP_FWD)
-        return tc_staged_bwd_workspace_bytes(tokens, m, op != MONARCH_OP_BWD_DX && g_fixed_order.load(std::memory_order_relaxed) != 0);
+        return tc_staged_bwd_workspace_bytes(tokens, m, op != MONARCH_OP_BWD_DX && fixed_order);
     if (which == kTcStaged && op == MONARCH_OP_FWD && m == 128) return chain_fwd_m128_workspace_bytes(tokens);
     if (op == MONARCH_OP_BWD) {
-        if (which == kFused) return fused_bwd_m64_workspace_bytes(tokens, g_fixed_order.load(std::memory_order_relaxed) != 0);
+        if (which == kFused) return fused_bwd_m64_workspace_bytes(tokens, fixed_order);
         const size_t a = staged_workspace_bytes(MONARCH_OP_BWD_DX, tokens, n, m, dtype);
         const size_t b = staged_workspace_bytes(MONARCH_OP_BWD_DW, tokens, n, m, dtype);
         return a > b ? a : b;
@@ -185,8 +222,20 @@ size_t monarch_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int
                : op == MONARCH_OP_MLP_FWD ? fused_mlp_fwd_m64_workspace_bytes(tokens)
                : op == MONARCH_OP_FWD    ? fused_fwd_m64_workspace_bytes(tokens)
                : op == MONARCH_OP_BWD_DX ? fused_bwd_dx_m64_workspace_bytes(tokens)
-                                         : fused_bwd_dw_m64_workspace_bytes(tokens, g_fixed_order.load(std::memory_order_relaxed) != 0);
+                                         : fused_bwd_dw_m64_workspace_bytes(tokens, fixed_order);
     return staged_workspace_bytes(op, tokens, n, m, dtype);
+}
+}  // namespace
+
+size_t monarch_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int dtype)
+{
+    if (op < MONARCH_OP_FWD || op > MONARCH_OP_CPLX) return 0;
+    if (check_shape(tokens, n, m, dtype) != MONARCH_OK) return 0;
+    const size_t plain = large_workspace_bytes(op, tokens, n, m, dtype, false);
+    const size_t need = op == MONARCH_OP_CPLX ? plain : with_units(plain, op, tokens, m, dtype);
+    if (plain == 0 || g_fixed_order.load(std::memory_order_relaxed) == 0) return need;
+    // the partial sums of monarch_set_deterministic come on top
+    return need + (large_workspace_bytes(op, tokens, n, m, dtype, true) - plain);
 }
 
 int monarch_fwd(const void *x, const void *L, const void *R, void *y, int64_t tokens, int32_t n,
@@ -200,6 +249,8 @@ int monarch_fwd(const void *x, const void *L, const void *R, void *y, int64_t to
     if (which < 0) return MONARCH_ERR_UNSUPPORTED;
     MONARCH_TRY(check_buffers(in, 3, out, 1, workspace, workspace_bytes,
                               monarch_workspace_bytes(MONARCH_OP_FWD, tokens, n, m, dtype)));
+    if (use_units(MONARCH_OP_FWD, m, dtype, tokens))
+        return units::fwd(x, L, R, y, tokens, m, dtype, units::saved_u(workspace), workspace, (cudaStream_t)stream);
     if (which == kFused)
         return m == 32 ? fused_fwd_m32(x, L, R, y, tokens, workspace, (cudaStream_t)stream)
                        : fused_fwd_m64(x, L, R, y, tokens, workspace, (cudaStream_t)stream);
@@ -222,6 +273,8 @@ int monarch_bwd_dx(const void *dy, const void *L, const void *R, void *dx, int64
     if (which < 0) return MONARCH_ERR_UNSUPPORTED;
     MONARCH_TRY(check_buffers(in, 3, out, 1, workspace, workspace_bytes,
                               monarch_workspace_bytes(MONARCH_OP_BWD_DX, tokens, n, m, dtype)));
+    if (use_units(MONARCH_OP_BWD_DX, m, dtype, tokens))
+        return units::bwd(nullptr, dy, L, R, nullptr, dx, nullptr, nullptr, 0, tokens, m, dtype, workspace, (cudaStream_t)stream);
     if (which == kFused)
         return fused_bwd_dx_m64(dy, L, R, dx, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
@@ -244,6 +297,8 @@ int monarch_bwd_dw(const void *x, const void *dy, const void *L, const void *R, 
     if (which < 0) return MONARCH_ERR_UNSUPPORTED;
     MONARCH_TRY(check_buffers(in, 4, out, 2, workspace, workspace_bytes,
                               monarch_workspace_bytes(MONARCH_OP_BWD_DW, tokens, n, m, dtype)));
+    if (use_units(MONARCH_OP_BWD_DW, m, dtype, tokens))
+        return units::bwd(x, dy, L, R, nullptr, nullptr, dL, dR, accumulate, tokens, m, dtype, workspace, (cudaStream_t)stream);
     if (which == kFused)
         return fused_bwd_dw_m64(x, dy, L, R, dL, dR, accumulate, tokens, workspace, (cudaStream_t)stream,
                                 g_fixed_order.load(std::memory_order_relaxed) != 0);
@@ -270,6 +325,12 @@ int monarch_bwd(const void *x, const void *dy, const void *L, const void *R, con
     MONARCH_TRY(check_buffers(in, 4, out, 3, workspace, workspace_bytes,
                               monarch_workspace_bytes(MONARCH_OP_BWD, tokens, n, m, dtype)));
     cudaStream_t s = (cudaStream_t)stream;
+    // which kernels the forward call ran on, and so in which layout it left u
+    const bool saved_by_units = fwd_workspace != nullptr && use_units(MONARCH_OP_FWD, m, dtype, tokens);
+    if (use_units(MONARCH_OP_BWD, m, dtype, tokens))
+        return units::bwd(x, dy, L, R, saved_by_units ? units::saved_u(fwd_workspace) : nullptr, dx, dL, dR, accumulate, tokens, m,
+                          dtype, workspace, s);
+    if (saved_by_units) fwd_workspace = nullptr;
     if (which == kFused) {
         const bool saved = fwd_workspace != nullptr && pick(MONARCH_OP_FWD, m, dtype) == kFused;
         return fused_bwd_m64(x, dy, L, R, saved ? fused_fwd_m64_saved_u(fwd_workspace) : nullptr, dx, dL,
@@ -298,6 +359,8 @@ int monarch_mlp_fwd(const void *x, const void *L1, const void *R1, const void *b
     if (which < 0) return MONARCH_ERR_UNSUPPORTED;
     MONARCH_TRY(check_buffers(in, 7, out, 1, workspace, workspace_bytes,
                               monarch_workspace_bytes(MONARCH_OP_MLP_FWD, tokens, n, m, dtype)));
+    if (use_units(MONARCH_OP_MLP_FWD, m, dtype, tokens))
+        return units::mlp_fwd(x, L1, R1, b1, L2, R2, b2, y, tokens, m, dtype, workspace, (cudaStream_t)stream);
     if (which == kFused)
         return fused_mlp_fwd_m64(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
@@ -321,8 +384,11 @@ int monarch_mlp_bwd(const void *x, const void *dy, const void *L1, const void *R
     const Range out[] = {{dx, act}, {dL1, gb}, {dR1, gb}, {db1, gbias}, {dL2, gb}, {dR2, gb}, {db2, gbias}};
     const MlpBwdLayout lay = mlp_bwd_layout(tokens, n, m, dtype);
     if (lay.ws_b == 0 || lay.ws_f == 0) return MONARCH_ERR_UNSUPPORTED;
-    MONARCH_TRY(check_buffers(in, 7, out, 7, workspace, workspace_bytes, lay.total));
+    MONARCH_TRY(check_buffers(in, 7, out, 7, workspace, workspace_bytes,
+                              monarch_workspace_bytes(MONARCH_OP_MLP_BWD, tokens, n, m, dtype)));
     cudaStream_t s = (cudaStream_t)stream;
+    if (use_units(MONARCH_OP_MLP_BWD, m, dtype, tokens))
+        return units::mlp_bwd(x, dy, L1, R1, b1, L2, R2, dx, dL1, dR1, db1, dL2, dR2, db2, accumulate, tokens, m, dtype, workspace, s);
     if (!accumulate) {
         MONARCH_CUDA_TRY(cudaMemsetAsync(db1, 0, gbias, s));
         MONARCH_CUDA_TRY(cudaMemsetAsync(db2, 0, gbias, s));
@@ -334,7 +400,7 @@ int monarch_mlp_bwd(const void *x, const void *dy, const void *L1, const void *R
     MONARCH_TRY(monarch_workspace_init(ws_f, lay.ws_f, stream));
     // a = M1 x + b1: the fused m = 64 forward adds the bias in its epilogue, the others leave it to the
     // elementwise kernels (a then holds M1 x)
-    const bool bias_in_a = pick(MONARCH_OP_FWD, m, dtype) == kFused && m == 64;
+    const bool bias_in_a = pick(MONARCH_OP_FWD, m, dtype) == kFused && m == 64 && !use_units(MONARCH_OP_FWD, m, dtype, tokens);
     if (bias_in_a)
         MONARCH_TRY(fused_fwd_bias_m64(x, L1, R1, b1, 0, a, tokens, ws_f, s));
     else

@@ -931,6 +931,65 @@ def test_project_leading_pair(P, m, dtype, kind):
         assert tail * (1 - 1e-9) <= res <= tail * (1 + 1e-5) + rounding + (1e-6 * sv[0]) ** 2
 
 
+@pytest.mark.parametrize("m,T,dtype", [(16, 2500, "bf16"), (16, 1100, "f32"), (32, 1185, "bf16"), (32, 1601, "bf16"),
+                                       (32, 833, "f32"), (64, 255, "bf16"), (64, 320, "bf16"), (64, 321, "bf16"), (64, 593, "f32"),
+                                       (128, 17, "bf16"), (128, 75, "f32")])
+def test_one_launch_over_units(P, m, T, dtype):
+    """Sizes at which a call changes its tiles, splits the tokens of a weight gradient or changes kernels between the
+    forward and the backward: every call against the oracle, with u saved and recomputed, from one pair of workspaces."""
+    import torch
+    n, code = m * m, _code(P, dtype)
+    d = _small_inputs(m, T, dtype, seed=31 * m + T)
+    x, dy, L, R = (to_device(d[k], dtype) for k in ("x", "dy", "L", "R"))
+    ref_y, ref = O.fwd(d["x"], d["L"], d["R"]), O.bwd(d["x"], d["dy"], d["L"], d["R"])
+    ws_f = P.Workspace(P.monarch_workspace_bytes(P.OP_FWD, T, n, m, code))
+    ws_b = P.Workspace(max(P.monarch_workspace_bytes(op, T, n, m, code) for op in (P.OP_BWD, P.OP_BWD_DX, P.OP_BWD_DW)))
+    yf, y = _guarded((T, n), _tdtype(dtype))
+    dxf, dx = _guarded((T, n), _tdtype(dtype))
+    dLf, dL = _guarded((m, m, m), torch.float32)
+    dRf, dR = _guarded((m, m, m), torch.float32)
+    P.monarch_fwd(x, L, R, y, T, n, m, ws_f)
+    for saved, accumulate in ((ws_f, 0), (None, 1)):
+        P.monarch_bwd(x, dy, L, R, dx, dL, dR, accumulate, T, n, m, ws_b, fwd_workspace=saved)
+        torch.cuda.synchronize()
+        for got, want, what in ((y, ref_y, "y"), (dx, ref["dx"], "dx"), (dL, (1 + accumulate) * ref["dL"], "dL"),
+                                (dR, (1 + accumulate) * ref["dR"], "dR")):
+            assert_close(to_host64(got), want, dtype, f"{what} saved={saved is not None}")
+        dx.fill_(float("nan"))
+    P.monarch_bwd_dx(dy, L, R, dx, T, n, m, ws_b)
+    P.monarch_bwd_dw(x, dy, L, R, dL, dR, 0, T, n, m, ws_b)
+    torch.cuda.synchronize()
+    assert P.monarch_last_device_status(ws_f) == 0 and P.monarch_last_device_status(ws_b) == 0
+    assert_close(to_host64(dx), ref["dx"], dtype, "dx alone")
+    assert_close(to_host64(dL), ref["dL"], dtype, "dL alone")
+    assert_close(to_host64(dR), ref["dR"], dtype, "dR alone")
+    for flat, what in ((yf, "y"), (dxf, "dx"), (dLf, "dL"), (dRf, "dR")):
+        _check_guard(flat, what)
+
+
+@pytest.mark.parametrize("m,T,dtype", [(16, 1300, "bf16"), (32, 1190, "bf16"), (64, 449, "bf16"), (128, 97, "bf16"), (64, 300, "f32")])
+def test_one_launch_feed_forward(P, m, T, dtype):
+    """The feed-forward block and its gradients at sizes with split token ranges and at the first size beyond the units."""
+    import torch
+    n, code = m * m, _code(P, dtype)
+    d = _small_inputs(m, T, dtype, seed=37 * m + T)
+    t = {k: to_device(d[k], dtype) for k in ("x", "dy", "L", "R", "b1", "L2", "R2", "b2")}
+    yf, y = _guarded((T, n), _tdtype(dtype))
+    ws = P.Workspace(max(P.monarch_workspace_bytes(op, T, n, m, code) for op in (P.OP_MLP_FWD, P.OP_MLP_BWD)))
+    bufs = _mlp_bwd_buffers(m, T, dtype)
+    P.monarch_mlp_fwd(t["x"], t["L"], t["R"], t["b1"], t["L2"], t["R2"], t["b2"], y, T, n, m, ws)
+    _call_mlp_bwd(P, t, bufs, 0, T, n, m, ws)
+    torch.cuda.synchronize()
+    assert P.monarch_last_device_status(ws) == 0
+    assert_close(to_host64(y), O.mlp_fwd(d["x"], d["L"], d["R"], d["b1"], d["L2"], d["R2"], d["b2"]), dtype, "mlp y")
+    ref = O.mlp_bwd(d["x"], d["dy"], d["L"], d["R"], d["b1"], d["L2"], d["R2"])
+    assert_close(to_host64(bufs["dx"][1]), ref["dx"], dtype, "mlp dx")
+    _assert_mlp_grads(bufs, ref, dtype, "mlp")
+    _check_guard(yf, "mlp y")
+    for k, (flat, _) in bufs.items():
+        _check_guard(flat, f"mlp {k}")
+
+
 # ----------------------------------------------------------------- the five workloads
 
 def _sample_tokens(T, count, seed):
