@@ -2,7 +2,9 @@
 
 Tensors are torch CUDA tensors used as typed device buffers; the binding checks dtype,
 contiguity and device, takes their pointers, and calls the C entry point on the current
-CUDA stream (or the one given).  A non-zero status raises MonarchError.
+CUDA stream (or the one given).  A non-zero status raises MonarchError.  The calls on device
+tensors marshal their arguments natively (csrc/pycalls.c): on a few tokens the checks and
+ctypes conversions took the host longer than the kernels take the GPU.
 """
 from __future__ import annotations
 
@@ -15,6 +17,7 @@ IMPL_AUTO, IMPL_STAGED, IMPL_FUSED = 0, 1, 2
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libmonarch.so")
 _lib = None
+_calls = {}         # name -> native call object, made on first use
 
 _vp, _i64, _i32, _int, _sz = (ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_int,
                               ctypes.c_size_t)
@@ -187,69 +190,73 @@ def monarch_status_string(status: int) -> str:
     return lib().monarch_status_string(status).decode()
 
 
+# Native calls: how the arguments of each are passed (see csrc/pycalls.c), and the tensors' names for messages.
+_SPECS = {
+    "monarch_fwd": ("ttttiiiDws", "x L R y tokens n m workspace stream"),
+    "monarch_bwd_dx": ("ttttiiiDws", "dy L R dx tokens n m workspace stream"),
+    "monarch_bwd_dw": ("ttttffiiiiDws", "x dy L R dL dR accumulate tokens n m workspace stream"),
+    "monarch_bwd": ("ttttvtffiiiiDws", "x dy L R fwd_workspace dx dL dR accumulate tokens n m workspace stream"),
+    "monarch_mlp_fwd": ("ttttttttiiiDws", "x L1 R1 b1 L2 R2 b2 y tokens n m workspace stream"),
+    "monarch_mlp_bwd": ("ttttttttffffffiiiiDws",
+                        "x dy L1 R1 b1 L2 R2 dx dL1 dR1 db1 dL2 dR2 db2 accumulate tokens n m workspace stream"),
+    "monarch_rect_fwd": ("ttttiiiiiDws", "x L R y tokens q b1 b r workspace stream"),
+    "monarch_rect_bwd": ("ttttvtffiiiiiiDws", "x dy L R fwd_workspace dx dL dR accumulate tokens q b1 b r workspace stream"),
+    "monarch_cplx_fwd": ("ttttiiiiDws", "x L R y adjoint tokens n m workspace stream"),
+    "monarch_dense": ("tttiiDs", "L R M n m stream"),
+    "monarch_project": ("tttiiDqs", "A L R n m rotation_count stream"),
+}
+
+
+def _current_stream() -> int:
+    import torch
+    return torch.cuda.current_stream().cuda_stream
+
+
+def _native(name: str):
+    """The native call object of ``name`` (slow path of the calls below: first use)."""
+    import torch
+    from . import _pycalls
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    current = (lambda: raw(device())) if raw is not None and device is not None else _current_stream
+    spec, names = _SPECS[name]
+    address = ctypes.cast(getattr(lib(), name), _vp).value
+    call = _pycalls.Call(name, address, spec, tuple(names.split()), (torch.float32, torch.bfloat16, torch.int64), _check, current)
+    _calls[name] = call
+    return call
+
+
 def monarch_fwd(x, L, R, y, tokens, n, m, workspace, stream=None) -> None:
     """y = P L P^T R x for ``tokens`` rows of x (see include/monarch.h)."""
-    dt = x.dtype
-    p, b = _ws(workspace)
-    _check(lib().monarch_fwd(_ptr(x, "x"), _ptr(L, "L", dt), _ptr(R, "R", dt), _ptr(y, "y", dt),
-                             tokens, n, m, _dtype_code(x), p, b, _stream(stream)), "monarch_fwd")
+    (_calls.get("monarch_fwd") or _native("monarch_fwd"))(x, L, R, y, tokens, n, m, workspace, stream)
 
 
 def monarch_bwd_dx(dy, L, R, dx, tokens, n, m, workspace, stream=None) -> None:
     """dx = M^T dy."""
-    dt = dy.dtype
-    p, b = _ws(workspace)
-    _check(lib().monarch_bwd_dx(_ptr(dy, "dy"), _ptr(L, "L", dt), _ptr(R, "R", dt),
-                                _ptr(dx, "dx", dt), tokens, n, m, _dtype_code(dy), p, b,
-                                _stream(stream)), "monarch_bwd_dx")
+    (_calls.get("monarch_bwd_dx") or _native("monarch_bwd_dx"))(dy, L, R, dx, tokens, n, m, workspace, stream)
 
 
 def monarch_bwd_dw(x, dy, L, R, dL, dR, accumulate, tokens, n, m, workspace, stream=None) -> None:
     """dL, dR (float32) summed over tokens; accumulate=1 adds to their contents."""
-    import torch
-    dt = x.dtype
-    p, b = _ws(workspace)
-    _check(lib().monarch_bwd_dw(_ptr(x, "x"), _ptr(dy, "dy", dt), _ptr(L, "L", dt),
-                                _ptr(R, "R", dt), _ptr(dL, "dL", torch.float32),
-                                _ptr(dR, "dR", torch.float32), int(accumulate), tokens, n, m,
-                                _dtype_code(x), p, b, _stream(stream)), "monarch_bwd_dw")
+    (_calls.get("monarch_bwd_dw") or _native("monarch_bwd_dw"))(x, dy, L, R, dL, dR, int(accumulate), tokens, n, m, workspace, stream)
 
 
 def monarch_bwd(x, dy, L, R, dx, dL, dR, accumulate, tokens, n, m, workspace, fwd_workspace=None,
                 stream=None) -> None:
     """dx, dL, dR in one call; fwd_workspace = the Workspace monarch_fwd used for the same x, L, R."""
-    import torch
-    dt = x.dtype
-    p, b = _ws(workspace)
-    fp = _ws(fwd_workspace)[0] if fwd_workspace is not None else None
-    _check(lib().monarch_bwd(_ptr(x, "x"), _ptr(dy, "dy", dt), _ptr(L, "L", dt), _ptr(R, "R", dt), fp,
-                             _ptr(dx, "dx", dt), _ptr(dL, "dL", torch.float32),
-                             _ptr(dR, "dR", torch.float32), int(accumulate), tokens, n, m,
-                             _dtype_code(x), p, b, _stream(stream)), "monarch_bwd")
+    (_calls.get("monarch_bwd") or _native("monarch_bwd"))(x, dy, L, R, fwd_workspace, dx, dL, dR, int(accumulate), tokens, n, m,
+                                                          workspace, stream)
 
 
 def monarch_mlp_fwd(x, L1, R1, b1, L2, R2, b2, y, tokens, n, m, workspace, stream=None) -> None:
     """y = M2 GELU(M1 x + b1) + b2."""
-    dt = x.dtype
-    p, b = _ws(workspace)
-    _check(lib().monarch_mlp_fwd(_ptr(x, "x"), _ptr(L1, "L1", dt), _ptr(R1, "R1", dt),
-                                 _ptr(b1, "b1", dt), _ptr(L2, "L2", dt), _ptr(R2, "R2", dt),
-                                 _ptr(b2, "b2", dt), _ptr(y, "y", dt), tokens, n, m,
-                                 _dtype_code(x), p, b, _stream(stream)), "monarch_mlp_fwd")
+    (_calls.get("monarch_mlp_fwd") or _native("monarch_mlp_fwd"))(x, L1, R1, b1, L2, R2, b2, y, tokens, n, m, workspace, stream)
 
 
 def monarch_mlp_bwd(x, dy, L1, R1, b1, L2, R2, dx, dL1, dR1, db1, dL2, dR2, db2, accumulate, tokens, n, m,
                     workspace, stream=None) -> None:
     """Gradients of <dy, y> for y = M2 GELU(M1 x + b1) + b2; weight and bias gradients are float32."""
-    import torch
-    dt, f32 = x.dtype, torch.float32
-    p, b = _ws(workspace)
-    _check(lib().monarch_mlp_bwd(_ptr(x, "x"), _ptr(dy, "dy", dt), _ptr(L1, "L1", dt), _ptr(R1, "R1", dt),
-                                 _ptr(b1, "b1", dt), _ptr(L2, "L2", dt), _ptr(R2, "R2", dt),
-                                 _ptr(dx, "dx", dt), _ptr(dL1, "dL1", f32), _ptr(dR1, "dR1", f32),
-                                 _ptr(db1, "db1", f32), _ptr(dL2, "dL2", f32), _ptr(dR2, "dR2", f32),
-                                 _ptr(db2, "db2", f32), int(accumulate), tokens, n, m, _dtype_code(x),
-                                 p, b, _stream(stream)), "monarch_mlp_bwd")
+    (_calls.get("monarch_mlp_bwd") or _native("monarch_mlp_bwd"))(x, dy, L1, R1, b1, L2, R2, dx, dL1, dR1, db1, dL2, dR2, db2,
+                                                                  int(accumulate), tokens, n, m, workspace, stream)
 
 
 def monarch_rect_workspace_bytes(tokens: int, q: int, b1: int, b: int, r: int, dtype: int) -> int:
@@ -258,35 +265,23 @@ def monarch_rect_workspace_bytes(tokens: int, q: int, b1: int, b: int, r: int, d
 
 def monarch_rect_fwd(x, L, R, y, tokens, q, b1, b, r, workspace, stream=None) -> None:
     """General (rectangular) Monarch multiply: x [tokens, q*b1], R [q, b, b1], L [b, r, q] -> y [tokens, r*b]."""
-    dt = x.dtype
-    p, nb = _ws(workspace)
-    _check(lib().monarch_rect_fwd(_ptr(x, "x"), _ptr(L, "L", dt), _ptr(R, "R", dt), _ptr(y, "y", dt), tokens,
-                                  q, b1, b, r, _dtype_code(x), p, nb, _stream(stream)), "monarch_rect_fwd")
+    (_calls.get("monarch_rect_fwd") or _native("monarch_rect_fwd"))(x, L, R, y, tokens, q, b1, b, r, workspace, stream)
 
 
 def monarch_cplx_fwd(x, L, R, y, adjoint, tokens, n, m, workspace, stream=None) -> None:
     """Complex multiply on planar tensors: x, y [2, tokens, n]; L, R [2, m, m, m]; adjoint=1 applies M^H."""
-    dt = x.dtype
-    p, b = _ws(workspace)
-    _check(lib().monarch_cplx_fwd(_ptr(x, "x"), _ptr(L, "L", dt), _ptr(R, "R", dt), _ptr(y, "y", dt), int(adjoint),
-                                  tokens, n, m, _dtype_code(x), p, b, _stream(stream)), "monarch_cplx_fwd")
+    (_calls.get("monarch_cplx_fwd") or _native("monarch_cplx_fwd"))(x, L, R, y, int(adjoint), tokens, n, m, workspace, stream)
 
 
 def monarch_dense(L, R, M, n, m, stream=None) -> None:
     """M[l*m+j, k*m+i] = L[j, l, k] * R[k, j, i] (Eq. 2); M is [n, n] in the dtype of L."""
-    dt = L.dtype
-    _check(lib().monarch_dense(_ptr(L, "L"), _ptr(R, "R", dt), _ptr(M, "M", dt), n, m, _dtype_code(L),
-                               _stream(stream)), "monarch_dense")
+    (_calls.get("monarch_dense") or _native("monarch_dense"))(L, R, M, n, m, stream)
 
 
 def monarch_project(A, L, R, n, m, rotation_count=None, stream=None) -> None:
     """Algorithm 1: factors L, R of the Monarch matrix closest to the dense A in Frobenius norm.
     rotation_count: optional one-element int64 CUDA tensor, incremented by the number of Jacobi rotations."""
-    import torch
-    dt = A.dtype
-    rc = _ptr(rotation_count, "rotation_count", torch.int64) if rotation_count is not None else None
-    _check(lib().monarch_project(_ptr(A, "A"), _ptr(L, "L", dt), _ptr(R, "R", dt), n, m, _dtype_code(A), rc,
-                                 _stream(stream)), "monarch_project")
+    (_calls.get("monarch_project") or _native("monarch_project"))(A, L, R, n, m, rotation_count, stream)
 
 
 def monarch_rect_bwd_workspace_bytes(tokens: int, q: int, b1: int, b: int, r: int, dtype: int) -> int:
@@ -297,13 +292,8 @@ def monarch_rect_bwd(x, dy, L, R, dx, dL, dR, accumulate, tokens, q, b1, b, r, w
                      stream=None) -> None:
     """Gradients of <dy, L R x> for the general class: dx like x; dL [b, r, q] and dR [q, b, b1] in float32.
     fwd_workspace = the Workspace monarch_rect_fwd used for the same x, R (its intermediate is then reused)."""
-    import torch
-    dt, f32 = x.dtype, torch.float32
-    p, nb = _ws(workspace)
-    fp = _ws(fwd_workspace)[0] if fwd_workspace is not None else None
-    _check(lib().monarch_rect_bwd(_ptr(x, "x"), _ptr(dy, "dy", dt), _ptr(L, "L", dt), _ptr(R, "R", dt), fp,
-                                  _ptr(dx, "dx", dt), _ptr(dL, "dL", f32), _ptr(dR, "dR", f32), int(accumulate),
-                                  tokens, q, b1, b, r, _dtype_code(x), p, nb, _stream(stream)), "monarch_rect_bwd")
+    (_calls.get("monarch_rect_bwd") or _native("monarch_rect_bwd"))(x, dy, L, R, fwd_workspace, dx, dL, dR, int(accumulate), tokens,
+                                                                    q, b1, b, r, workspace, stream)
 
 
 def monarch_rectw_workspace_bytes(tokens: int, q: int, b1: int, b2: int, b3: int, r: int, dtype: int) -> int:

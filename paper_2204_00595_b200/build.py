@@ -5,11 +5,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 CSRC = os.path.join(_PKG, "csrc")
 LIB = os.path.join(_PKG, "libmonarch.so")
+PYCALLS = os.path.join(_PKG, "_pycalls.so")      # argument marshalling of the hot calls (plain C, CPython API)
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -23,6 +25,17 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def _build_pycalls() -> None:
+    src = os.path.join(CSRC, "pycalls.c")
+    deps = [src, os.path.join(_ROOT, "include", "monarch.h"), os.path.abspath(__file__)]
+    if os.path.exists(PYCALLS) and all(os.path.getmtime(d) <= os.path.getmtime(PYCALLS) for d in deps):
+        return
+    tmp = PYCALLS + f".tmp{os.getpid()}"
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                    "-I", os.path.join(_ROOT, "include"), "-o", tmp, src], check=True)
+    os.replace(tmp, PYCALLS)
+
+
 def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
@@ -33,7 +46,8 @@ def _stale() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into libmonarch.so (only if sources changed)."""
+    """Compile every .cu under csrc/ into libmonarch.so and pycalls.c into _pycalls.so (only if sources changed)."""
+    _build_pycalls()
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
