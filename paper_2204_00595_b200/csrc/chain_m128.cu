@@ -601,6 +601,8 @@ struct FusedParams {
     unsigned *cnt1, *cnt2;                   // per tile: store warps (two per CTA) whose stage-1 / stage-2 rows are in memory
     char *u, *w, *y;                         // u' planes, w' ring, output
     const char *x;                           // input, for the L2 prefetch hints only (the data path goes through TMA)
+    const __nv_bfloat16 *bias;               // ACT: added to y, [n]
+    int gelu;                                // ACT: y = GELU(M x + bias)
     long long tokens;
     int ntiles;
     long long *trace;                        // debug builds: per-CTA cycle sums of the waits, else null
@@ -653,6 +655,9 @@ __device__ __forceinline__ bool wait_counter(unsigned *ctr, unsigned need, unsig
     return true;
 }
 
+// ACT: a bias and GELU on y, applied to the fp32 accumulators of stage 2 (thread row l of CTA j holds column l*128 + j of
+// every token of the tile, so the bias is one value per thread).
+template <bool ACT>
 __global__ void __launch_bounds__(kFusedThreads, 1)
 chain_fused_fwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_R,
                        const __grid_constant__ CUtensorMap tm_L, const FusedParams p)
@@ -777,6 +782,7 @@ chain_fused_fwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_co
         const uint32_t lane_base = tmem_base + ((uint32_t)(warp * 32) << 16);
         uint32_t g = 0;
         bool ok = true;
+        const float bias = ACT ? __bfloat162float(p.bias[row * kB + b]) : 0.0f;
         [[maybe_unused]] long long wa = 0, ws = 0;
         [[maybe_unused]] const long long te0 = clock64();
         for (int s = 0; ok && s < nsteps; ++s) {
@@ -798,6 +804,15 @@ chain_fused_fwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_co
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(acce0 + buf * 8);
+                    }
+                    if (ACT && kind == 1) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) {
+                                const float a = __uint_as_float(v[q][e]) + bias;
+                                v[q][e] = __float_as_uint(p.gelu ? gelu_fast(a) : a);
+                            }
                     }
                     // staging half h is free once the store of the previous item's half h has read it
                     { FT0(); if (!mbar_wait(stfree0 + h * 8, (g & 1) ^ 1, p.status, dead, kErrSlotWait)) { ok = false; break; } FACC(ws); }
@@ -1100,12 +1115,66 @@ size_t chain_bwd_m128_workspace_bytes(int64_t tokens)
     return MONARCH_STATUS_BYTES + kChainCounterBytes + 3 * tc::planes_bytes(tokens);
 }
 
+namespace tc {
+namespace {
+// one persistent launch; every CTA must be resident at once (one per SM).  bias (optional): y = act(M x + bias)
+int launch_fused_fwd(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws,
+                     cudaStream_t s)
+{
+    char *up = (char *)ws + MONARCH_STATUS_BYTES + kChainCounterBytes;
+    CUtensorMap mx, mR, mL;
+    MONARCH_TRY(map_tokens(&mx, x, tokens));
+    MONARCH_TRY(map_weights(&mR, R));
+    MONARCH_TRY(map_weights(&mL, L));
+    FusedParams fp;
+    fp.status = (unsigned *)ws;
+    fp.cnt1 = (unsigned *)((char *)ws + MONARCH_STATUS_BYTES);
+    fp.cnt2 = fp.cnt1 + kFusedCounters;
+    fp.ntiles = (int)((tokens + 127) / 128);
+    fp.u = up;
+    fp.w = up + planes_bytes(tokens);
+    fp.y = (char *)y;
+    fp.x = (const char *)x;
+    fp.bias = (const __nv_bfloat16 *)bias;
+    fp.gelu = gelu;
+    fp.tokens = tokens;
+    fp.trace = nullptr;
+#ifdef MONARCH_TRACE
+    if (const char *e = getenv("MONARCH_TRACE_PTR")) fp.trace = (long long *)strtoull(e, nullptr, 0);
+#endif
+    auto kern = bias != nullptr ? chain_fused_fwd_kernel<true> : chain_fused_fwd_kernel<false>;
+    MONARCH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmem));
+    MONARCH_CUDA_TRY(launch_chained(kern, kB, kFusedThreads, kFusedSmem, s, mx, mR, mL, fp));
+    note_launch();
+    return MONARCH_OK;
+}
+}  // namespace
+}  // namespace tc
+
+// The feed-forward block as two passes of the one-launch forward (4096 tokens: 248 us; as four launches of the stage
+// kernel 512 tokens took 116 us, now 50); workspace 0 where that form cannot run.
+size_t chain_mlp_fwd_m128_workspace_bytes(int64_t tokens)
+{
+    if (!tc::fwd_runs_fused(tokens)) return 0;
+    return chain_fwd_m128_workspace_bytes(tokens) + (((size_t)tokens * tc::kB * tc::kB * 2 + 255) & ~(size_t)255);
+}
+int chain_mlp_fwd_m128(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2,
+                       void *y, int64_t tokens, void *ws, cudaStream_t s)
+{
+    if (tokens == 0) return MONARCH_OK;
+    void *h = (char *)ws + chain_fwd_m128_workspace_bytes(tokens);
+    MONARCH_TRY(tc::launch_fused_fwd(x, L1, R1, b1, 1, h, tokens, ws, s));
+    return tc::launch_fused_fwd(h, L2, R2, b2, 0, y, tokens, ws, s);
+}
+
 // y = P L P^T R x (Def. 3.1; Section 3.3 steps 1-3): one persistent launch, or three launches.
 int chain_fwd_m128(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s)
 {
     using namespace tc;
     if (tokens == 0) return MONARCH_OK;
     if (tokens > (int64_t)1 << 30) return MONARCH_ERR_UNSUPPORTED;
+    if (fwd_runs_fused(tokens) && g_skip_load.load(std::memory_order_relaxed) < 0)
+        return launch_fused_fwd(x, L, R, nullptr, 0, y, tokens, ws, s);
     const int ntiles = (int)((tokens + 127) / 128);
     unsigned *status = (unsigned *)ws;
     char *up = (char *)ws + MONARCH_STATUS_BYTES + kChainCounterBytes, *wp = up + planes_bytes(tokens);
@@ -1113,27 +1182,6 @@ int chain_fwd_m128(const void *x, const void *L, const void *R, void *y, int64_t
     MONARCH_TRY(map_tokens(&mx, x, tokens));
     MONARCH_TRY(map_weights(&mR, R));
     MONARCH_TRY(map_weights(&mL, L));
-    if (fwd_runs_fused(tokens) && g_skip_load.load(std::memory_order_relaxed) < 0) {
-        // one persistent launch; every CTA must be resident at once (one per SM)
-        MONARCH_CUDA_TRY(cudaFuncSetAttribute(chain_fused_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmem));
-        FusedParams fp;
-        fp.status = status;
-        fp.cnt1 = (unsigned *)((char *)ws + MONARCH_STATUS_BYTES);
-        fp.cnt2 = fp.cnt1 + kFusedCounters;
-        fp.ntiles = ntiles;
-        fp.u = up;
-        fp.w = wp;
-        fp.y = (char *)y;
-        fp.x = (const char *)x;
-        fp.tokens = tokens;
-        fp.trace = nullptr;
-#ifdef MONARCH_TRACE
-        if (const char *e = getenv("MONARCH_TRACE_PTR")) fp.trace = (long long *)strtoull(e, nullptr, 0);
-#endif
-        MONARCH_CUDA_TRY(launch_chained(chain_fused_fwd_kernel, kB, kFusedThreads, kFusedSmem, s, mx, mR, mL, fp));
-        note_launch();
-        return MONARCH_OK;
-    }
     MONARCH_TRY(map_tokens(&my, y, tokens));
     MONARCH_TRY(map_pieces(&mu_st, up, ntiles));
     MONARCH_TRY(map_pieces(&mw_st, wp, ntiles));

@@ -148,6 +148,10 @@ int tc_staged_mlp_fwd(const void *x, const void *L1, const void *R1, const void 
 size_t chain_fwd_m128_workspace_bytes(int64_t tokens);
 size_t chain_bwd_m128_workspace_bytes(int64_t tokens);
 int chain_fwd_m128(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s);
+// y = M2 GELU(M1 x + b1) + b2 in two launches; workspace 0 where the one-launch forward cannot run
+size_t chain_mlp_fwd_m128_workspace_bytes(int64_t tokens);
+int chain_mlp_fwd_m128(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2,
+                       void *y, int64_t tokens, void *ws, cudaStream_t s);
 // saved_up: the u' the forward call left in its workspace (chain_fwd_m128_saved_u), or null
 int chain_bwd_m128(const void *x, const void *dy, const void *L, const void *R, const void *saved_up, void *dx, float *dL,
                    float *dR, int accumulate, int want_dx, int want_dw, int64_t tokens, void *ws, cudaStream_t s);

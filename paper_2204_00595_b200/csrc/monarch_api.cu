@@ -211,6 +211,10 @@ size_t large_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int d
     if (which == kTcStaged && op != MONARCH_OP_FWD && op != MONARCH_OP_MLP_FWD)
         return tc_staged_bwd_workspace_bytes(tokens, m, op != MONARCH_OP_BWD_DX && fixed_order);
     if (which == kTcStaged && op == MONARCH_OP_FWD && m == 128) return chain_fwd_m128_workspace_bytes(tokens);
+    if (which == kTcStaged && op == MONARCH_OP_MLP_FWD && m == 128) {
+        const size_t a = staged_workspace_bytes(op, tokens, n, m, dtype), b = chain_mlp_fwd_m128_workspace_bytes(tokens);
+        return a > b ? a : b;
+    }
     if (op == MONARCH_OP_BWD) {
         if (which == kFused) return fused_bwd_m64_workspace_bytes(tokens, fixed_order);
         const size_t a = staged_workspace_bytes(MONARCH_OP_BWD_DX, tokens, n, m, dtype);
@@ -363,6 +367,8 @@ int monarch_mlp_fwd(const void *x, const void *L1, const void *R1, const void *b
         return units::mlp_fwd(x, L1, R1, b1, L2, R2, b2, y, tokens, m, dtype, workspace, (cudaStream_t)stream);
     if (which == kFused)
         return fused_mlp_fwd_m64(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
+    if (which == kTcStaged && m == 128 && chain_mlp_fwd_m128_workspace_bytes(tokens) != 0)
+        return chain_mlp_fwd_m128(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
         return tc_staged_mlp_fwd(x, L1, R1, b1, L2, R2, b2, y, tokens, m, workspace,
                                  (cudaStream_t)stream);
