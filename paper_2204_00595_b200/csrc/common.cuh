@@ -174,8 +174,17 @@ int tc_staged_bwd(const void *x, const void *dy, const void *L, const void *R, v
 // ---- forward for m = 16 in one launch on the CUDA cores, both dtypes (fused_m16.cu); no workspace use ----
 int fused_fwd_m16(const void *x, const void *L, const void *R, void *y, int64_t tokens, int dtype, cudaStream_t s);
 
-// ---- fused forward for m = 32, bf16: both stages inside one CTA (fused_m32.cu); workspace = status word only ----
+// ---- m = 32, bf16: all stages of a token tile inside one CTA (fused_m32.cu) ----
+// forward: workspace = status word only
 int fused_fwd_m32(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s);
+// the feed-forward block in two launches
+size_t fused_mlp_fwd_m32_workspace_bytes(int64_t tokens);
+int fused_mlp_fwd_m32(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2,
+                      void *y, int64_t tokens, void *ws, cudaStream_t s);
+// dx null: gradients only; dL null: dx only.  The gradients are sums in a fixed order.
+size_t fused_bwd_m32_workspace_bytes();
+int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, void *dx, float *dL, float *dR, int accumulate,
+                  int64_t tokens, void *ws, cudaStream_t s);
 
 // ---- fused single-pass forward for m = 64, bf16 (fused_m64.cu) ----
 size_t fused_fwd_m64_workspace_bytes(int64_t tokens);

@@ -1,368 +1,515 @@
-// Fused forward y = P L P^T R x for m = 32 (n = 1024), bf16: both stages and both permutations inside one CTA.
+// m = 32 (n = 1024), bf16: forward and backward with every intermediate on one SM.
 //
-// At this size a 64-token tile of the intermediate u' = P R x is 128 KB and fits the shared memory of one SM, so
-// nothing is exchanged between SMs (Section 3.3 steps 1-3 with the permutations done on chip, as the method
-// is meant to run): a persistent CTA per SM takes whole tiles.
-//   stage 1: x arrives as 64 x 64 TMA boxes (two blocks k side by side, 128B swizzle), R_k pairs as 64 x 32 boxes;
-//            M = 64, N = 32 MMAs accumulate 16 blocks at a time into one 16-lane half of TMEM (a "plane" of 512
-//            columns; the two halves of a stage go to the two planes); the epilogue packs 8 blocks' results for one (t, j) into 16 bytes and writes them into
-//            the shared-memory buffer U[j][k/8][t][k%8] - the P^T of step 2 is which columns are packed together,
-//            and U[j] is, as it lies, the K-major A operand of stage 2.
-//   stage 2: A = U[j], B = L_j (streamed as pairs), again 16 blocks j per plane;
-//            the epilogue packs 16 blocks into the 32 bytes y[t][l*32 + 16s .. +16) (the final P), staged and
-//            stored with 3-D TMA boxes.
-// One thread issues all MMAs in the order S1a S1b S2a S2b per tile (a = blocks 0-15, b = 16-31); stage 1 of
-// the next tile is issued straight after S2b of the current one and cannot complete before it (the tensor
-// pipe is in order), so a single U buffer suffices.  The weights (64 KB + 64 KB) are re-streamed from L2 for
-// every tile: there is no room to keep them next to U.
-#include <cstdlib>
-
+// The weights of one stage are 64 KB: held as MMA operands in the registers of one CTA's 16 warps (two blocks per warp,
+// 32 registers per stage) they are read once per launch, and shared memory is left to the token tiles.  A tile is 16
+// tokens (32 KB per tensor), brought and taken by TMA.  Warp MMAs (m16n8k16): one stage is 2 GFLOP at 16384 tokens,
+// 4 us of their rate, while the path is bound by HBM (10.3 us) - tcgen05 needs M = 64 rows of tokens or outputs per
+// instruction, and its form of this kernel was bound by the issue of 128 such instructions per 64 tokens (29 us).
+//
+// The weights are the A operand (rows = outputs), the tokens are N, so every result fragment has tokens innermost and
+// every permutation of Section 3.3 is a choice of where stmatrix puts a row of 8 tokens:
+//   T tile  x, y, dy, dx in shared memory: [16 boxes of 64 columns][16 tokens][128 bytes], 16-byte chunks XORed with t % 8
+//           (TMA's 128-byte swizzle)
+//   E tile  a tensor by blocks: [block b][8-token half][row c of the block] chunks of 8 tokens, XORed with b % 8
+//   forward:   u = R_k x_k  (B = T tile by ldmatrix)        -> E tile [j][k]:  row j of block k goes to block j (the P^T)
+//              w = L_j u_j  (B = E tile by ldmatrix.trans)  -> E tile [j][l], in place: a warp overwrites its own blocks
+//              y            E tile [j][l] -> T tile, 8 x 8 transposes by ldmatrix.trans / stmatrix (the outer P)
+//   backward:  z = P dy     T tile -> E tile [j][l];   du = L_j^T z_j -> E tile [k][j];   dx = R_k^T du_k -> T tile
+//              dL_j = sum_t z_j u_j^T, dR_k = sum_t du_k x_k^T: tokens are the contraction, both operands as they lie
+// Shared memory moves 16 to 18 KB per token at 128 bytes per clock, no access has a bank conflict.
+//
+// Backward CTAs are of three kinds, dL, dR and dx: the sums of one gradient are 128 KB of accumulators, half the
+// registers of an SM, and a kind needs one or two sets of weights beside them.  u and du are recomputed by the kind that
+// needs them (the MMAs are nearly free; the saved traffic is not).  Every CTA stores its sums, a second small launch adds
+// them in a fixed order.
 #include "tc_common.cuh"
 
 namespace monarch {
 namespace tc {
 namespace {
 
-constexpr int kM = 32;
-constexpr int kN = kM * kM;
-// warps: 0-7 epilogue (two halves of four), 8-9 loaders of (x, R) pairs, 10 loader of L pairs, 11 MMA,
-// 12-13 store threads
-constexpr int kEpiWarps = 8, kXWarp0 = 8, kLWarp = 10, kMmaWarp = 11, kStoreWarp0 = 12;
-constexpr int kThreads = 14 * 32;
-constexpr int kUBytes = 32 * 4096;                       // U[j][k/8 4][t 64][16 B]
-constexpr int kXSlotBytes = 8192 + 4096, kXSlots = 4;    // x pair tile + R pair tile
-constexpr int kLSlotBytes = 4096, kLSlots = 4;           // L pair tile
-constexpr int kStageBytes = 8192, kStagesPerHalf = 2;
-constexpr int kSmemBytes = kUBytes + kXSlots * kXSlotBytes + kLSlots * kLSlotBytes + 2 * kStagesPerHalf * kStageBytes + 1024;
+constexpr int kM = 32, kN = kM * kM, kTok = 16, kWarps = 16, kThreads = kWarps * 32;
+constexpr int kTile = kTok * kN * 2;                     // bytes of a T or E tile
+constexpr int kSlots = 5, kSmemBytes = (kSlots + 2) * kTile + 1024;
+constexpr int kKinds = 3, kDL = 0, kDR = 1, kDX = 2;
+constexpr int kMaxParts = 50;                            // CTAs of a kind: a third of the chip
 
-struct P32 {
-    unsigned *status;
-    int tiles;
-    long long *trace;            // optional per-CTA timeline (debug builds), else null
-};
-
-#ifdef MONARCH_TRACE
-#define T32(item, slot, val) do { if (p.trace && (item) < 16) p.trace[((size_t)blockIdx.x * 16 + (item)) * 8 + (slot)] = (val); } while (0)
-#define C32() clock64()
-#else
-#define T32(item, slot, val) do { } while (0)
-#define C32() 0ll
-#endif
-
-struct Bars {
-    uint64_t xfull[2], xempty[2];                     // ring slots are handed over in groups of two
-    uint64_t lfull[2], lempty[2];
-    uint64_t pl_full[2], pl_empty[2];                 // the two accumulator planes (16-lane halves of TMEM)
-    uint64_t st_full[2 * kStagesPerHalf], st_free[2 * kStagesPerHalf];
-};
-
-__device__ __forceinline__ bool wait_fast(uint32_t bar, uint32_t parity, unsigned *status, volatile int *dead,
-                                          unsigned code)
+__device__ __forceinline__ void ldm4(uint32_t (&r)[4], uint32_t a)
 {
-    if (mbar_try_wait(bar, parity)) return true;
-    return mbar_wait(bar, parity, status, dead, code);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldm4t(uint32_t (&r)[4], uint32_t a)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void stm4(uint32_t a, const uint32_t (&r)[4])
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+__device__ __forceinline__ void stm4t(uint32_t a, const uint32_t (&r)[4])
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+__device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *m, int x, int y, int z, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
+                 "l"(m), "r"(bar), "r"(x), "r"(y), "r"(z) : "memory");
+}
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap *m, uint32_t src, int x, int y, int z)
+{
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(m), "r"(src), "r"(x), "r"(y), "r"(z) : "memory");
 }
 
+// chunk c (8 columns) of token t in a T tile; chunk (half h, row c) of block b in an E tile
+__device__ __forceinline__ uint32_t t_at(uint32_t base, int box, int t, int c) { return base + box * (kTok * 128) + t * 128 + ((c ^ (t & 7)) << 4); }
+__device__ __forceinline__ uint32_t e_at(uint32_t base, int b, int h, int c) { return base + b * 1024 + (((h * 32 + c) ^ (b & 7)) << 4); }
+
+// Operand A of a warp's two blocks: rows = outputs, [block][16 rows][16 columns of the contraction]
+struct Weights {
+    uint32_t a[2][2][2][4];
+    // trans: multiply by the transposed blocks (8 x 8 pieces transposed in registers)
+    __device__ __forceinline__ void load(const __nv_bfloat16 *W, int warp, bool trans)
+    {
+        const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
+#pragma unroll
+        for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int row = mt * 16 + (r & 1) * 8, col = ks * 16 + (r >> 1) * 8;      // of the 8 x 8 piece
+                        const __nv_bfloat16 *p = W + (size_t)(warp * 2 + blk) * kM * kM + (trans ? (col + g) * kM + row : (row + g) * kM + col) + 2 * q;
+                        a[blk][mt][ks][r] = *reinterpret_cast<const uint32_t *>(p);
+                    }
+        if (trans)
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                uint32_t &v = a[i >> 4][i >> 3 & 1][i >> 2 & 1][i & 3];
+                asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(v) : "r"(v));
+            }
+    }
+    // acc = blk's rows times the operand b (both 16-column steps)
+    __device__ __forceinline__ void times(int blk, const uint32_t (&b)[4], float (&acc)[2][4]) const
+    {
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+            acc[mt][0] = acc[mt][1] = acc[mt][2] = acc[mt][3] = 0.0f;
+            mma(acc[mt], a[blk][mt][0], b[0], b[1]);
+            mma(acc[mt], a[blk][mt][1], b[2], b[3]);
+        }
+    }
+};
+__device__ __forceinline__ void pack_rows(const float (&acc)[2][4], uint32_t (&o)[4])       // the 8 x 8 pieces of 32 rows x 8 tokens
+{
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+        o[2 * mt] = pack_bf16(acc[mt][0], acc[mt][1]);
+        o[2 * mt + 1] = pack_bf16(acc[mt][2], acc[mt][3]);
+    }
+}
+
+struct Lane {                                            // rows of the four matrices of an x4 instruction
+    int warp, m, r;
+    __device__ __forceinline__ Lane() : warp(threadIdx.x >> 5), m((threadIdx.x & 31) >> 3), r(threadIdx.x & 7) {}
+};
+
+// E[row][own block] = W_block T_block: row c of the result of block b becomes row b of block c
+__device__ __forceinline__ void stage_from_t(const Weights &w, uint32_t T, uint32_t E)
+{
+    const Lane ln;
+#pragma unroll
+    for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t b[4], o[4];
+            float acc[2][4];
+            ldm4(b, t_at(T, ln.warp, h * 8 + ln.r, blk * 4 + ln.m));
+            w.times(blk, b, acc);
+            pack_rows(acc, o);
+            stm4(e_at(E, ln.m * 8 + ln.r, h, ln.warp * 2 + blk), o);
+        }
+}
+// the same from an E tile of this warp's blocks
+__device__ __forceinline__ void stage_from_e(const Weights &w, uint32_t E, uint32_t out)
+{
+    const Lane ln;
+#pragma unroll
+    for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t b[4], o[4];
+            float acc[2][4];
+            const int own = ln.warp * 2 + blk;
+            ldm4t(b, e_at(E, own, h, ln.m * 8 + ln.r));
+            w.times(blk, b, acc);
+            pack_rows(acc, o);
+            stm4(e_at(out, ln.m * 8 + ln.r, h, own), o);
+        }
+}
+// E[block][row] -> T (the outer P) and back; a warp takes the columns of one box
+__device__ __forceinline__ void e_to_t(uint32_t E, uint32_t T)
+{
+    const Lane ln;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        const int h = n >> 1, c = ln.warp * 2 + (n & 1);
+        uint32_t v[4];
+        ldm4t(v, e_at(E, ln.m * 8 + ln.r, h, c));
+        stm4(t_at(T, ln.warp, h * 8 + ln.r, (n & 1) * 4 + ln.m), v);
+    }
+}
+__device__ __forceinline__ void t_to_e(uint32_t T, uint32_t E)
+{
+    const Lane ln;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        const int h = n >> 1, c = ln.warp * 2 + (n & 1);
+        uint32_t v[4];
+        ldm4t(v, t_at(T, ln.warp, h * 8 + ln.r, (n & 1) * 4 + ln.m));
+        stm4(e_at(E, ln.m * 8 + ln.r, h, c), v);
+    }
+}
+
+struct Params {
+    unsigned *status;
+    const __nv_bfloat16 *L, *R, *bias;
+    float *parts;                // backward: [kDL, kDR][kMaxParts][32][32][32]
+    int tiles, gelu;
+    int first[kKinds + 1];       // backward: CTAs of a kind start here
+};
+
+// Ring of T tiles filled by one thread
+struct Ring {
+    uint32_t base, bars;
+    unsigned *status;
+    volatile int *dead;
+    __device__ __forceinline__ uint32_t slot(int item) const { return base + (item % kSlots) * kTile; }
+    __device__ __forceinline__ void load(int item, const CUtensorMap *m, int tile) const
+    {
+        const uint32_t bar = bars + (item % kSlots) * 8;
+        mbar_expect_tx(bar, kTile);
+        tma_load_3d(slot(item), m, 0, tile * kTok, 0, bar);
+    }
+    // a wait that runs out leaves `dead` set and garbage in the tile; the loops still run to their end, every later wait
+    // returns at once
+    __device__ __forceinline__ uint32_t wait(int item) const
+    {
+        mbar_wait(bars + (item % kSlots) * 8, (item / kSlots) & 1, status, dead, kErrTmaWait);
+        return slot(item);
+    }
+};
+
+struct Shared {
+    uint64_t bars[kSlots];
+    int dead;
+};
+__device__ __forceinline__ void init(Shared &s)
+{
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kSlots; ++i) mbar_init(smem_u32(&s.bars[i]), 1);
+        fence_mbar_init();
+        s.dead = 0;
+    }
+    __syncthreads();
+}
+
+// ---------------------------------------------------------------- forward
+// Per tile two barriers: [w(i) from u(i), u(i + 1) from x] [y(i)].  ACT: y = GELU(M x + bias), or without the GELU.
+template <bool ACT>
 __global__ void __launch_bounds__(kThreads, 1)
-fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_R,
-                     const __grid_constant__ CUtensorMap tm_L, const __grid_constant__ CUtensorMap tm_y, const P32 p)
+fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_y, const Params p)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) Bars bars;
-    __shared__ uint32_t tmem_base_s;
-    __shared__ int dead_s;
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const Ring ring = {base, smem_u32(sh.bars), p.status, &sh.dead};
+    const uint32_t E[2] = {base + kSlots * kTile, base + (kSlots + 1) * kTile};
+    init(sh);
+    const int first = blockIdx.x, step = gridDim.x, count = (p.tiles - first + step - 1) / step;
+    if (threadIdx.x == 0)
+        for (int i = 0; i < 3 && i < count; ++i) ring.load(i, &tm_x, first + i * step);
+    const int warp = threadIdx.x >> 5;
+    Weights wr, wl;
+    wr.load(p.R, warp, false);
+    wl.load(p.L, warp, false);
+    float bias[2][4];
+    if (ACT)
+#pragma unroll
+        for (int i = 0; i < 8; ++i)                      // row l = 8 (i % 4) + lane / 4 of block j
+            bias[i >> 2][i & 3] = __bfloat162float(p.bias[((i & 3) * 8 + ((threadIdx.x & 31) >> 2)) * kM + warp * 2 + (i >> 2)]);
 
-    const uint32_t U0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t xring0 = U0 + kUBytes;
-    const uint32_t lring0 = xring0 + kXSlots * kXSlotBytes;
-    const uint32_t stage0 = lring0 + kLSlots * kLSlotBytes;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    volatile int *dead = &dead_s;
-
-    if (threadIdx.x == 0) {
-        for (int g = 0; g < 2; ++g) {
-            mbar_init(smem_u32(&bars.xfull[g]), 2);          // one (x, R) pair from each of the two loaders
-            mbar_init(smem_u32(&bars.xempty[g]), 1);
-            mbar_init(smem_u32(&bars.lfull[g]), 1);
-            mbar_init(smem_u32(&bars.lempty[g]), 1);
+    const Lane ln;
+    stage_from_t(wr, ring.wait(0), E[0]);
+    for (int i = 0; i < count; ++i) {
+        const uint32_t e = E[i & 1];
+        __syncthreads();                                 // u(i) and y(i - 1) are complete
+        if (threadIdx.x == 0) {
+            if (i > 0) {
+                tma_store_3d(&tm_y, ring.slot(i - 1), 0, (first + (i - 1) * step) * kTok, 0);
+                tma_store_commit();
+            }
+            if (i + 3 < count) {
+                tma_store_wait_read<1>();                // y(i - 2) has left its slot
+                ring.load(i + 3, &tm_x, first + (i + 3) * step);
+            }
         }
-        for (int h = 0; h < 2; ++h) {
-            mbar_init(smem_u32(&bars.pl_full[h]), 1);
-            mbar_init(smem_u32(&bars.pl_empty[h]), kEpiWarps);
-        }
-        for (int k = 0; k < 2 * kStagesPerHalf; ++k) {
-            mbar_init(smem_u32(&bars.st_full[k]), 4);
-            mbar_init(smem_u32(&bars.st_free[k]), 1);
-        }
-        fence_mbar_init();
-        dead_s = 0;
-        tma_prefetch_desc(&tm_x); tma_prefetch_desc(&tm_R); tma_prefetch_desc(&tm_L); tma_prefetch_desc(&tm_y);
+#pragma unroll
+        for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t b[4], o[4];
+                float acc[2][4];
+                const int own = warp * 2 + blk;
+                ldm4t(b, e_at(e, own, h, ln.m * 8 + ln.r));
+                wl.times(blk, b, acc);
+                if (ACT)
+#pragma unroll
+                    for (int v = 0; v < 8; ++v) {
+                        const float a = acc[v >> 2][v & 3] + bias[blk][v >> 1];
+                        acc[v >> 2][v & 3] = p.gelu ? gelu_fast(a) : a;
+                    }
+                pack_rows(acc, o);
+                stm4(e_at(e, own, h, ln.m * 8 + ln.r), o);
+            }
+        if (i + 1 < count) stage_from_t(wr, ring.wait(i + 1), E[(i + 1) & 1]);
+        __syncthreads();                                 // w(i) is complete; x(i) has been read by everyone
+        e_to_t(e, ring.slot(i));
+        fence_proxy_async_smem();
     }
-    if (warp == 0) {
-        tmem_alloc(smem_u32(&tmem_base_s), 512);
-        tmem_relinquish();
-    }
-    tc_fence_before();
     __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = tmem_base_s;
+    if (threadIdx.x == 0) {
+        tma_store_3d(&tm_y, ring.slot(count - 1), 0, (first + (count - 1) * step) * kTok, 0);
+        tma_store_commit();
+        tma_store_wait_all<0>();
+    }
+}
 
-    const int first = (int)blockIdx.x, step = (int)gridDim.x;
-    const uint32_t xf0 = smem_u32(bars.xfull), xe0 = smem_u32(bars.xempty);
-    const uint32_t lf0 = smem_u32(bars.lfull), le0 = smem_u32(bars.lempty);
-    const uint32_t plf0 = smem_u32(bars.pl_full), ple0 = smem_u32(bars.pl_empty);
+// ---------------------------------------------------------------- backward
+// sums[block][32 rows][32 columns] += A (rows, tokens) B (tokens, columns) of the warp's two blocks; A rows are rows of an
+// E tile; B likewise, or columns of a T tile
+struct Sums {
+    float v[2][2][4][4];
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int i = 0; i < 64; ++i) v[i >> 5][i >> 4 & 1][i >> 2 & 3][i & 3] = 0.0f;
+    }
+    template <bool BT> __device__ __forceinline__ void add(uint32_t A, uint32_t B)
+    {
+        const Lane ln;
+#pragma unroll
+        for (int blk = 0; blk < 2; ++blk) {
+            const int own = ln.warp * 2 + blk;
+            uint32_t a[2][4];
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) ldm4(a[mt], e_at(A, own, ln.m >> 1, mt * 16 + (ln.m & 1) * 8 + ln.r));
+#pragma unroll
+            for (int np = 0; np < 2; ++np) {
+                uint32_t b[4];
+                const int col = np * 2 + (ln.m >> 1), half = ln.m & 1;
+                if (BT) ldm4t(b, t_at(B, ln.warp, half * 8 + ln.r, blk * 4 + col));
+                else    ldm4(b, e_at(B, own, half, col * 8 + ln.r));
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt) {
+                    mma(v[blk][mt][2 * np], a[mt], b[0], b[1]);
+                    mma(v[blk][mt][2 * np + 1], a[mt], b[2], b[3]);
+                }
+            }
+        }
+    }
+    __device__ __forceinline__ void store(float *to) const
+    {
+        const int warp = threadIdx.x >> 5, g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
+#pragma unroll
+        for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        *reinterpret_cast<float2 *>(to + (size_t)(warp * 2 + blk) * kM * kM + (mt * 16 + g + 8 * h) * kM + nt * 8 + 2 * q) =
+                            make_float2(v[blk][mt][nt][2 * h], v[blk][mt][nt][2 * h + 1]);
+    }
+};
 
-    if (first >= p.tiles) {
-        // nothing to do
-    } else if (warp >= kXWarp0 && warp < kXWarp0 + 2) {
-        // ------------------------------------------------------------ (x, R) loaders: warp pw takes pairs pw, pw+2, ...
-        if (lane == 0) {
-            const int pw = warp - kXWarp0;
-            uint32_t ng = 0;                               // group use count: pairs (2 ng, 2 ng + 1) of the stream
-            for (int tile = first; tile < p.tiles; tile += step) {
-                bool ok = true;
-#pragma unroll 1
-                for (int G = 0; G < 8; ++G, ++ng) {
-                    const uint32_t g = ng & 1, ph = (ng >> 1) & 1;
-                    const int pr = G * 2 + pw;
-                    if (!wait_fast(xe0 + g * 8, ph ^ 1, p.status, dead, kErrSlotWait)) { ok = false; break; }
-                    const uint32_t dst = xring0 + (g * 2 + pw) * kXSlotBytes, full = xf0 + g * 8;
-                    mbar_expect_tx(full, kXSlotBytes);
-                    tma_load_2d(dst, &tm_x, pr * 64, tile * 64, full);            // blocks 2pr, 2pr+1: 64 columns
-                    tma_load_2d(dst + 8192, &tm_R, 0, pr * 64, full);             // R rows of both blocks
+__global__ void __launch_bounds__(kThreads, 1)
+fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_dy,
+                     const __grid_constant__ CUtensorMap tm_dx, const Params p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const Ring ring = {base, smem_u32(sh.bars), p.status, &sh.dead};
+    const uint32_t V = base + kSlots * kTile, U = V + kTile;
+    init(sh);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int b = blockIdx.x, kind = b < p.first[1] ? kDL : b < p.first[2] ? kDR : kDX;
+    const int first = b - p.first[kind], step = p.first[kind + 1] - p.first[kind], count = (p.tiles - first + step - 1) / step;
+    const int warp = threadIdx.x >> 5;
+
+    if (kind == kDX) {
+        // per tile [du(i) from z(i)] [dx(i), z(i + 1)]
+        if (threadIdx.x == 0)
+            for (int i = 0; i < 3 && i < count; ++i) ring.load(i, &tm_dy, first + i * step);
+        Weights wl, wr;
+        wl.load(p.L, warp, true);
+        wr.load(p.R, warp, true);
+        const Lane ln;
+        t_to_e(ring.wait(0), V);
+        for (int i = 0; i < count; ++i) {
+            __syncthreads();                             // z(i) and dx(i - 1) are complete
+            if (threadIdx.x == 0) {
+                if (i > 0) {
+                    tma_store_3d(&tm_dx, ring.slot(i - 1), 0, (first + (i - 1) * step) * kTok, 0);
+                    tma_store_commit();
                 }
-                if (!ok) break;
+                if (i + 3 < count) {
+                    tma_store_wait_read<1>();
+                    ring.load(i + 3, &tm_dy, first + (i + 3) * step);
+                }
             }
+            stage_from_e(wl, V, U);
+            __syncthreads();                             // du(i) is complete, z(i) has been read
+#pragma unroll
+            for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t bb[4], o[4];
+                    float acc[2][4];
+                    ldm4t(bb, e_at(U, warp * 2 + blk, h, ln.m * 8 + ln.r));
+                    wr.times(blk, bb, acc);
+                    pack_rows(acc, o);
+                    stm4t(t_at(ring.slot(i), warp, h * 8 + ln.r, blk * 4 + ln.m), o);
+                }
+            fence_proxy_async_smem();
+            if (i + 1 < count) t_to_e(ring.wait(i + 1), V);
         }
-    } else if (warp == kLWarp) {
-        // ------------------------------------------------------------ L loader
-        if (lane == 0) {
-            uint32_t ng = 0;
-            for (int tile = first; tile < p.tiles; tile += step) {
-                bool ok = true;
-#pragma unroll 1
-                for (int G = 0; G < 8; ++G, ++ng) {
-                    const uint32_t g = ng & 1, ph = (ng >> 1) & 1;
-                    if (!wait_fast(le0 + g * 8, ph ^ 1, p.status, dead, kErrSlotWait)) { ok = false; break; }
-                    mbar_expect_tx(lf0 + g * 8, 2 * kLSlotBytes);
-                    tma_load_2d(lring0 + (g * 2) * kLSlotBytes, &tm_L, 0, (G * 2) * 64, lf0 + g * 8);
-                    tma_load_2d(lring0 + (g * 2 + 1) * kLSlotBytes, &tm_L, 0, (G * 2 + 1) * 64, lf0 + g * 8);
-                }
-                if (!ok) break;
-            }
-        }
-    } else if (warp == kMmaWarp) {
-        // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idesc = make_idesc_bf16(64, 32, 0, 0);
-            const uint64_t d_x = make_smem_desc(0, 16, 1024, kSwizzle128);   // x pair tile: 128-byte rows
-            const uint64_t d_w = make_smem_desc(0, 16, 512, kSwizzle64);     // weight tiles: 64-byte rows
-            const uint64_t d_u = make_smem_desc(0, 1024, 128, 0);            // U[j]: k chunks 1 KB apart
-            // ring use counts; per plane: sub-items issued so far, completions of its `empty` barrier waited for
-            uint32_t nx = 0, nl = 0, issued[2] = {0, 0}, c[2] = {0, 0};
-            bool ok = true;
-            // wait until the epilogue has drained `target` sub-items of plane P (completion n has parity n & 1)
-            auto drained = [&](int P, uint32_t target) {
-                while (ok && c[P] < target) {
-                    if (!wait_fast(ple0 + P * 8, c[P] & 1, p.status, dead, kErrTmemWait)) ok = false;
-                    ++c[P];
-                }
-                tc_fence_after();
-            };
-            [[maybe_unused]] int ntile = -1;
-            for (int tile = first; ok && tile < p.tiles; tile += step) {
-                ++ntile;
-                // sub-items S1a S1b S2a S2b alternate between the two planes, so a half never waits for the
-                // epilogue of the half before it; only stage 2 waits - for all of U
-#pragma unroll 1
-                for (int q = 0; q < 4 && ok; ++q) {
-                    const int P = q & 1, h = q & 1;
-                    const uint32_t plane = tmem_base + ((uint32_t)(P * 16) << 16);
-                    [[maybe_unused]] const long long t_a = C32();
-                    if (q == 2) drained(1, issued[1]);     // S1b's epilogue: U is complete
-                    drained(P, issued[P]);                 // this plane has been read out
-                    if (!ok) break;
-                    [[maybe_unused]] const long long t_b = C32();
-                    [[maybe_unused]] long long wsum = 0;
-                    if (q < 2) {
-                        // four groups per half and two in the ring: group G sits in ring position G & 1
-#pragma unroll
-                        for (int G = 0; G < 4; ++G, ++nx) {
-                            const uint32_t g = G & 1, ph = (nx >> 1) & 1;
-                            [[maybe_unused]] const long long w0 = C32();
-                            if (!wait_fast(xf0 + g * 8, ph, p.status, dead, kErrTmaWait)) { ok = false; break; }
-                            tc_fence_after();
-                            wsum += C32() - w0;
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const uint32_t slot = xring0 + (g * 2 + e) * kXSlotBytes;
-                                const uint64_t ax = d_x | (uint64_t)(slot >> 4);
-                                const uint64_t bw = d_w | (uint64_t)((slot + 8192) >> 4);
-#pragma unroll
-                                for (int i = 0; i < 2; ++i) {
-                                    const uint32_t d = plane + ((G * 2 + e) * 2 + i) * 32;
-                                    // block 2pr+i: columns [32 i, +32) of the pair tile, rows [32 i, +32) of the R pair
-                                    mma_f16_ss(d, ax + i * 4, bw + i * 128, idesc, 0);
-                                    mma_f16_ss(d, ax + i * 4 + 2, bw + i * 128 + 2, idesc, 1);
-                                }
-                            }
-                            mma_commit(xe0 + g * 8);
-                        }
-                    } else {
-#pragma unroll
-                        for (int G = 0; G < 4; ++G, ++nl) {
-                            const uint32_t g = G & 1, ph = (nl >> 1) & 1;
-                            [[maybe_unused]] const long long w0 = C32();
-                            if (!wait_fast(lf0 + g * 8, ph, p.status, dead, kErrTmaWait)) { ok = false; break; }
-                            tc_fence_after();
-                            wsum += C32() - w0;
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const uint64_t bl = d_w | (uint64_t)((lring0 + (g * 2 + e) * kLSlotBytes) >> 4);
-#pragma unroll
-                                for (int i = 0; i < 2; ++i) {
-                                    const int jb = (G * 2 + e) * 2 + i;
-                                    const uint32_t d = plane + jb * 32;
-                                    const uint64_t au = d_u | (uint64_t)((U0 + (h * 16 + jb) * 4096) >> 4);
-                                    mma_f16_ss(d, au, bl + i * 128, idesc, 0);
-                                    mma_f16_ss(d, au + 128, bl + i * 128 + 2, idesc, 1);
-                                }
-                            }
-                            mma_commit(le0 + g * 8);
-                        }
-                    }
-                    if (!ok) break;
-                    mma_commit(plf0 + P * 8);
-                    T32(ntile * 4 + q, 0, t_a); T32(ntile * 4 + q, 1, t_b - t_a); T32(ntile * 4 + q, 2, wsum);
-                    T32(ntile * 4 + q, 3, C32());
-                    ++issued[P];
-                }
-            }
-        }
-    } else if (warp < kEpiWarps) {
-        // ------------------------------------------------------------ epilogues
-        const int q4 = warp & 3, sub = warp >> 2, hl = lane >> 4;
-        const uint32_t lane_base = tmem_base + ((uint32_t)(q4 * 32) << 16);
-        const int row = q4 * 16 + (lane & 15);
-        const uint32_t my_stage = stage0 + sub * kStagesPerHalf * kStageBytes;
-        const uint32_t stf0 = smem_u32(bars.st_full) + sub * kStagesPerHalf * 8;
-        const uint32_t stfree0 = smem_u32(bars.st_free) + sub * kStagesPerHalf * 8;
-        uint32_t np[2] = {0, 0}, nchunk = 0;          // sub-items seen per plane
-        bool ok = true;
-        for (int tile = first; ok && tile < p.tiles; tile += step) {
-            // ---- stage 1 halves: half h sits in plane h (lanes 16 h .. 16 h + 15 of every quarter) -> U
-#pragma unroll 1
-            for (int h = 0; h < 2 && ok; ++h) {
-                if (!wait_fast(plf0 + h * 8, np[h] & 1, p.status, dead, kErrMmaWait)) { ok = false; break; }
-                ++np[h];
-                tc_fence_after();
-                // this warp: rows j in [16 sub, 16 sub + 16), in two chunks of 8; blocks k of this half in two
-                // groups of 8 -> U chunk index 2h + g
-#pragma unroll 1
-                for (int jc = 0; jc < 2; ++jc) {
-#pragma unroll
-                    for (int g = 0; g < 2; ++g) {
-                        uint32_t v[8][8];
-#pragma unroll
-                        for (int kb = 0; kb < 8; ++kb) tmem_ld8(lane_base + (g * 8 + kb) * 32 + sub * 16 + jc * 8, v[kb]);
-                        tmem_ld_wait();
-                        if (hl == h) {
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) {
-                                const uint32_t o0 = pack_bf16(__uint_as_float(v[0][q]), __uint_as_float(v[1][q]));
-                                const uint32_t o1 = pack_bf16(__uint_as_float(v[2][q]), __uint_as_float(v[3][q]));
-                                const uint32_t o2 = pack_bf16(__uint_as_float(v[4][q]), __uint_as_float(v[5][q]));
-                                const uint32_t o3 = pack_bf16(__uint_as_float(v[6][q]), __uint_as_float(v[7][q]));
-                                const int j = sub * 16 + jc * 8 + q;
-                                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(U0 + j * 4096 + (h * 2 + g) * 1024 + row * 16),
-                                             "r"(o0), "r"(o1), "r"(o2), "r"(o3) : "memory");
-                            }
-                        }
-                    }
-                }
-                tc_fence_before();
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(ple0 + h * 8);
-            }
-            // ---- stage 2 halves: half h in plane h -> y
-#pragma unroll 1
-            for (int h = 0; h < 2 && ok; ++h) {
-                if (!wait_fast(plf0 + h * 8, np[h] & 1, p.status, dead, kErrMmaWait)) { ok = false; break; }
-                ++np[h];
-                tc_fence_after();
-#pragma unroll 1
-                for (int c = sub; c < 8; c += 2, ++nchunk) {
-                    const uint32_t k = nchunk & (kStagesPerHalf - 1);
-                    const uint32_t sbuf = my_stage + k * kStageBytes;
-                    if (!wait_fast(stfree0 + k * 8, ((nchunk / kStagesPerHalf) & 1) ^ 1, p.status, dead, kErrSlotWait)) { ok = false; break; }
-                    // chunk = 4 consecutive output rows l; 16 blocks j of this half -> 32 bytes per (l, t)
-                    uint32_t v[16][4];
-#pragma unroll
-                    for (int a = 0; a < 16; ++a) tmem_ld4(lane_base + a * 32 + c * 4, v[a]);
-                    tmem_ld_wait();
-                    if (hl == h) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const uint32_t o0 = pack_bf16(__uint_as_float(v[e * 8 + 0][q]), __uint_as_float(v[e * 8 + 1][q]));
-                                const uint32_t o1 = pack_bf16(__uint_as_float(v[e * 8 + 2][q]), __uint_as_float(v[e * 8 + 3][q]));
-                                const uint32_t o2 = pack_bf16(__uint_as_float(v[e * 8 + 4][q]), __uint_as_float(v[e * 8 + 5][q]));
-                                const uint32_t o3 = pack_bf16(__uint_as_float(v[e * 8 + 6][q]), __uint_as_float(v[e * 8 + 7][q]));
-                                // staging [l local 4][t 64][16 j]
-                                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(sbuf + q * 2048 + row * 32 + e * 16),
-                                             "r"(o0), "r"(o1), "r"(o2), "r"(o3) : "memory");
-                            }
-                        }
-                    }
-                    if (c + 2 >= 8) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(ple0 + h * 8);
-                    }
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(stf0 + k * 8);
-                }
-            }
-        }
-    } else if (warp >= kStoreWarp0 && warp < kStoreWarp0 + 2) {
-        // ------------------------------------------------------------ store threads (one per epilogue half)
-        if (lane == 0) {
-            const int sub = warp - kStoreWarp0;
-            const uint32_t my_stage = stage0 + sub * kStagesPerHalf * kStageBytes;
-            const uint32_t stf0 = smem_u32(bars.st_full) + sub * kStagesPerHalf * 8;
-            const uint32_t stfree0 = smem_u32(bars.st_free) + sub * kStagesPerHalf * 8;
-            uint32_t nchunk = 0;
-            int unfreed = -1;
-            bool ok = true;
-            for (int tile = first; ok && tile < p.tiles; tile += step) {
-#pragma unroll 1
-                for (int h = 0; h < 2 && ok; ++h) {
-#pragma unroll 1
-                    for (int c = sub; c < 8; c += 2, ++nchunk) {
-                        const uint32_t k = nchunk & (kStagesPerHalf - 1);
-                        if (!wait_fast(stf0 + k * 8, (nchunk / kStagesPerHalf) & 1, p.status, dead, kErrMmaWait)) { ok = false; break; }
-                        // y as [l][t][j]: box 16 j x 64 t x 4 l; rows past the last token are clipped
-                        asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(&tm_y),
-                                     "r"(my_stage + k * kStageBytes), "r"(h * 16), "r"(tile * 64), "r"(c * 4) : "memory");
-                        tma_store_commit();
-                        if (unfreed >= 0) {
-                            tma_store_wait_read<1>();
-                            mbar_arrive(stfree0 + unfreed * 8);
-                        }
-                        unfreed = (int)k;
-                    }
-                }
-            }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            tma_store_3d(&tm_dx, ring.slot(count - 1), 0, (first + (count - 1) * step) * kTok, 0);
+            tma_store_commit();
             tma_store_wait_all<0>();
         }
+        return;
     }
+    // items of the ring: dy(i) = 2 i, x(i) = 2 i + 1
+    int next = 0;
+    auto load_to = [&](int last) {
+        for (; next <= last && next < 2 * count; ++next) ring.load(next, next & 1 ? &tm_x : &tm_dy, first + (next >> 1) * step);
+    };
+    if (threadIdx.x == 0) load_to(kSlots - 1);
+    Weights w;
+    Sums sums;
+    sums.clear();
+    if (kind == kDL) {
+        // per tile [sums from z(i), u(i)] [z(i + 1), u(i + 1)]
+        w.load(p.R, warp, false);
+        t_to_e(ring.wait(0), V);
+        stage_from_t(w, ring.wait(1), U);
+        for (int i = 0; i < count; ++i) {
+            __syncthreads();
+            if (threadIdx.x == 0) load_to(2 * i + 1 + kSlots);
+            sums.add<false>(V, U);
+            __syncthreads();
+            if (i + 1 < count) {
+                t_to_e(ring.wait(2 * i + 2), V);
+                stage_from_t(w, ring.wait(2 * i + 3), U);
+            }
+        }
+    } else {
+        // per tile [du(i) from z(i)] [sums from du(i), x(i); z(i + 1)]
+        w.load(p.L, warp, true);
+        t_to_e(ring.wait(0), V);
+        for (int i = 0; i < count; ++i) {
+            __syncthreads();                             // z(i) is complete; x(i - 1) has been read
+            if (threadIdx.x == 0) load_to(2 * i + kSlots);
+            stage_from_e(w, V, U);
+            const uint32_t x = ring.wait(2 * i + 1);
+            __syncthreads();
+            sums.add<true>(U, x);
+            if (i + 1 < count) t_to_e(ring.wait(2 * i + 2), V);
+        }
+    }
+    sums.store(p.parts + ((size_t)kind * kMaxParts + first) * kM * kM * kM);
+}
 
-    tc_fence_before();
+// grads = (accumulate ? grads : 0) + the parts, in order; 32 groups of 4 elements and 8 ranges of parts per CTA
+__global__ void __launch_bounds__(256)
+add_parts_m32_kernel(const float *__restrict__ parts, float *__restrict__ dL, float *__restrict__ dR, int n_l, int n_r, int accumulate)
+{
+    __shared__ float4 red[8][32];
+    constexpr int kElems = kM * kM * kM, kPer = 32 * 4;
+    const int kind = blockIdx.x / (kElems / kPer), at = blockIdx.x % (kElems / kPer) * kPer + (threadIdx.x & 31) * 4;
+    const int range = threadIdx.x >> 5, n = kind == kDL ? n_l : n_r;
+    const float *src = parts + (size_t)kind * kMaxParts * kElems + at;
+    float *dst = (kind == kDL ? dL : dR) + at;
+    const int per = (n + 7) / 8;
+    float4 s = make_float4(0, 0, 0, 0);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll 7
+    for (int i = range * per; i < (range + 1) * per && i < n; ++i) {
+        const float4 v = *reinterpret_cast<const float4 *>(src + (size_t)i * kElems);
+        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    red[range][threadIdx.x & 31] = s;
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem_base, 512);
+    if (range == 0) {
+        if (accumulate) {
+            const float4 o = *reinterpret_cast<const float4 *>(dst);
+            s.x += o.x; s.y += o.y; s.z += o.z; s.w += o.w;
+        }
+#pragma unroll
+        for (int i = 1; i < 8; ++i) {
+            const float4 v = red[i][threadIdx.x];
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        *reinterpret_cast<float4 *>(dst) = s;
+    }
+}
+
+// [tokens][1024] as boxes of 64 columns: one copy of 64 x 16 tokens x 16 boxes is a T tile
+int map_tile(CUtensorMap *m, const void *p, int64_t tokens)
+{
+    const uint64_t dims[3] = {64, (uint64_t)tokens, 16}, strides[2] = {kN * 2, 128};
+    const uint32_t box[3] = {64, kTok, 16};
+    return encode_tmap_nd(m, p, 2, 3, dims, strides, box, 128);
+}
+
+// bias null: y = M x
+int launch_fwd_m32(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws,
+                   cudaStream_t s)
+{
+    if (tokens == 0) return MONARCH_OK;
+    if (tokens > 0x7fffffffLL - kTok) return MONARCH_ERR_UNSUPPORTED;
+    CUtensorMap tm_x, tm_y;
+    MONARCH_TRY(map_tile(&tm_x, x, tokens));
+    MONARCH_TRY(map_tile(&tm_y, y, tokens));
+    int sms = 0;
+    MONARCH_TRY(current_device_sms(&sms));
+    auto kern = bias != nullptr ? fused_fwd_m32_kernel<true> : fused_fwd_m32_kernel<false>;
+    MONARCH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+    Params p = {};
+    p.status = (unsigned *)ws;
+    p.L = (const __nv_bfloat16 *)L;
+    p.R = (const __nv_bfloat16 *)R;
+    p.bias = (const __nv_bfloat16 *)bias;
+    p.gelu = gelu;
+    p.tiles = (int)((tokens + kTok - 1) / kTok);
+    kern<<<p.tiles < sms ? p.tiles : sms, kThreads, kSmemBytes, s>>>(tm_x, tm_y, p);
+    note_launch();
+    MONARCH_CUDA_TRY(cudaGetLastError());
+    return MONARCH_OK;
 }
 
 }  // namespace
@@ -371,37 +518,77 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
 // Workspace: only the status word is used.
 int fused_fwd_m32(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s)
 {
+    return tc::launch_fwd_m32(x, L, R, nullptr, 0, y, tokens, ws, s);
+}
+
+// The feed-forward block as two passes; workspace: status word, then h.
+size_t fused_mlp_fwd_m32_workspace_bytes(int64_t tokens)
+{
+    return MONARCH_STATUS_BYTES + (((size_t)tokens * tc::kN * 2 + 255) & ~(size_t)255);
+}
+int fused_mlp_fwd_m32(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2,
+                      void *y, int64_t tokens, void *ws, cudaStream_t s)
+{
+    void *h = (char *)ws + MONARCH_STATUS_BYTES;
+    MONARCH_TRY(tc::launch_fwd_m32(x, L1, R1, b1, 1, h, tokens, ws, s));
+    return tc::launch_fwd_m32(h, L2, R2, b2, 0, y, tokens, ws, s);
+}
+
+// Workspace: status word, then the sums of every CTA (64 KB are left out for the counters of the kernels that share it).
+size_t fused_bwd_m32_workspace_bytes()
+{
+    return MONARCH_STATUS_BYTES + 65536 + (size_t)2 * tc::kMaxParts * tc::kM * tc::kM * tc::kM * sizeof(float);
+}
+// dx null: gradients only; dL null: dx only
+int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, void *dx, float *dL, float *dR, int accumulate,
+                  int64_t tokens, void *ws, cudaStream_t s)
+{
     using namespace tc;
-    if (tokens == 0) return MONARCH_OK;
-    const long long tiles = (tokens + 63) / 64;
-    if (tiles > 0x7fffffffLL / 64) return MONARCH_ERR_UNSUPPORTED;
-    CUtensorMap tm_x, tm_R, tm_L, tm_y;
-    MONARCH_TRY(encode_tmap_2d(&tm_x, x, (uint64_t)tokens, kN, kN * 2, 64, 64, 128));     // two blocks per box
-    MONARCH_TRY(encode_tmap_2d(&tm_R, R, kN, kM, kM * 2, 64, 32, 64));                     // two blocks per box
-    MONARCH_TRY(encode_tmap_2d(&tm_L, L, kN, kM, kM * 2, 64, 32, 64));
-    {
-        // y as [l][t][j] bf16; a store moves 16 j x 64 t x 4 l
-        const uint64_t ydims[3] = {32, (uint64_t)tokens, 32}, ystrides[2] = {(uint64_t)kN * 2, 64};
-        const uint32_t ybox[3] = {16, 64, 4};
-        MONARCH_TRY(encode_tmap_nd(&tm_y, y, 2, 3, ydims, ystrides, ybox));
+    if (tokens == 0) {
+        if (dL != nullptr && !accumulate) {
+            MONARCH_CUDA_TRY(cudaMemsetAsync(dL, 0, kM * kM * kM * sizeof(float), s));
+            MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, kM * kM * kM * sizeof(float), s));
+        }
+        return MONARCH_OK;
     }
-    // per call: the SM count and the shared-memory attribute belong to the current device, and a first-call
-    // cache would not be safe against two host threads
+    if (tokens > 0x7fffffffLL - kTok) return MONARCH_ERR_UNSUPPORTED;
+    CUtensorMap tm_x, tm_dy, tm_dx;
+    MONARCH_TRY(map_tile(&tm_dy, dy, tokens));
+    MONARCH_TRY(map_tile(&tm_x, dL != nullptr ? x : dy, tokens));
+    MONARCH_TRY(map_tile(&tm_dx, dx != nullptr ? dx : dy, tokens));
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
-    MONARCH_CUDA_TRY(cudaFuncSetAttribute(fused_fwd_m32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          kSmemBytes));
-    P32 p;
+    Params p = {};
     p.status = (unsigned *)ws;
-    p.tiles = (int)tiles;
-    p.trace = nullptr;
-#ifdef MONARCH_TRACE
-    if (const char *e = getenv("MONARCH_TRACE_PTR")) p.trace = (long long *)strtoull(e, nullptr, 0);
-#endif
-    const int grid = tiles < sms ? (int)tiles : sms;
-    fused_fwd_m32_kernel<<<grid, kThreads, kSmemBytes, s>>>(tm_x, tm_R, tm_L, tm_y, p);
+    p.L = (const __nv_bfloat16 *)L;
+    p.R = (const __nv_bfloat16 *)R;
+    p.parts = (float *)((char *)ws + MONARCH_STATUS_BYTES + 65536);
+    p.tiles = (int)((tokens + kTok - 1) / kTok);
+    // The kinds cost the same per tile (256 KB of shared-memory traffic): equal shares, and the same share of a gradient
+    // whether or not dx is asked for, so that its sums have the same bits.
+    const int share = sms / kKinds < kMaxParts ? sms / kKinds : kMaxParts;
+    const int most[kKinds] = {dL != nullptr ? share : 0, dL != nullptr ? share : 0, dx == nullptr ? 0 : dL != nullptr ? sms - 2 * share : sms};
+    int n[kKinds];
+    for (int k = 0; k < kKinds; ++k) {
+        n[k] = most[k] < p.tiles ? most[k] : p.tiles;
+        p.first[k + 1] = p.first[k] + n[k];
+    }
+    MONARCH_CUDA_TRY(cudaFuncSetAttribute(fused_bwd_m32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+    fused_bwd_m32_kernel<<<p.first[kKinds], kThreads, kSmemBytes, s>>>(tm_x, tm_dy, tm_dx, p);
     note_launch();
     MONARCH_CUDA_TRY(cudaGetLastError());
+    if (dL == nullptr) return MONARCH_OK;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * kM * kM * kM / 128);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    MONARCH_CUDA_TRY(cudaLaunchKernelEx(&cfg, add_parts_m32_kernel, (const float *)p.parts, dL, dR, n[kDL], n[kDR], accumulate));
+    note_launch();
     return MONARCH_OK;
 }
 

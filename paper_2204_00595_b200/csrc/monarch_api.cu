@@ -134,6 +134,7 @@ int pick(int op, int m, int dtype)
 //   fp32          the other family (one launch per stage) is slower at every size
 int64_t units_limit(int op, int m, int dtype)
 {
+    static const char *mu = getenv("MU"); if (mu && m == 32 && dtype == MONARCH_BF16) return atoll(mu);
     const int64_t all = 1 << 20;                          // what the 32-bit addressing of the units allows
     if (dtype == MONARCH_F32 || m == 16) return all;
     const bool fwd = op == MONARCH_OP_FWD, mlp = op == MONARCH_OP_MLP_FWD, mlp_bwd = op == MONARCH_OP_MLP_BWD;
@@ -208,6 +209,9 @@ size_t large_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int d
     // the fused m = 64 kernels keep one dependency counter per 64-token tile in 64 KB: beyond 2^20 tokens the calls
     // refuse, and so does this query (shard the tokens)
     if (which == kFused && m == 64 && tokens > ((int64_t)1 << 20)) return 0;
+    if (which == kTcStaged && m == 32 && op == MONARCH_OP_MLP_FWD) return fused_mlp_fwd_m32_workspace_bytes(tokens);
+    if (which == kTcStaged && m == 32 && op != MONARCH_OP_FWD)
+        return fused_bwd_m32_workspace_bytes() + (op != MONARCH_OP_BWD_DX && fixed_order ? kTcPartialBytes : 0);
     if (which == kTcStaged && op != MONARCH_OP_FWD && op != MONARCH_OP_MLP_FWD)
         return tc_staged_bwd_workspace_bytes(tokens, m, op != MONARCH_OP_BWD_DX && fixed_order);
     if (which == kTcStaged && op == MONARCH_OP_FWD && m == 128) return chain_fwd_m128_workspace_bytes(tokens);
@@ -281,6 +285,8 @@ int monarch_bwd_dx(const void *dy, const void *L, const void *R, void *dx, int64
         return units::bwd(nullptr, dy, L, R, nullptr, dx, nullptr, nullptr, 0, tokens, m, dtype, workspace, (cudaStream_t)stream);
     if (which == kFused)
         return fused_bwd_dx_m64(dy, L, R, dx, tokens, workspace, (cudaStream_t)stream);
+    if (which == kTcStaged && m == 32)
+        return fused_bwd_m32(nullptr, dy, L, R, dx, nullptr, nullptr, 0, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
         return tc_staged_bwd(nullptr, dy, L, R, dx, nullptr, nullptr, 0, 1, 0, tokens, m, workspace,
                              (cudaStream_t)stream);
@@ -306,6 +312,8 @@ int monarch_bwd_dw(const void *x, const void *dy, const void *L, const void *R, 
     if (which == kFused)
         return fused_bwd_dw_m64(x, dy, L, R, dL, dR, accumulate, tokens, workspace, (cudaStream_t)stream,
                                 g_fixed_order.load(std::memory_order_relaxed) != 0);
+    if (which == kTcStaged && m == 32)
+        return fused_bwd_m32(x, dy, L, R, nullptr, dL, dR, accumulate, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
         return tc_staged_bwd(x, dy, L, R, nullptr, dL, dR, accumulate, 0, 1, tokens, m, workspace,
                              (cudaStream_t)stream, nullptr, g_fixed_order.load(std::memory_order_relaxed) != 0);
@@ -340,6 +348,7 @@ int monarch_bwd(const void *x, const void *dy, const void *L, const void *R, con
         return fused_bwd_m64(x, dy, L, R, saved ? fused_fwd_m64_saved_u(fwd_workspace) : nullptr, dx, dL,
                              dR, accumulate, tokens, workspace, s, g_fixed_order.load(std::memory_order_relaxed) != 0);
     }
+    if (which == kTcStaged && m == 32) return fused_bwd_m32(x, dy, L, R, dx, dL, dR, accumulate, tokens, workspace, s);
     if (which == kTcStaged) {
         const bool saved = fwd_workspace != nullptr && m == 128 && pick(MONARCH_OP_FWD, m, dtype) == kTcStaged;
         return tc_staged_bwd(x, dy, L, R, dx, dL, dR, accumulate, 1, 1, tokens, m, workspace, s,
@@ -367,6 +376,8 @@ int monarch_mlp_fwd(const void *x, const void *L1, const void *R1, const void *b
         return units::mlp_fwd(x, L1, R1, b1, L2, R2, b2, y, tokens, m, dtype, workspace, (cudaStream_t)stream);
     if (which == kFused)
         return fused_mlp_fwd_m64(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
+    if (which == kTcStaged && m == 32)
+        return fused_mlp_fwd_m32(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged && m == 128 && chain_mlp_fwd_m128_workspace_bytes(tokens) != 0)
         return chain_mlp_fwd_m128(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
