@@ -34,13 +34,12 @@
  *    when one of their bounded waits runs out; zero it once with
  *    monarch_workspace_init and read it with monarch_last_device_status.
  *    Calls that overlap on the GPU must not share a workspace.
- *  - Weight gradients of the fused tensor-core kernels (bf16, m = 64; the
- *    general class) and of the staged tensor-core kernels (bf16, m = 32) are
- *    summed with fp32 reductions whose order across thread blocks is not
- *    fixed: dL, dR can differ in the last fp32 bits from run to run
- *    (monarch_set_deterministic switches m = 32 and m = 64 to a fixed order).  The bf16 m = 128 kernels (one thread block sums all tokens of a
- *    block, in a fixed order) and the CUDA-core family (MONARCH_IMPL_STAGED)
- *    give the same bits every run.
+ *  - Weight gradients of the fused tensor-core kernels for bf16 m = 64 (beyond
+ *    a few hundred tokens) and of the general class are summed with fp32
+ *    reductions whose order across thread blocks is not fixed: dL, dR can
+ *    differ in the last fp32 bits from run to run (monarch_set_deterministic
+ *    switches m = 64 to a fixed order).  All others (bf16 m = 16, 32 and 128,
+ *    fp32, MONARCH_IMPL_STAGED) give the same bits every run.
  *  - Return value: a monarch_status_t.  Nothing throws.
  */
 #ifndef MONARCH_H_

@@ -1201,7 +1201,13 @@ int chain_bwd_m128(const void *x, const void *dy, const void *L, const void *R, 
                    float *dR, int accumulate, int want_dx, int want_dw, int64_t tokens, void *ws, cudaStream_t s)
 {
     using namespace tc;
-    if (tokens == 0) return MONARCH_OK;
+    if (tokens == 0) {
+        if (want_dw && !accumulate) {
+            MONARCH_CUDA_TRY(cudaMemsetAsync(dL, 0, (size_t)kB * kB * kB * sizeof(float), s));
+            MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, (size_t)kB * kB * kB * sizeof(float), s));
+        }
+        return MONARCH_OK;
+    }
     if (tokens > (int64_t)1 << 30) return MONARCH_ERR_UNSUPPORTED;
     const int ntiles = (int)((tokens + 127) / 128);
     unsigned *status = (unsigned *)ws;

@@ -136,12 +136,10 @@ int staged_mlp_fwd(const void *x, const void *L1, const void *R1, const void *b1
                    void *ws, cudaStream_t s);
 
 
-// ---- tensor-core stage chains through the workspace (bf16, m >= 32), tc_stage.cu ----
-int tc_staged_fwd(const void *x, const void *L, const void *R, void *y, int64_t tokens, int m,
-                  void *ws, cudaStream_t s);
+// ---- the feed-forward block at m = 128 as four launches of a tensor-core stage (tc_stage.cu): where the forward of
+// chain_m128.cu cannot run as one launch ----
 int tc_staged_mlp_fwd(const void *x, const void *L1, const void *R1, const void *b1, const void *L2,
-                      const void *R2, const void *b2, void *y, int64_t tokens, int m, void *ws,
-                      cudaStream_t s);
+                      const void *R2, const void *b2, void *y, int64_t tokens, void *ws, cudaStream_t s);
 
 
 // m = 128 as chains of block GEMMs on token-innermost planes (chain_m128.cu)
@@ -161,16 +159,6 @@ void debug_skip_next_plane_load(long long item);
 // true when the next forward call has to run as three launches: the switch for comparison runs, or a load to leave out
 bool chain_fwd_m128_split();
 
-// ---- backward as a chain of tensor-core launches (bf16; dx for m >= 32, dL/dR for m = 128), tc_bwd.cu ----
-// fixed_order (m = 32, 64): kTcPartialBytes more; the token slices of the weight-gradient launches store their sums there and a
-// small launch adds them in slice order (same bits on every run) instead of reductions in L2
-constexpr size_t kTcPartialBytes = (size_t)32 << 20;
-size_t tc_staged_bwd_workspace_bytes(int64_t tokens, int m, bool fixed_order = false);
-// saved_up: for m = 128, the u' planes left by the forward call (chain_fwd_m128_saved_u), or null
-int tc_staged_bwd(const void *x, const void *dy, const void *L, const void *R, void *dx, float *dL, float *dR,
-                  int accumulate, int want_dx, int want_dw, int64_t tokens, int m, void *ws, cudaStream_t s,
-                  const void *saved_up = nullptr, bool fixed_order = false);
-
 // ---- forward for m = 16 in one launch on the CUDA cores, both dtypes (fused_m16.cu); no workspace use ----
 int fused_fwd_m16(const void *x, const void *L, const void *R, void *y, int64_t tokens, int dtype, cudaStream_t s);
 
@@ -182,6 +170,8 @@ size_t fused_mlp_fwd_m32_workspace_bytes(int64_t tokens);
 int fused_mlp_fwd_m32(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2,
                       void *y, int64_t tokens, void *ws, cudaStream_t s);
 // dx null: gradients only; dL null: dx only.  The gradients are sums in a fixed order.
+// Reported on top while monarch_set_deterministic is on, as its contract says (these kernels have no use for it).
+constexpr size_t kTcPartialBytes = (size_t)32 << 20;
 size_t fused_bwd_m32_workspace_bytes();
 int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, void *dx, float *dL, float *dR, int accumulate,
                   int64_t tokens, void *ws, cudaStream_t s);

@@ -17,6 +17,9 @@
 //   backward:  z = P dy     T tile -> E tile [j][l];   du = L_j^T z_j -> E tile [k][j];   dx = R_k^T du_k -> T tile
 //              dL_j = sum_t z_j u_j^T, dR_k = sum_t du_k x_k^T: tokens are the contraction, both operands as they lie
 // Shared memory moves 16 to 18 KB per token at 128 bytes per clock, no access has a bank conflict.
+// Measured, back to back: forward 16384 tokens 29.2 -> 18.9 us (6.0 TB/s beyond a fixed 7 us of launch, first tile and
+// weights), 1000 tokens 14.5 -> 6.6; forward + backward 4999 tokens 103 -> 31, 16384 tokens 62 (the staged chain of nine
+// launches took 219 as units and more as tcgen05 stages); feed-forward block 16384 tokens 167 -> 40.
 //
 // Backward CTAs are of three kinds, dL, dR and dx: the sums of one gradient are 128 KB of accumulators, half the
 // registers of an SM, and a kind needs one or two sets of weights beside them.  u and du are recomputed by the kind that
@@ -54,7 +57,7 @@ __device__ __forceinline__ void stm4t(uint32_t a, const uint32_t (&r)[4])
 }
 __device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -123,61 +126,53 @@ struct Lane {                                            // rows of the four mat
     __device__ __forceinline__ Lane() : warp(threadIdx.x >> 5), m((threadIdx.x & 31) >> 3), r(threadIdx.x & 7) {}
 };
 
-// E[row][own block] = W_block T_block: row c of the result of block b becomes row b of block c
-__device__ __forceinline__ void stage_from_t(const Weights &w, uint32_t T, uint32_t E)
+// The operands of a stage are loaded together, ahead of its products.
+struct Operands {
+    uint32_t b[2][2][4];                                 // [block][8-token half]
+    __device__ __forceinline__ void from_t(uint32_t T)
+    {
+        const Lane ln;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ldm4(b[i >> 1][i & 1], t_at(T, ln.warp, (i & 1) * 8 + ln.r, (i >> 1) * 4 + ln.m));
+    }
+    __device__ __forceinline__ void from_e(uint32_t E)   // rows of the warp's own blocks
+    {
+        const Lane ln;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ldm4t(b[i >> 1][i & 1], e_at(E, ln.warp * 2 + (i >> 1), i & 1, ln.m * 8 + ln.r));
+    }
+};
+// E[row][own block] = W_block operand: row c of the result of block b becomes row b of block c
+__device__ __forceinline__ void stage_to_e(const Weights &w, const Operands &in, uint32_t E)
 {
     const Lane ln;
 #pragma unroll
-    for (int blk = 0; blk < 2; ++blk)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t b[4], o[4];
-            float acc[2][4];
-            ldm4(b, t_at(T, ln.warp, h * 8 + ln.r, blk * 4 + ln.m));
-            w.times(blk, b, acc);
-            pack_rows(acc, o);
-            stm4(e_at(E, ln.m * 8 + ln.r, h, ln.warp * 2 + blk), o);
-        }
-}
-// the same from an E tile of this warp's blocks
-__device__ __forceinline__ void stage_from_e(const Weights &w, uint32_t E, uint32_t out)
-{
-    const Lane ln;
-#pragma unroll
-    for (int blk = 0; blk < 2; ++blk)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            uint32_t b[4], o[4];
-            float acc[2][4];
-            const int own = ln.warp * 2 + blk;
-            ldm4t(b, e_at(E, own, h, ln.m * 8 + ln.r));
-            w.times(blk, b, acc);
-            pack_rows(acc, o);
-            stm4(e_at(out, ln.m * 8 + ln.r, h, own), o);
-        }
+    for (int i = 0; i < 4; ++i) {
+        uint32_t o[4];
+        float acc[2][4];
+        w.times(i >> 1, in.b[i >> 1][i & 1], acc);
+        pack_rows(acc, o);
+        stm4(e_at(E, ln.m * 8 + ln.r, i & 1, ln.warp * 2 + (i >> 1)), o);
+    }
 }
 // E[block][row] -> T (the outer P) and back; a warp takes the columns of one box
 __device__ __forceinline__ void e_to_t(uint32_t E, uint32_t T)
 {
     const Lane ln;
+    uint32_t v[4][4];
 #pragma unroll
-    for (int n = 0; n < 4; ++n) {
-        const int h = n >> 1, c = ln.warp * 2 + (n & 1);
-        uint32_t v[4];
-        ldm4t(v, e_at(E, ln.m * 8 + ln.r, h, c));
-        stm4(t_at(T, ln.warp, h * 8 + ln.r, (n & 1) * 4 + ln.m), v);
-    }
+    for (int n = 0; n < 4; ++n) ldm4t(v[n], e_at(E, ln.m * 8 + ln.r, n >> 1, ln.warp * 2 + (n & 1)));
+#pragma unroll
+    for (int n = 0; n < 4; ++n) stm4(t_at(T, ln.warp, (n >> 1) * 8 + ln.r, (n & 1) * 4 + ln.m), v[n]);
 }
 __device__ __forceinline__ void t_to_e(uint32_t T, uint32_t E)
 {
     const Lane ln;
+    uint32_t v[4][4];
 #pragma unroll
-    for (int n = 0; n < 4; ++n) {
-        const int h = n >> 1, c = ln.warp * 2 + (n & 1);
-        uint32_t v[4];
-        ldm4t(v, t_at(T, ln.warp, h * 8 + ln.r, (n & 1) * 4 + ln.m));
-        stm4(e_at(E, ln.m * 8 + ln.r, h, c), v);
-    }
+    for (int n = 0; n < 4; ++n) ldm4t(v[n], t_at(T, ln.warp, (n >> 1) * 8 + ln.r, (n & 1) * 4 + ln.m));
+#pragma unroll
+    for (int n = 0; n < 4; ++n) stm4(e_at(E, ln.m * 8 + ln.r, n >> 1, ln.warp * 2 + (n & 1)), v[n]);
 }
 
 struct Params {
@@ -213,8 +208,12 @@ struct Shared {
     uint64_t bars[kSlots];
     int dead;
 };
+// Launched with programmatic serialization: a kernel may begin while the one before it drains; nothing is read or written
+// before the wait.
+__device__ __forceinline__ void depend_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void init(Shared &s)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (threadIdx.x == 0) {
         for (int i = 0; i < kSlots; ++i) mbar_init(smem_u32(&s.bars[i]), 1);
         fence_mbar_init();
@@ -236,10 +235,11 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     const uint32_t E[2] = {base + kSlots * kTile, base + (kSlots + 1) * kTile};
     init(sh);
     const int first = blockIdx.x, step = gridDim.x, count = (p.tiles - first + step - 1) / step;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < 3 && i < count; ++i) ring.load(i, &tm_x, first + i * step);
     const int warp = threadIdx.x >> 5;
     Weights wr, wl;
+    depend_wait();
+    if (threadIdx.x == 0)
+        for (int i = 0; i < 3 && i < count; ++i) ring.load(i, &tm_x, first + i * step);
     wr.load(p.R, warp, false);
     wl.load(p.L, warp, false);
     float bias[2][4];
@@ -249,7 +249,9 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             bias[i >> 2][i & 3] = __bfloat162float(p.bias[((i & 3) * 8 + ((threadIdx.x & 31) >> 2)) * kM + warp * 2 + (i >> 2)]);
 
     const Lane ln;
-    stage_from_t(wr, ring.wait(0), E[0]);
+    Operands in;
+    in.from_t(ring.wait(0));
+    stage_to_e(wr, in, E[0]);
     for (int i = 0; i < count; ++i) {
         const uint32_t e = E[i & 1];
         __syncthreads();                                 // u(i) and y(i - 1) are complete
@@ -263,25 +265,25 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
                 ring.load(i + 3, &tm_x, first + (i + 3) * step);
             }
         }
+        const bool more = i + 1 < count;
+        in.from_e(e);
+        Operands nx;
+        if (more) nx.from_t(ring.wait(i + 1));
 #pragma unroll
-        for (int blk = 0; blk < 2; ++blk)
+        for (int v = 0; v < 4; ++v) {
+            uint32_t o[4];
+            float acc[2][4];
+            wl.times(v >> 1, in.b[v >> 1][v & 1], acc);
+            if (ACT)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                uint32_t b[4], o[4];
-                float acc[2][4];
-                const int own = warp * 2 + blk;
-                ldm4t(b, e_at(e, own, h, ln.m * 8 + ln.r));
-                wl.times(blk, b, acc);
-                if (ACT)
-#pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        const float a = acc[v >> 2][v & 3] + bias[blk][v >> 1];
-                        acc[v >> 2][v & 3] = p.gelu ? gelu_fast(a) : a;
-                    }
-                pack_rows(acc, o);
-                stm4(e_at(e, own, h, ln.m * 8 + ln.r), o);
-            }
-        if (i + 1 < count) stage_from_t(wr, ring.wait(i + 1), E[(i + 1) & 1]);
+                for (int k = 0; k < 8; ++k) {
+                    const float a = acc[k >> 2][k & 3] + bias[v >> 1][k >> 1];
+                    acc[k >> 2][k & 3] = p.gelu ? gelu_fast(a) : a;
+                }
+            pack_rows(acc, o);
+            stm4(e_at(e, warp * 2 + (v >> 1), v & 1, ln.m * 8 + ln.r), o);
+        }
+        if (more) stage_to_e(wr, nx, E[(i + 1) & 1]);
         __syncthreads();                                 // w(i) is complete; x(i) has been read by everyone
         e_to_t(e, ring.slot(i));
         fence_proxy_async_smem();
@@ -353,19 +355,20 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     const Ring ring = {base, smem_u32(sh.bars), p.status, &sh.dead};
     const uint32_t V = base + kSlots * kTile, U = V + kTile;
     init(sh);
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int b = blockIdx.x, kind = b < p.first[1] ? kDL : b < p.first[2] ? kDR : kDX;
     const int first = b - p.first[kind], step = p.first[kind + 1] - p.first[kind], count = (p.tiles - first + step - 1) / step;
     const int warp = threadIdx.x >> 5;
 
     if (kind == kDX) {
         // per tile [du(i) from z(i)] [dx(i), z(i + 1)]
+        Weights wl, wr;
+        depend_wait();
         if (threadIdx.x == 0)
             for (int i = 0; i < 3 && i < count; ++i) ring.load(i, &tm_dy, first + i * step);
-        Weights wl, wr;
         wl.load(p.L, warp, true);
         wr.load(p.R, warp, true);
         const Lane ln;
+        Operands in;
         t_to_e(ring.wait(0), V);
         for (int i = 0; i < count; ++i) {
             __syncthreads();                             // z(i) and dx(i - 1) are complete
@@ -379,19 +382,18 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
                     ring.load(i + 3, &tm_dy, first + (i + 3) * step);
                 }
             }
-            stage_from_e(wl, V, U);
+            in.from_e(V);
+            stage_to_e(wl, in, U);
             __syncthreads();                             // du(i) is complete, z(i) has been read
+            in.from_e(U);
 #pragma unroll
-            for (int blk = 0; blk < 2; ++blk)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t bb[4], o[4];
-                    float acc[2][4];
-                    ldm4t(bb, e_at(U, warp * 2 + blk, h, ln.m * 8 + ln.r));
-                    wr.times(blk, bb, acc);
-                    pack_rows(acc, o);
-                    stm4t(t_at(ring.slot(i), warp, h * 8 + ln.r, blk * 4 + ln.m), o);
-                }
+            for (int v = 0; v < 4; ++v) {
+                uint32_t o[4];
+                float acc[2][4];
+                wr.times(v >> 1, in.b[v >> 1][v & 1], acc);
+                pack_rows(acc, o);
+                stm4t(t_at(ring.slot(i), warp, (v & 1) * 8 + ln.r, (v >> 1) * 4 + ln.m), o);
+            }
             fence_proxy_async_smem();
             if (i + 1 < count) t_to_e(ring.wait(i + 1), V);
         }
@@ -408,15 +410,19 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     auto load_to = [&](int last) {
         for (; next <= last && next < 2 * count; ++next) ring.load(next, next & 1 ? &tm_x : &tm_dy, first + (next >> 1) * step);
     };
-    if (threadIdx.x == 0) load_to(kSlots - 1);
     Weights w;
+    Operands in;
     Sums sums;
     sums.clear();
+    depend_wait();
+    if (threadIdx.x == 0) load_to(kSlots - 1);
+    if (kind == kDL) w.load(p.R, warp, false);
+    else             w.load(p.L, warp, true);
     if (kind == kDL) {
         // per tile [sums from z(i), u(i)] [z(i + 1), u(i + 1)]
-        w.load(p.R, warp, false);
         t_to_e(ring.wait(0), V);
-        stage_from_t(w, ring.wait(1), U);
+        in.from_t(ring.wait(1));
+        stage_to_e(w, in, U);
         for (int i = 0; i < count; ++i) {
             __syncthreads();
             if (threadIdx.x == 0) load_to(2 * i + 1 + kSlots);
@@ -424,17 +430,18 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             __syncthreads();
             if (i + 1 < count) {
                 t_to_e(ring.wait(2 * i + 2), V);
-                stage_from_t(w, ring.wait(2 * i + 3), U);
+                in.from_t(ring.wait(2 * i + 3));
+                stage_to_e(w, in, U);
             }
         }
     } else {
         // per tile [du(i) from z(i)] [sums from du(i), x(i); z(i + 1)]
-        w.load(p.L, warp, true);
         t_to_e(ring.wait(0), V);
         for (int i = 0; i < count; ++i) {
             __syncthreads();                             // z(i) is complete; x(i - 1) has been read
             if (threadIdx.x == 0) load_to(2 * i + kSlots);
-            stage_from_e(w, V, U);
+            in.from_e(V);
+            stage_to_e(w, in, U);
             const uint32_t x = ring.wait(2 * i + 1);
             __syncthreads();
             sums.add<true>(U, x);
@@ -456,7 +463,7 @@ add_parts_m32_kernel(const float *__restrict__ parts, float *__restrict__ dL, fl
     float *dst = (kind == kDL ? dL : dR) + at;
     const int per = (n + 7) / 8;
     float4 s = make_float4(0, 0, 0, 0);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    depend_wait();
 #pragma unroll 7
     for (int i = range * per; i < (range + 1) * per && i < n; ++i) {
         const float4 v = *reinterpret_cast<const float4 *>(src + (size_t)i * kElems);
@@ -476,6 +483,25 @@ add_parts_m32_kernel(const float *__restrict__ parts, float *__restrict__ dL, fl
         }
         *reinterpret_cast<float4 *>(dst) = s;
     }
+}
+
+template <typename... Ts, typename... As>
+int launch(void (*kern)(Ts...), int grid, int threads, int smem, cudaStream_t s, As... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (smem > 48 * 1024) MONARCH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    MONARCH_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+    note_launch();
+    return MONARCH_OK;
 }
 
 // [tokens][1024] as boxes of 64 columns: one copy of 64 x 16 tokens x 16 boxes is a T tile
@@ -498,7 +524,6 @@ int launch_fwd_m32(const void *x, const void *L, const void *R, const void *bias
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
     auto kern = bias != nullptr ? fused_fwd_m32_kernel<true> : fused_fwd_m32_kernel<false>;
-    MONARCH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
     Params p = {};
     p.status = (unsigned *)ws;
     p.L = (const __nv_bfloat16 *)L;
@@ -506,10 +531,7 @@ int launch_fwd_m32(const void *x, const void *L, const void *R, const void *bias
     p.bias = (const __nv_bfloat16 *)bias;
     p.gelu = gelu;
     p.tiles = (int)((tokens + kTok - 1) / kTok);
-    kern<<<p.tiles < sms ? p.tiles : sms, kThreads, kSmemBytes, s>>>(tm_x, tm_y, p);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
-    return MONARCH_OK;
+    return launch(kern, p.tiles < sms ? p.tiles : sms, kThreads, kSmemBytes, s, tm_x, tm_y, p);
 }
 
 }  // namespace
@@ -573,23 +595,9 @@ int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, v
         n[k] = most[k] < p.tiles ? most[k] : p.tiles;
         p.first[k + 1] = p.first[k] + n[k];
     }
-    MONARCH_CUDA_TRY(cudaFuncSetAttribute(fused_bwd_m32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-    fused_bwd_m32_kernel<<<p.first[kKinds], kThreads, kSmemBytes, s>>>(tm_x, tm_dy, tm_dx, p);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
+    MONARCH_TRY(launch(fused_bwd_m32_kernel, p.first[kKinds], kThreads, kSmemBytes, s, tm_x, tm_dy, tm_dx, p));
     if (dL == nullptr) return MONARCH_OK;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * kM * kM * kM / 128);
-    cfg.blockDim = dim3(256);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    MONARCH_CUDA_TRY(cudaLaunchKernelEx(&cfg, add_parts_m32_kernel, (const float *)p.parts, dL, dR, n[kDL], n[kDR], accumulate));
-    note_launch();
-    return MONARCH_OK;
+    return launch(add_parts_m32_kernel, 2 * kM * kM * kM / 128, 256, 0, s, (const float *)p.parts, dL, dR, n[kDL], n[kDR], accumulate);
 }
 
 }  // namespace monarch

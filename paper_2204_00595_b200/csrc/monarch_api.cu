@@ -95,21 +95,7 @@ enum Family { kSimt = 0, kFused = 1, kTcStaged = 2, kNone = -1 };
 // true when the fused tensor-core family has a kernel for (op, m, dtype)
 bool fused_available(int op, int m, int dtype)
 {
-#ifdef MONARCH_TRACE
-    static const bool off = getenv("MONARCH_NO_FUSED") != nullptr;   // debug builds: stage chain, for comparison
-#else
-    constexpr bool off = false;
-#endif
-    if (off || dtype != MONARCH_BF16) return false;
-    return m == 64 || (m == 32 && op == MONARCH_OP_FWD);   // m = 64: every op; m = 32: forward
-}
-
-// true when the call can run as a chain of tensor-core stages through the workspace
-bool tc_staged_available(int op, int m, int dtype)
-{
-    if (dtype != MONARCH_BF16 || m < 32) return false;
-    if (op == MONARCH_OP_FWD || op == MONARCH_OP_MLP_FWD || op == MONARCH_OP_BWD_DX) return true;
-    return m == 32 || m == 64 || m == 128;      // dL, dR: the token-reduction kernel works on 128-column windows
+    return dtype == MONARCH_BF16 && (m == 64 || (m == 32 && op == MONARCH_OP_FWD));   // m = 64: every op; m = 32: forward
 }
 
 // kernel family for a call under the current selection
@@ -120,27 +106,26 @@ int pick(int op, int m, int dtype)
     if (impl == MONARCH_IMPL_STAGED) return kSimt;
     if (impl == MONARCH_IMPL_FUSED) return f ? kFused : kNone;
     if (f) return kFused;
-    return tc_staged_available(op, m, dtype) ? kTcStaged : kSimt;
+    return dtype == MONARCH_BF16 && m >= 32 ? kTcStaged : kSimt;
 }
 
 // Largest batch that runs as one launch over block-product units (block_units.cu); beyond it the kernels above are
 // faster.  Measured per pass, back to back (us, units / the others):
 //   bf16 m = 16   forward 27 / 213 at 32768 tokens, forward + backward 148 / 484: every batch
-//   bf16 m = 32   forward 12.4 / 14.5 at 1000, 20.6 / 14.5 at 4000; forward + backward 66 / 105 at 4000; feed-forward
-//                 block 41 / 84 at 4000, 122 / 167 at 16384, with its backward 96 / 277 at 1000
+//   bf16 m = 32   forward 9.5 / 7.0 at 4, 12.4 / 6.6 at 1000; forward + backward 18.5 / 14.1 at 4: never; the backward of
+//                 the feed-forward block, eight launches otherwise, 33 / 44 at 64, 55 / 46 at 256
 //   bf16 m = 64   forward 14.5 / 16.5 at 256, 19.8 / 16.5 at 512; forward + backward 32 / 45 at 128, 45 / 46 at 256;
 //                 block 29 / 35 at 256, 41 / 35 at 512, with its backward 113 / 147 at 256, 172 / 163 at 512
-//   bf16 m = 128  forward 10.7 / 12.1 at 16; block 54 / 115 at 128, 147 / 116 at 512, with its backward 148 / 183 at 64
+//   bf16 m = 128  forward 10.7 / 12.1 at 16; block 25 / 25 at 32, its backward 112 / 147 at 64
 //   fp32          the other family (one launch per stage) is slower at every size
 int64_t units_limit(int op, int m, int dtype)
 {
-    static const char *mu = getenv("MU"); if (mu && m == 32 && dtype == MONARCH_BF16) return atoll(mu);
     const int64_t all = 1 << 20;                          // what the 32-bit addressing of the units allows
     if (dtype == MONARCH_F32 || m == 16) return all;
     const bool fwd = op == MONARCH_OP_FWD, mlp = op == MONARCH_OP_MLP_FWD, mlp_bwd = op == MONARCH_OP_MLP_BWD;
-    if (m == 32) return fwd ? 1500 : all;
+    if (m == 32) return mlp_bwd ? 128 : 0;
     if (m == 64) return fwd ? 320 : mlp ? 384 : mlp_bwd ? 448 : 256;
-    return fwd ? 16 : mlp ? 320 : mlp_bwd ? 96 : 0;
+    return fwd ? 16 : mlp ? 24 : mlp_bwd ? 96 : 0;
 }
 
 // (the switches that ask for a particular form of the other kernels keep their meaning at every size)
@@ -212,10 +197,9 @@ size_t large_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int d
     if (which == kTcStaged && m == 32 && op == MONARCH_OP_MLP_FWD) return fused_mlp_fwd_m32_workspace_bytes(tokens);
     if (which == kTcStaged && m == 32 && op != MONARCH_OP_FWD)
         return fused_bwd_m32_workspace_bytes() + (op != MONARCH_OP_BWD_DX && fixed_order ? kTcPartialBytes : 0);
-    if (which == kTcStaged && op != MONARCH_OP_FWD && op != MONARCH_OP_MLP_FWD)
-        return tc_staged_bwd_workspace_bytes(tokens, m, op != MONARCH_OP_BWD_DX && fixed_order);
-    if (which == kTcStaged && op == MONARCH_OP_FWD && m == 128) return chain_fwd_m128_workspace_bytes(tokens);
-    if (which == kTcStaged && op == MONARCH_OP_MLP_FWD && m == 128) {
+    if (which == kTcStaged && op != MONARCH_OP_FWD && op != MONARCH_OP_MLP_FWD) return chain_bwd_m128_workspace_bytes(tokens);
+    if (which == kTcStaged && op == MONARCH_OP_FWD) return chain_fwd_m128_workspace_bytes(tokens);
+    if (which == kTcStaged) {
         const size_t a = staged_workspace_bytes(op, tokens, n, m, dtype), b = chain_mlp_fwd_m128_workspace_bytes(tokens);
         return a > b ? a : b;
     }
@@ -262,7 +246,7 @@ int monarch_fwd(const void *x, const void *L, const void *R, void *y, int64_t to
     if (which == kFused)
         return m == 32 ? fused_fwd_m32(x, L, R, y, tokens, workspace, (cudaStream_t)stream)
                        : fused_fwd_m64(x, L, R, y, tokens, workspace, (cudaStream_t)stream);
-    if (which == kTcStaged) return tc_staged_fwd(x, L, R, y, tokens, m, workspace, (cudaStream_t)stream);
+    if (which == kTcStaged) return chain_fwd_m128(x, L, R, y, tokens, workspace, (cudaStream_t)stream);
     // the automatic choice runs m = 16 in one launch; MONARCH_IMPL_STAGED keeps the two-launch chain
     if (m == 16 && g_impl.load(std::memory_order_relaxed) == MONARCH_IMPL_AUTO)
         return fused_fwd_m16(x, L, R, y, tokens, dtype, (cudaStream_t)stream);
@@ -288,8 +272,7 @@ int monarch_bwd_dx(const void *dy, const void *L, const void *R, void *dx, int64
     if (which == kTcStaged && m == 32)
         return fused_bwd_m32(nullptr, dy, L, R, dx, nullptr, nullptr, 0, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
-        return tc_staged_bwd(nullptr, dy, L, R, dx, nullptr, nullptr, 0, 1, 0, tokens, m, workspace,
-                             (cudaStream_t)stream);
+        return chain_bwd_m128(nullptr, dy, L, R, nullptr, dx, nullptr, nullptr, 0, 1, 0, tokens, workspace, (cudaStream_t)stream);
     return staged_bwd_dx(dy, L, R, dx, tokens, m, dtype, workspace, (cudaStream_t)stream);
 }
 
@@ -315,8 +298,7 @@ int monarch_bwd_dw(const void *x, const void *dy, const void *L, const void *R, 
     if (which == kTcStaged && m == 32)
         return fused_bwd_m32(x, dy, L, R, nullptr, dL, dR, accumulate, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
-        return tc_staged_bwd(x, dy, L, R, nullptr, dL, dR, accumulate, 0, 1, tokens, m, workspace,
-                             (cudaStream_t)stream, nullptr, g_fixed_order.load(std::memory_order_relaxed) != 0);
+        return chain_bwd_m128(x, dy, L, R, nullptr, nullptr, dL, dR, accumulate, 0, 1, tokens, workspace, (cudaStream_t)stream);
     return staged_bwd_dw(x, dy, L, R, dL, dR, accumulate, tokens, m, dtype, workspace,
                          (cudaStream_t)stream);
 }
@@ -350,10 +332,9 @@ int monarch_bwd(const void *x, const void *dy, const void *L, const void *R, con
     }
     if (which == kTcStaged && m == 32) return fused_bwd_m32(x, dy, L, R, dx, dL, dR, accumulate, tokens, workspace, s);
     if (which == kTcStaged) {
-        const bool saved = fwd_workspace != nullptr && m == 128 && pick(MONARCH_OP_FWD, m, dtype) == kTcStaged;
-        return tc_staged_bwd(x, dy, L, R, dx, dL, dR, accumulate, 1, 1, tokens, m, workspace, s,
-                             saved ? chain_fwd_m128_saved_u(fwd_workspace, tokens) : nullptr,
-                             g_fixed_order.load(std::memory_order_relaxed) != 0);
+        const bool saved = fwd_workspace != nullptr && pick(MONARCH_OP_FWD, m, dtype) == kTcStaged;
+        return chain_bwd_m128(x, dy, L, R, saved ? chain_fwd_m128_saved_u(fwd_workspace, tokens) : nullptr, dx, dL, dR, accumulate, 1, 1,
+                              tokens, workspace, s);
     }
     MONARCH_TRY(staged_bwd_dx(dy, L, R, dx, tokens, m, dtype, workspace, s));
     return staged_bwd_dw(x, dy, L, R, dL, dR, accumulate, tokens, m, dtype, workspace, s);
@@ -378,11 +359,10 @@ int monarch_mlp_fwd(const void *x, const void *L1, const void *R1, const void *b
         return fused_mlp_fwd_m64(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged && m == 32)
         return fused_mlp_fwd_m32(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
-    if (which == kTcStaged && m == 128 && chain_mlp_fwd_m128_workspace_bytes(tokens) != 0)
+    if (which == kTcStaged && chain_mlp_fwd_m128_workspace_bytes(tokens) != 0)
         return chain_mlp_fwd_m128(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
-        return tc_staged_mlp_fwd(x, L1, R1, b1, L2, R2, b2, y, tokens, m, workspace,
-                                 (cudaStream_t)stream);
+        return tc_staged_mlp_fwd(x, L1, R1, b1, L2, R2, b2, y, tokens, workspace, (cudaStream_t)stream);
     return staged_mlp_fwd(x, L1, R1, b1, L2, R2, b2, y, tokens, m, dtype, workspace,
                           (cudaStream_t)stream);
 }

@@ -1,13 +1,11 @@
 // One block-diagonal stage on the tcgen05 tensor cores (bf16 in, fp32 accumulate in TMEM):
 //   out[t][e*m + b] = act( sum_c W[b][e][c] * in[t][b*m + c] + bias[e*m + b] )
 // i.e. multiply every length-m segment of a token row by its block, then scatter with the
-// stride permutation P (or, with `natural` set, leave the result in place: out[t][b*m + e]).  Two launches give the forward pass (M = (P L)(P R)), four the
-// feed-forward block.  The intermediate goes through the caller's workspace, so this family
-// is bounded by twice the HBM traffic of the fused kernels; it serves the sizes and calls
-// that have no fused kernel.
+// stride permutation P.  Four launches give the feed-forward block at m = 128 on a device (or for a token count)
+// that the one-launch forward of chain_m128.cu cannot serve; the intermediates go through the caller's workspace.
 //
 // CTA = 128 tokens x 16 consecutive blocks x 32 output rows.  TMA brings each block's token
-// tile [128 x m] and weight rows [NJ x m] into 128-byte (64-byte for m = 32) swizzled
+// tile [128 x m] and weight rows [NJ x m] into 128-byte swizzled
 // K-major tiles through a 4-slot ring; one thread issues the MMAs (M = 128 tokens, N = NJ,
 // K = 16 per instruction), block b accumulating into TMEM columns [b*NJ, (b+1)*NJ).  With all
 // sixteen accumulators resident, the thread that owns a token (a TMEM lane) picks element e of
@@ -43,7 +41,7 @@ template <int M>
 __global__ void __launch_bounds__(128)
 tc_stage_kernel(const __grid_constant__ CUtensorMap tm_in, const __grid_constant__ CUtensorMap tm_w,
                 __nv_bfloat16 *__restrict__ out, const __nv_bfloat16 *__restrict__ bias, int gelu,
-                int natural, long long tokens, unsigned *status)
+                long long tokens, unsigned *status)
 {
     using C = StageCfg<M>;
     constexpr int n = M * M;
@@ -125,31 +123,7 @@ tc_stage_kernel(const __grid_constant__ CUtensorMap tm_in, const __grid_constant
     tc_fence_after();
     const long long t = t0 + threadIdx.x;
     const uint32_t lane_base = tmem_base + ((uint32_t)(warp * 32) << 16);
-    if (have && natural) {
-        // no permutation: the NJ results of block b are contiguous, out[t][(b0+b)*m + e0 ..]
-        for (int b = 0; b < C::NB; ++b) {
-#pragma unroll
-            for (int ec = 0; ec < C::NJ / 16; ++ec) {
-                uint32_t v[16];
-                tmem_ld16(lane_base + b * C::NJ + ec * 16, v);
-                tmem_ld_wait();
-                if (t < tokens) {
-                    uint4 o0, o1;
-                    o0.x = pack_bf16(__uint_as_float(v[0]), __uint_as_float(v[1]));
-                    o0.y = pack_bf16(__uint_as_float(v[2]), __uint_as_float(v[3]));
-                    o0.z = pack_bf16(__uint_as_float(v[4]), __uint_as_float(v[5]));
-                    o0.w = pack_bf16(__uint_as_float(v[6]), __uint_as_float(v[7]));
-                    o1.x = pack_bf16(__uint_as_float(v[8]), __uint_as_float(v[9]));
-                    o1.y = pack_bf16(__uint_as_float(v[10]), __uint_as_float(v[11]));
-                    o1.z = pack_bf16(__uint_as_float(v[12]), __uint_as_float(v[13]));
-                    o1.w = pack_bf16(__uint_as_float(v[14]), __uint_as_float(v[15]));
-                    uint4 *dst = reinterpret_cast<uint4 *>(out + (size_t)t * n + (b0 + b) * M + e0 + ec * 16);
-                    dst[0] = o0;
-                    dst[1] = o1;
-                }
-            }
-        }
-    } else if (have) {
+    if (have) {
         for (int ec = 0; ec < C::NJ / 4; ++ec) {
             uint32_t v[C::NB][4];
 #pragma unroll
@@ -198,7 +172,7 @@ tc_stage_kernel(const __grid_constant__ CUtensorMap tm_in, const __grid_constant
 }
 
 template <int M>
-int launch_tc_stage(const void *in, const void *W, void *out, const void *bias, int gelu, int natural,
+int launch_tc_stage(const void *in, const void *W, void *out, const void *bias, int gelu,
                     int64_t tokens, unsigned *status, cudaStream_t s)
 {
     using C = StageCfg<M>;
@@ -212,7 +186,7 @@ int launch_tc_stage(const void *in, const void *W, void *out, const void *bias, 
     MONARCH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
     dim3 grid((unsigned)((tokens + C::TOK - 1) / C::TOK), M / C::NB, M / C::NJ);
     kern<<<grid, 128, C::SMEM_BYTES, s>>>(tm_in, tm_w, (__nv_bfloat16 *)out,
-                                          (const __nv_bfloat16 *)bias, gelu, natural, tokens, status);
+                                          (const __nv_bfloat16 *)bias, gelu, tokens, status);
     note_launch();
     MONARCH_CUDA_TRY(cudaGetLastError());
     return MONARCH_OK;
@@ -221,17 +195,6 @@ int launch_tc_stage(const void *in, const void *W, void *out, const void *bias, 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace
-
-int tc_stage(int m, const void *in, const void *W, void *out, const void *bias, int gelu,
-             int64_t tokens, unsigned *status, cudaStream_t s, int natural)
-{
-    switch (m) {
-        case 32:  return launch_tc_stage<32>(in, W, out, bias, gelu, natural, tokens, status, s);
-        case 64:  return launch_tc_stage<64>(in, W, out, bias, gelu, natural, tokens, status, s);
-        case 128: return launch_tc_stage<128>(in, W, out, bias, gelu, natural, tokens, status, s);
-    }
-    return MONARCH_ERR_UNSUPPORTED;
-}
 
 // ---- host: tensor-map encoder through the driver entry point (no link-time libcuda) ----
 typedef CUresult (*tmap_encode_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -297,30 +260,21 @@ int encode_tmap_nd(CUtensorMap *out, const void *base, int elem_bytes, int rank,
 
 }  // namespace tc
 
-// Forward pass and feed-forward block as chains of tensor-core stages (bf16, m >= 32); same
-// workspace layout as the CUDA-core staged family.
-int tc_staged_fwd(const void *x, const void *L, const void *R, void *y, int64_t tokens, int m,
-                  void *ws, cudaStream_t s)
-{
-    if (m == 128) return chain_fwd_m128(x, L, R, y, tokens, ws, s);          // workspace: two plane buffers
-    unsigned *status = (unsigned *)ws;
-    void *u = (char *)ws + MONARCH_STATUS_BYTES;
-    MONARCH_TRY(tc::tc_stage(m, x, R, u, nullptr, 0, tokens, status, s));
-    return tc::tc_stage(m, u, L, y, nullptr, 0, tokens, status, s);
-}
-
+// The feed-forward block as a chain of stages (bf16, m = 128); same workspace layout as the CUDA-core staged family.
 int tc_staged_mlp_fwd(const void *x, const void *L1, const void *R1, const void *b1, const void *L2,
-                      const void *R2, const void *b2, void *y, int64_t tokens, int m, void *ws,
+                      const void *R2, const void *b2, void *y, int64_t tokens, void *ws,
                       cudaStream_t s)
 {
+    constexpr int m = 128;
+    auto stage = tc::launch_tc_stage<m>;
     unsigned *status = (unsigned *)ws;
     const size_t act = tc::align256((size_t)tokens * m * m * 2);
     char *base = (char *)ws + MONARCH_STATUS_BYTES;
     void *w = base, *h = base + act;
-    MONARCH_TRY(tc::tc_stage(m, x, R1, w, nullptr, 0, tokens, status, s));
-    MONARCH_TRY(tc::tc_stage(m, w, L1, h, b1, 1, tokens, status, s));
-    MONARCH_TRY(tc::tc_stage(m, h, R2, w, nullptr, 0, tokens, status, s));
-    return tc::tc_stage(m, w, L2, y, b2, 0, tokens, status, s);
+    MONARCH_TRY(stage(x, R1, w, nullptr, 0, tokens, status, s));
+    MONARCH_TRY(stage(w, L1, h, b1, 1, tokens, status, s));
+    MONARCH_TRY(stage(h, R2, w, nullptr, 0, tokens, status, s));
+    return stage(w, L2, y, b2, 0, tokens, status, s);
 }
 
 }  // namespace monarch
