@@ -249,16 +249,16 @@ int rect_stage1_tc(const void *x, const void *R, void *u, int64_t tokens, int q,
                    cudaStream_t s);
 int rect_stage1_adjoint_tc(const void *du, const void *R, void *dx, int64_t tokens, int q, int b1, int b,
                            unsigned *status, cudaStream_t s);
-// dL for blocks up to 4 x 4 as a TMA-fed streaming pass (rect_tc.cu): sizes as rect_stage2_stream_available
-int rect_dl_stream(const void *dy, const void *u, float *dL, int64_t tokens, int q, int b, int r, unsigned *status,
-                   cudaStream_t s);
+// du = L^T dy and dL += for blocks up to 4 x 4 in one TMA-fed streaming pass (rect_tc.cu): sizes as rect_stage2_stream_available
+int rect_bwd_stream(const void *dy, const void *u, const void *Lp, void *du, float *dL, int64_t tokens, int q, int b, int r,
+                    unsigned *status, cudaStream_t s);
 bool rect_wgrad_R_tc_available(int q, int b1, int b, int dtype);
-int rect_wgrad_R_tc(const void *du, const void *x, float *dR, int64_t tokens, int q, int b1, int b, unsigned *status,
+// dR = (accumulate ? dR : 0) + ...
+int rect_wgrad_R_tc(const void *du, const void *x, float *dR, int accumulate, int64_t tokens, int q, int b1, int b, unsigned *status,
                     cudaStream_t s);
-// stage 2 as a TMA-fed streaming pass (rect_tc.cu): bf16, q and r at most 4, b a multiple of 8 and at least 256
+// stage 2 as a TMA-fed streaming pass (rect_tc.cu): bf16, q and r at most 4, b a multiple of 8 and at least 128
 bool rect_stage2_stream_available(int q, int b, int r, int dtype);
-int rect_stage2_stream(const void *u, const void *Lp, void *y, int64_t tokens, int q, int b, int r, int wt,
-                       unsigned *status, cudaStream_t s);
+int rect_stage2_stream(const void *u, const void *Lp, void *y, int64_t tokens, int q, int b, int r, unsigned *status, cudaStream_t s);
 
 // ---- rectangular class with wrapped-diagonal blocks, b2 != b3 (rect_wrapped.cu) ----
 size_t rectw_workspace_bytes(int64_t tokens, int q, int b2, int b3, int r, int dtype);

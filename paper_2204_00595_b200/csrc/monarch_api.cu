@@ -439,7 +439,7 @@ int monarch_rect_fwd(const void *x, const void *L, const void *R, void *y, int64
     else
         MONARCH_TRY(rect_stage1_simt(x, R, u, tokens, q, b1, b, dtype, 0, s));
     if (fast && rect_stage2_stream_available(q, b, r, dtype))
-        return rect_stage2_stream(u, L, y, tokens, q, b, r, 0, status, s);
+        return rect_stage2_stream(u, L, y, tokens, q, b, r, status, s);
     return rect_stage2_simt(u, L, y, tokens, q, b, r, dtype, 0, s);
 }
 
@@ -506,15 +506,16 @@ int monarch_rect_bwd(const void *x, const void *dy, const void *L, const void *R
     MONARCH_TRY(check_buffers(in, 4, out, 3, workspace, workspace_bytes,
                               monarch_rect_bwd_workspace_bytes(tokens, q, b1, b, r, dtype)));
     cudaStream_t s = (cudaStream_t)stream;
+    const bool fast = g_impl.load(std::memory_order_relaxed) != MONARCH_IMPL_STAGED;
+    const bool tc_dR = fast && rect_wgrad_R_tc_available(q, b1, b, dtype);
     if (!accumulate) {
         MONARCH_CUDA_TRY(cudaMemsetAsync(dL, 0, lb * sizeof(float), s));
-        MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, rb * sizeof(float), s));
+        if (!tc_dR || tokens == 0) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, rb * sizeof(float), s));
     }
     if (tokens == 0) return MONARCH_OK;
     unsigned *status = (unsigned *)workspace;
     char *u_own = (char *)workspace + MONARCH_STATUS_BYTES;
     char *du = u_own + round256((size_t)tokens * q * b * es);
-    const bool fast = g_impl.load(std::memory_order_relaxed) != MONARCH_IMPL_STAGED;
     // u = blockdiag(R) x: what the forward call left in its workspace ([status][u]), else recomputed
     const char *u = fwd_workspace ? (const char *)fwd_workspace + MONARCH_STATUS_BYTES : u_own;
     if (!fwd_workspace) {
@@ -523,9 +524,10 @@ int monarch_rect_bwd(const void *x, const void *dy, const void *L, const void *R
         else
             MONARCH_TRY(rect_stage1_simt(x, R, u_own, tokens, q, b1, b, dtype, 0, s));
     }
-    // du = L^T dy: stage 2 with the roles of q and r exchanged and the blocks read transposed
-    if (fast && rect_stage2_stream_available(r, b, q, dtype))
-        MONARCH_TRY(rect_stage2_stream(dy, L, du, tokens, r, b, q, 1, status, s));
+    // du = L^T dy (stage 2 with the roles of q and r exchanged and the blocks read transposed), with dL where both stream
+    const bool streamed = fast && rect_stage2_stream_available(q, b, r, dtype);
+    if (streamed)
+        MONARCH_TRY(rect_bwd_stream(dy, u, L, du, dL, tokens, q, b, r, status, s));
     else
         MONARCH_TRY(rect_stage2_simt(dy, L, du, tokens, r, b, q, dtype, 1, s));
     // dx = blockdiag(R)^T du: stage 1 with the roles of b1 and b exchanged and the blocks read transposed
@@ -533,11 +535,8 @@ int monarch_rect_bwd(const void *x, const void *dy, const void *L, const void *R
         MONARCH_TRY(rect_stage1_adjoint_tc(du, R, dx, tokens, q, b1, b, status, s));
     else
         MONARCH_TRY(rect_stage1_simt(du, R, dx, tokens, q, b, b1, dtype, 1, s));
-    const bool tc_dR = fast && rect_wgrad_R_tc_available(q, b1, b, dtype);
-    if (tc_dR) MONARCH_TRY(rect_wgrad_R_tc(du, x, dR, tokens, q, b1, b, status, s));
-    const bool stream_dL = fast && rect_stage2_stream_available(q, b, r, dtype);
-    if (stream_dL) MONARCH_TRY(rect_dl_stream(dy, u, dL, tokens, q, b, r, status, s));
-    return rect_wgrad_simt(x, dy, u, du, dL, dR, tokens, q, b1, b, r, dtype, !stream_dL, !tc_dR, s);
+    if (tc_dR) MONARCH_TRY(rect_wgrad_R_tc(du, x, dR, accumulate, tokens, q, b1, b, status, s));
+    return rect_wgrad_simt(x, dy, u, du, dL, dR, tokens, q, b1, b, r, dtype, !streamed, !tc_dR, s);
 }
 
 int monarch_cplx_fwd(const void *x, const void *L, const void *R, void *y, int adjoint, int64_t tokens,

@@ -375,6 +375,31 @@ rect_stage1_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_c
     if (warp == 0) tmem_dealloc_pair(tmem_base, 2 * NT);
 }
 
+// pairs of CTAs that can be resident at once (0: none)
+template <typename K> int max_pairs_of(K kern, PerDeviceCache &cache, int smem, int *out)
+{
+    int n = cache.get();
+    if (n < 0) {
+        MONARCH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2, 1, 1);
+        cfg.blockDim = dim3(kThreads, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+        cache.set(n);
+    }
+    *out = n;
+    return MONARCH_OK;
+}
+
 template <bool BT>
 int launch_pair(const void *in, const void *W, void *out, int64_t tokens, int q, int kdim, int ndim, unsigned *status,
                 cudaStream_t s, bool *used)
@@ -388,26 +413,8 @@ int launch_pair(const void *in, const void *W, void *out, int64_t tokens, int q,
         MONARCH_TRY(encode_tmap_2d(&tm_R, W, (uint64_t)q * ndim, (uint64_t)kdim, (uint64_t)kdim * 2, 128, kKChunk, 128));
     MONARCH_TRY(encode_tmap_2d(&tm_u, out, (uint64_t)tokens, (uint64_t)q * ndim, (uint64_t)q * ndim * 2, kTokTile, 64, 128));
     static PerDeviceCache max_pairs_cache;
-    int max_pairs = max_pairs_cache.get();
-    if (max_pairs < 0) {
-        MONARCH_CUDA_TRY(cudaFuncSetAttribute(rect_stage1_pair_kernel<BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem));
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2, 1, 1);
-        cfg.blockDim = dim3(kThreads, 1, 1);
-        cfg.dynamicSmemBytes = kPairSmem;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 2; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, rect_stage1_pair_kernel<BT>, &cfg) != cudaSuccess) {
-            (void)cudaGetLastError();
-            n = 0;
-        }
-        max_pairs = n;
-        max_pairs_cache.set(n);
-    }
+    int max_pairs = 0;
+    MONARCH_TRY(max_pairs_of(rect_stage1_pair_kernel<BT>, max_pairs_cache, kPairSmem, &max_pairs));
     if (max_pairs < 1) return MONARCH_OK;                                 // the caller falls back to single CTAs
     RectParams p;
     p.status = status;
@@ -463,7 +470,8 @@ int launch(const void *in, const void *W, void *out, int64_t tokens, int q, int 
 // A CTA owns 256 columns j and a slab of tokens; TMA brings 16-token tiles of the q slices u[t][k*b + j0 ..] into a
 // three-stage ring (no thread holds a load in flight, so the pass is not limited by registers x occupancy), the
 // blocks sit in shared memory as fp32, and each thread turns 8 columns of two tokens into r x 8 outputs per step,
-// written back with 16-byte stores (a warp writes 512 contiguous bytes of a slice y[t][l*b + .]).
+// written back with 16-byte stores (a warp writes 512 contiguous bytes of a slice y[t][l*b + .]).  y is stored streaming:
+// u is still in L2 from stage 1 (67 MB at 8192 tokens of 4 x 1024 columns) and the backward call reads it again.
 constexpr int kS2Cols = 256, kS2Tok = 16, kS2Stages = 3, kS2Threads = 256;
 constexpr int kS2SliceBytes = kS2Tok * kS2Cols * 2;                 // one k slice of a tile
 constexpr int kS2SmemBytes = kS2Stages * 4 * kS2SliceBytes + 128;     // two CTAs per SM with the 16 KB of blocks
@@ -489,7 +497,7 @@ __device__ __forceinline__ float bf_elem(const uint4 &v, int e)
 __global__ void __launch_bounds__(kS2Threads, 2)
 rect_stage2_stream_kernel(const __grid_constant__ CUtensorMap tm_u, const __nv_bfloat16 *__restrict__ Lp,
                           __nv_bfloat16 *__restrict__ y, unsigned *status, long long tokens, int q, int b, int r,
-                          int tokens_per_slab, int wt)
+                          int tokens_per_slab)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ float4 ws[4][4][2][32];            // [l][k][half][lane]: columns 8 lane + 4 half + (0..3)
@@ -508,8 +516,7 @@ rect_stage2_stream_kernel(const __grid_constant__ CUtensorMap tm_u, const __nv_b
     for (int i = threadIdx.x; i < 16 * kS2Cols; i += kS2Threads) {
         const int jl = i >> 4, l = (i >> 2) & 3, k = i & 3;
         float v = 0.0f;
-        // wt: the blocks are stored [j][k][l] (the adjoint pass reads L's blocks transposed)
-        if (j0 + jl < b && l < r && k < q) v = __bfloat162float(Lp[(size_t)(j0 + jl) * r * q + (wt ? k * r + l : l * q + k)]);
+        if (j0 + jl < b && l < r && k < q) v = __bfloat162float(Lp[(size_t)(j0 + jl) * r * q + l * q + k]);
         reinterpret_cast<float *>(&ws[l][k][(jl >> 2) & 1][jl >> 3])[jl & 3] = v;
     }
     __syncthreads();
@@ -570,7 +577,7 @@ rect_stage2_stream_kernel(const __grid_constant__ CUtensorMap tm_u, const __nv_b
                     if (tt == 1 && !two) break;
                     const uint4 o = make_uint4(pack_bf16(acc[tt][0], acc[tt][1]), pack_bf16(acc[tt][2], acc[tt][3]),
                                                pack_bf16(acc[tt][4], acc[tt][5]), pack_bf16(acc[tt][6], acc[tt][7]));
-                    *reinterpret_cast<uint4 *>(y + (size_t)(tt ? tb : ta) * r * b + (size_t)l * b + j0 + lane * 8) = o;
+                    __stcs(reinterpret_cast<uint4 *>(y + (size_t)(tt ? tb : ta) * r * b + (size_t)l * b + j0 + lane * 8), o);
                 }
             }
         }
@@ -579,14 +586,18 @@ rect_stage2_stream_kernel(const __grid_constant__ CUtensorMap tm_u, const __nv_b
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// dL[j][l][k] += sum_t dy[t][l*b + j] u[t][k*b + j] for blocks of at most 4 x 4, as a streaming pass like the one
-// above: TMA brings 16-token tiles of the r slices of dy and the q slices of u into a three-stage ring; a thread owns
-// 8 columns and keeps their r x q x 8 partial sums in registers (one CTA per SM), adding them to dL at the end.
+// du[t][k*b + j] = sum_l Lp[j][l][k] dy[t][l*b + j]  and  dL[j][l][k] += sum_t dy[t][l*b + j] u[t][k*b + j]  for blocks of
+// at most 4 x 4, in one streaming pass like the one above (as two passes dy was read twice): TMA brings 16-token tiles
+// of the r slices of dy and the q slices of u into a three-stage ring; a thread owns 8 columns of two tokens per step and
+// keeps their r x q x 8 partial sums of dL in registers (one CTA per SM), adding them to dL at the end.  Bound by HBM:
+// three token tensors, 201 MB at 8192 tokens of 4 x 1024 columns.
 __global__ void __launch_bounds__(kS2Threads, 1)
-rect_dl_stream_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_constant__ CUtensorMap tm_u,
-                      float *__restrict__ dL, unsigned *status, long long tokens, int q, int b, int r, int tokens_per_slab)
+rect_bwd_stream_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_constant__ CUtensorMap tm_u,
+                       const __nv_bfloat16 *__restrict__ Lp, __nv_bfloat16 *__restrict__ du, float *__restrict__ dL,
+                       unsigned *status, long long tokens, int q, int b, int r, int tokens_per_slab)
 {
     extern __shared__ uint8_t smem_raw[];
+    __shared__ float4 ws[4][4][2][32];            // [l][k][half][lane]: columns 8 lane + 4 half + (0..3)
     __shared__ __align__(8) uint64_t full[kS2Stages];
     __shared__ int dead_s;
     const uint32_t ring0 = (smem_u32(smem_raw) + 127u) & ~127u;
@@ -596,8 +607,6 @@ rect_dl_stream_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_co
         for (int s = 0; s < kS2Stages; ++s) mbar_init(smem_u32(&full[s]), 1);
         fence_mbar_init();
         dead_s = 0;
-        tma_prefetch_desc(&tm_dy);
-        tma_prefetch_desc(&tm_u);
     }
     __syncthreads();
     const long long t0 = (long long)blockIdx.y * tokens_per_slab;
@@ -616,9 +625,16 @@ rect_dl_stream_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_co
     };
     if (threadIdx.x == 0)
         for (int tile = 0; tile < kS2Stages - 1 && tile < ntiles; ++tile) issue(tile);
+    for (int i = threadIdx.x; i < 16 * kS2Cols; i += kS2Threads) {
+        const int jl = i >> 4, l = (i >> 2) & 3, k = i & 3;
+        const float v = j0 + jl < b && l < r && k < q ? __bfloat162float(Lp[(size_t)(j0 + jl) * r * q + l * q + k]) : 0.0f;
+        reinterpret_cast<float *>(&ws[l][k][(jl >> 2) & 1][jl >> 3])[jl & 3] = v;
+    }
+    __syncthreads();
 
     const int lane = threadIdx.x & 31, tr = threadIdx.x >> 5;
     const bool active = j0 + lane * 8 < b;
+    const uint32_t ws0 = smem_u32(ws);
     float gsum[4][4][8];
 #pragma unroll
     for (int l = 0; l < 4; ++l)
@@ -631,30 +647,42 @@ rect_dl_stream_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_co
         const uint32_t s = tile % kS2Stages;
         if (!mbar_wait(full0 + s * 8, (tile / kS2Stages) & 1, status, dead, kErrTmaWait)) break;
         const long long ta = t0 + (long long)tile * kS2Tok + tr;
-        if (active) {
-            const uint32_t src = ring0 + s * 8 * kS2SliceBytes + lane * 16;
+        const uint32_t src = ring0 + s * 8 * kS2SliceBytes + lane * 16 + tr * (kS2Cols * 2);
+        // rows of the next slab count there; rows past the last token arrive as zeros
+        const bool one = active && ta < t1, two = active && ta + 8 < t1;
+        if (one) {
+            uint4 g[2][4];
 #pragma unroll
-            for (int tt = 0; tt < 2; ++tt) {
-                if (ta + 8 * tt >= t1) break;                     // rows of the next slab, or past the last token
-                const uint32_t rowoff = (tr + 8 * tt) * (kS2Cols * 2);
-                float gf[4][8];
+            for (int l = 0; l < 4; ++l) {
+                g[0][l] = l < r ? lds128u(src + l * kS2SliceBytes) : make_uint4(0u, 0u, 0u, 0u);
+                g[1][l] = l < r && two ? lds128u(src + l * kS2SliceBytes + 8 * (kS2Cols * 2)) : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (k >= q) break;
+                const uint4 ua = lds128u(src + (4 + k) * kS2SliceBytes), ub = lds128u(src + (4 + k) * kS2SliceBytes + 8 * (kS2Cols * 2));
+                float acc[2][8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) acc[0][e] = acc[1][e] = 0.0f;
 #pragma unroll
                 for (int l = 0; l < 4; ++l) {
-                    const uint4 g = l < r ? lds128u(src + l * kS2SliceBytes + rowoff) : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) gf[l][e] = bf_elem(g, e);
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (k >= q) break;
-                    const uint4 uv = lds128u(src + (4 + k) * kS2SliceBytes + rowoff);
+                    const float4 wa = lds128f(ws0 + ((l * 4 + k) * 2 + 0) * 512 + lane * 16);
+                    const float4 wb = lds128f(ws0 + ((l * 4 + k) * 2 + 1) * 512 + lane * 16);
+                    const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        const float uf = bf_elem(uv, e);
-#pragma unroll
-                        for (int l = 0; l < 4; ++l) gsum[l][k][e] = fmaf(gf[l][e], uf, gsum[l][k][e]);
+                        const float ga = bf_elem(g[0][l], e), gb = bf_elem(g[1][l], e);
+                        acc[0][e] = fmaf(wv[e], ga, acc[0][e]);
+                        acc[1][e] = fmaf(wv[e], gb, acc[1][e]);
+                        gsum[l][k][e] = fmaf(ga, bf_elem(ua, e), fmaf(gb, bf_elem(ub, e), gsum[l][k][e]));
                     }
                 }
+#pragma unroll
+                for (int tt = 0; tt < 2; ++tt)
+                    if (tt == 0 || two)
+                        *reinterpret_cast<uint4 *>(du + (size_t)(ta + 8 * tt) * q * b + (size_t)k * b + j0 + lane * 8) =
+                            make_uint4(pack_bf16(acc[tt][0], acc[tt][1]), pack_bf16(acc[tt][2], acc[tt][3]),
+                                       pack_bf16(acc[tt][4], acc[tt][5]), pack_bf16(acc[tt][6], acc[tt][7]));
             }
         }
         __syncthreads();
@@ -783,6 +811,7 @@ rect_wgrad_kernel(const __grid_constant__ CUtensorMap tm_du, const __grid_consta
                     uint32_t v[16];
                     tmem_ld16(lane_base + c, v);
                     tmem_ld_wait();
+                    if (j0 + warp * 32 + lane >= p.b) continue;          // the next block's rows
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
                         asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(out + c + e * 4),
@@ -796,6 +825,144 @@ rect_wgrad_kernel(const __grid_constant__ CUtensorMap tm_du, const __grid_consta
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem_base, NT);
+}
+
+// The same on CTA pairs: a 256 (j) x 256 (i) tile, each CTA loading its own 128 columns of du and HALF of the 256 columns
+// of x.  A single CTA needs 48 KB of operands per 512 cycles of MMA, more than the 60 to 70 bytes per clock that L2 gives
+// an SM (62.6 us for 69 GFLOP); a pair needs 32 KB per CTA.
+// add: the sums go to the output with vector reductions (token slices, or accumulation); else they are stored.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+rect_wgrad_pair_kernel(const __grid_constant__ CUtensorMap tm_du, const __grid_constant__ CUtensorMap tm_x, const WgParams p, int add)
+{
+    constexpr int NT = 256;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) PairBars bars;
+    __shared__ uint32_t tmem_base_s;
+    __shared__ int dead_s;
+    const uint32_t ring0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();
+    volatile int *dead = &dead_s;
+    int tile = blockIdx.x >> 1;
+    const int i0 = tile % p.itiles * NT;
+    tile /= p.itiles;
+    const int j0 = tile % p.jtiles * 256 + (int)rank * 128, k = tile / p.jtiles;
+    const int first = blockIdx.y;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kPairStages; ++s) {
+            mbar_init(smem_u32(&bars.full[s]), 1);
+            mbar_init(smem_u32(&bars.empty[s]), 1);
+        }
+        mbar_init(smem_u32(&bars.acc_full[0]), 1);
+        fence_mbar_init();
+        dead_s = 0;
+        tma_prefetch_desc(&tm_du);
+        tma_prefetch_desc(&tm_x);
+    }
+    if (warp == 0) {
+        tmem_alloc_pair(smem_u32(&tmem_base_s), NT);
+        tmem_relinquish_pair();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_arrive_release();                                             // both CTAs' barriers exist before any remote arrive
+    cluster_wait_acquire();
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_base_s;
+    const uint32_t full0 = smem_u32(bars.full), empty0 = smem_u32(bars.empty), acc = smem_u32(&bars.acc_full[0]);
+
+    if (warp == 4) {
+        if (lane == 0) {
+            uint32_t n = 0;
+            for (int c = first; c < p.chunks; c += p.slices, ++n) {
+                const uint32_t s = n % kPairStages;
+                if (!mbar_wait(empty0 + s * 8, ((n / kPairStages) & 1) ^ 1, p.status, dead, kErrSlotWait)) break;
+                const uint32_t dst = ring0 + s * kPairStageBytes, full = full0 + s * 8;
+                if (rank == 0) mbar_expect_tx(full, 2 * kPairStageBytes);
+#pragma unroll
+                for (int a = 0; a < 2; ++a) {
+                    tma_load_2d_pair(dst + a * 8192, &tm_du, k * p.b + j0 + a * 64, c * 64, full);
+                    tma_load_2d_pair(dst + kPairStageBytes / 2 + a * 8192, &tm_x, k * p.b1 + i0 + (int)rank * (NT / 2) + a * 64, c * 64, full);
+                }
+            }
+        }
+    } else if (warp == 5) {
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc = make_idesc_bf16(256, NT, 1, 1);
+            uint32_t n = 0;
+            bool ok = true;
+            for (int c = first; c < p.chunks; c += p.slices, ++n) {
+                const uint32_t s = n % kPairStages;
+                if (!mbar_wait<true>(full0 + s * 8, (n / kPairStages) & 1, p.status, dead, kErrTmaWait)) { ok = false; break; }
+                tc_fence_after();
+                const uint64_t ad = make_smem_desc(ring0 + s * kPairStageBytes, 8192, 1024, kSwizzle128);
+                const uint64_t bd = make_smem_desc(ring0 + s * kPairStageBytes + kPairStageBytes / 2, 8192, 1024, kSwizzle128);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) mma_f16_ss_pair(tmem_base, ad + 128 * kk, bd + 128 * kk, idesc, (n | kk) != 0);
+                mma_commit_pair(empty0 + s * 8, 3);
+            }
+            if (ok) mma_commit_pair(acc, 3);
+        }
+    } else if (mbar_wait(acc, 0, p.status, dead, kErrMmaWait)) {
+        tc_fence_after();
+        const uint32_t lane_base = tmem_base + ((uint32_t)(warp * 32) << 16);
+        float *out = p.out + ((size_t)k * p.b + j0 + warp * 32 + lane) * p.b1 + i0;
+#pragma unroll 2
+        for (int c = 0; c < NT; c += 16) {
+            uint32_t v[16];
+            tmem_ld16(lane_base + c, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float a0 = __uint_as_float(v[e * 4]), a1 = __uint_as_float(v[e * 4 + 1]), a2 = __uint_as_float(v[e * 4 + 2]),
+                            a3 = __uint_as_float(v[e * 4 + 3]);
+                if (add)
+                    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(out + c + e * 4), "f"(a0), "f"(a1), "f"(a2), "f"(a3) : "memory");
+                else
+                    *reinterpret_cast<float4 *>(out + c + e * 4) = make_float4(a0, a1, a2, a3);
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_arrive_release();
+    cluster_wait_acquire();
+    if (warp == 0) tmem_dealloc_pair(tmem_base, NT);
+}
+
+// dR = (accumulate ? dR : 0) + ...; b and b1 multiples of 256; *used = false where no pair can be resident
+int launch_wgrad_pair(const void *du, const void *x, float *dR, int accumulate, int64_t tokens, int q, int b1, int b, unsigned *status,
+                      cudaStream_t s, bool *used)
+{
+    static PerDeviceCache cache;
+    constexpr int smem = kPairStages * kPairStageBytes + 1024;
+    int pairs = 0;
+    *used = false;
+    MONARCH_TRY(max_pairs_of(rect_wgrad_pair_kernel, cache, smem, &pairs));
+    if (pairs < 1) return MONARCH_OK;
+    CUtensorMap tm_du, tm_x;
+    MONARCH_TRY(encode_tmap_2d(&tm_du, du, (uint64_t)tokens, (uint64_t)q * b, (uint64_t)q * b * 2, 64, 64, 128));
+    MONARCH_TRY(encode_tmap_2d(&tm_x, x, (uint64_t)tokens, (uint64_t)q * b1, (uint64_t)q * b1 * 2, 64, 64, 128));
+    WgParams p;
+    p.out = dR;
+    p.status = status;
+    p.q = q; p.b = b; p.b1 = b1;
+    p.chunks = (int)((tokens + 63) / 64);
+    p.jtiles = b / 256;
+    p.itiles = b1 / 256;
+    const long long tiles = (long long)q * p.jtiles * p.itiles;
+    long long slices = pairs / tiles;
+    if (slices < 1) slices = 1;
+    if (slices > p.chunks) slices = p.chunks;
+    if (tiles > 0x3fffffffLL || slices > 65535) return MONARCH_ERR_UNSUPPORTED;
+    p.slices = (int)slices;
+    if (slices > 1 && !accumulate) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, (size_t)q * b * b1 * sizeof(float), s));
+    rect_wgrad_pair_kernel<<<dim3((unsigned)(2 * tiles), (unsigned)slices), kThreads, smem, s>>>(tm_du, tm_x, p, slices > 1 || accumulate);
+    note_launch();
+    MONARCH_CUDA_TRY(cudaGetLastError());
+    *used = true;
+    return MONARCH_OK;
 }
 
 template <int NT>
@@ -816,7 +983,7 @@ int launch_wgrad(const void *du, const void *x, float *dR, int64_t tokens, int q
     p.status = status;
     p.q = q; p.b = b; p.b1 = b1;
     p.chunks = (int)((tokens + 63) / 64);
-    p.jtiles = b / 128;
+    p.jtiles = (b + 127) / 128;
     p.itiles = b1 / NT;
     const long long tiles = (long long)q * p.jtiles * p.itiles;
     long long slices = sms / tiles;
@@ -841,11 +1008,11 @@ bool rect_stage1_tc_available(int q, int b1, int b, int dtype)
 
 bool rect_stage2_stream_available(int q, int b, int r, int dtype)
 {
-    return dtype == MONARCH_BF16 && q <= 4 && r <= 4 && b % 8 == 0 && b >= 256;     // a 256-column box fits a slice
+    // a 256-column box fits a row; one that is wider than a slice (b < 256) brings columns that nobody looks at
+    return dtype == MONARCH_BF16 && q <= 4 && r <= 4 && b % 8 == 0 && b >= 128 && (int64_t)q * b >= 256 && (int64_t)r * b >= 256;
 }
 
-int rect_stage2_stream(const void *u, const void *Lp, void *y, int64_t tokens, int q, int b, int r, int wt,
-                       unsigned *status, cudaStream_t s)
+int rect_stage2_stream(const void *u, const void *Lp, void *y, int64_t tokens, int q, int b, int r, unsigned *status, cudaStream_t s)
 {
     using namespace tc;
     if (tokens == 0) return MONARCH_OK;
@@ -865,7 +1032,7 @@ int rect_stage2_stream(const void *u, const void *Lp, void *y, int64_t tokens, i
     slabs = (tokens + per - 1) / per;
     if (slabs > 65535) return MONARCH_ERR_UNSUPPORTED;
     rect_stage2_stream_kernel<<<dim3((unsigned)cx, (unsigned)slabs), kS2Threads, kS2SmemBytes, s>>>(
-        tm_u, (const __nv_bfloat16 *)Lp, (__nv_bfloat16 *)y, status, tokens, q, b, r, (int)per, wt);
+        tm_u, (const __nv_bfloat16 *)Lp, (__nv_bfloat16 *)y, status, tokens, q, b, r, (int)per);
     note_launch();
     MONARCH_CUDA_TRY(cudaGetLastError());
     return MONARCH_OK;
@@ -886,9 +1053,9 @@ int rect_stage1_tc(const void *x, const void *R, void *u, int64_t tokens, int q,
                         : tc::launch<64, false>(x, R, u, tokens, q, b1, b, status, s);
 }
 
-// dL as a TMA-fed streaming pass: same sizes as the streaming stage 2
-int rect_dl_stream(const void *dy, const void *u, float *dL, int64_t tokens, int q, int b, int r, unsigned *status,
-                   cudaStream_t s)
+// du and dL in one TMA-fed streaming pass: same sizes as the streaming stage 2
+int rect_bwd_stream(const void *dy, const void *u, const void *Lp, void *du, float *dL, int64_t tokens, int q, int b, int r,
+                    unsigned *status, cudaStream_t s)
 {
     using namespace tc;
     if (tokens == 0) return MONARCH_OK;
@@ -900,7 +1067,7 @@ int rect_dl_stream(const void *dy, const void *u, float *dL, int64_t tokens, int
     // cache would not be safe against two host threads
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
-    MONARCH_CUDA_TRY(cudaFuncSetAttribute(rect_dl_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    MONARCH_CUDA_TRY(cudaFuncSetAttribute(rect_bwd_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int cx = (b + kS2Cols - 1) / kS2Cols;
     long long slabs = (sms + cx - 1) / cx;                            // one CTA per SM, one wave
     if (slabs > (tokens + kS2Tok - 1) / kS2Tok) slabs = (tokens + kS2Tok - 1) / kS2Tok;
@@ -908,23 +1075,29 @@ int rect_dl_stream(const void *dy, const void *u, float *dL, int64_t tokens, int
     per = (per + kS2Tok - 1) / kS2Tok * kS2Tok;
     slabs = (tokens + per - 1) / per;
     if (slabs > 65535) return MONARCH_ERR_UNSUPPORTED;
-    rect_dl_stream_kernel<<<dim3((unsigned)cx, (unsigned)slabs), kS2Threads, smem, s>>>(tm_dy, tm_u, dL, status, tokens, q,
-                                                                                      b, r, (int)per);
+    rect_bwd_stream_kernel<<<dim3((unsigned)cx, (unsigned)slabs), kS2Threads, smem, s>>>(
+        tm_dy, tm_u, (const __nv_bfloat16 *)Lp, (__nv_bfloat16 *)du, dL, status, tokens, q, b, r, (int)per);
     note_launch();
     MONARCH_CUDA_TRY(cudaGetLastError());
     return MONARCH_OK;
 }
 
-// dR on the tensor cores: bf16, b a multiple of 128 (the 128 TMEM lanes), b1 a multiple of 64
+// dR on the tensor cores: bf16, b and b1 multiples of 64 (the rows of a last half tile of 128 are not stored)
 bool rect_wgrad_R_tc_available(int q, int b1, int b, int dtype)
 {
     (void)q;
-    return dtype == MONARCH_BF16 && b % 128 == 0 && b1 % 64 == 0;
+    return dtype == MONARCH_BF16 && b % 64 == 0 && b1 % 64 == 0;
 }
 
-int rect_wgrad_R_tc(const void *du, const void *x, float *dR, int64_t tokens, int q, int b1, int b, unsigned *status,
+int rect_wgrad_R_tc(const void *du, const void *x, float *dR, int accumulate, int64_t tokens, int q, int b1, int b, unsigned *status,
                     cudaStream_t s)
 {
+    if (tokens > 0 && b % 256 == 0 && b1 % 256 == 0) {
+        bool used = false;
+        MONARCH_TRY(tc::launch_wgrad_pair(du, x, dR, accumulate, tokens, q, b1, b, status, s, &used));
+        if (used) return MONARCH_OK;
+    }
+    if (!accumulate) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, (size_t)q * b * b1 * sizeof(float), s));
     if (tokens == 0) return MONARCH_OK;
     if (b1 % 256 == 0) return tc::launch_wgrad<256>(du, x, dR, tokens, q, b1, b, status, s);
     return b1 % 128 == 0 ? tc::launch_wgrad<128>(du, x, dR, tokens, q, b1, b, status, s)

@@ -148,12 +148,12 @@ int stage1(const void *x, const void *R, void *u, int64_t tokens, int q, int b1,
     return rect_stage1_simt(x, R, u, tokens, q, b1, b2, dtype, 0, s);
 }
 
-// stage 2 of the diagonal-block case (wt = 1: its adjoint, with the roles of q and r exchanged by the caller)
-int stage2_diag(const void *in, const void *Lp, void *out, int64_t tokens, int q, int b, int r, int dtype, int wt, bool fast,
+// stage 2 of the diagonal-block case
+int stage2_diag(const void *in, const void *Lp, void *out, int64_t tokens, int q, int b, int r, int dtype, bool fast,
                 unsigned *status, cudaStream_t s)
 {
-    if (fast && rect_stage2_stream_available(q, b, r, dtype)) return rect_stage2_stream(in, Lp, out, tokens, q, b, r, wt, status, s);
-    return rect_stage2_simt(in, Lp, out, tokens, q, b, r, dtype, wt, s);
+    if (fast && rect_stage2_stream_available(q, b, r, dtype)) return rect_stage2_stream(in, Lp, out, tokens, q, b, r, status, s);
+    return rect_stage2_simt(in, Lp, out, tokens, q, b, r, dtype, 0, s);
 }
 
 }  // namespace
@@ -187,7 +187,7 @@ int rectw_fwd(const void *x, const void *Lw, const void *R, void *y, int64_t tok
         else relabel_kernel<__nv_bfloat16><<<g, kThreads, 0, s>>>((const __nv_bfloat16 *)Lw, (__nv_bfloat16 *)Lp, m);
         note_launch();
         MONARCH_CUDA_TRY(cudaGetLastError());
-        return stage2_diag(u, Lp, y, tokens, m.q2, m.bb, m.r2, dtype, 0, fast, status, s);
+        return stage2_diag(u, Lp, y, tokens, m.q2, m.bb, m.r2, dtype, fast, status, s);
     }
     const int g = grid_for(tokens * r * b3);
     if (dtype == MONARCH_F32)
@@ -205,9 +205,10 @@ int rectw_bwd(const void *x, const void *dy, const void *Lw, const void *R, void
 {
     const size_t es = dtype == MONARCH_F32 ? 4 : 2, bmax = b2 > b3 ? b2 : b3;
     const size_t lw = (size_t)r * q * bmax, rb = (size_t)q * b2 * b1;
+    const bool tc_dR = fast && rect_wgrad_R_tc_available(q, b1, b2, dtype);
     if (!accumulate) {
         MONARCH_CUDA_TRY(cudaMemsetAsync(dLw, 0, lw * sizeof(float), s));
-        MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, rb * sizeof(float), s));
+        if (!tc_dR || tokens == 0) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, rb * sizeof(float), s));
     }
     if (tokens == 0) return MONARCH_OK;
     unsigned *status = (unsigned *)ws;
@@ -218,14 +219,18 @@ int rectw_bwd(const void *x, const void *dy, const void *Lw, const void *R, void
     MONARCH_TRY(stage1(x, R, u, tokens, q, b1, b2, dtype, fast, status, s));
     const bool div = divisible(b2, b3);
     const Relabel m = relabel_of(q, b2, b3, r);
+    const bool stream = div && fast && rect_stage2_stream_available(m.q2, m.bb, m.r2, dtype);
     if (div) {
         const int g = grid_for((long long)lw);
         if (dtype == MONARCH_F32) relabel_kernel<float><<<g, kThreads, 0, s>>>((const float *)Lw, (float *)Lp, m);
         else relabel_kernel<__nv_bfloat16><<<g, kThreads, 0, s>>>((const __nv_bfloat16 *)Lw, (__nv_bfloat16 *)Lp, m);
         note_launch();
         MONARCH_CUDA_TRY(cudaGetLastError());
-        // du = L^T dy: stage 2 with the roles of q and r exchanged and the blocks read transposed
-        MONARCH_TRY(stage2_diag(dy, Lp, du, tokens, m.r2, m.bb, m.q2, dtype, 1, fast, status, s));
+        // dLp of the re-labelled problem goes into zeroed scratch.  du = L^T dy: stage 2 with the roles of q and r exchanged
+        // and the blocks read transposed.
+        MONARCH_CUDA_TRY(cudaMemsetAsync(dLp, 0, lw * sizeof(float), s));
+        if (stream) MONARCH_TRY(rect_bwd_stream(dy, u, Lp, du, dLp, tokens, m.q2, m.bb, m.r2, status, s));
+        else MONARCH_TRY(rect_stage2_simt(dy, Lp, du, tokens, m.r2, m.bb, m.q2, dtype, 1, s));
     } else {
         const int g = grid_for(tokens * q * b2);
         if (dtype == MONARCH_F32)
@@ -241,15 +246,11 @@ int rectw_bwd(const void *x, const void *dy, const void *Lw, const void *R, void
         MONARCH_TRY(rect_stage1_adjoint_tc(du, R, dx, tokens, q, b1, b2, status, s));
     else
         MONARCH_TRY(rect_stage1_simt(du, R, dx, tokens, q, b2, b1, dtype, 1, s));
-    const bool tc_dR = fast && rect_wgrad_R_tc_available(q, b1, b2, dtype);
-    if (tc_dR) MONARCH_TRY(rect_wgrad_R_tc(du, x, dR, tokens, q, b1, b2, status, s));
+    if (tc_dR) MONARCH_TRY(rect_wgrad_R_tc(du, x, dR, accumulate, tokens, q, b1, b2, status, s));
     else MONARCH_TRY(rect_wgrad_simt(x, dy, u, du, nullptr, dR, tokens, q, b1, b2, 1, dtype, 0, 1, s));
     if (div) {
-        // dLp of the re-labelled problem (into zeroed scratch), then back into the caller's layout
-        MONARCH_CUDA_TRY(cudaMemsetAsync(dLp, 0, lw * sizeof(float), s));
-        const bool stream_dL = fast && rect_stage2_stream_available(m.q2, m.bb, m.r2, dtype);
-        if (stream_dL) MONARCH_TRY(rect_dl_stream(dy, u, dLp, tokens, m.q2, m.bb, m.r2, status, s));
-        else MONARCH_TRY(rect_wgrad_simt(x, dy, u, du, dLp, nullptr, tokens, m.q2, 1, m.bb, m.r2, dtype, 1, 0, s));
+        // dLp, then back into the caller's layout
+        if (!stream) MONARCH_TRY(rect_wgrad_simt(x, dy, u, du, dLp, nullptr, tokens, m.q2, 1, m.bb, m.r2, dtype, 1, 0, s));
         relabel_back_kernel<<<grid_for((long long)lw), kThreads, 0, s>>>(dLp, dLw, m, 1);
         note_launch();
         MONARCH_CUDA_TRY(cudaGetLastError());

@@ -557,6 +557,13 @@ def test_rect_bwd(P, q, b1, b, r, T, dtype):
     assert_close(_instances(to_host64(dR)), _instances(2 * ref["dR"]), dtype, "rect dR accumulate")
 
 
+@pytest.mark.parametrize("q,b1,b,r,T", [(4, 256, 256, 4, 63), (2, 512, 256, 2, 1000), (1, 256, 768, 4, 129), (4, 192, 192, 4, 300),
+                                        (4, 384, 192, 2, 65), (3, 64, 136, 2, 50), (2, 320, 320, 4, 16)])
+def test_rect_bwd_tiles(P, q, b1, b, r, T):
+    """dR on CTA pairs (one and several token slices), a last half tile of rows, streamed slices narrower than a box."""
+    test_rect_bwd(P, q, b1, b, r, T, "bf16")
+
+
 # (q, b1, b2, b3, r, T): b3 a multiple of b2, b2 a multiple of b3, neither; tiny, ragged and tensor-core sizes
 RECTW_CASES = [
     (3, 2, 2, 4, 2, 7), (2, 3, 4, 2, 3, 65), (2, 2, 3, 5, 2, 130), (3, 1, 5, 3, 2, 70), (2, 4, 2, 6, 1, 33),
