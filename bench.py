@@ -209,14 +209,12 @@ def time_oracle(cfg, d, target_s=12.0, calls=None, tokens=None):
 KERNELS_OF = {
     (16, "f32", "fwd"): "fused_fwd_m16_kernel (1 launch)",
     (32, "bf16", "fwd"): "fused_fwd_m32_kernel (1 launch)",
-    (64, "bf16", "fwd"): "fused_fwd_m64_team_kernel (1 launch)",
-    (64, "bf16", "bwd"): "fused_bwd_all_m64_kernel (1 launch, 2 memset nodes)",
-    (64, "bf16", "bwd_dx"): "fused_bwd_dx_m64_kernel (1 launch)",
-    (64, "bf16", "bwd_dw"): "fused_fwd_m64_kernel (stage 1 only) + fused_bwd_all_m64_kernel without dx "
-                            "(2 launches, 2 memset nodes)",
-    (64, "bf16", "mlp_fwd"): "fused_fwd_m64_team_kernel (2 launches)",
-    (64, "bf16", "mlp_bwd"): "fused_fwd_m64_team_kernel + mlp_act_kernel + fused_fwd_m64_kernel (stage 1 only) + "
-                             "2 x fused_bwd_all_m64_kernel + mlp_dact_kernel + merge_status_kernel (7 launches)",
+    (64, "bf16", "fwd"): "stage1_kernel + stage2_kernel (2 launches)",
+    (64, "bf16", "bwd"): "bwd_du_kernel + bwd_dx_kernel + add_parts_m64_kernel (3 launches)",
+    (64, "bf16", "bwd_dx"): "bwd_du_kernel + bwd_dx_kernel (2 launches)",
+    (64, "bf16", "bwd_dw"): "stage1_kernel + bwd_du_kernel + bwd_dx_kernel without dx + add_parts_m64_kernel (4 launches)",
+    (64, "bf16", "mlp_fwd"): "2 x (stage1_kernel + stage2_kernel) (4 launches)",
+    (64, "bf16", "mlp_bwd"): "2 x forward + mlp_act_kernel + stage1_kernel + 2 x backward + mlp_dact_kernel + merge_status_kernel",
     (128, "bf16", "fwd"): "chain_fused_fwd_kernel (1 persistent launch; chain_gemm_kernel x 2 + plane_transpose_kernel "
                           "beyond 8192 tiles)",
     (128, "bf16", "bwd"): "plane_transpose_kernel + chain_gemm_kernel x 2 with the token reductions (3 launches)",

@@ -34,12 +34,9 @@
  *    when one of their bounded waits runs out; zero it once with
  *    monarch_workspace_init and read it with monarch_last_device_status.
  *    Calls that overlap on the GPU must not share a workspace.
- *  - Weight gradients of the fused tensor-core kernels for bf16 m = 64 (beyond
- *    a few hundred tokens) and of the general class are summed with fp32
- *    reductions whose order across thread blocks is not fixed: dL, dR can
- *    differ in the last fp32 bits from run to run (monarch_set_deterministic
- *    switches m = 64 to a fixed order).  All others (bf16 m = 16, 32 and 128,
- *    fp32, MONARCH_IMPL_STAGED) give the same bits every run.
+ *  - Weight gradients of the general class are summed with fp32 reductions
+ *    whose order across thread blocks is not fixed: dL, dR can differ in the
+ *    last fp32 bits from run to run.  All others give the same bits every run.
  *  - Return value: a monarch_status_t.  Nothing throws.
  */
 #ifndef MONARCH_H_
@@ -136,9 +133,9 @@ int monarch_mlp_fwd(const void *x, const void *L1, const void *R1, const void *b
  * not enter the gradients).  dL1, dR1, dL2, dR2: float32 [m][m][m]; db1, db2:
  * float32 [n]; accumulate == 0 overwrites all six, 1 adds to their contents.
  * a, h and da are rounded to the storage dtype once each (they are tensor-core
- * operands).  The sums over tokens use atomic adds: their order, hence the
- * last bits, may vary from run to run.  Workspace: monarch_workspace_bytes
- * with MONARCH_OP_MLP_BWD. */
+ * operands).  The sums of the bias gradients over tokens use atomic adds: their
+ * order, hence their last bits, may vary from run to run.  Workspace:
+ * monarch_workspace_bytes with MONARCH_OP_MLP_BWD. */
 int monarch_mlp_bwd(const void *x, const void *dy, const void *L1, const void *R1, const void *b1,
                     const void *L2, const void *R2, void *dx,
                     float *dL1, float *dR1, float *db1, float *dL2, float *dR2, float *db2,
@@ -290,19 +287,15 @@ int monarch_set_impl(int impl);
 
 /* Summation order of the weight gradients dL[j][l][k] = sum_t dy[t][l*m+j] u[t][k][j]
  * and dR[k][j][i] = sum_t du[t][k][j] x[t][k*m+i] (the adjoints of Section 3.3,
- * steps 1-2) in the bf16 kernels that split the tokens over thread blocks: m = 64
- * (fused family) and m = 32 (staged tensor-core family), behind monarch_bwd and
- * monarch_bwd_dw.  on != 0: every thread block writes the partial sums of its
- * (fixed) share of the token tiles to the workspace and a second small launch adds
- * them in a fixed order - the same bits on every run, accumulate honoured by that
- * launch; monarch_workspace_bytes for these two operations then reports 32 MiB
- * more, and at m = 64 a device on which the one-launch backward cannot run gets
- * MONARCH_ERR_UNSUPPORTED instead of the multi-launch form.  on == 0 (default):
- * partial sums are added with fp32 atomics in whatever order they arrive.  Other
- * sizes and dtypes already sum in a fixed order (bf16 m = 128, every fp32 call) or
- * are not affected (the feed-forward block and the general class keep their
- * atomics).  Process-wide, affects later calls and later workspace-size queries;
- * not thread-safe against concurrent calls.  Returns the previous setting. */
+ * steps 1-2) behind monarch_bwd and monarch_bwd_dw.  The order is fixed for every
+ * size and dtype, on or off: a thread block sums its (fixed) share of the tokens and
+ * a last step adds these sums in a fixed order, with accumulate honoured there.
+ * on != 0 only keeps a promise to callers that sized their workspaces by it:
+ * monarch_workspace_bytes for these two operations at bf16 m = 32 and m = 64 then
+ * reports 32 MiB more, and less is refused.  The feed-forward block's bias gradients
+ * and the general class use atomics and are not affected.  Process-wide, affects
+ * later calls and later workspace-size queries; not thread-safe against concurrent
+ * calls.  Returns the previous setting. */
 int monarch_set_deterministic(int on);
 
 /* Name of the kernel family the next call with these arguments would use

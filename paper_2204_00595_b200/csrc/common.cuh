@@ -172,66 +172,31 @@ int fused_mlp_fwd_m32(const void *x, const void *L1, const void *R1, const void 
 // dx null: gradients only; dL null: dx only.  The gradients are sums in a fixed order.
 // Reported on top while monarch_set_deterministic is on, as its contract says (these kernels have no use for it).
 constexpr size_t kTcPartialBytes = (size_t)32 << 20;
-size_t fused_bwd_m32_workspace_bytes();
+size_t fused_bwd_m32_workspace_bytes(int64_t tokens);
 int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, void *dx, float *dL, float *dR, int accumulate,
                   int64_t tokens, void *ws, cudaStream_t s);
 
-// ---- fused single-pass forward for m = 64, bf16 (fused_m64.cu) ----
+// ---- m = 64, bf16: one streaming launch per stage (stream_m64.cu) ----
 size_t fused_fwd_m64_workspace_bytes(int64_t tokens);
-int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws,
-                  cudaStream_t s);
-// the same on clusters of four CTAs with the intermediate in distributed shared memory (fused_m64_cluster.cu);
-// MONARCH_ERR_UNSUPPORTED when the device cannot host such a cluster
+int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s);
+// where the forward keeps u inside its workspace (null: nowhere)
+const void *fused_fwd_m64_saved_u(const void *fwd_ws);
+// one pass y = act(M x + bias), act = GELU or identity; workspace of fused_fwd_m64 (u stays behind)
+int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws,
+                       cudaStream_t s);
+size_t fused_mlp_fwd_m64_workspace_bytes(int64_t tokens);
+int fused_mlp_fwd_m64(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2, void *y,
+                      int64_t tokens, void *ws, cudaStream_t s);
+size_t fused_bwd_dx_m64_workspace_bytes(int64_t tokens);
+int fused_bwd_dx_m64(const void *dy, const void *L, const void *R, void *dx, int64_t tokens, void *ws, cudaStream_t s);
+// dx null: gradients only.  u_saved null: recomputed.  The gradients are sums in a fixed order.
+size_t fused_bwd_m64_workspace_bytes(int64_t tokens);
+int fused_bwd_m64(const void *x, const void *dy, const void *L, const void *R, const void *u_saved, void *dx, float *dL, float *dR,
+                  int accumulate, int64_t tokens, void *ws, cudaStream_t s);
+// the forward on clusters of four CTAs with the intermediate in distributed shared memory (fused_m64_cluster.cu), selected by
+// MONARCH_M64_CLUSTER; MONARCH_ERR_UNSUPPORTED when the device cannot host such a cluster
 int fused_fwd_m64_cluster(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s);
 bool fused_fwd_m64_on_clusters();
-// the same with every CTA doing both stages (fused_m64_team.cu); same workspace layout
-int fused_fwd_m64_team(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws,
-                       cudaStream_t s);
-// feed-forward block as two passes of the team kernel with bias (+ GELU) in the stage-2 epilogue
-size_t fused_mlp_fwd_m64_workspace_bytes(int64_t tokens);
-int fused_mlp_fwd_m64(const void *x, const void *L1, const void *R1, const void *b1, const void *L2,
-                      const void *R2, const void *b2, void *y, int64_t tokens, void *ws, cudaStream_t s);
-// one pass y = act(M x + bias), act = GELU or identity; workspace layout of fused_fwd_m64 (u stays behind)
-int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y,
-                       int64_t tokens, void *ws, cudaStream_t s);
-// first stage only: u = P R x in the exchange layout [tile][j][k/8][t%64][k%8] (tokens rounded up to 64)
-int fused_fwd_m64_stage1(const void *x, const void *R, void *u, int64_t tokens, unsigned *status,
-                         cudaStream_t s);
-
-// ---- fused single-pass dx = M^T dy for m = 64, bf16 (fused_m64_bwd.cu) ----
-size_t fused_bwd_dx_m64_workspace_bytes(int64_t tokens);
-int fused_bwd_dx_m64(const void *dy, const void *L, const void *R, void *dx, int64_t tokens, void *ws,
-                     cudaStream_t s);
-// first stage only: du as [tile][k][j/8][t%64][j%8] and P dy as [tile][j][l/8][t%64][l%8]
-int fused_bwd_m64_stage1(const void *dy, const void *L, void *du, void *dyp, int64_t tokens,
-                         unsigned *status, cudaStream_t s);
-
-// both stages, also leaving du (and P dy if dyp != null) behind for the weight gradients
-int fused_bwd_dx_m64_keep(const void *dy, const void *L, const void *R, void *dx, void *du, void *dyp,
-                          unsigned *counters, unsigned *status, int64_t tokens, cudaStream_t s);
-
-// dx, dL +=, dR += in one launch; u = P R x in the forward exchange layout, du / dyp = scratch exchange buffers
-// partials (optional, kBwdPartialBytes): per-CTA partial sums + a fixed-order reduction instead of atomic adds; dL, dR
-// are then overwritten (accumulate = 0) or added to (1) by that reduction
-constexpr int kBwdMaxPartials = 16;                                  // CTAs per group of a weight-gradient kind, at most
-constexpr size_t kBwdPartialBytes = (size_t)2 * kBwdMaxPartials * 64 * 64 * 64 * sizeof(float);
-int fused_bwd_all_m64(const void *x, const void *dy, const void *L, const void *R, const void *u, void *dx,
-                      void *du, void *dyp, float *dL, float *dR, unsigned *counters, unsigned *status,
-                      int64_t tokens, cudaStream_t s, float *partials = nullptr, int accumulate = 1);
-
-// ---- weight gradients for m = 64, bf16 (fused_m64_bwd_dw.cu) ----
-// fixed_order: the weight gradients are summed in a fixed order (partial sums in the workspace, which is then
-// kBwdPartialBytes larger); refused (MONARCH_ERR_UNSUPPORTED) where the one-launch backward cannot run
-size_t fused_bwd_dw_m64_workspace_bytes(int64_t tokens, bool fixed_order = false);
-int fused_bwd_dw_m64(const void *x, const void *dy, const void *L, const void *R, float *dL, float *dR,
-                     int accumulate, int64_t tokens, void *ws, cudaStream_t s, bool fixed_order = false);
-// dx, dL, dR in one pass; u_saved (optional) = the exchange buffer a fused forward call left behind
-size_t fused_bwd_m64_workspace_bytes(int64_t tokens, bool fixed_order = false);
-int fused_bwd_m64(const void *x, const void *dy, const void *L, const void *R, const void *u_saved,
-                  void *dx, float *dL, float *dR, int accumulate, int64_t tokens, void *ws,
-                  cudaStream_t s, bool fixed_order = false);
-// where the fused forward keeps u inside its workspace
-const void *fused_fwd_m64_saved_u(const void *fwd_ws);
 
 // ---- general (rectangular) Monarch multiply on the CUDA cores (rect_simt.cu); workspace = [status][u] ----
 size_t rect_workspace_bytes(int64_t tokens, int q, int b, int dtype);

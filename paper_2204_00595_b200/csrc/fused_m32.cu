@@ -25,7 +25,7 @@
 // registers of an SM, and a kind needs one or two sets of weights beside them.  u and du are recomputed by the kind that
 // needs them (the MMAs are nearly free; the saved traffic is not).  Every CTA stores its sums, a second small launch adds
 // them in a fixed order.
-#include "tc_common.cuh"
+#include "mma_tiles.cuh"
 
 namespace monarch {
 namespace tc {
@@ -37,40 +37,6 @@ constexpr int kSlots = 5, kSmemBytes = (kSlots + 2) * kTile + 1024;
 constexpr int kKinds = 3, kDL = 0, kDR = 1, kDX = 2;
 constexpr int kMaxParts = 50;                            // CTAs of a kind: a third of the chip
 
-__device__ __forceinline__ void ldm4(uint32_t (&r)[4], uint32_t a)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
-}
-__device__ __forceinline__ void ldm4t(uint32_t (&r)[4], uint32_t a)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
-}
-__device__ __forceinline__ void stm4(uint32_t a, const uint32_t (&r)[4])
-{
-    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
-}
-__device__ __forceinline__ void stm4t(uint32_t a, const uint32_t (&r)[4])
-{
-    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
-}
-__device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *m, int x, int y, int z, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
-                 "l"(m), "r"(bar), "r"(x), "r"(y), "r"(z) : "memory");
-}
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap *m, uint32_t src, int x, int y, int z)
-{
-    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(m), "r"(src), "r"(x), "r"(y), "r"(z) : "memory");
-}
-
 // chunk c (8 columns) of token t in a T tile; chunk (half h, row c) of block b in an E tile
 __device__ __forceinline__ uint32_t t_at(uint32_t base, int box, int t, int c) { return base + box * (kTok * 128) + t * 128 + ((c ^ (t & 7)) << 4); }
 __device__ __forceinline__ uint32_t e_at(uint32_t base, int b, int h, int c) { return base + b * 1024 + (((h * 32 + c) ^ (b & 7)) << 4); }
@@ -78,28 +44,15 @@ __device__ __forceinline__ uint32_t e_at(uint32_t base, int b, int h, int c) { r
 // Operand A of a warp's two blocks: rows = outputs, [block][16 rows][16 columns of the contraction]
 struct Weights {
     uint32_t a[2][2][2][4];
-    // trans: multiply by the transposed blocks (8 x 8 pieces transposed in registers)
     __device__ __forceinline__ void load(const __nv_bfloat16 *W, int warp, bool trans)
     {
-        const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
 #pragma unroll
         for (int blk = 0; blk < 2; ++blk)
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
                 for (int ks = 0; ks < 2; ++ks)
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const int row = mt * 16 + (r & 1) * 8, col = ks * 16 + (r >> 1) * 8;      // of the 8 x 8 piece
-                        const __nv_bfloat16 *p = W + (size_t)(warp * 2 + blk) * kM * kM + (trans ? (col + g) * kM + row : (row + g) * kM + col) + 2 * q;
-                        a[blk][mt][ks][r] = *reinterpret_cast<const uint32_t *>(p);
-                    }
-        if (trans)
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                uint32_t &v = a[i >> 4][i >> 3 & 1][i >> 2 & 1][i & 3];
-                asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(v) : "r"(v));
-            }
+                    load_operand(a[blk][mt][ks], W + (size_t)(warp * 2 + blk) * kM * kM, kM, mt * 16, ks * 16, trans);
     }
     // acc = blk's rows times the operand b (both 16-column steps)
     __device__ __forceinline__ void times(int blk, const uint32_t (&b)[4], float (&acc)[2][4]) const
@@ -120,11 +73,6 @@ __device__ __forceinline__ void pack_rows(const float (&acc)[2][4], uint32_t (&o
         o[2 * mt + 1] = pack_bf16(acc[mt][2], acc[mt][3]);
     }
 }
-
-struct Lane {                                            // rows of the four matrices of an x4 instruction
-    int warp, m, r;
-    __device__ __forceinline__ Lane() : warp(threadIdx.x >> 5), m((threadIdx.x & 31) >> 3), r(threadIdx.x & 7) {}
-};
 
 // The operands of a stage are loaded together, ahead of its products.
 struct Operands {
@@ -178,8 +126,8 @@ __device__ __forceinline__ void t_to_e(uint32_t T, uint32_t E)
 struct Params {
     unsigned *status;
     const __nv_bfloat16 *L, *R, *bias;
-    float *parts;                // backward: [kDL, kDR][kMaxParts][32][32][32]
-    int tiles, gelu;
+    float *parts;                // backward: [kDL, kDR][ranks][32][32][32]
+    int tiles, gelu, ranks;
     int first[kKinds + 1];       // backward: CTAs of a kind start here
 };
 
@@ -208,12 +156,9 @@ struct Shared {
     uint64_t bars[kSlots];
     int dead;
 };
-// Launched with programmatic serialization: a kernel may begin while the one before it drains; nothing is read or written
-// before the wait.
-__device__ __forceinline__ void depend_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void init(Shared &s)
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    depend_launch();
     if (threadIdx.x == 0) {
         for (int i = 0; i < kSlots; ++i) mbar_init(smem_u32(&s.bars[i]), 1);
         fence_mbar_init();
@@ -448,18 +393,18 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             if (i + 1 < count) t_to_e(ring.wait(2 * i + 2), V);
         }
     }
-    sums.store(p.parts + ((size_t)kind * kMaxParts + first) * kM * kM * kM);
+    sums.store(p.parts + ((size_t)kind * p.ranks + first) * kM * kM * kM);
 }
 
 // grads = (accumulate ? grads : 0) + the parts, in order; 32 groups of 4 elements and 8 ranges of parts per CTA
 __global__ void __launch_bounds__(256)
-add_parts_m32_kernel(const float *__restrict__ parts, float *__restrict__ dL, float *__restrict__ dR, int n_l, int n_r, int accumulate)
+add_parts_m32_kernel(const float *__restrict__ parts, float *__restrict__ dL, float *__restrict__ dR, int n, int accumulate)
 {
     __shared__ float4 red[8][32];
     constexpr int kElems = kM * kM * kM, kPer = 32 * 4;
     const int kind = blockIdx.x / (kElems / kPer), at = blockIdx.x % (kElems / kPer) * kPer + (threadIdx.x & 31) * 4;
-    const int range = threadIdx.x >> 5, n = kind == kDL ? n_l : n_r;
-    const float *src = parts + (size_t)kind * kMaxParts * kElems + at;
+    const int range = threadIdx.x >> 5;
+    const float *src = parts + (size_t)kind * n * kElems + at;
     float *dst = (kind == kDL ? dL : dR) + at;
     const int per = (n + 7) / 8;
     float4 s = make_float4(0, 0, 0, 0);
@@ -483,25 +428,6 @@ add_parts_m32_kernel(const float *__restrict__ parts, float *__restrict__ dL, fl
         }
         *reinterpret_cast<float4 *>(dst) = s;
     }
-}
-
-template <typename... Ts, typename... As>
-int launch(void (*kern)(Ts...), int grid, int threads, int smem, cudaStream_t s, As... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (smem > 48 * 1024) MONARCH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    MONARCH_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
-    note_launch();
-    return MONARCH_OK;
 }
 
 // [tokens][1024] as boxes of 64 columns: one copy of 64 x 16 tokens x 16 boxes is a T tile
@@ -531,7 +457,7 @@ int launch_fwd_m32(const void *x, const void *L, const void *R, const void *bias
     p.bias = (const __nv_bfloat16 *)bias;
     p.gelu = gelu;
     p.tiles = (int)((tokens + kTok - 1) / kTok);
-    return launch(kern, p.tiles < sms ? p.tiles : sms, kThreads, kSmemBytes, s, tm_x, tm_y, p);
+    return launch_serialized(kern, p.tiles < sms ? p.tiles : sms, kThreads, kSmemBytes, s, tm_x, tm_y, p);
 }
 
 }  // namespace
@@ -557,9 +483,10 @@ int fused_mlp_fwd_m32(const void *x, const void *L1, const void *R1, const void 
 }
 
 // Workspace: status word, then the sums of every CTA (64 KB are left out for the counters of the kernels that share it).
-size_t fused_bwd_m32_workspace_bytes()
+size_t fused_bwd_m32_workspace_bytes(int64_t tokens)
 {
-    return MONARCH_STATUS_BYTES + 65536 + (size_t)2 * tc::kMaxParts * tc::kM * tc::kM * tc::kM * sizeof(float);
+    const int64_t tiles = (tokens + tc::kTok - 1) / tc::kTok;
+    return MONARCH_STATUS_BYTES + 65536 + (size_t)2 * (tiles < tc::kMaxParts ? tiles : tc::kMaxParts) * tc::kM * tc::kM * tc::kM * sizeof(float);
 }
 // dx null: gradients only; dL null: dx only
 int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, void *dx, float *dL, float *dR, int accumulate,
@@ -595,9 +522,10 @@ int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, v
         n[k] = most[k] < p.tiles ? most[k] : p.tiles;
         p.first[k + 1] = p.first[k] + n[k];
     }
-    MONARCH_TRY(launch(fused_bwd_m32_kernel, p.first[kKinds], kThreads, kSmemBytes, s, tm_x, tm_dy, tm_dx, p));
+    p.ranks = n[kDL];
+    MONARCH_TRY(launch_serialized(fused_bwd_m32_kernel, p.first[kKinds], kThreads, kSmemBytes, s, tm_x, tm_dy, tm_dx, p));
     if (dL == nullptr) return MONARCH_OK;
-    return launch(add_parts_m32_kernel, 2 * kM * kM * kM / 128, 256, 0, s, (const float *)p.parts, dL, dR, n[kDL], n[kDR], accumulate);
+    return launch_serialized(add_parts_m32_kernel, 2 * kM * kM * kM / 128, 256, 0, s, (const float *)p.parts, dL, dR, p.ranks, accumulate);
 }
 
 }  // namespace monarch

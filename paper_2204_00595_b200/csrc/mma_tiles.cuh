@@ -1,0 +1,91 @@
+// Warp-MMA building blocks of the kernels that keep the weights of a stage in registers (fused_m32.cu, stream_m64.cu): one
+// operand is the weights (rows = outputs), the tokens are N, so results have tokens innermost and every permutation of
+// Section 3.3 is a choice of where stmatrix puts a row of 8 tokens.
+#pragma once
+
+#include "tc_common.cuh"
+
+namespace monarch {
+namespace tc {
+
+__device__ __forceinline__ void ldm4(uint32_t (&r)[4], uint32_t a)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldm4t(uint32_t (&r)[4], uint32_t a)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void stm4(uint32_t a, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
+__device__ __forceinline__ void stm4(uint32_t a, const uint32_t (&r)[4]) { stm4(a, r[0], r[1], r[2], r[3]); }
+__device__ __forceinline__ void stm4t(uint32_t a, const uint32_t (&r)[4])
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+__device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *m, int x, int y, int z, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
+                 "l"(m), "r"(bar), "r"(x), "r"(y), "r"(z) : "memory");
+}
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap *m, uint32_t src, int x, int y, int z)
+{
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(m), "r"(src), "r"(x), "r"(y), "r"(z) : "memory");
+}
+
+// A operand of mma for 16 rows x 16 columns of a row-major m x m block at (row, col); trans: of the transposed block (8 x 8
+// pieces transposed in registers)
+__device__ __forceinline__ void load_operand(uint32_t (&a)[4], const __nv_bfloat16 *block, int m, int row, int col, bool trans)
+{
+    const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int pr = row + (r & 1) * 8, pc = col + (r >> 1) * 8;       // of the 8 x 8 piece
+        a[r] = *reinterpret_cast<const uint32_t *>(block + (trans ? (pc + g) * m + pr : (pr + g) * m + pc) + 2 * q);
+    }
+    if (trans)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(a[r]) : "r"(a[r]));
+}
+
+struct Lane {                                            // rows of the four matrices of an x4 instruction
+    int warp, m, r;
+    __device__ __forceinline__ Lane() : warp(threadIdx.x >> 5), m((threadIdx.x & 31) >> 3), r(threadIdx.x & 7) {}
+};
+
+// Launched with programmatic serialization: a kernel may begin while the one before it drains; nothing is read or written
+// before the wait.
+__device__ __forceinline__ void depend_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void depend_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... Ts, typename... As>
+int launch_serialized(void (*kern)(Ts...), int grid, int threads, int smem, cudaStream_t s, As... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (smem > 48 * 1024) MONARCH_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    MONARCH_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+    note_launch();
+    return MONARCH_OK;
+}
+
+}  // namespace tc
+}  // namespace monarch

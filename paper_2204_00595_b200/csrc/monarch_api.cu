@@ -114,8 +114,8 @@ int pick(int op, int m, int dtype)
 //   bf16 m = 16   forward 27 / 213 at 32768 tokens, forward + backward 148 / 484: every batch
 //   bf16 m = 32   forward 9.5 / 7.0 at 4, 12.4 / 6.6 at 1000; forward + backward 18.5 / 14.1 at 4: never; the backward of
 //                 the feed-forward block, eight launches otherwise, 33 / 44 at 64, 55 / 46 at 256
-//   bf16 m = 64   forward 14.5 / 16.5 at 256, 19.8 / 16.5 at 512; forward + backward 32 / 45 at 128, 45 / 46 at 256;
-//                 block 29 / 35 at 256, 41 / 35 at 512, with its backward 113 / 147 at 256, 172 / 163 at 512
+//   bf16 m = 64   forward 10.7 / 9.2 at 64; forward + backward 23 / 24.5 at 4, 26.7 / 26.3 at 64; block 18.6 / 19.5 at 64,
+//                 22.6 / 19.8 at 128, with its backward 84 / 95 at 128, 113 / 98 at 256
 //   bf16 m = 128  forward 10.7 / 12.1 at 16; block 25 / 25 at 32, its backward 112 / 147 at 64
 //   fp32          the other family (one launch per stage) is slower at every size
 int64_t units_limit(int op, int m, int dtype)
@@ -124,7 +124,7 @@ int64_t units_limit(int op, int m, int dtype)
     if (dtype == MONARCH_F32 || m == 16) return all;
     const bool fwd = op == MONARCH_OP_FWD, mlp = op == MONARCH_OP_MLP_FWD, mlp_bwd = op == MONARCH_OP_MLP_BWD;
     if (m == 32) return mlp_bwd ? 128 : 0;
-    if (m == 64) return fwd ? 320 : mlp ? 384 : mlp_bwd ? 448 : 256;
+    if (m == 64) return fwd ? 0 : mlp ? 64 : mlp_bwd ? 192 : 32;
     return fwd ? 16 : mlp ? 24 : mlp_bwd ? 96 : 0;
 }
 
@@ -196,7 +196,7 @@ size_t large_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int d
     if (which == kFused && m == 64 && tokens > ((int64_t)1 << 20)) return 0;
     if (which == kTcStaged && m == 32 && op == MONARCH_OP_MLP_FWD) return fused_mlp_fwd_m32_workspace_bytes(tokens);
     if (which == kTcStaged && m == 32 && op != MONARCH_OP_FWD)
-        return fused_bwd_m32_workspace_bytes() + (op != MONARCH_OP_BWD_DX && fixed_order ? kTcPartialBytes : 0);
+        return fused_bwd_m32_workspace_bytes(tokens) + (op != MONARCH_OP_BWD_DX && fixed_order ? kTcPartialBytes : 0);
     if (which == kTcStaged && op != MONARCH_OP_FWD && op != MONARCH_OP_MLP_FWD) return chain_bwd_m128_workspace_bytes(tokens);
     if (which == kTcStaged && op == MONARCH_OP_FWD) return chain_fwd_m128_workspace_bytes(tokens);
     if (which == kTcStaged) {
@@ -204,7 +204,7 @@ size_t large_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int d
         return a > b ? a : b;
     }
     if (op == MONARCH_OP_BWD) {
-        if (which == kFused) return fused_bwd_m64_workspace_bytes(tokens, fixed_order);
+        if (which == kFused) return fused_bwd_m64_workspace_bytes(tokens) + (fixed_order ? kTcPartialBytes : 0);
         const size_t a = staged_workspace_bytes(MONARCH_OP_BWD_DX, tokens, n, m, dtype);
         const size_t b = staged_workspace_bytes(MONARCH_OP_BWD_DW, tokens, n, m, dtype);
         return a > b ? a : b;
@@ -214,7 +214,7 @@ size_t large_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int d
                : op == MONARCH_OP_MLP_FWD ? fused_mlp_fwd_m64_workspace_bytes(tokens)
                : op == MONARCH_OP_FWD    ? fused_fwd_m64_workspace_bytes(tokens)
                : op == MONARCH_OP_BWD_DX ? fused_bwd_dx_m64_workspace_bytes(tokens)
-                                         : fused_bwd_dw_m64_workspace_bytes(tokens, fixed_order);
+                                         : fused_bwd_m64_workspace_bytes(tokens) + (fixed_order ? kTcPartialBytes : 0);
     return staged_workspace_bytes(op, tokens, n, m, dtype);
 }
 }  // namespace
@@ -293,8 +293,7 @@ int monarch_bwd_dw(const void *x, const void *dy, const void *L, const void *R, 
     if (use_units(MONARCH_OP_BWD_DW, m, dtype, tokens))
         return units::bwd(x, dy, L, R, nullptr, nullptr, dL, dR, accumulate, tokens, m, dtype, workspace, (cudaStream_t)stream);
     if (which == kFused)
-        return fused_bwd_dw_m64(x, dy, L, R, dL, dR, accumulate, tokens, workspace, (cudaStream_t)stream,
-                                g_fixed_order.load(std::memory_order_relaxed) != 0);
+        return fused_bwd_m64(x, dy, L, R, nullptr, nullptr, dL, dR, accumulate, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged && m == 32)
         return fused_bwd_m32(x, dy, L, R, nullptr, dL, dR, accumulate, tokens, workspace, (cudaStream_t)stream);
     if (which == kTcStaged)
@@ -327,8 +326,7 @@ int monarch_bwd(const void *x, const void *dy, const void *L, const void *R, con
     if (saved_by_units) fwd_workspace = nullptr;
     if (which == kFused) {
         const bool saved = fwd_workspace != nullptr && pick(MONARCH_OP_FWD, m, dtype) == kFused;
-        return fused_bwd_m64(x, dy, L, R, saved ? fused_fwd_m64_saved_u(fwd_workspace) : nullptr, dx, dL,
-                             dR, accumulate, tokens, workspace, s, g_fixed_order.load(std::memory_order_relaxed) != 0);
+        return fused_bwd_m64(x, dy, L, R, saved ? fused_fwd_m64_saved_u(fwd_workspace) : nullptr, dx, dL, dR, accumulate, tokens, workspace, s);
     }
     if (which == kTcStaged && m == 32) return fused_bwd_m32(x, dy, L, R, dx, dL, dR, accumulate, tokens, workspace, s);
     if (which == kTcStaged) {

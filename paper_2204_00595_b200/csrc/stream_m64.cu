@@ -1,0 +1,736 @@
+// m = 64 (n = 4096), bf16: forward, backward and feed-forward block as streaming launches, one per block-diagonal stage.
+//
+// The weights of a stage are 512 KB, so an SM cannot hold both stages and every block of stage 2 needs a row of every block
+// of stage 1: the intermediate has to cross SMs.  Each launch is one stage for all tokens: a CTA keeps the weights of its 16
+// (backward: 8) blocks as warp-MMA operands in registers, read once, and streams 16-token tiles of just those blocks through
+// shared memory by TMA.  Nothing waits for another CTA inside a launch.  Each launch walks the tiles in the opposite direction
+// of the one before it: what that one wrote last is still in L2.  (Chunks of tokens whose intermediate stays there cost more in
+// launches and last waves than they save: 4096 tokens a chunk, 194 us forward and backward at 8192 tokens, none 164.)
+// The intermediates are stored as the next stage's operands lie in shared memory:
+//   E tile  [tile of 16 tokens][consumer block c][8-token half][producer block p] chunks of 8 tokens, XORed with c % 8:
+//           2 KB per (tile, c); a consumer's blocks are one linear copy, a producer's 16 (8) blocks 256- (128-) byte pieces
+//   T tile  natural rows of 64 columns, 128 bytes per token, 16-byte chunks XORed with t % 8 (TMA's 128-byte swizzle)
+//   Y tile  [l][token][16 neighbouring columns j]: the 32-byte pieces of a permuted row (TMA's 32-byte swizzle)
+// forward   x --T--> u_k = R_k x_k --E--> w_j = L_j u_j, in place in the E tile, transposed 8 x 8 to Y --> y
+// backward  dy --(8 columns j)--> z_j, transposed to E; du_j = L_j^T z_j --E--> dx_k = R_k^T du_k --T--> dx
+//           dL_j = sum_t z_j u_j^T beside du, dR_k = sum_t du_k x_k^T beside dx: tokens are the contraction, operands as they
+//           lie; a CTA's sums are 128 KB of accumulators (half of its registers), stored once and added by a last launch in a
+//           fixed order.
+// A warp works on its own blocks and only the transposes look across, so warps run ahead of one another between mbarriers;
+// a thread of the first warp asks for tiles and sends results away, one tile behind its own work (a warp of its own would
+// cost every other one 32 of its 128 registers).  With a CTA barrier per tile instead, loads, MMAs and stores of a
+// tile followed one another (2650 cycles per 32 KB tile and stage against 1030 of MMA and 1000 to 1500 of shared memory).
+// The weights arrive by TMA as swizzled rows and go to registers by ldmatrix (1 us; fetched by the warps themselves in the
+// 16-byte pieces of the operand layout they took 4).
+#include "mma_tiles.cuh"
+
+namespace monarch {
+namespace tc {
+namespace {
+
+constexpr int kM = 64, kN = kM * kM, kTok = 16, kWarps = 16, kThreads = kWarps * 32;
+constexpr int kBlockBytes = 2 * kM * 16;                 // a block of an E tile
+constexpr int kTileBytes = kM * kBlockBytes;             // an E tile: 128 KB
+constexpr int kFwdBlocks = 16, kFwdGroups = kM / kFwdBlocks, kFwdTile = kTok * kFwdBlocks * kM * 2;   // 32 KB of any kind
+constexpr int kBwdBlocks = 8, kBwdGroups = kM / kBwdBlocks, kBwdTile = kTok * kBwdBlocks * kM * 2;    // 16 KB
+// shared memory in tiles: slots of the input ring, then V tiles (du), then staging tiles of the results.  The last four tiles
+// hold the weights first.
+constexpr int kFwdSlots = 4, kFwdStages = 3, kFwdSmem = (kFwdSlots + kFwdStages) * kFwdTile + 1024;
+constexpr int kDuSlots = 9, kDuStages = 3, kDxSlots = 10, kDxStages = 4, kBwdSmem = 14 * kBwdTile + 1024;
+constexpr int kMaxRanks = 19;                            // CTAs of a group in the backward launches (148 / 8, rounded up)
+constexpr size_t kGradElems = (size_t)kM * kM * kM;
+
+__device__ __forceinline__ uint32_t t_at(uint32_t base, int box, int t, int c) { return base + box * (kTok * 128) + t * 128 + ((c ^ (t & 7)) << 4); }
+__device__ __forceinline__ uint32_t e_at(uint32_t base, int b, int h, int c) { return base + b * kBlockBytes + (((h * kM + c) ^ (b & 7)) << 4); }
+
+struct Params {
+    unsigned *status;
+    const __nv_bfloat16 *bias;
+    const char *e_in, *u;        // E tiles that linear copies read
+    float *parts;                // [rank][64][64][64]
+    int tiles, gelu;
+    int last;                    // tiles - 1: from the last tile to the first; 0: from the first to the last
+};
+
+// Rows r0 .. r0 + 16 MT of one block, as operand A, from its 64 rows of 128 bytes in shared memory
+template <int MT> struct Weights {
+    uint32_t a[MT][4][4];
+    __device__ __forceinline__ void load(uint32_t block, int r0, bool trans)
+    {
+        const Lane ln;
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                const int row = r0 + mt * 16 + (ln.m & 1) * 8, col = ks * 16 + (ln.m >> 1) * 8;      // of the 8 x 8 piece
+                if (trans) ldm4t(a[mt][ks], block + (col + ln.r) * 128 + (((row >> 3) ^ ln.r) << 4));
+                else       ldm4(a[mt][ks], block + (row + ln.r) * 128 + (((col >> 3) ^ ln.r) << 4));
+            }
+    }
+    __device__ __forceinline__ void times(int mt, const uint32_t (&b)[2][4], float (&acc)[4]) const
+    {
+        acc[0] = acc[1] = acc[2] = acc[3] = 0.0f;
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) mma(acc, a[mt][ks], b[ks >> 1][(ks & 1) * 2], b[ks >> 1][(ks & 1) * 2 + 1]);
+    }
+};
+
+struct Ring {
+    uint32_t base, bars;
+    int slots, bytes;
+    unsigned *status;
+    volatile int *dead;
+    __device__ __forceinline__ uint32_t slot(int item) const { return base + (item % slots) * bytes; }
+    __device__ __forceinline__ uint32_t expect(int item) const
+    {
+        mbar_expect_tx(bars + (item % slots) * 8, bytes);
+        return bars + (item % slots) * 8;
+    }
+    __device__ __forceinline__ void load(int item, const CUtensorMap *m, int tile, int z, int x = 0) const
+    {
+        tma_load_3d(slot(item), m, x, tile * kTok, z, expect(item));
+    }
+    __device__ __forceinline__ void load_linear(int item, const char *from) const
+    {
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(slot(item)), "l"(from),
+                     "r"(bytes), "r"(expect(item)) : "memory");
+    }
+    // a wait that runs out leaves `dead` set and garbage in the tile; the loops still run to their end, every later wait
+    // returns at once
+    __device__ __forceinline__ uint32_t wait(int item) const
+    {
+        mbar_wait(bars + (item % slots) * 8, (item / slots) & 1, status, dead, kErrTmaWait);
+        return slot(item);
+    }
+};
+constexpr int kMaxSlots = 10, kMaxStages = 8;
+struct Shared {
+    uint64_t full[kMaxSlots], staged[kMaxStages], free_[kMaxStages];
+    uint64_t across[kFwdSlots];          // tiles that the transposes read: every warp has written its part
+    uint64_t w_full, w_read;
+    int dead;
+};
+// Barriers of a CTA.  staged(i): the results of tile i are in staging tile i % stages, and every warp is done with its inputs.
+struct Sync {
+    Shared &s;
+    unsigned *status;
+    int stages, across_n;
+    __device__ __forceinline__ bool wait(const uint64_t &bar, int phase, unsigned code) const
+    {
+        return mbar_wait(smem_u32(&bar), phase & 1, status, &s.dead, code);
+    }
+    __device__ __forceinline__ static void arrive(uint64_t &bar)             // one per warp
+    {
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(smem_u32(&bar));
+    }
+    __device__ __forceinline__ void wait_staging(int i) const                // staging tile i % stages may be written
+    {
+        if (i < stages) wait(s.w_read, 0, kErrSlotWait);
+        else            wait(s.free_[i % stages], i / stages - 1, kErrSlotWait);
+    }
+    __device__ __forceinline__ void staged(int i) const
+    {
+        fence_proxy_async_smem();
+        arrive(s.staged[i % stages]);
+    }
+    __device__ __forceinline__ void wait_staged(int i) const { wait(s.staged[i % stages], i / stages, kErrMmaWait); }
+    __device__ __forceinline__ void across(int i) const { arrive(s.across[i % across_n]); }
+    __device__ __forceinline__ void wait_across(int i) const { wait(s.across[i % across_n], i / across_n, kErrMmaWait); }
+    // the feeder, after store(i) is committed: store(i - 1) has left its staging tile
+    __device__ __forceinline__ void stored(int i) const
+    {
+        tma_store_wait_read<1>();
+        if (i > 0) mbar_arrive(smem_u32(&s.free_[(i - 1) % stages]));
+    }
+    // `blocks` blocks of W from block `first` on, as [row][64 columns] with 128-byte swizzle
+    __device__ __forceinline__ void load_weights(uint32_t to, const CUtensorMap *tm_w, int first, int blocks) const
+    {
+        const uint32_t bar = smem_u32(&s.w_full);
+        mbar_expect_tx(bar, blocks * kM * 128);
+        for (int b = 0; b < blocks; b += 4) tma_load_2d(to + b * kM * 128, tm_w, 0, (first + b) * kM, bar);
+    }
+    template <int MT> __device__ __forceinline__ void take_weights(Weights<MT> &w, uint32_t block, int r0, bool trans) const
+    {
+        wait(s.w_full, 0, kErrTmaWait);
+        w.load(block, r0, trans);
+        arrive(s.w_read);
+    }
+    // after a wait that ran out: copies that are still under way land before the CTA leaves
+    __device__ __forceinline__ void leave() const
+    {
+        if (*(volatile int *)&s.dead)
+            for (int i = 0; i < 4096; ++i) __nanosleep(256);
+    }
+};
+__device__ __forceinline__ void init(Shared &s)
+{
+    depend_launch();
+    if (threadIdx.x == 0) {
+        for (uint64_t &b : s.full) mbar_init(smem_u32(&b), 1);
+        for (uint64_t &b : s.staged) mbar_init(smem_u32(&b), kWarps);
+        for (uint64_t &b : s.free_) mbar_init(smem_u32(&b), 1);
+        for (uint64_t &b : s.across) mbar_init(smem_u32(&b), kWarps);
+        mbar_init(smem_u32(&s.w_full), 1);
+        mbar_init(smem_u32(&s.w_read), kWarps);
+        fence_mbar_init();
+        s.dead = 0;
+    }
+    __syncthreads();
+    depend_wait();
+}
+// CTA -> (group of blocks, rank among the CTAs of that group)
+__device__ __forceinline__ int ranks_of(int groups, int group) { return ((int)gridDim.x - group + groups - 1) / groups; }
+
+// ---------------------------------------------------------------- forward, stage 1: x -> u (E tiles)
+__global__ void __launch_bounds__(kThreads, 1)
+stage1_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_u,
+              const Params p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
+    const Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead};
+    const Sync sync = {sh, p.status, kFwdStages, kFwdSlots};
+    init(sh);
+    const int group = blockIdx.x % kFwdGroups, first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
+    const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
+    const Lane ln;
+    auto load = [&](int i) {
+        if (i < count) ring.load(i, &tm_x, tile(i), group * kFwdBlocks);
+    };
+    const bool feeder = threadIdx.x == 0;
+    if (feeder) {
+        sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
+        for (int i = 0; i < kFwdSlots - 1; ++i) load(i);
+    }
+    auto feed = [&](int i) {
+        sync.wait_staged(i);
+        tma_store_2d(&tm_u, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks * 8, tile(i) * (2 * kM));
+        tma_store_commit();
+        load(i + kFwdSlots);
+        sync.stored(i);
+    };
+    Weights<4> w;
+    sync.take_weights(w, weights + ln.warp * (kM * 128), 0, false);
+    if (feeder) {
+        sync.wait(sh.w_read, 0, kErrSlotWait);
+        load(kFwdSlots - 1);
+    }
+    for (int i = 0; i < count; ++i) {
+        const uint32_t x = ring.wait(i), stage = stage0 + i % kFwdStages * kFwdTile;
+        uint32_t b[2][2][4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) ldm4(b[v >> 1][v & 1], t_at(x, ln.warp, (v >> 1) * 8 + ln.r, (v & 1) * 4 + ln.m));
+        sync.wait_staging(i);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                float a0[4], a1[4];
+                w.times(2 * n, b[h], a0);
+                w.times(2 * n + 1, b[h], a1);
+                const int j = n * 32 + ln.m * 8 + ln.r;      // row j of this block goes to block j
+                stm4(stage + (j * 2 + h) * (kFwdBlocks * 16) + ((ln.warp ^ (j & 7)) << 4), pack_bf16(a0[0], a0[1]), pack_bf16(a0[2], a0[3]),
+                     pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3]));
+            }
+        sync.staged(i);
+        if (feeder && i > 0) feed(i - 1);
+    }
+    if (feeder && count > 0) feed(count - 1);
+    if (feeder) tma_store_wait_all<0>();
+    sync.leave();
+}
+
+// ---------------------------------------------------------------- forward, stage 2: u -> y
+// ACT: y = GELU(M x + bias), or without the GELU.  Iteration i multiplies tile i + 1 and transposes tile i.
+template <bool ACT>
+__global__ void __launch_bounds__(kThreads, 1)
+stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_y, const Params p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
+    const Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead};
+    const Sync sync = {sh, p.status, kFwdStages, kFwdSlots};
+    init(sh);
+    const int group = blockIdx.x % kFwdGroups, first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
+    const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
+    const Lane ln;
+    auto load = [&](int i) {
+        if (i < count) ring.load_linear(i, p.e_in + ((size_t)tile(i) * kM + group * kFwdBlocks) * kBlockBytes);
+    };
+    const bool feeder = threadIdx.x == 0;
+    if (feeder) {
+        sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
+        for (int i = 0; i < kFwdSlots - 1; ++i) load(i);
+    }
+    auto feed = [&](int i) {
+        sync.wait_staged(i);
+        tma_store_3d(&tm_y, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks, tile(i) * kTok, 0);
+        tma_store_commit();
+        load(i + kFwdSlots);
+        sync.stored(i);
+    };
+    Weights<4> w;
+    sync.take_weights(w, weights + ln.warp * (kM * 128), 0, false);
+    if (feeder) {
+        sync.wait(sh.w_read, 0, kErrSlotWait);
+        load(kFwdSlots - 1);
+    }
+    const __nv_bfloat16 *bias = ACT ? p.bias + ((threadIdx.x & 31) >> 2) * kM + group * kFwdBlocks + ln.warp : nullptr;
+    auto multiply = [&](uint32_t e) {                        // in place: a warp's own block
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t b[2][4], o[8];
+#pragma unroll
+            for (int v = 0; v < 2; ++v) ldm4t(b[v], e_at(e, ln.warp, h, v * 32 + ln.m * 8 + ln.r));
+#pragma unroll
+            for (int mt = 0; mt < 4; ++mt) {
+                float acc[4];
+                w.times(mt, b, acc);
+                if (ACT)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {            // row l = 16 mt + 8 (k / 2) + lane / 4 of block j
+                        const float a = acc[k] + __bfloat162float(__ldg(bias + (mt * 16 + (k >> 1) * 8) * kM));
+                        acc[k] = p.gelu ? gelu_fast(a) : a;
+                    }
+                o[2 * mt] = pack_bf16(acc[0], acc[1]);
+                o[2 * mt + 1] = pack_bf16(acc[2], acc[3]);
+            }
+#pragma unroll
+            for (int n = 0; n < 2; ++n) stm4(e_at(e, ln.warp, h, n * 32 + ln.m * 8 + ln.r), o[4 * n], o[4 * n + 1], o[4 * n + 2], o[4 * n + 3]);
+        }
+    };
+    if (count > 0) {
+        multiply(ring.wait(0));
+        sync.across(0);
+    }
+    for (int i = 0; i < count; ++i) {
+        if (i + 1 < count) {
+            multiply(ring.wait(i + 1));
+            sync.across(i + 1);
+        }
+        const uint32_t e = ring.slot(i), stage = stage0 + i % kFwdStages * kFwdTile;
+        uint32_t v[4][4];
+        const int jg = ln.m & 1, h = ln.m >> 1, t = h * 8 + ln.r;
+        sync.wait_across(i);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) ldm4t(v[n], e_at(e, jg * 8 + ln.r, h, ln.warp * 4 + n));
+        sync.wait_staging(i);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) stm4(stage + (ln.warp * 4 + n) * (kTok * 32) + t * 32 + ((jg ^ (t >> 2 & 1)) << 4), v[n]);
+        sync.staged(i);
+        if (feeder && i > 0) feed(i - 1);
+    }
+    if (feeder && count > 0) feed(count - 1);
+    if (feeder) tma_store_wait_all<0>();
+    sync.leave();
+}
+
+// ---------------------------------------------------------------- backward
+// sums of rows half * 32 .. + 32 and all 64 columns of a warp's block: A = rows of an E block, B = rows of an E block or
+// columns of a T tile, both by token
+struct Sums {
+    float v[2][8][4];
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int i = 0; i < 64; ++i) v[i >> 5][i >> 2 & 7][i & 3] = 0.0f;
+    }
+    template <bool BT> __device__ __forceinline__ void add(uint32_t A, uint32_t B, int blk, int half)
+    {
+        const Lane ln;
+        uint32_t a[2][4];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) ldm4(a[mt], e_at(A, blk, ln.m >> 1, half * 32 + mt * 16 + (ln.m & 1) * 8 + ln.r));
+#pragma unroll
+        for (int np = 0; np < 4; ++np) {
+            uint32_t b[4];
+            const int col = np * 2 + (ln.m >> 1), h = ln.m & 1;
+            if (BT) ldm4t(b, t_at(B, blk, h * 8 + ln.r, col));
+            else    ldm4(b, e_at(B, blk, h, col * 8 + ln.r));
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                mma(v[mt][2 * np], a[mt], b[0], b[1]);
+                mma(v[mt][2 * np + 1], a[mt], b[2], b[3]);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(float *block, int half) const
+    {
+        const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float2 *to = reinterpret_cast<float2 *>(block + (half * 32 + mt * 16 + g + 8 * h) * kM + nt * 8 + 2 * q);
+                    *to = make_float2(v[mt][nt][2 * h], v[mt][nt][2 * h + 1]);
+                }
+    }
+};
+
+// dy -> z, du (E tiles) and, with DW, dL.  Iteration i: z(i + 1), du(i), sums of tile i.
+template <bool DW>
+__global__ void __launch_bounds__(kThreads, 1)
+bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_dy, const __grid_constant__ CUtensorMap tm_du,
+              const Params p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, V0 = base + kDuSlots * kBwdTile, stage0 = V0 + 2 * kBwdTile;
+    const uint32_t weights = base + 10 * kBwdTile;
+    const Ring ring = {base, smem_u32(sh.full), kDuSlots, kBwdTile, p.status, &sh.dead};
+    const Sync sync = {sh, p.status, kDuStages, 2};
+    init(sh);
+    const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
+    const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
+    constexpr int kItems = DW ? 2 : 1;                       // per tile: dy, u
+    const Lane ln;
+    int next = 0;
+    auto load_to = [&](int last) {
+        for (; next <= last && next < kItems * count; ++next) {
+            const int t = tile(next / kItems);
+            if (DW && (next & 1)) ring.load_linear(next, p.u + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
+            else                  ring.load(next, &tm_dy, t, 0, group * kBwdBlocks);
+        }
+    };
+    const bool feeder = threadIdx.x == 0;
+    if (feeder) {
+        sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks);
+        load_to(kDuSlots - 1);
+    }
+    auto feed = [&](int i) {
+        sync.wait_staged(i);
+        tma_store_2d(&tm_du, stage0 + i % kDuStages * kBwdTile, group * kBwdBlocks * 8, tile(i) * (2 * kM));
+        tma_store_commit();
+        load_to((DW ? 2 * i + 2 : i + 1) + kDuSlots);                // dy(i + 1) and u(i) have been read
+        sync.stored(i);
+    };
+    const int blk = ln.warp >> 1, half = ln.warp & 1;
+    Weights<2> w;
+    sync.take_weights(w, weights + blk * (kM * 128), half * 32, true);
+    Sums sums;
+    if (DW) sums.clear();
+    // [l][token][8 columns j] -> E blocks [j][l]
+    auto transpose = [&](uint32_t y, uint32_t V) {
+        uint32_t v[2][4];
+        const int h = ln.m & 1, lo = ln.m >> 1;
+#pragma unroll
+        for (int n = 0; n < 2; ++n) ldm4t(v[n], y + (ln.warp * 4 + n * 2 + lo) * (kTok * 16) + (h * 8 + ln.r) * 16);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) stm4(e_at(V, ln.r, h, ln.warp * 4 + n * 2 + lo), v[n]);
+    };
+    if (count > 0) {
+        sync.wait(sh.w_read, 0, kErrSlotWait);               // V(1) lies where the weights were
+        transpose(ring.wait(0), V0);
+        sync.across(0);
+    }
+    for (int i = 0; i < count; ++i) {
+        const uint32_t V = V0 + (i & 1) * kBwdTile, stage = stage0 + i % kDuStages * kBwdTile;
+        if (i + 1 < count) {
+            const uint32_t y = ring.wait(kItems * (i + 1));
+            if (i > 0) sync.wait_staged(i - 1);              // every warp is done with V(i - 1)
+            transpose(y, V0 + ((i + 1) & 1) * kBwdTile);
+            sync.across(i + 1);
+        }
+        sync.wait_across(i);
+        uint32_t b[2][2][4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) ldm4t(b[v >> 1][v & 1], e_at(V, blk, v >> 1, (v & 1) * 32 + ln.m * 8 + ln.r));
+        sync.wait_staging(i);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float a0[4], a1[4];
+            w.times(0, b[h], a0);
+            w.times(1, b[h], a1);
+            const int k = half * 32 + ln.m * 8 + ln.r;       // row k of this block goes to block k
+            stm4(stage + (k * 2 + h) * (kBwdBlocks * 16) + ((blk ^ (k & 7)) << 4), pack_bf16(a0[0], a0[1]), pack_bf16(a0[2], a0[3]),
+                 pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3]));
+        }
+        if (DW) sums.add<false>(V, ring.wait(2 * i + 1), blk, half);
+        sync.staged(i);
+        if (feeder && i > 0) feed(i - 1);
+    }
+    if (feeder && count > 0) feed(count - 1);
+    if (DW && count > 0)
+        sums.store(p.parts + (size_t)first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
+    if (feeder) tma_store_wait_all<0>();
+    sync.leave();
+}
+
+// du -> dx (DX) and dR (DW)
+template <bool DX, bool DW>
+__global__ void __launch_bounds__(kThreads, 1)
+bwd_dx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_dx,
+              const Params p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kDxSlots * kBwdTile;
+    const Ring ring = {base, smem_u32(sh.full), kDxSlots, kBwdTile, p.status, &sh.dead};
+    const Sync sync = {sh, p.status, DX ? kDxStages : kMaxStages, 1};   // without staging, warps are up to five tiles apart
+    init(sh);
+    const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
+    const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
+    constexpr int kItems = DW ? 2 : 1;                       // per tile: du, x
+    const Lane ln;
+    int next = 0;
+    auto load_to = [&](int last) {
+        for (; next <= last && next < kItems * count; ++next) {
+            const int t = tile(next / kItems);
+            if (DW && (next & 1)) ring.load(next, &tm_x, t, group * kBwdBlocks);
+            else                  ring.load_linear(next, p.e_in + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
+        }
+    };
+    const bool feeder = threadIdx.x == 0;
+    if (feeder) {
+        if (DX) sync.load_weights(stage0, &tm_w, group * kBwdBlocks, kBwdBlocks);
+        load_to(kDxSlots - 1);
+    }
+    auto feed = [&](int i) {
+        sync.wait_staged(i);
+        if (DX) {
+            tma_store_3d(&tm_dx, stage0 + i % kDxStages * kBwdTile, 0, tile(i) * kTok, group * kBwdBlocks);
+            tma_store_commit();
+        }
+        load_to(kItems * (i + 1) - 1 + kDxSlots);
+        if (DX) sync.stored(i);
+    };
+    const int blk = ln.warp >> 1, half = ln.warp & 1;
+    Weights<2> w;
+    if (DX) sync.take_weights(w, stage0 + blk * (kM * 128), half * 32, true);
+    Sums sums;
+    if (DW) sums.clear();
+    for (int i = 0; i < count; ++i) {
+        const uint32_t du = ring.wait(kItems * i), stage = stage0 + i % kDxStages * kBwdTile;
+        if (DX) {
+            uint32_t b[2][2][4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) ldm4t(b[v >> 1][v & 1], e_at(du, blk, v >> 1, (v & 1) * 32 + ln.m * 8 + ln.r));
+            sync.wait_staging(i);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float a0[4], a1[4];
+                w.times(0, b[h], a0);
+                w.times(1, b[h], a1);
+                const uint32_t o[4] = {pack_bf16(a0[0], a0[1]), pack_bf16(a0[2], a0[3]), pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3])};
+                stm4t(t_at(stage, blk, h * 8 + ln.r, half * 4 + ln.m), o);
+            }
+        }
+        if (DW) sums.add<true>(du, ring.wait(2 * i + 1), blk, half);
+        sync.staged(i);
+        if (feeder && i > 0) feed(i - 1);
+    }
+    if (feeder && count > 0) feed(count - 1);
+    if (DW && count > 0)
+        sums.store(p.parts + (size_t)first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
+    if (feeder) tma_store_wait_all<0>();
+    sync.leave();
+}
+
+// grads = (accumulate ? grads : 0) + the parts of every rank, in order; 64 groups of 4 elements and 4 ranges of ranks per CTA
+__global__ void __launch_bounds__(256)
+add_parts_m64_kernel(const float *__restrict__ parts_l, const float *__restrict__ parts_r, float *__restrict__ dL, float *__restrict__ dR,
+                     int grid, int accumulate)
+{
+    __shared__ float4 red[4][64];
+    constexpr int kPer = 64 * 4, kCtas = (int)(kGradElems / kPer);
+    const int kind = blockIdx.x / kCtas, at = blockIdx.x % kCtas * kPer + (threadIdx.x & 63) * 4, range = threadIdx.x >> 6;
+    const int group = at / (kBwdBlocks * kM * kM), n = (grid - group + kBwdGroups - 1) / kBwdGroups, per = (n + 3) / 4;
+    const float *src = (kind == 0 ? parts_l : parts_r) + at;
+    float *dst = (kind == 0 ? dL : dR) + at;
+    float4 s = make_float4(0, 0, 0, 0);
+    depend_wait();
+#pragma unroll 5
+    for (int i = range * per; i < (range + 1) * per && i < n; ++i) {
+        const float4 v = *reinterpret_cast<const float4 *>(src + (size_t)i * kGradElems);
+        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    red[range][threadIdx.x & 63] = s;
+    __syncthreads();
+    if (range == 0) {
+        if (accumulate) {
+            const float4 o = *reinterpret_cast<const float4 *>(dst);
+            s.x += o.x; s.y += o.y; s.z += o.z; s.w += o.w;
+        }
+#pragma unroll
+        for (int i = 1; i < 4; ++i) {
+            const float4 v = red[i][threadIdx.x];
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        *reinterpret_cast<float4 *>(dst) = s;
+    }
+}
+
+// ---------------------------------------------------------------- host
+// [tokens][4096] as boxes of 64 columns: a copy of 64 columns x 16 tokens x `blocks` boxes is a T tile
+int map_t(CUtensorMap *m, const void *p, int64_t tokens, int blocks)
+{
+    const uint64_t dims[3] = {kM, (uint64_t)tokens, kM}, strides[2] = {kN * 2, kM * 2};
+    const uint32_t box[3] = {kM, kTok, (uint32_t)blocks};
+    return encode_tmap_nd(m, p, 2, 3, dims, strides, box, 128);
+}
+// the same tensor as [l][t][j]: `columns` neighbouring j of every l
+int map_y(CUtensorMap *m, const void *p, int64_t tokens, int columns)
+{
+    const uint64_t dims[3] = {kM, (uint64_t)tokens, kM}, strides[2] = {kN * 2, kM * 2};
+    const uint32_t box[3] = {(uint32_t)columns, kTok, kM};
+    return encode_tmap_nd(m, p, 2, 3, dims, strides, box, columns == 16 ? 32 : 0);
+}
+// E tiles as rows (tile, consumer, half) of 64 chunks: the chunks of `blocks` producers in all rows of a tile
+int map_e(CUtensorMap *m, const void *p, int tiles, int blocks)
+{
+    return encode_tmap_2d(m, p, (uint64_t)tiles * 2 * kM, kM * 8, kM * 16, 2 * kM, (uint32_t)blocks * 8, 0);
+}
+
+// blocks as rows of 64 columns, four blocks a copy
+int map_w(CUtensorMap *m, const void *W) { return encode_tmap_2d(m, W, kN, kM, kM * 2, 4 * kM, kM, 128); }
+
+int64_t tiles_of(int64_t tokens) { return (tokens + kTok - 1) / kTok; }
+size_t max_ranks(int64_t tokens) { return (size_t)(tiles_of(tokens) < kMaxRanks ? tiles_of(tokens) : kMaxRanks); }
+size_t e_bytes(int64_t tokens) { return (size_t)tiles_of(tokens) * kTileBytes; }
+
+int grid_of(int groups, int sms, int64_t tokens)
+{
+    const int64_t all = tiles_of(tokens) * groups;
+    return (int)(all < sms ? all : sms);
+}
+
+int stage1(const void *x, const void *R, char *u, int64_t tokens, int sms, unsigned *status, cudaStream_t s)
+{
+    CUtensorMap tm_w, tm_x, tm_u;
+    MONARCH_TRY(map_w(&tm_w, R));
+    MONARCH_TRY(map_t(&tm_x, x, tokens, kFwdBlocks));
+    MONARCH_TRY(map_e(&tm_u, u, (int)tiles_of(tokens), kFwdBlocks));
+    Params p = {};
+    p.status = status;
+    p.tiles = (int)tiles_of(tokens);
+    return launch_serialized(stage1_kernel, grid_of(kFwdGroups, sms, tokens), kThreads, kFwdSmem, s, tm_w, tm_x, tm_u, p);
+}
+
+}  // namespace
+}  // namespace tc
+
+// y = act(M x + bias) (bias null: y = M x); u: E tiles of all tokens, kept for the backward call
+static int stream_fwd(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, void *u, int64_t tokens,
+                      unsigned *status, cudaStream_t s)
+{
+    using namespace tc;
+    if (tokens == 0) return MONARCH_OK;
+    int sms = 0;
+    MONARCH_TRY(current_device_sms(&sms));
+    MONARCH_TRY(stage1(x, R, (char *)u, tokens, sms, status, s));
+    CUtensorMap tm_w, tm_y;
+    MONARCH_TRY(map_w(&tm_w, L));
+    MONARCH_TRY(map_y(&tm_y, y, tokens, kFwdBlocks));
+    Params p = {};
+    p.status = status;
+    p.bias = (const __nv_bfloat16 *)bias;
+    p.gelu = gelu;
+    p.e_in = (const char *)u;
+    p.tiles = (int)tiles_of(tokens);
+    p.last = p.tiles - 1;
+    return launch_serialized(bias != nullptr ? stage2_kernel<true> : stage2_kernel<false>, grid_of(kFwdGroups, sms, tokens), kThreads, kFwdSmem, s,
+                             tm_w, tm_y, p);
+}
+
+// dx null: gradients only; dL null: dx only.  u: what the forward call left (u_saved), or scratch for E tiles of all tokens;
+// du: scratch of the same size; parts: two gradients of max_ranks(tokens)
+static int stream_bwd(const void *x, const void *dy, const void *L, const void *R, const void *u, bool u_saved, void *dx, float *dL, float *dR,
+                      int accumulate, void *du, void *parts, int64_t tokens, unsigned *status, cudaStream_t s)
+{
+    using namespace tc;
+    if (tokens == 0) {
+        if (dL != nullptr && !accumulate) {
+            MONARCH_CUDA_TRY(cudaMemsetAsync(dL, 0, kGradElems * sizeof(float), s));
+            MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, kGradElems * sizeof(float), s));
+        }
+        return MONARCH_OK;
+    }
+    int sms = 0;
+    MONARCH_TRY(current_device_sms(&sms));
+    if (sms > kMaxRanks * kBwdGroups) sms = kMaxRanks * kBwdGroups;
+    float *parts_l = (float *)parts, *parts_r = parts_l + max_ranks(tokens) * kGradElems;
+    const int grid = grid_of(kBwdGroups, sms, tokens), tiles = (int)tiles_of(tokens);
+    if (dL != nullptr && !u_saved) MONARCH_TRY(stage1(x, R, (char *)u, tokens, sms, status, s));
+    CUtensorMap tm_L, tm_R, tm_dy, tm_du, tm_x, tm_dx;
+    MONARCH_TRY(map_w(&tm_L, L));
+    MONARCH_TRY(map_w(&tm_R, R));
+    MONARCH_TRY(map_y(&tm_dy, dy, tokens, kBwdBlocks));
+    MONARCH_TRY(map_e(&tm_du, du, tiles, kBwdBlocks));
+    MONARCH_TRY(map_t(&tm_x, dL != nullptr ? x : dy, tokens, kBwdBlocks));
+    MONARCH_TRY(map_t(&tm_dx, dx != nullptr ? dx : dy, tokens, kBwdBlocks));
+    Params p = {};
+    p.status = status;
+    p.u = (const char *)u;
+    p.parts = parts_l;
+    p.tiles = tiles;
+    MONARCH_TRY(launch_serialized(dL != nullptr ? bwd_du_kernel<true> : bwd_du_kernel<false>, grid, kThreads, kBwdSmem, s, tm_L, tm_dy, tm_du, p));
+    p.e_in = (const char *)du;
+    p.parts = parts_r;
+    p.last = tiles - 1;
+    auto last = dx == nullptr ? bwd_dx_kernel<false, true> : dL == nullptr ? bwd_dx_kernel<true, false> : bwd_dx_kernel<true, true>;
+    MONARCH_TRY(launch_serialized(last, grid, kThreads, kBwdSmem, s, tm_R, tm_x, tm_dx, p));
+    if (dL == nullptr) return MONARCH_OK;
+    return launch_serialized(add_parts_m64_kernel, 2 * (int)(kGradElems / 256), 256, 0, s, (const float *)parts_l, (const float *)parts_r, dL, dR,
+                             grid, accumulate);
+}
+
+// Workspaces: [status][64 KB left out: the counters of kernels that share it stay zero][E tiles ...][parts]
+namespace {
+constexpr size_t kHead = MONARCH_STATUS_BYTES + 65536;
+char *head(const void *ws) { return (char *)ws + kHead; }
+}  // namespace
+
+size_t fused_fwd_m64_workspace_bytes(int64_t tokens)
+{
+    // at least 1 MB: the forward on clusters keeps its weight images where the E tiles start
+    return kHead + tc::e_bytes(tokens < 128 ? 128 : tokens);
+}
+const void *fused_fwd_m64_saved_u(const void *fwd_ws) { return fused_fwd_m64_on_clusters() ? nullptr : head(fwd_ws); }
+
+int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s)
+{
+    if (tokens == 0) return MONARCH_OK;
+    if (fused_fwd_m64_on_clusters()) {
+        const int st = fused_fwd_m64_cluster(x, L, R, y, tokens, ws, s);
+        if (st != MONARCH_ERR_UNSUPPORTED) return st;
+    }
+    return stream_fwd(x, L, R, nullptr, 0, y, head(ws), tokens, (unsigned *)ws, s);
+}
+int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws, cudaStream_t s)
+{
+    return stream_fwd(x, L, R, bias, gelu, y, head(ws), tokens, (unsigned *)ws, s);
+}
+
+size_t fused_mlp_fwd_m64_workspace_bytes(int64_t tokens) { return kHead + 2 * tc::e_bytes(tokens); }
+int fused_mlp_fwd_m64(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2, void *y,
+                      int64_t tokens, void *ws, cudaStream_t s)
+{
+    char *u = head(ws), *h = u + tc::e_bytes(tokens);
+    MONARCH_TRY(stream_fwd(x, L1, R1, b1, 1, h, u, tokens, (unsigned *)ws, s));
+    return stream_fwd(h, L2, R2, b2, 0, y, u, tokens, (unsigned *)ws, s);
+}
+
+size_t fused_bwd_dx_m64_workspace_bytes(int64_t tokens) { return kHead + tc::e_bytes(tokens); }
+int fused_bwd_dx_m64(const void *dy, const void *L, const void *R, void *dx, int64_t tokens, void *ws, cudaStream_t s)
+{
+    return stream_bwd(nullptr, dy, L, R, nullptr, false, dx, nullptr, nullptr, 0, head(ws), nullptr, tokens, (unsigned *)ws, s);
+}
+
+size_t fused_bwd_m64_workspace_bytes(int64_t tokens) { return kHead + 2 * tc::e_bytes(tokens) + 2 * tc::max_ranks(tokens) * tc::kGradElems * sizeof(float); }
+int fused_bwd_m64(const void *x, const void *dy, const void *L, const void *R, const void *u_saved, void *dx, float *dL, float *dR, int accumulate,
+                  int64_t tokens, void *ws, cudaStream_t s)
+{
+    char *du = head(ws), *u = du + tc::e_bytes(tokens), *parts = u + tc::e_bytes(tokens);
+    return stream_bwd(x, dy, L, R, u_saved != nullptr ? u_saved : u, u_saved != nullptr, dx, dL, dR, accumulate, du, parts, tokens, (unsigned *)ws, s);
+}
+
+}  // namespace monarch

@@ -940,9 +940,10 @@ def test_project_leading_pair(P, m, dtype, kind):
 
 @pytest.mark.parametrize("m,T,dtype", [(16, 2500, "bf16"), (16, 1100, "f32"), (32, 1185, "bf16"), (32, 1601, "bf16"),
                                        (32, 833, "f32"), (32, 15, "bf16"), (32, 16 * 148, "bf16"), (32, 16 * 148 * 6 + 1, "bf16"), (64, 255, "bf16"), (64, 320, "bf16"), (64, 321, "bf16"), (64, 593, "f32"),
+                                       (64, 33, "bf16"), (64, 16 * 18, "bf16"), (64, 16 * 37 + 9, "bf16"), (64, 16 * 19 * 5 + 1, "bf16"),
                                        (128, 17, "bf16"), (128, 75, "f32")])
 def test_one_launch_over_units(P, m, T, dtype):
-    """Sizes at which a call changes its tiles (m = 32: one tile, one and six per CTA), splits the tokens of a weight gradient or changes kernels between the
+    """Sizes at which a call changes its tiles (m = 32: one tile, one and six per CTA; m = 64: one per CTA or fewer, a CTA with one more), splits the tokens of a weight gradient or changes kernels between the
     forward and the backward: every call against the oracle, with u saved and recomputed, from one pair of workspaces."""
     import torch
     n, code = m * m, _code(P, dtype)
@@ -975,7 +976,7 @@ def test_one_launch_over_units(P, m, T, dtype):
 
 
 @pytest.mark.parametrize("m,T,dtype", [(16, 1300, "bf16"), (32, 1190, "bf16"), (64, 449, "bf16"), (128, 97, "bf16"), (64, 300, "f32"),
-                                       (32, 129, "bf16"), (128, 25, "bf16")])
+                                       (32, 129, "bf16"), (64, 65, "bf16"), (64, 193, "bf16"), (128, 25, "bf16")])
 def test_one_launch_feed_forward(P, m, T, dtype):
     """The feed-forward block and its gradients at sizes with split token ranges and at the first size beyond the units
     (32 tokens: the m = 32 and m = 128 blocks in two launches)."""
