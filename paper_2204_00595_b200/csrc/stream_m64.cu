@@ -114,6 +114,16 @@ struct Shared {
     uint64_t w_full, w_read;
     int dead;
 };
+// A CTA's place: a group of blocks, and a rank among the CTAs of that group and stage; its tiles
+struct Place {
+    int group, first, step, count, last;
+    __device__ __forceinline__ Place(int groups, int cta, int ctas, const Params &p)
+        : group(cta % groups), first(cta / groups), step((ctas - group + groups - 1) / groups),
+          count(first < p.tiles ? (p.tiles - first + step - 1) / step : 0), last(p.last)
+    {
+    }
+    __device__ __forceinline__ int tile(int i) const { return last != 0 ? last - first - i * step : first + i * step; }
+};
 // Barriers of a CTA.  staged(i): the results of tile i are in staging tile i % stages, and every warp is done with its inputs.
 struct Sync {
     Shared &s;
@@ -147,21 +157,47 @@ struct Sync {
         tma_store_wait_read<1>();
         if (i > 0) mbar_arrive(smem_u32(&s.free_[(i - 1) % stages]));
     }
-    // ... and what was stored two tiles ago is there for every SM
+    // The results of a first stage leave by turns, warp i % 16 for tile i: it stores the tile (after tile i + 1 is staged), frees
+    // the staging tile one iteration later and raises the flag two more later.  Each of these waits for the memory system for
+    // about as long as a tile takes (fences included), which one warp at a time does not slow the others.
+    template <typename Store> __device__ __forceinline__ void pass_on(int k, Store store, unsigned *flags, const Place &place, unsigned ones) const
+    {
+        if ((threadIdx.x & 31) == 0) {
+            const int warp = threadIdx.x >> 5;
+            if (k >= 1 && warp == ((k - 1) & (kWarps - 1))) {
+                wait_staged(k - 1);
+                store(k - 1);
+                tma_store_commit();
+            }
+            if (k >= 2 && warp == ((k - 2) & (kWarps - 1))) {
+                tma_store_wait_read<0>();
+                mbar_arrive(smem_u32(&s.free_[(k - 2) % stages]));
+            }
+            if (flags != nullptr && k >= 4 && warp == ((k - 4) & (kWarps - 1))) publish(flags + place.tile(k - 4), ones);
+        }
+        __syncwarp();
+    }
+    template <typename Store> __device__ __forceinline__ void pass_last(int count, Store store, unsigned *flags, const Place &place, unsigned ones) const
+    {
+        if ((threadIdx.x & 31) == 0) {
+            const int warp = threadIdx.x >> 5;
+            if (count >= 1 && warp == ((count - 1) & (kWarps - 1))) {
+                wait_staged(count - 1);
+                store(count - 1);
+                tma_store_commit();
+            }
+            for (int i = count < 4 ? 0 : count - 4; i < count; ++i)
+                if (flags != nullptr && warp == (i & (kWarps - 1))) publish(flags + place.tile(i), ones);
+            tma_store_wait_all<0>();
+        }
+        __syncwarp();
+    }
     __device__ __forceinline__ static void publish(unsigned *flag, unsigned ones)
     {
+        tma_store_wait_all<0>();
         asm volatile("fence.proxy.async.global;" ::: "memory");
         __threadfence();
         atomicAdd(flag, ones);
-    }
-    template <typename Tile> __device__ __forceinline__ static void finish(unsigned *flags, int count, Tile tile, unsigned ones)
-    {
-        if (flags != nullptr && count >= 2) {
-            tma_store_wait_all<1>();
-            publish(flags + tile(count - 2), ones);
-        }
-        tma_store_wait_all<0>();
-        if (flags != nullptr && count >= 1) publish(flags + tile(count - 1), ones);
     }
     // `blocks` blocks of W from block `first` on, as [row][64 columns] with 128-byte swizzle
     __device__ __forceinline__ void load_weights(uint32_t to, const CUtensorMap *tm_w, int first, int blocks) const
@@ -183,42 +219,26 @@ struct Sync {
             for (int i = 0; i < 4096; ++i) __nanosleep(256);
     }
 };
-// The consuming side, one warp: which of a CTA's tiles are complete.  32 tiles per look, so a CTA that is behind the producers
-// seldom has to.  A tile's four bits are this CTA's alone: it clears them for the next launch.
-struct Gate {
-    unsigned *flags, full;
-    int shift, ready;
-    unsigned *status;
-    volatile int *dead;
-    template <typename Tile> __device__ __forceinline__ bool open(int i, int count, Tile tile, bool must)
-    {
-        if (flags == nullptr || i < ready) return true;
-        const int lane = threadIdx.x & 31;
-        unsigned long long t0 = 0;
-        while (true) {
-            const int n = ready + lane;
-            unsigned *f = flags + tile(n < count ? n : count - 1), v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-            const unsigned closed = ~__ballot_sync(~0u, n >= count || (v >> shift & 15) == full);
-            const int got = closed == 0 ? 32 : __ffs(closed) - 1;
-            if (lane < got && n < count) atomicSub(f, full << shift);
-            ready += got;
-            if (i < ready) {
-                asm volatile("fence.proxy.async.global;" ::: "memory");
-                __syncwarp();
-                return true;
-            }
-            if (!must) return false;
-            const unsigned long long now = global_timer_ns();
-            if (t0 == 0) t0 = now;
-            if (__any_sync(~0u, *dead || now - t0 > wait_limit_ns(status))) {
-                *dead = 1;
-                atomicCAS(status, 0u, kErrPeerWait);
-                return true;
-            }
+// The consuming side, one thread: every producer has stored its part of a tile.  The tile's four bits are this CTA's alone: it
+// clears them for the next launch.
+__device__ __forceinline__ void wait_flag(unsigned *flag, unsigned full, int shift, unsigned *status, volatile int *dead)
+{
+    unsigned long long t0 = 0;
+    while (true) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+        if ((v >> shift & 15) == full) break;
+        const unsigned long long now = global_timer_ns();
+        if (t0 == 0) t0 = now;
+        if (*dead || now - t0 > wait_limit_ns(status)) {
+            *dead = 1;
+            atomicCAS(status, 0u, kErrPeerWait);
+            return;
         }
     }
-};
+    atomicSub(flag, full << shift);
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+}
 __device__ __forceinline__ void init(Shared &s)
 {
     depend_launch();
@@ -235,17 +255,6 @@ __device__ __forceinline__ void init(Shared &s)
     __syncthreads();
     depend_wait();
 }
-// A CTA's place: a group of blocks, and a rank among the CTAs of that group and stage; its tiles
-struct Place {
-    int group, first, step, count, last;
-    __device__ __forceinline__ Place(int groups, int cta, int ctas, const Params &p)
-        : group(cta % groups), first(cta / groups), step((ctas - group + groups - 1) / groups),
-          count(first < p.tiles ? (p.tiles - first + step - 1) / step : 0), last(p.last)
-    {
-    }
-    __device__ __forceinline__ int tile(int i) const { return last != 0 ? last - first - i * step : first + i * step; }
-};
-
 // ---------------------------------------------------------------- forward, stage 1: x -> u (E tiles)
 __device__ __forceinline__ void stage1(const CUtensorMap &tm_w, const CUtensorMap &tm_x, const CUtensorMap &tm_u, const Params &p, const uint32_t base,
                                        Shared &sh)
@@ -265,16 +274,8 @@ __device__ __forceinline__ void stage1(const CUtensorMap &tm_w, const CUtensorMa
         sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
         for (int i = 0; i < kFwdSlots - 1; ++i) load(i);
     }
-    auto feed = [&](int i) {
-        sync.wait_staged(i);
+    auto store = [&](int i) {
         tma_store_2d(&tm_u, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks * 8, tile(i) * (2 * kM));
-        tma_store_commit();
-        load(i + kFwdSlots);
-        sync.stored(i);
-        if (p.flags != nullptr && i >= 2) {
-            tma_store_wait_all<2>();
-            sync.publish(p.flags + tile(i - 2), kFwdOnes);
-        }
     };
     Weights<4> w;
     sync.take_weights(w, weights + ln.warp * (kM * 128), 0, false);
@@ -300,10 +301,13 @@ __device__ __forceinline__ void stage1(const CUtensorMap &tm_w, const CUtensorMa
                      pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3]));
             }
         sync.staged(i);
-        if (feeder && i > 0) feed(i - 1);
+        if (feeder && i > 0) {
+            sync.wait_staged(i - 1);
+            load(i - 1 + kFwdSlots);
+        }
+        sync.pass_on(i, store, p.flags, place, kFwdOnes);
     }
-    if (feeder && count > 0) feed(count - 1);
-    if (feeder) sync.finish(p.flags, count, tile, kFwdOnes);
+    sync.pass_last(count, store, p.flags, place, kFwdOnes);
     sync.leave();
 }
 
@@ -320,33 +324,26 @@ __device__ __forceinline__ void stage2(const CUtensorMap &tm_w, const CUtensorMa
     auto tile = [&](int i) { return place.tile(i); };
     const Lane ln;
     const bool feeder = threadIdx.x == 0;
-    Gate gate = {p.flags, kFwdGroups, group * 4, 0, p.status, &sh.dead};
-    int next = 0, allowed = kFwdSlots - 2;                   // tile to load; last one whose slot is free
-    auto fill = [&](int must) {                              // the first warp
-        for (; next <= allowed && next < count && gate.open(next, count, tile, next <= must); ++next)
-            if (feeder) ring.load_linear(next, p.e_in + ((size_t)tile(next) * kM + group * kFwdBlocks) * kBlockBytes);
-    };
-    if (ln.warp == 0) {
-        if (feeder) sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
-        fill(-1);
-    }
-    auto feed = [&](int i) {                                 // the first warp
-        if (feeder) {
-            sync.wait_staged(i);
-            tma_store_3d(&tm_y, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks, tile(i) * kTok, 0);
-            tma_store_commit();
+    auto load = [&](int i) {                                 // by turns, warp i % 16
+        if (i < count && threadIdx.x == (i & (kWarps - 1)) * 32) {
+            if (p.flags != nullptr) wait_flag(p.flags + tile(i), kFwdGroups, group * 4, p.status, &sh.dead);
+            ring.load_linear(i, p.e_in + ((size_t)tile(i) * kM + group * kFwdBlocks) * kBlockBytes);
         }
-        __syncwarp();
-        allowed = i + kFwdSlots;
-        fill(-1);
-        if (feeder) sync.stored(i);
+    };
+    if (feeder) sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
+    auto feed = [&](int i) {
+        sync.wait_staged(i);
+        tma_store_3d(&tm_y, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks, tile(i) * kTok, 0);
+        tma_store_commit();
+        sync.stored(i);
     };
     Weights<4> w;
     sync.take_weights(w, weights + ln.warp * (kM * 128), 0, false);
-    if (ln.warp == 0) {
-        sync.wait(sh.w_read, 0, kErrSlotWait);
-        allowed = kFwdSlots - 1;
+    for (int i = 0; i < kFwdSlots; ++i) {
+        if (i == kFwdSlots - 1 && ln.warp == i) sync.wait(sh.w_read, 0, kErrSlotWait);       // the last slot lies where the weights were
+        load(i);
     }
+    __syncwarp();
     const __nv_bfloat16 *bias = ACT ? p.bias + ((threadIdx.x & 31) >> 2) * kM + group * kFwdBlocks + ln.warp : nullptr;
     auto multiply = [&](uint32_t e) {                        // in place: a warp's own block
 #pragma unroll
@@ -372,13 +369,11 @@ __device__ __forceinline__ void stage2(const CUtensorMap &tm_w, const CUtensorMa
         }
     };
     if (count > 0) {
-        if (ln.warp == 0) fill(0);
         multiply(ring.wait(0));
         sync.across(0);
     }
     for (int i = 0; i < count; ++i) {
         if (i + 1 < count) {
-            if (ln.warp == 0) fill(i + 1);
             multiply(ring.wait(i + 1));
             sync.across(i + 1);
         }
@@ -392,9 +387,14 @@ __device__ __forceinline__ void stage2(const CUtensorMap &tm_w, const CUtensorMa
 #pragma unroll
         for (int n = 0; n < 4; ++n) stm4(stage + (ln.warp * 4 + n) * (kTok * 32) + t * 32 + ((jg ^ (t >> 2 & 1)) << 4), v[n]);
         sync.staged(i);
-        if (ln.warp == 0 && i > 0) feed(i - 1);
+        if (feeder && i > 0) feed(i - 1);
+        if (i > 0 && ln.warp == ((i - 1 + kFwdSlots) & (kWarps - 1))) {
+            sync.wait_staged(i - 1);
+            load(i - 1 + kFwdSlots);
+            __syncwarp();
+        }
     }
-    if (ln.warp == 0 && count > 0) feed(count - 1);
+    if (feeder && count > 0) feed(count - 1);
     if (feeder) tma_store_wait_all<0>();
     sync.leave();
 }
@@ -484,16 +484,8 @@ __device__ __forceinline__ void bwd_du(const CUtensorMap &tm_w, const CUtensorMa
         sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks);
         load_to(kDuSlots - 1);
     }
-    auto feed = [&](int i) {
-        sync.wait_staged(i);
+    auto store = [&](int i) {
         tma_store_2d(&tm_du, stage0 + i % kDuStages * kBwdTile, group * kBwdBlocks * 8, tile(i) * (2 * kM));
-        tma_store_commit();
-        load_to((DW ? 2 * i + 2 : i + 1) + kDuSlots);                // dy(i + 1) and u(i) have been read
-        sync.stored(i);
-        if (p.flags != nullptr && i >= 2) {
-            tma_store_wait_all<2>();
-            sync.publish(p.flags + tile(i - 2), kBwdOnes);
-        }
     };
     const int blk = ln.warp >> 1, half = ln.warp & 1;
     Weights<2> w;
@@ -538,10 +530,13 @@ __device__ __forceinline__ void bwd_du(const CUtensorMap &tm_w, const CUtensorMa
         }
         if (DW) sums.add<false>(V, ring.wait(2 * i + 1), blk, half);
         sync.staged(i);
-        if (feeder && i > 0) feed(i - 1);
+        if (feeder && i > 0) {
+            sync.wait_staged(i - 1);
+            load_to((DW ? 2 * i : i) + kDuSlots);            // dy(i) and u(i - 1) have been read
+        }
+        sync.pass_on(i, store, p.flags, place, kBwdOnes);
     }
-    if (feeder && count > 0) feed(count - 1);
-    if (feeder) sync.finish(p.flags, count, tile, kBwdOnes);
+    sync.pass_last(count, store, p.flags, place, kBwdOnes);
     if (DW && count > 0)
         sums.store(p.parts_l + (size_t)place.first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
     sync.leave();
@@ -561,42 +556,30 @@ __device__ __forceinline__ void bwd_dx(const CUtensorMap &tm_w, const CUtensorMa
     constexpr int kItems = DW ? 2 : 1;                       // per tile: du, x
     const Lane ln;
     const bool feeder = threadIdx.x == 0;
-    Gate gate = {p.flags, kBwdGroups, group * 4, 0, p.status, &sh.dead};
-    int next = 0, allowed = kDxSlots - 1;                    // item to load; last one whose slot is free
-    auto fill = [&](int must) {                              // the first warp
-        for (; next <= allowed && next < kItems * count; ++next) {
-            const bool rows = DW && (next & 1);
-            if (!rows && !gate.open(next / kItems, count, tile, next <= must)) break;
-            const int t = tile(next / kItems);
-            if (!feeder) continue;
-            if (rows) ring.load(next, &tm_x, t, group * kBwdBlocks);
-            else      ring.load_linear(next, p.e_in + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
+    constexpr int kAhead = kDxSlots / kItems;
+    auto load = [&](int i) {                                 // by turns, warp i % 16
+        if (i < count && threadIdx.x == (i & (kWarps - 1)) * 32) {
+            const int t = tile(i);
+            if (DW) ring.load(kItems * i + 1, &tm_x, t, group * kBwdBlocks);
+            if (p.flags != nullptr) wait_flag(p.flags + t, kBwdGroups, group * 4, p.status, &sh.dead);
+            ring.load_linear(kItems * i, p.e_in + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
         }
     };
-    if (ln.warp == 0) {
-        if (DX && feeder) sync.load_weights(stage0, &tm_w, group * kBwdBlocks, kBwdBlocks);
-        fill(-1);
-    }
-    auto feed = [&](int i) {                                 // the first warp
-        if (feeder) {
-            sync.wait_staged(i);
-            if (DX) {
-                tma_store_3d(&tm_dx, stage0 + i % kDxStages * kBwdTile, 0, tile(i) * kTok, group * kBwdBlocks);
-                tma_store_commit();
-            }
-        }
-        __syncwarp();
-        allowed = kItems * (i + 1) - 1 + kDxSlots;
-        fill(-1);
-        if (DX && feeder) sync.stored(i);
+    if (DX && feeder) sync.load_weights(stage0, &tm_w, group * kBwdBlocks, kBwdBlocks);
+    auto feed = [&](int i) {
+        sync.wait_staged(i);
+        tma_store_3d(&tm_dx, stage0 + i % kDxStages * kBwdTile, 0, tile(i) * kTok, group * kBwdBlocks);
+        tma_store_commit();
+        sync.stored(i);
     };
     const int blk = ln.warp >> 1, half = ln.warp & 1;
     Weights<2> w;
     if (DX) sync.take_weights(w, stage0 + blk * (kM * 128), half * 32, true);
+    for (int i = 0; i < kAhead; ++i) load(i);
+    __syncwarp();
     Sums sums;
     if (DW) sums.clear();
     for (int i = 0; i < count; ++i) {
-        if (ln.warp == 0) fill(kItems * (i + 1) - 1);
         const uint32_t du = ring.wait(kItems * i), stage = stage0 + i % kDxStages * kBwdTile;
         if (DX) {
             uint32_t b[2][2][4];
@@ -614,9 +597,14 @@ __device__ __forceinline__ void bwd_dx(const CUtensorMap &tm_w, const CUtensorMa
         }
         if (DW) sums.add<true>(du, ring.wait(2 * i + 1), blk, half);
         sync.staged(i);
-        if (ln.warp == 0 && i > 0) feed(i - 1);
+        if (DX && feeder && i > 0) feed(i - 1);
+        if (i > 0 && ln.warp == ((i - 1 + kAhead) & (kWarps - 1))) {
+            sync.wait_staged(i - 1);
+            load(i - 1 + kAhead);
+            __syncwarp();
+        }
     }
-    if (ln.warp == 0 && count > 0) feed(count - 1);
+    if (DX && feeder && count > 0) feed(count - 1);
     if (DW && count > 0)
         sums.store(p.parts_r + (size_t)place.first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
     if (feeder) tma_store_wait_all<0>();
