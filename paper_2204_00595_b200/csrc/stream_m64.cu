@@ -22,7 +22,6 @@
 // tile followed one another (2650 cycles per 32 KB tile and stage against 1030 of MMA and 1000 to 1500 of shared memory).
 // The weights arrive by TMA as swizzled rows and go to registers by ldmatrix (1 us; fetched by the warps themselves in the
 // 16-byte pieces of the operand layout they took 4).
-#include <cstdlib>
 #include "mma_tiles.cuh"
 
 namespace monarch {
@@ -38,7 +37,6 @@ constexpr int kBwdBlocks = 8, kBwdGroups = kM / kBwdBlocks, kBwdTile = kTok * kB
 // hold the weights first.
 constexpr int kFwdSlots = 4, kFwdStages = 3, kFwdSmem = (kFwdSlots + kFwdStages) * kFwdTile + 1024;
 constexpr int kDuSlots = 9, kDuStages = 3, kDxSlots = 10, kDxStages = 4, kBwdSmem = 14 * kBwdTile + 1024;
-constexpr unsigned kFwdOnes = 0x1111u, kBwdOnes = 0x11111111u;  // one of a tile's producers, for every consuming group
 constexpr int kMaxRanks = 19;                            // CTAs of a group in the backward launches (148 / 8, rounded up)
 constexpr size_t kGradElems = (size_t)kM * kM * kM;
 
@@ -49,9 +47,7 @@ struct Params {
     unsigned *status;
     const __nv_bfloat16 *bias;
     const char *e_in, *u;        // E tiles that linear copies read
-    float *parts_l, *parts_r;    // [rank][64][64][64]
-    unsigned *flags;             // per tile, four bits per consuming group: producers that have stored their part; null: all have
-    int producers;               // CTAs of the first stage, the others run the second
+    float *parts;                // [rank][64][64][64]
     int tiles, gelu;
     int last;                    // tiles - 1: from the last tile to the first; 0: from the first to the last
 };
@@ -114,16 +110,6 @@ struct Shared {
     uint64_t w_full, w_read;
     int dead;
 };
-// A CTA's place: a group of blocks, and a rank among the CTAs of that group and stage; its tiles
-struct Place {
-    int group, first, step, count, last;
-    __device__ __forceinline__ Place(int groups, int cta, int ctas, const Params &p)
-        : group(cta % groups), first(cta / groups), step((ctas - group + groups - 1) / groups),
-          count(first < p.tiles ? (p.tiles - first + step - 1) / step : 0), last(p.last)
-    {
-    }
-    __device__ __forceinline__ int tile(int i) const { return last != 0 ? last - first - i * step : first + i * step; }
-};
 // Barriers of a CTA.  staged(i): the results of tile i are in staging tile i % stages, and every warp is done with its inputs.
 struct Sync {
     Shared &s;
@@ -157,48 +143,6 @@ struct Sync {
         tma_store_wait_read<1>();
         if (i > 0) mbar_arrive(smem_u32(&s.free_[(i - 1) % stages]));
     }
-    // The results of a first stage leave by turns, warp i % 16 for tile i: it stores the tile (after tile i + 1 is staged), frees
-    // the staging tile one iteration later and raises the flag two more later.  Each of these waits for the memory system for
-    // about as long as a tile takes (fences included), which one warp at a time does not slow the others.
-    template <typename Store> __device__ __forceinline__ void pass_on(int k, Store store, unsigned *flags, const Place &place, unsigned ones) const
-    {
-        if ((threadIdx.x & 31) == 0) {
-            const int warp = threadIdx.x >> 5;
-            if (k >= 1 && warp == ((k - 1) & (kWarps - 1))) {
-                wait_staged(k - 1);
-                store(k - 1);
-                tma_store_commit();
-            }
-            if (k >= 2 && warp == ((k - 2) & (kWarps - 1))) {
-                tma_store_wait_read<0>();
-                mbar_arrive(smem_u32(&s.free_[(k - 2) % stages]));
-            }
-            if (flags != nullptr && k >= 4 && warp == ((k - 4) & (kWarps - 1))) publish(flags + place.tile(k - 4), ones);
-        }
-        __syncwarp();
-    }
-    template <typename Store> __device__ __forceinline__ void pass_last(int count, Store store, unsigned *flags, const Place &place, unsigned ones) const
-    {
-        if ((threadIdx.x & 31) == 0) {
-            const int warp = threadIdx.x >> 5;
-            if (count >= 1 && warp == ((count - 1) & (kWarps - 1))) {
-                wait_staged(count - 1);
-                store(count - 1);
-                tma_store_commit();
-            }
-            for (int i = count < 4 ? 0 : count - 4; i < count; ++i)
-                if (flags != nullptr && warp == (i & (kWarps - 1))) publish(flags + place.tile(i), ones);
-            tma_store_wait_all<0>();
-        }
-        __syncwarp();
-    }
-    __device__ __forceinline__ static void publish(unsigned *flag, unsigned ones)
-    {
-        tma_store_wait_all<0>();
-        asm volatile("fence.proxy.async.global;" ::: "memory");
-        __threadfence();
-        atomicAdd(flag, ones);
-    }
     // `blocks` blocks of W from block `first` on, as [row][64 columns] with 128-byte swizzle
     __device__ __forceinline__ void load_weights(uint32_t to, const CUtensorMap *tm_w, int first, int blocks) const
     {
@@ -219,26 +163,6 @@ struct Sync {
             for (int i = 0; i < 4096; ++i) __nanosleep(256);
     }
 };
-// The consuming side, one thread: every producer has stored its part of a tile.  The tile's four bits are this CTA's alone: it
-// clears them for the next launch.
-__device__ __forceinline__ void wait_flag(unsigned *flag, unsigned full, int shift, unsigned *status, volatile int *dead)
-{
-    unsigned long long t0 = 0;
-    while (true) {
-        unsigned v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-        if ((v >> shift & 15) == full) break;
-        const unsigned long long now = global_timer_ns();
-        if (t0 == 0) t0 = now;
-        if (*dead || now - t0 > wait_limit_ns(status)) {
-            *dead = 1;
-            atomicCAS(status, 0u, kErrPeerWait);
-            return;
-        }
-    }
-    atomicSub(flag, full << shift);
-    asm volatile("fence.proxy.async.global;" ::: "memory");
-}
 __device__ __forceinline__ void init(Shared &s)
 {
     depend_launch();
@@ -255,16 +179,23 @@ __device__ __forceinline__ void init(Shared &s)
     __syncthreads();
     depend_wait();
 }
+// CTA -> (group of blocks, rank among the CTAs of that group)
+__device__ __forceinline__ int ranks_of(int groups, int group) { return ((int)gridDim.x - group + groups - 1) / groups; }
+
 // ---------------------------------------------------------------- forward, stage 1: x -> u (E tiles)
-__device__ __forceinline__ void stage1(const CUtensorMap &tm_w, const CUtensorMap &tm_x, const CUtensorMap &tm_u, const Params &p, const uint32_t base,
-                                       Shared &sh)
+__global__ void __launch_bounds__(kThreads, 1)
+stage1_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_u,
+              const Params p)
 {
-    const uint32_t stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
     const Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead};
     const Sync sync = {sh, p.status, kFwdStages, kFwdSlots};
-    const Place place(kFwdGroups, blockIdx.x, p.producers, p);
-    const int group = place.group, count = place.count;
-    auto tile = [&](int i) { return place.tile(i); };
+    init(sh);
+    const int group = blockIdx.x % kFwdGroups, first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
+    const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     const Lane ln;
     auto load = [&](int i) {
         if (i < count) ring.load(i, &tm_x, tile(i), group * kFwdBlocks);
@@ -274,8 +205,12 @@ __device__ __forceinline__ void stage1(const CUtensorMap &tm_w, const CUtensorMa
         sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
         for (int i = 0; i < kFwdSlots - 1; ++i) load(i);
     }
-    auto store = [&](int i) {
+    auto feed = [&](int i) {
+        sync.wait_staged(i);
         tma_store_2d(&tm_u, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks * 8, tile(i) * (2 * kM));
+        tma_store_commit();
+        load(i + kFwdSlots);
+        sync.stored(i);
     };
     Weights<4> w;
     sync.take_weights(w, weights + ln.warp * (kM * 128), 0, false);
@@ -301,49 +236,50 @@ __device__ __forceinline__ void stage1(const CUtensorMap &tm_w, const CUtensorMa
                      pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3]));
             }
         sync.staged(i);
-        if (feeder && i > 0) {
-            sync.wait_staged(i - 1);
-            load(i - 1 + kFwdSlots);
-        }
-        sync.pass_on(i, store, p.flags, place, kFwdOnes);
+        if (feeder && i > 0) feed(i - 1);
     }
-    sync.pass_last(count, store, p.flags, place, kFwdOnes);
+    if (feeder && count > 0) feed(count - 1);
+    if (feeder) tma_store_wait_all<0>();
     sync.leave();
 }
 
 // ---------------------------------------------------------------- forward, stage 2: u -> y
 // ACT: y = GELU(M x + bias), or without the GELU.  Iteration i multiplies tile i + 1 and transposes tile i.
 template <bool ACT>
-__device__ __forceinline__ void stage2(const CUtensorMap &tm_w, const CUtensorMap &tm_y, const Params &p, const uint32_t base, Shared &sh)
+__global__ void __launch_bounds__(kThreads, 1)
+stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_y, const Params p)
 {
-    const uint32_t stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
     const Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead};
     const Sync sync = {sh, p.status, kFwdStages, kFwdSlots};
-    const Place place(kFwdGroups, blockIdx.x - p.producers, gridDim.x - p.producers, p);
-    const int group = place.group, count = place.count;
-    auto tile = [&](int i) { return place.tile(i); };
+    init(sh);
+    const int group = blockIdx.x % kFwdGroups, first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
+    const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     const Lane ln;
-    const bool feeder = threadIdx.x == 0;
-    auto load = [&](int i) {                                 // by turns, warp i % 16
-        if (i < count && threadIdx.x == (i & (kWarps - 1)) * 32) {
-            if (p.flags != nullptr) wait_flag(p.flags + tile(i), kFwdGroups, group * 4, p.status, &sh.dead);
-            ring.load_linear(i, p.e_in + ((size_t)tile(i) * kM + group * kFwdBlocks) * kBlockBytes);
-        }
+    auto load = [&](int i) {
+        if (i < count) ring.load_linear(i, p.e_in + ((size_t)tile(i) * kM + group * kFwdBlocks) * kBlockBytes);
     };
-    if (feeder) sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
+    const bool feeder = threadIdx.x == 0;
+    if (feeder) {
+        sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
+        for (int i = 0; i < kFwdSlots - 1; ++i) load(i);
+    }
     auto feed = [&](int i) {
         sync.wait_staged(i);
         tma_store_3d(&tm_y, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks, tile(i) * kTok, 0);
         tma_store_commit();
+        load(i + kFwdSlots);
         sync.stored(i);
     };
     Weights<4> w;
     sync.take_weights(w, weights + ln.warp * (kM * 128), 0, false);
-    for (int i = 0; i < kFwdSlots; ++i) {
-        if (i == kFwdSlots - 1 && ln.warp == i) sync.wait(sh.w_read, 0, kErrSlotWait);       // the last slot lies where the weights were
-        load(i);
+    if (feeder) {
+        sync.wait(sh.w_read, 0, kErrSlotWait);
+        load(kFwdSlots - 1);
     }
-    __syncwarp();
     const __nv_bfloat16 *bias = ACT ? p.bias + ((threadIdx.x & 31) >> 2) * kM + group * kFwdBlocks + ln.warp : nullptr;
     auto multiply = [&](uint32_t e) {                        // in place: a warp's own block
 #pragma unroll
@@ -388,29 +324,10 @@ __device__ __forceinline__ void stage2(const CUtensorMap &tm_w, const CUtensorMa
         for (int n = 0; n < 4; ++n) stm4(stage + (ln.warp * 4 + n) * (kTok * 32) + t * 32 + ((jg ^ (t >> 2 & 1)) << 4), v[n]);
         sync.staged(i);
         if (feeder && i > 0) feed(i - 1);
-        if (i > 0 && ln.warp == ((i - 1 + kFwdSlots) & (kWarps - 1))) {
-            sync.wait_staged(i - 1);
-            load(i - 1 + kFwdSlots);
-            __syncwarp();
-        }
     }
     if (feeder && count > 0) feed(count - 1);
     if (feeder) tma_store_wait_all<0>();
     sync.leave();
-}
-
-// The first CTAs run stage 1, the others stage 2 behind them: nothing waits for a CTA with a higher index
-template <bool ACT>
-__global__ void __launch_bounds__(kThreads, 1)
-fwd_kernel(const __grid_constant__ CUtensorMap tm_R, const __grid_constant__ CUtensorMap tm_L, const __grid_constant__ CUtensorMap tm_x,
-           const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_y, const Params p)
-{
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ Shared sh;
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    init(sh);
-    if ((int)blockIdx.x < p.producers) stage1(tm_R, tm_x, tm_u, p, base, sh);
-    else                               stage2<ACT>(tm_L, tm_y, p, base, sh);
 }
 
 // ---------------------------------------------------------------- backward
@@ -459,16 +376,20 @@ struct Sums {
 
 // dy -> z, du (E tiles) and, with DW, dL.  Iteration i: z(i + 1), du(i), sums of tile i.
 template <bool DW>
-__device__ __forceinline__ void bwd_du(const CUtensorMap &tm_w, const CUtensorMap &tm_dy, const CUtensorMap &tm_du, const Params &p, const uint32_t base,
-                                       Shared &sh)
+__global__ void __launch_bounds__(kThreads, 1)
+bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_dy, const __grid_constant__ CUtensorMap tm_du,
+              const Params p)
 {
-    const uint32_t V0 = base + kDuSlots * kBwdTile, stage0 = V0 + 2 * kBwdTile;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, V0 = base + kDuSlots * kBwdTile, stage0 = V0 + 2 * kBwdTile;
     const uint32_t weights = base + 10 * kBwdTile;
     const Ring ring = {base, smem_u32(sh.full), kDuSlots, kBwdTile, p.status, &sh.dead};
     const Sync sync = {sh, p.status, kDuStages, 2};
-    const Place place(kBwdGroups, blockIdx.x, p.producers, p);
-    const int group = place.group, count = place.count;
-    auto tile = [&](int i) { return place.tile(i); };
+    init(sh);
+    const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
+    const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     constexpr int kItems = DW ? 2 : 1;                       // per tile: dy, u
     const Lane ln;
     int next = 0;
@@ -484,8 +405,12 @@ __device__ __forceinline__ void bwd_du(const CUtensorMap &tm_w, const CUtensorMa
         sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks);
         load_to(kDuSlots - 1);
     }
-    auto store = [&](int i) {
+    auto feed = [&](int i) {
+        sync.wait_staged(i);
         tma_store_2d(&tm_du, stage0 + i % kDuStages * kBwdTile, group * kBwdBlocks * 8, tile(i) * (2 * kM));
+        tma_store_commit();
+        load_to((DW ? 2 * i + 2 : i + 1) + kDuSlots);                // dy(i + 1) and u(i) have been read
+        sync.stored(i);
     };
     const int blk = ln.warp >> 1, half = ln.warp & 1;
     Weights<2> w;
@@ -530,53 +455,57 @@ __device__ __forceinline__ void bwd_du(const CUtensorMap &tm_w, const CUtensorMa
         }
         if (DW) sums.add<false>(V, ring.wait(2 * i + 1), blk, half);
         sync.staged(i);
-        if (feeder && i > 0) {
-            sync.wait_staged(i - 1);
-            load_to((DW ? 2 * i : i) + kDuSlots);            // dy(i) and u(i - 1) have been read
-        }
-        sync.pass_on(i, store, p.flags, place, kBwdOnes);
+        if (feeder && i > 0) feed(i - 1);
     }
-    sync.pass_last(count, store, p.flags, place, kBwdOnes);
+    if (feeder && count > 0) feed(count - 1);
     if (DW && count > 0)
-        sums.store(p.parts_l + (size_t)place.first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
+        sums.store(p.parts + (size_t)first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
+    if (feeder) tma_store_wait_all<0>();
     sync.leave();
 }
 
 // du -> dx (DX) and dR (DW)
 template <bool DX, bool DW>
-__device__ __forceinline__ void bwd_dx(const CUtensorMap &tm_w, const CUtensorMap &tm_x, const CUtensorMap &tm_dx, const Params &p, const uint32_t base,
-                                       Shared &sh)
+__global__ void __launch_bounds__(kThreads, 1)
+bwd_dx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_dx,
+              const Params p)
 {
-    const uint32_t stage0 = base + kDxSlots * kBwdTile;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ Shared sh;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kDxSlots * kBwdTile;
     const Ring ring = {base, smem_u32(sh.full), kDxSlots, kBwdTile, p.status, &sh.dead};
     const Sync sync = {sh, p.status, DX ? kDxStages : kMaxStages, 1};   // without staging, warps are up to five tiles apart
-    const Place place(kBwdGroups, blockIdx.x - p.producers, gridDim.x - p.producers, p);
-    const int group = place.group, count = place.count;
-    auto tile = [&](int i) { return place.tile(i); };
+    init(sh);
+    const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
+    const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     constexpr int kItems = DW ? 2 : 1;                       // per tile: du, x
     const Lane ln;
-    const bool feeder = threadIdx.x == 0;
-    constexpr int kAhead = kDxSlots / kItems;
-    auto load = [&](int i) {                                 // by turns, warp i % 16
-        if (i < count && threadIdx.x == (i & (kWarps - 1)) * 32) {
-            const int t = tile(i);
-            if (DW) ring.load(kItems * i + 1, &tm_x, t, group * kBwdBlocks);
-            if (p.flags != nullptr) wait_flag(p.flags + t, kBwdGroups, group * 4, p.status, &sh.dead);
-            ring.load_linear(kItems * i, p.e_in + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
+    int next = 0;
+    auto load_to = [&](int last) {
+        for (; next <= last && next < kItems * count; ++next) {
+            const int t = tile(next / kItems);
+            if (DW && (next & 1)) ring.load(next, &tm_x, t, group * kBwdBlocks);
+            else                  ring.load_linear(next, p.e_in + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
         }
     };
-    if (DX && feeder) sync.load_weights(stage0, &tm_w, group * kBwdBlocks, kBwdBlocks);
+    const bool feeder = threadIdx.x == 0;
+    if (feeder) {
+        if (DX) sync.load_weights(stage0, &tm_w, group * kBwdBlocks, kBwdBlocks);
+        load_to(kDxSlots - 1);
+    }
     auto feed = [&](int i) {
         sync.wait_staged(i);
-        tma_store_3d(&tm_dx, stage0 + i % kDxStages * kBwdTile, 0, tile(i) * kTok, group * kBwdBlocks);
-        tma_store_commit();
-        sync.stored(i);
+        if (DX) {
+            tma_store_3d(&tm_dx, stage0 + i % kDxStages * kBwdTile, 0, tile(i) * kTok, group * kBwdBlocks);
+            tma_store_commit();
+        }
+        load_to(kItems * (i + 1) - 1 + kDxSlots);
+        if (DX) sync.stored(i);
     };
     const int blk = ln.warp >> 1, half = ln.warp & 1;
     Weights<2> w;
     if (DX) sync.take_weights(w, stage0 + blk * (kM * 128), half * 32, true);
-    for (int i = 0; i < kAhead; ++i) load(i);
-    __syncwarp();
     Sums sums;
     if (DW) sums.clear();
     for (int i = 0; i < count; ++i) {
@@ -597,43 +526,24 @@ __device__ __forceinline__ void bwd_dx(const CUtensorMap &tm_w, const CUtensorMa
         }
         if (DW) sums.add<true>(du, ring.wait(2 * i + 1), blk, half);
         sync.staged(i);
-        if (DX && feeder && i > 0) feed(i - 1);
-        if (i > 0 && ln.warp == ((i - 1 + kAhead) & (kWarps - 1))) {
-            sync.wait_staged(i - 1);
-            load(i - 1 + kAhead);
-            __syncwarp();
-        }
+        if (feeder && i > 0) feed(i - 1);
     }
-    if (DX && feeder && count > 0) feed(count - 1);
+    if (feeder && count > 0) feed(count - 1);
     if (DW && count > 0)
-        sums.store(p.parts_r + (size_t)place.first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
+        sums.store(p.parts + (size_t)first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
     if (feeder) tma_store_wait_all<0>();
     sync.leave();
-}
-
-template <bool DX, bool DW>
-__global__ void __launch_bounds__(kThreads, 1)
-bwd_kernel(const __grid_constant__ CUtensorMap tm_L, const __grid_constant__ CUtensorMap tm_R, const __grid_constant__ CUtensorMap tm_dy,
-           const __grid_constant__ CUtensorMap tm_du, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_dx,
-           const Params p)
-{
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ Shared sh;
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    init(sh);
-    if ((int)blockIdx.x < p.producers) bwd_du<DW>(tm_L, tm_dy, tm_du, p, base, sh);
-    else                               bwd_dx<DX, DW>(tm_R, tm_x, tm_dx, p, base, sh);
 }
 
 // grads = (accumulate ? grads : 0) + the parts of every rank, in order; 64 groups of 4 elements and 4 ranges of ranks per CTA
 __global__ void __launch_bounds__(256)
 add_parts_m64_kernel(const float *__restrict__ parts_l, const float *__restrict__ parts_r, float *__restrict__ dL, float *__restrict__ dR,
-                     int grid_l, int grid_r, int accumulate)
+                     int grid, int accumulate)
 {
     __shared__ float4 red[4][64];
     constexpr int kPer = 64 * 4, kCtas = (int)(kGradElems / kPer);
     const int kind = blockIdx.x / kCtas, at = blockIdx.x % kCtas * kPer + (threadIdx.x & 63) * 4, range = threadIdx.x >> 6;
-    const int group = at / (kBwdBlocks * kM * kM), n = ((kind == 0 ? grid_l : grid_r) - group + kBwdGroups - 1) / kBwdGroups, per = (n + 3) / 4;
+    const int group = at / (kBwdBlocks * kM * kM), n = (grid - group + kBwdGroups - 1) / kBwdGroups, per = (n + 3) / 4;
     const float *src = (kind == 0 ? parts_l : parts_r) + at;
     float *dst = (kind == 0 ? dL : dR) + at;
     float4 s = make_float4(0, 0, 0, 0);
@@ -687,67 +597,56 @@ int64_t tiles_of(int64_t tokens) { return (tokens + kTok - 1) / kTok; }
 size_t max_ranks(int64_t tokens) { return (size_t)(tiles_of(tokens) < kMaxRanks ? tiles_of(tokens) : kMaxRanks); }
 size_t e_bytes(int64_t tokens) { return (size_t)tiles_of(tokens) * kTileBytes; }
 
-// CTAs of the two stages of a launch.  One per tile and group while there are SMs for both; beyond that a share of the SMs each,
-// by what a tile costs (measured: `share` hundredths for the first stage).  Without flags (more tiles than the 64 KB of
-// counters serve, or one stage only) each stage is a launch on all SMs.
-struct Split {
-    int producers, consumers;
-    Split(int groups, int tiles, int sms, int share)
-    {
-        const int64_t all = (int64_t)tiles * groups;
-        producers = consumers = (int)(all < sms ? all : sms);
-        if (producers + consumers <= sms) return;
-        producers = sms * share / 100;
-        if (consumers > sms - producers) consumers = sms - producers;
-        if (producers < sms - consumers) producers = sms - consumers;
-    }
-};
-constexpr int kMaxFlags = 65536 / 4;
+int grid_of(int groups, int sms, int64_t tokens)
+{
+    const int64_t all = tiles_of(tokens) * groups;
+    return (int)(all < sms ? all : sms);
+}
+
+int stage1(const void *x, const void *R, char *u, int64_t tokens, int sms, unsigned *status, cudaStream_t s)
+{
+    CUtensorMap tm_w, tm_x, tm_u;
+    MONARCH_TRY(map_w(&tm_w, R));
+    MONARCH_TRY(map_t(&tm_x, x, tokens, kFwdBlocks));
+    MONARCH_TRY(map_e(&tm_u, u, (int)tiles_of(tokens), kFwdBlocks));
+    Params p = {};
+    p.status = status;
+    p.tiles = (int)tiles_of(tokens);
+    return launch_serialized(stage1_kernel, grid_of(kFwdGroups, sms, tokens), kThreads, kFwdSmem, s, tm_w, tm_x, tm_u, p);
+}
 
 }  // namespace
+}  // namespace tc
 
-// y = act(M x + bias) (bias null: y = M x); u: E tiles of all tokens, kept for the backward call.  y null: u only.
+// y = act(M x + bias) (bias null: y = M x); u: E tiles of all tokens, kept for the backward call
 static int stream_fwd(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, void *u, int64_t tokens,
-                      int backwards, char *ws, cudaStream_t s)
+                      unsigned *status, cudaStream_t s)
 {
+    using namespace tc;
     if (tokens == 0) return MONARCH_OK;
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
-    CUtensorMap tm_R, tm_L, tm_x, tm_u, tm_y;
-    MONARCH_TRY(map_w(&tm_R, R));
-    MONARCH_TRY(map_w(&tm_L, L));
-    MONARCH_TRY(map_t(&tm_x, x, tokens, kFwdBlocks));
-    MONARCH_TRY(map_e(&tm_u, u, (int)tiles_of(tokens), kFwdBlocks));
-    MONARCH_TRY(map_y(&tm_y, y != nullptr ? y : x, tokens, kFwdBlocks));
+    MONARCH_TRY(stage1(x, R, (char *)u, tokens, sms, status, s));
+    CUtensorMap tm_w, tm_y;
+    MONARCH_TRY(map_w(&tm_w, L));
+    MONARCH_TRY(map_y(&tm_y, y, tokens, kFwdBlocks));
     Params p = {};
-    p.status = (unsigned *)ws;
+    p.status = status;
     p.bias = (const __nv_bfloat16 *)bias;
     p.gelu = gelu;
     p.e_in = (const char *)u;
     p.tiles = (int)tiles_of(tokens);
-    p.last = backwards ? p.tiles - 1 : 0;
-    auto kernel = bias != nullptr ? fwd_kernel<true> : fwd_kernel<false>;
-    static const int share = getenv("FSH") ? atoi(getenv("FSH")) : 45;
-    const int64_t all = (int64_t)p.tiles * kFwdGroups;
-    Split split(kFwdGroups, p.tiles, sms, share);
-    if (y == nullptr || p.tiles > kMaxFlags || getenv("NOFL")) {
-        split.producers = split.consumers = (int)(all < sms ? all : sms);
-        p.producers = split.producers;
-        MONARCH_TRY(launch_serialized(kernel, split.producers, kThreads, kFwdSmem, s, tm_R, tm_L, tm_x, tm_u, tm_y, p));
-        p.producers = 0;
-        p.last = p.last != 0 ? 0 : p.tiles - 1;
-        return y == nullptr ? MONARCH_OK : launch_serialized(kernel, split.consumers, kThreads, kFwdSmem, s, tm_R, tm_L, tm_x, tm_u, tm_y, p);
-    }
-    p.flags = (unsigned *)(ws + MONARCH_STATUS_BYTES);
-    p.producers = split.producers;
-    return launch_serialized(kernel, split.producers + split.consumers, kThreads, kFwdSmem, s, tm_R, tm_L, tm_x, tm_u, tm_y, p);
+    p.last = p.tiles - 1;
+    return launch_serialized(bias != nullptr ? stage2_kernel<true> : stage2_kernel<false>, grid_of(kFwdGroups, sms, tokens), kThreads, kFwdSmem, s,
+                             tm_w, tm_y, p);
 }
 
 // dx null: gradients only; dL null: dx only.  u: what the forward call left (u_saved), or scratch for E tiles of all tokens;
 // du: scratch of the same size; parts: two gradients of max_ranks(tokens)
 static int stream_bwd(const void *x, const void *dy, const void *L, const void *R, const void *u, bool u_saved, void *dx, float *dL, float *dR,
-                      int accumulate, void *du, void *parts, int64_t tokens, char *ws, cudaStream_t s)
+                      int accumulate, void *du, void *parts, int64_t tokens, unsigned *status, cudaStream_t s)
 {
+    using namespace tc;
     if (tokens == 0) {
         if (dL != nullptr && !accumulate) {
             MONARCH_CUDA_TRY(cudaMemsetAsync(dL, 0, kGradElems * sizeof(float), s));
@@ -758,43 +657,31 @@ static int stream_bwd(const void *x, const void *dy, const void *L, const void *
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
     if (sms > kMaxRanks * kBwdGroups) sms = kMaxRanks * kBwdGroups;
-    if (dL != nullptr && !u_saved) MONARCH_TRY(stream_fwd(x, L, R, nullptr, 0, nullptr, (void *)u, tokens, 0, ws, s));
-    Params p = {};
-    p.status = (unsigned *)ws;
-    p.tiles = (int)tiles_of(tokens);
+    float *parts_l = (float *)parts, *parts_r = parts_l + max_ranks(tokens) * kGradElems;
+    const int grid = grid_of(kBwdGroups, sms, tokens), tiles = (int)tiles_of(tokens);
+    if (dL != nullptr && !u_saved) MONARCH_TRY(stage1(x, R, (char *)u, tokens, sms, status, s));
     CUtensorMap tm_L, tm_R, tm_dy, tm_du, tm_x, tm_dx;
     MONARCH_TRY(map_w(&tm_L, L));
     MONARCH_TRY(map_w(&tm_R, R));
     MONARCH_TRY(map_y(&tm_dy, dy, tokens, kBwdBlocks));
-    MONARCH_TRY(map_e(&tm_du, du, p.tiles, kBwdBlocks));
+    MONARCH_TRY(map_e(&tm_du, du, tiles, kBwdBlocks));
     MONARCH_TRY(map_t(&tm_x, dL != nullptr ? x : dy, tokens, kBwdBlocks));
     MONARCH_TRY(map_t(&tm_dx, dx != nullptr ? dx : dy, tokens, kBwdBlocks));
+    Params p = {};
+    p.status = status;
     p.u = (const char *)u;
+    p.parts = parts_l;
+    p.tiles = tiles;
+    MONARCH_TRY(launch_serialized(dL != nullptr ? bwd_du_kernel<true> : bwd_du_kernel<false>, grid, kThreads, kBwdSmem, s, tm_L, tm_dy, tm_du, p));
     p.e_in = (const char *)du;
-    p.parts_l = (float *)parts;
-    p.parts_r = p.parts_l + max_ranks(tokens) * kGradElems;
-    p.last = p.tiles - 1;
-    auto kernel = dx == nullptr ? bwd_kernel<false, true> : dL == nullptr ? bwd_kernel<true, false> : bwd_kernel<true, true>;
-    static const int share = getenv("BSH") ? atoi(getenv("BSH")) : 50;
-    const int64_t all = (int64_t)p.tiles * kBwdGroups;
-    Split split(kBwdGroups, p.tiles, sms, share);
-    if (p.tiles > kMaxFlags || getenv("NOFL")) {
-        split.producers = split.consumers = (int)(all < sms ? all : sms);
-        p.producers = split.producers;
-        MONARCH_TRY(launch_serialized(kernel, split.producers, kThreads, kBwdSmem, s, tm_L, tm_R, tm_dy, tm_du, tm_x, tm_dx, p));
-        p.producers = 0;
-        p.last = 0;
-        MONARCH_TRY(launch_serialized(kernel, split.consumers, kThreads, kBwdSmem, s, tm_L, tm_R, tm_dy, tm_du, tm_x, tm_dx, p));
-    } else {
-        p.flags = (unsigned *)(ws + MONARCH_STATUS_BYTES);
-        p.producers = split.producers;
-        MONARCH_TRY(launch_serialized(kernel, split.producers + split.consumers, kThreads, kBwdSmem, s, tm_L, tm_R, tm_dy, tm_du, tm_x, tm_dx, p));
-    }
+    p.parts = parts_r;
+    p.last = tiles - 1;
+    auto last = dx == nullptr ? bwd_dx_kernel<false, true> : dL == nullptr ? bwd_dx_kernel<true, false> : bwd_dx_kernel<true, true>;
+    MONARCH_TRY(launch_serialized(last, grid, kThreads, kBwdSmem, s, tm_R, tm_x, tm_dx, p));
     if (dL == nullptr) return MONARCH_OK;
-    return launch_serialized(add_parts_m64_kernel, 2 * (int)(kGradElems / 256), 256, 0, s, (const float *)p.parts_l, (const float *)p.parts_r, dL, dR,
-                             split.producers, split.consumers, accumulate);
+    return launch_serialized(add_parts_m64_kernel, 2 * (int)(kGradElems / 256), 256, 0, s, (const float *)parts_l, (const float *)parts_r, dL, dR,
+                             grid, accumulate);
 }
-}  // namespace tc
 
 // Workspaces: [status][64 KB left out: the counters of kernels that share it stay zero][E tiles ...][parts]
 namespace {
@@ -816,11 +703,11 @@ int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t 
         const int st = fused_fwd_m64_cluster(x, L, R, y, tokens, ws, s);
         if (st != MONARCH_ERR_UNSUPPORTED) return st;
     }
-    return tc::stream_fwd(x, L, R, nullptr, 0, y, head(ws), tokens, 0, (char *)ws, s);
+    return stream_fwd(x, L, R, nullptr, 0, y, head(ws), tokens, (unsigned *)ws, s);
 }
 int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws, cudaStream_t s)
 {
-    return tc::stream_fwd(x, L, R, bias, gelu, y, head(ws), tokens, 0, (char *)ws, s);
+    return stream_fwd(x, L, R, bias, gelu, y, head(ws), tokens, (unsigned *)ws, s);
 }
 
 size_t fused_mlp_fwd_m64_workspace_bytes(int64_t tokens) { return kHead + 2 * tc::e_bytes(tokens); }
@@ -828,14 +715,14 @@ int fused_mlp_fwd_m64(const void *x, const void *L1, const void *R1, const void 
                       int64_t tokens, void *ws, cudaStream_t s)
 {
     char *u = head(ws), *h = u + tc::e_bytes(tokens);
-    MONARCH_TRY(tc::stream_fwd(x, L1, R1, b1, 1, h, u, tokens, 0, (char *)ws, s));
-    return tc::stream_fwd(h, L2, R2, b2, 0, y, u, tokens, 1, (char *)ws, s);
+    MONARCH_TRY(stream_fwd(x, L1, R1, b1, 1, h, u, tokens, (unsigned *)ws, s));
+    return stream_fwd(h, L2, R2, b2, 0, y, u, tokens, (unsigned *)ws, s);
 }
 
 size_t fused_bwd_dx_m64_workspace_bytes(int64_t tokens) { return kHead + tc::e_bytes(tokens); }
 int fused_bwd_dx_m64(const void *dy, const void *L, const void *R, void *dx, int64_t tokens, void *ws, cudaStream_t s)
 {
-    return tc::stream_bwd(nullptr, dy, L, R, nullptr, false, dx, nullptr, nullptr, 0, head(ws), nullptr, tokens, (char *)ws, s);
+    return stream_bwd(nullptr, dy, L, R, nullptr, false, dx, nullptr, nullptr, 0, head(ws), nullptr, tokens, (unsigned *)ws, s);
 }
 
 size_t fused_bwd_m64_workspace_bytes(int64_t tokens) { return kHead + 2 * tc::e_bytes(tokens) + 2 * tc::max_ranks(tokens) * tc::kGradElems * sizeof(float); }
@@ -843,7 +730,7 @@ int fused_bwd_m64(const void *x, const void *dy, const void *L, const void *R, c
                   int64_t tokens, void *ws, cudaStream_t s)
 {
     char *du = head(ws), *u = du + tc::e_bytes(tokens), *parts = u + tc::e_bytes(tokens);
-    return tc::stream_bwd(x, dy, L, R, u_saved != nullptr ? u_saved : u, u_saved != nullptr, dx, dL, dR, accumulate, du, parts, tokens, (char *)ws, s);
+    return stream_bwd(x, dy, L, R, u_saved != nullptr ? u_saved : u, u_saved != nullptr, dx, dL, dR, accumulate, du, parts, tokens, (unsigned *)ws, s);
 }
 
 }  // namespace monarch
