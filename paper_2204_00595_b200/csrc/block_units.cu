@@ -19,16 +19,17 @@ constexpr int kSms = 148;                              // of the part this libra
 
 // Tile sizes of a launch.  Small: as many CTAs as possible share the weights of a few tokens.  Large: fewer, larger
 // units, so that weights and inputs are read less often.
-struct Sizes { int TT, ES, LS, KS; };
+struct Sizes { int TT, ES, LS, KS, TW; };
 template <typename T, int M> struct Small { typedef Cfg<T, M, 16, 16, M < 32 ? M : 32, M < 32 ? M : 32> C; };
 template <typename T, int M> struct Large { typedef typename Small<T, M>::C C; };
 template <> struct Large<bf16, 16> { typedef Cfg<bf16, 16, 64, 16, 16, 16> C; };
 template <> struct Large<bf16, 32> { typedef Cfg<bf16, 32, 64, 32, 32, 32> C; };
 template <> struct Large<bf16, 64> { typedef Cfg<bf16, 64, 32, 64, 32, 32> C; };
-template <> struct Large<float, 32> { typedef Cfg<float, 32, 32, 32, 32, 32> C; };
-template <> struct Large<float, 64> { typedef Cfg<float, 64, 16, 32, 32, 32> C; };
+template <> struct Large<float, 32> { typedef Cfg<float, 32, 32, 32, 32, 32, 16> C; };
+template <> struct Large<float, 64> { typedef Cfg<float, 64, 32, 64, 64, 64, 16> C; };
+template <> struct Large<float, 128> { typedef Cfg<float, 128, 32, 64, 64, 64, 16> C; };
 
-template <typename C> Sizes sizes_of() { return {C::TT, C::ES, C::LS, C::KS}; }
+template <typename C> Sizes sizes_of() { return {C::TT, C::ES, C::LS, C::KS, C::TW}; }
 template <typename T> Sizes sizes_t(int m, bool large)
 {
     switch (m) {
@@ -52,7 +53,7 @@ constexpr int kMaxSplits = 16;
 int wgrad_splits(int dtype, int m, int64_t tokens)
 {
     const Sizes s = sizes(dtype, m, use_large(dtype, m, tokens));
-    const long long base = (long long)(m / 8) * (m / s.LS) * (m / s.KS), steps = ceil_div(tokens, 32);
+    const long long base = (long long)(m / 8) * (m / s.LS) * (m / s.KS), steps = ceil_div(tokens, s.TW);
     long long n = kSms / base;
     if (n > steps / 4) n = steps / 4;
     if (n > kMaxSplits) n = kMaxSplits;
@@ -132,7 +133,7 @@ struct Builder {
     {
         const int n = wgrad_splits(dtype, m, p.tokens);
         Op &o = add(kWgrad, phase, (long long)(m / 8) * (m / sz.LS) * (m / sz.KS) * n,
-                    ceil_div(ceil_div(p.tokens, 32), n) * 32 * (sz.LS + sz.KS) * 8);
+                    ceil_div(p.tokens, n) * (sz.LS + sz.KS) * 8);
         o.perm = perm;
         o.in = rows;
         o.in2 = cols;

@@ -65,15 +65,18 @@ struct Params {
 constexpr int kBarrierWord = 8, kDoneWord = 9;
 constexpr unsigned kErrGridWait = 0x301;
 
-template <typename T_, int M_, int TT_, int ES_, int LS_, int KS_> struct Cfg {
+template <typename T_, int M_, int TT_, int ES_, int LS_, int KS_, int KC_ = 0> struct Cfg {
     typedef T_ T;
     static constexpr int M = M_, TT = TT_, ES = ES_, LS = LS_, KS = KS_, G = 8;
     static constexpr bool kBf = std::is_same<T, bf16>::value;
-    static constexpr int kWpb = 1, kThreads = 32 * G * kWpb;
+    static constexpr int kWpb = KC_ > 0 ? 2 : 1, kThreads = 32 * G * kWpb;   // warps per block
     static constexpr int EW = ES / kWpb, KW = KS / kWpb;      // outputs / gradient columns of one warp
     static constexpr int kPad = kBf ? 8 : 4;                  // rows 16 bytes longer: conflict-free ldmatrix / 16-byte reads
     static constexpr int PA = M + kPad, PE = ES + kPad, PL = LS + kPad, PK = KS + kPad;
-    static constexpr int TW = 32;                             // tokens per step of a weight gradient
+    // KC > 0 (fp32, many tokens): both operands of a stage stream through shared memory, KC columns at a time, which
+    // leaves room for 8 x 8 results per lane; one CTA per SM
+    static constexpr int KC = KC_, PC = KC + 4;
+    static constexpr int TW = KC ? 16 : 32;                   // tokens per step of a weight gradient
     static constexpr int cmax(int a, int b) { return a > b ? a : b; }
     // staging of results: permuted role - one plane of words per pair of bf16 blocks (per fp32 block), pitch 8 mod 32;
     // natural role - rows of ES outputs and rows of 8 blocks, each 16 bytes longer
@@ -85,14 +88,16 @@ template <typename T_, int M_, int TT_, int ES_, int LS_, int KS_> struct Cfg {
     static constexpr int kStepBytes = G * TW * (PL + PK) * (int)sizeof(T);
     // Two CTAs per SM work on different units while each waits for its own loads.  Within that share of shared memory: two
     // tiles (the next unit's input is on its way during this one's work), or one, or one that the results are staged over.
-    static constexpr int kHalf = 113 * 1024 - 512;
+    static constexpr int kChunkA = G * TT * PC * 4, kChunkW = cmax(G * ES * PC, G * KC * (ES + 4)) * 4, kChunk = kChunkA + kChunkW;
+    static constexpr int kHalf = KC ? 226 * 1024 : 113 * 1024 - 512;
     static constexpr int kBufs = 2 * kTileBytes + kWBytes + kStageBytes <= kHalf ? 2 : 1;
-    static constexpr bool kAlias = kTileBytes + kWBytes + kStageBytes > kHalf;
-    static constexpr int kWAt = kAlias ? cmax(kTileBytes, kStageBytes) : kBufs * kTileBytes, kStageAt = kAlias ? 0 : kWAt + kWBytes;
+    static constexpr bool kAlias = KC == 0 && kTileBytes + kWBytes + kStageBytes > kHalf;
+    static constexpr int kWAt = kAlias ? cmax(kTileBytes, kStageBytes) : kBufs * kTileBytes;
+    static constexpr int kStageAt = KC ? 2 * kChunk : kAlias ? 0 : kWAt + kWBytes;
     static constexpr int kStageSmem = kAlias ? kWAt + kWBytes : kStageAt + kStageBytes;
     static constexpr int kSteps = 2 * kStepBytes <= cmax(kStageSmem, kHalf) ? 2 : 1;   // buffers of a weight gradient
     static constexpr int kSmem = cmax(kStageSmem, kSteps * kStepBytes);
-    static constexpr int kCtas = kSmem <= kHalf ? 2 : 1;
+    static constexpr int kCtas = kSmem <= 113 * 1024 - 512 ? 2 : 1;
 };
 
 // ---------------------------------------------------------------- small device helpers
@@ -152,19 +157,19 @@ template <typename C, int R, int NC, int PITCH> struct TileLoad {
     {
         const uint4 *src = static_cast<const uint4 *>(v.p);
         if (!perm) {
-            constexpr int kPieces = R * NC;            // per token: 8 blocks x NC / 8
+            // 16 bytes per lane, neighbours in memory on neighbouring lanes; per token: 8 blocks x NC / 8 pieces of H
+            constexpr int kVecs = R * NC * H;
             const unsigned first = t0 * v.t_stride + b0 * v.b_stride + c8 * v.c_stride;
 #pragma unroll 4
-            for (int i = threadIdx.x; i < kPieces; i += kThreads) {
+            for (int j = threadIdx.x; j < kVecs; j += kThreads) {
+                const int h = j % H, i = j / H;
                 int b, c;
                 if (v.mid) { b = i % 8; c = i / 8 % (NC / 8); }
                 else       { c = i % (NC / 8); b = i / (NC / 8) % 8; }
                 const int t = i / NC;
                 const bool ok = t < left;
-                const uint4 *g = src + (size_t)(first + (ok ? t : 0) * v.t_stride + b * v.b_stride + c * v.c_stride) * H;
-                T *d = tile + (b * R + t) * PITCH + c * 8;
-                cp_async16(d, g, ok);
-                if (H == 2) cp_async16(d + 4, g + 1, ok);
+                cp_async16(tile + (b * R + t) * PITCH + c * 8 + h * 4,
+                           src + (size_t)(first + (ok ? t : 0) * v.t_stride + b * v.b_stride + c * v.c_stride) * H + h, ok);
             }
             return;
         }
@@ -276,13 +281,16 @@ template <typename C> struct Acc<C, true> {
 };
 template <typename C> struct Acc<C, false> {
     float v[C::TT / 4][C::EW / 8];
+    static constexpr int V = C::EW / 8 < 4 ? C::EW / 8 : 4;
+    int packed;                                        // outputs of a lane: V neighbours at a time, else every eighth
+    __device__ __forceinline__ int output(int el, int q) const { return packed ? V * el + 8 * V * (q / V) + q % V : el + 8 * q; }
     template <typename F> __device__ __forceinline__ void each(F f)
     {
         const int tl = (threadIdx.x & 31) >> 3, el = threadIdx.x & 7;
 #pragma unroll
         for (int i = 0; i < C::TT / 4; ++i)
 #pragma unroll
-            for (int q = 0; q < C::EW / 8; ++q) f(v[i][q], tl + 4 * i, el + 8 * q);
+            for (int q = 0; q < C::EW / 8; ++q) f(v[i][q], tl + 4 * i, output(el, q));
     }
     template <typename F> __device__ __forceinline__ void column_sums(F f)
     {
@@ -294,7 +302,7 @@ template <typename C> struct Acc<C, false> {
             for (int i = 0; i < C::TT / 4; ++i) s += v[i][q];
             s += __shfl_xor_sync(0xffffffffu, s, 8);
             s += __shfl_xor_sync(0xffffffffu, s, 16);
-            if (tl == 0) f(s, el + 8 * q);
+            if (tl == 0) f(s, output(el, q));
         }
     }
 };
@@ -336,33 +344,30 @@ __device__ __forceinline__ void copy_out(const unsigned char *stage, const View 
     typedef typename C::T T;
     constexpr int H = (int)sizeof(T) / 2;
     uint4 *dst = static_cast<uint4 *>(out.p);
-    constexpr int kPieces = C::TT * C::ES;             // natural: per token 8 blocks x ES / 8; permuted: ES
+    constexpr int kVecs = C::TT * C::ES * H;           // natural: per token 8 blocks x ES / 8 pieces; permuted: ES; H each
     if (!perm) {
         const unsigned first = t0 * out.t_stride + b0 * out.b_stride + e0 / 8 * out.c_stride;
 #pragma unroll 4
-        for (int i = threadIdx.x; i < kPieces; i += C::kThreads) {
+        for (int j = threadIdx.x; j < kVecs; j += C::kThreads) {
+            const int h = j % H, i = j / H;
             int b, c;
             if (out.mid) { b = i % 8; c = i / 8 % (C::ES / 8); }
             else         { c = i % (C::ES / 8); b = i / (C::ES / 8) % 8; }
             const int t = i / C::ES;
             if (t >= left) break;
-            const uint4 *s = reinterpret_cast<const uint4 *>(stage + t * C::kNatT + b * C::kNatB + c * 8 * sizeof(T));
-            uint4 *d = dst + (size_t)(first + t * out.t_stride + b * out.b_stride + c * out.c_stride) * H;
-            d[0] = s[0];
-            if (H == 2) d[1] = s[1];
+            dst[(size_t)(first + t * out.t_stride + b * out.b_stride + c * out.c_stride) * H + h] =
+                *reinterpret_cast<const uint4 *>(stage + t * C::kNatT + b * C::kNatB + c * 8 * sizeof(T) + h * 16);
         }
         return;
     }
     const unsigned first = t0 * out.t_stride + b0 / 8 * out.b_stride + e0 * out.c_stride;
 #pragma unroll 4
-    for (int i = threadIdx.x; i < kPieces; i += C::kThreads) {
-        const int e = i % C::ES, t = i / C::ES;
+    for (int j = threadIdx.x; j < kVecs; j += C::kThreads) {
+        const int h = j % H, e = j / H % C::ES, t = j / (H * C::ES);
         if (t >= left) break;
-        const uint32_t *s = reinterpret_cast<const uint32_t *>(stage) + t * C::PS + e;
-        uint4 *d = dst + (size_t)(first + t * out.t_stride + e * out.c_stride) * H;
         constexpr int kPlane = C::TT * C::PS;
-        d[0] = make_uint4(s[0], s[kPlane], s[2 * kPlane], s[3 * kPlane]);
-        if constexpr (!C::kBf) d[1] = make_uint4(s[4 * kPlane], s[5 * kPlane], s[6 * kPlane], s[7 * kPlane]);
+        const uint32_t *s = reinterpret_cast<const uint32_t *>(stage) + h * 4 * kPlane + t * C::PS + e;
+        dst[(size_t)(first + t * out.t_stride + e * out.c_stride) * H + h] = make_uint4(s[0], s[kPlane], s[2 * kPlane], s[3 * kPlane]);
     }
 }
 
@@ -450,7 +455,149 @@ __device__ __forceinline__ void multiply(Acc<C> &acc, const typename C::T *tile,
                 const float2 t = unpack2(s[i][q]);
                 acc.v[i][q] = t.x + t.y;
             }
+        acc.packed = 0;
     }
+}
+
+// ---- the same with both operands streamed in chunks of KC columns (fp32, many tokens)
+// Bound by FMA issue once a lane has 8 x 4 results: 12 loads of 16 bytes from shared memory feed 64 packed FMAs, where the
+// 4 x 4 results that fit beside resident operands take 8 for 32 and wait for shared memory (m = 64, us: forward of 1500
+// tokens 158 -> 107, forward + backward of 2048 tokens 544 -> 397; m = 128, 400 tokens 997 -> 742; m = 32, 8000 tokens
+// 379 -> 331).  Blocks as stored ([out][in]): the FMA packs two columns of the contraction; transposed blocks ([in][out]):
+// it packs two outputs.
+template <typename C> struct Chunks {
+    static constexpr int TT = C::TT, ES = C::ES, KC = C::KC, PC = C::PC, M = C::M, EW = C::EW, RT = TT / 4, RE = EW / 8;
+    f32x2 s[RT][RE];                                   // [out][in]: sums over even and odd columns; else [RT][RE / 2] used
+
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+#pragma unroll
+            for (int q = 0; q < RE; ++q) s[i][q] = 0;
+    }
+    static __device__ __forceinline__ void load_w(float *wt, const void *w, int trans, int b0, int e0, int c0)
+    {
+        const float *src = static_cast<const float *>(w) + (size_t)b0 * M * M;
+        constexpr int kVecs = 8 * ES * KC / 4;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < kVecs; i += C::kThreads) {
+            if (!trans) {
+                const int c = i % (KC / 4) * 4, e = i / (KC / 4) % ES, b = i / (KC / 4 * ES);
+                cp_async16(wt + (b * ES + e) * PC + c, src + (b * M + e0 + e) * M + c0 + c, true);
+            } else {
+                const int e = i % (ES / 4) * 4, c = i / (ES / 4) % KC, b = i / (ES / 4 * KC);
+                cp_async16(wt + (b * KC + c) * (ES + 4) + e, src + (b * M + c0 + c) * M + e0 + e, true);
+            }
+        }
+    }
+    __device__ __forceinline__ void multiply(const float *tile, const float *wt, int trans)
+    {
+        const int w = (threadIdx.x >> 5) / C::kWpb, e0 = (threadIdx.x >> 5) % C::kWpb * EW;
+        const int tl = (threadIdx.x & 31) >> 3, el = threadIdx.x & 7;
+        const float *a = tile + (w * TT + tl) * PC;
+        if (!trans) {
+            const float *b = wt + (w * ES + e0 + el) * PC;
+#pragma unroll
+            for (int c = 0; c < KC; c += 4) {
+                ulonglong2 fb[RE];
+#pragma unroll
+                for (int q = 0; q < RE; ++q) fb[q] = *reinterpret_cast<const ulonglong2 *>(b + 8 * q * PC + c);
+#pragma unroll
+                for (int i = 0; i < RT; ++i) {
+                    const ulonglong2 fa = *reinterpret_cast<const ulonglong2 *>(a + 4 * i * PC + c);
+#pragma unroll
+                    for (int q = 0; q < RE; ++q) s[i][q] = fma2(fa.y, fb[q].y, fma2(fa.x, fb[q].x, s[i][q]));
+                }
+            }
+        } else {
+            constexpr int V = RE < 4 ? RE : 4;             // neighbouring outputs of a lane
+            const float *b = wt + w * KC * (ES + 4) + e0 + V * el;
+#pragma unroll
+            for (int c = 0; c < KC; c += 4) {
+                f32x2 fb[4][RE / 2];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int q = 0; q < RE / V; ++q) {
+                        const float *at = b + (c + k) * (ES + 4) + 8 * V * q;
+                        if constexpr (V == 4) {
+                            const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(at);
+                            fb[k][2 * q] = t.x;
+                            fb[k][2 * q + 1] = t.y;
+                        } else {
+                            fb[k][q] = *reinterpret_cast<const f32x2 *>(at);
+                        }
+                    }
+#pragma unroll
+                for (int i = 0; i < RT; ++i) {
+                    const float4 fa = *reinterpret_cast<const float4 *>(a + 4 * i * PC + c);
+                    const float av[4] = {fa.x, fa.y, fa.z, fa.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const f32x2 d = pack2(av[k], av[k]);
+#pragma unroll
+                        for (int q = 0; q < RE / 2; ++q) s[i][q] = fma2(d, fb[k][q], s[i][q]);
+                    }
+                }
+            }
+        }
+    }
+    __device__ __forceinline__ void finish(Acc<C> &acc, int trans) const
+    {
+        acc.packed = trans;
+        if (trans) {
+#pragma unroll
+            for (int i = 0; i < RT; ++i)
+#pragma unroll
+                for (int q = 0; q < RE / 2; ++q) {
+                    const float2 t = unpack2(s[i][q]);
+                    acc.v[i][2 * q] = t.x;
+                    acc.v[i][2 * q + 1] = t.y;
+                }
+        } else {
+#pragma unroll
+            for (int i = 0; i < RT; ++i)
+#pragma unroll
+                for (int q = 0; q < RE; ++q) {
+                    const float2 t = unpack2(s[i][q]);
+                    acc.v[i][q] = t.x + t.y;
+                }
+        }
+    }
+};
+
+// bias, activation, staging and the copy to memory: shared by both forms.  On return the results are staged and a
+// barrier has been passed; the caller copies them out (copy_out) when it has started its next loads.
+template <typename C>
+__device__ __forceinline__ void finish_unit(const Op &op, Acc<C> &acc, unsigned char *stage, int b0, int e0, int tile_no, int tokens)
+{
+    typedef typename C::T T;
+    constexpr int M = C::M, N = M * M;
+    const int w = threadIdx.x >> 5, t0 = tile_no * C::TT, left = tokens - t0;
+    const int b = b0 + w / C::kWpb, ew = e0 + w % C::kWpb * C::EW;
+    if (op.bias != nullptr) {
+        const T *bias = static_cast<const T *>(op.bias);
+        acc.each([&](float &v, int, int e) { v += elem<T>::load(bias + (op.perm ? (ew + e) * M + b : b * M + ew + e)); });
+    }
+    if (C::kAlias) __syncthreads();                    // every warp is done with the tile
+    if (op.act == kGelu) {
+        if (op.in2.p != nullptr) {
+            stage_results<C>(acc, stage, op.perm);
+            __syncthreads();
+            copy_out<C>(stage, op.in2, op.perm, b0, e0, t0, left);
+            __syncthreads();
+        }
+        acc.each([&](float &v, int, int) { v = Math<T>::gelu(v); });
+    } else if (op.act == kGeluGrad) {
+        const T *a = static_cast<const T *>(op.in2.p);
+        acc.each([&](float &v, int t, int e) {
+            if (t < left) v *= Math<T>::grad(elem<T>::load(a + (size_t)(t0 + t) * N + b * M + ew + e));
+        });
+        acc.column_sums([&](float s, int e) { op.sums[(size_t)tile_no * N + b * M + ew + e] = s; });
+    }
+    stage_results<C>(acc, stage, op.perm);
+    __syncthreads();                                   // results staged; nobody reads the tile or the weights any more
 }
 
 // Units i0 .. i1 of a stage, in order: (8 blocks, ES outputs) major, token tile minor.  `held`: whose weights are in
@@ -459,10 +606,9 @@ template <typename C>
 __device__ __forceinline__ void stage_units(const Op &op, int i0, int i1, int tiles, int tokens, unsigned char *smem, int &held)
 {
     typedef typename C::T T;
-    constexpr int M = C::M, N = M * M, kSlices = M / C::ES;
+    constexpr int M = C::M, kSlices = M / C::ES;
     T *wt = reinterpret_cast<T *>(smem + C::kWAt);
     unsigned char *stage = smem + C::kStageAt;
-    const int w = threadIdx.x >> 5;
     TileLoad<C, C::TT, M, C::PA> load;
     int at = i0 / tiles, tile_no = i0 % tiles, buf = 0;
     __syncthreads();                                   // what ran before has left shared memory
@@ -487,29 +633,7 @@ __device__ __forceinline__ void stage_units(const Op &op, int i0, int i1, int ti
         if (early) load.begin(next, op.in, op.perm, at / kSlices * 8, 0, tile_no * C::TT, tokens - tile_no * C::TT);
         Acc<C> acc;
         multiply<C>(acc, tile, wt, op.trans);
-        const int b = b0 + w / C::kWpb, ew = e0 + w % C::kWpb * C::EW;
-        if (op.bias != nullptr) {
-            const T *bias = static_cast<const T *>(op.bias);
-            acc.each([&](float &v, int, int e) { v += elem<T>::load(bias + (op.perm ? (ew + e) * M + b : b * M + ew + e)); });
-        }
-        if (C::kAlias) __syncthreads();                // every warp is done with the tile
-        if (op.act == kGelu) {
-            if (op.in2.p != nullptr) {
-                stage_results<C>(acc, stage, op.perm);
-                __syncthreads();
-                copy_out<C>(stage, op.in2, op.perm, b0, e0, t0, left);
-                __syncthreads();
-            }
-            acc.each([&](float &v, int, int) { v = Math<T>::gelu(v); });
-        } else if (op.act == kGeluGrad) {
-            const T *a = static_cast<const T *>(op.in2.p);
-            acc.each([&](float &v, int t, int e) {
-                if (t < left) v *= Math<T>::grad(elem<T>::load(a + (size_t)(t0 + t) * N + b * M + ew + e));
-            });
-            acc.column_sums([&](float s, int e) { op.sums[(size_t)this_tile * N + b * M + ew + e] = s; });
-        }
-        stage_results<C>(acc, stage, op.perm);
-        __syncthreads();                               // results staged; nobody reads the tile or the weights any more
+        finish_unit<C>(op, acc, stage, b0, e0, this_tile, tokens);
         if (more) {
             if (held != at) {
                 load_weights<C>(wt, op.w, op.trans, at / kSlices * 8, at % kSlices * C::ES);
@@ -523,6 +647,45 @@ __device__ __forceinline__ void stage_units(const Op &op, int i0, int i1, int ti
             if (!early) load.begin(next, op.in, op.perm, at / kSlices * 8, 0, tile_no * C::TT, tokens - tile_no * C::TT);
         }
         if (more) load.end(next, op.perm);
+    }
+}
+
+template <typename C>
+__device__ __forceinline__ void stage_units_chunked(const Op &op, int i0, int i1, int tiles, int tokens, unsigned char *smem)
+{
+    constexpr int M = C::M, kSlices = M / C::ES, KC = C::KC, kChunks = M / KC;
+    unsigned char *stage = smem + C::kStageAt;
+    TileLoad<C, C::TT, KC, C::PC> load;
+    // where unit i, chunk k is loaded to and from
+    auto tile = [&](int n) { return reinterpret_cast<float *>(smem + (n & 1) * C::kChunk); };
+    auto wt = [&](int n) { return reinterpret_cast<float *>(smem + (n & 1) * C::kChunk + C::kChunkA); };
+    auto begin = [&](int n, int i, int k) {
+        const int at = i / tiles, tile_no = i % tiles, b0 = at / kSlices * 8, e0 = at % kSlices * C::ES;
+        load.begin(tile(n), op.in, op.perm, b0, k * KC / 8, tile_no * C::TT, tokens - tile_no * C::TT);
+        Chunks<C>::load_w(wt(n), op.w, op.trans, b0, e0, k * KC);
+    };
+    int n = 0;
+    __syncthreads();                                   // what ran before has left shared memory
+    begin(0, i0, 0);
+    load.end(tile(0), op.perm);
+    for (int i = i0; i < i1; ++i) {
+        Chunks<C> sums;
+        sums.clear();
+#pragma unroll 1
+        for (int k = 0; k < kChunks; ++k, ++n) {
+            cp_async_wait();
+            __syncthreads();                           // chunk n is here, chunk n - 1 has been read
+            const bool more = k + 1 < kChunks || i + 1 < i1;
+            if (more) begin(n + 1, k + 1 < kChunks ? i : i + 1, k + 1 < kChunks ? k + 1 : 0);
+            sums.multiply(tile(n), wt(n), op.trans);
+            if (more) load.end(tile(n + 1), op.perm);
+        }
+        const int at = i / tiles, tile_no = i % tiles, b0 = at / kSlices * 8, e0 = at % kSlices * C::ES;
+        Acc<C> acc;
+        sums.finish(acc, op.trans);
+        finish_unit<C>(op, acc, stage, b0, e0, tile_no, tokens);
+        copy_out<C>(stage, op.out, op.perm, b0, e0, tile_no * C::TT, tokens - tile_no * C::TT);
+        // (staged again only after the next unit's barriers)
     }
 }
 
@@ -550,7 +713,8 @@ __device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0,
         load_b.begin(tile_b(s & kMask), op.in2, op.perm, b0, k0 / 8, s * TW, tokens - s * TW);
         load_b.end(tile_b(s & kMask), op.perm);
     };
-    constexpr int RL = LS / 4, RK = KW / 8;            // fp32: rows and columns of a lane
+    constexpr int RL = LS / 4, RK = KW / 8;            // fp32: rows and columns of a lane, the columns VK neighbours at a time
+    constexpr int VK = RK < 4 ? RK : 4;
     float acc[C::kBf ? LS / 16 : RL][C::kBf ? KW / 8 : RK][C::kBf ? 4 : 1] = {};
 
     __syncthreads();                                   // what ran before has left shared memory
@@ -589,14 +753,17 @@ __device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0,
                 }
             }
         } else {
-            const float *a = tile_a(s & kMask) + bw * TW * C::PL + (lane >> 3) * RL, *b = tile_b(s & kMask) + bw * TW * C::PK + (lane & 7) * RK;
+            const float *a = tile_a(s & kMask) + bw * TW * C::PL + (lane >> 3) * RL, *b = tile_b(s & kMask) + bw * TW * C::PK + kw + (lane & 7) * VK;
 #pragma unroll 4
             for (int t = 0; t < TW; ++t) {
                 float fa[RL], fb[RK];
 #pragma unroll
                 for (int i = 0; i < RL; i += 4) *reinterpret_cast<float4 *>(fa + i) = *reinterpret_cast<const float4 *>(a + t * C::PL + i);
 #pragma unroll
-                for (int i = 0; i < RK; i += 2) *reinterpret_cast<float2 *>(fb + i) = *reinterpret_cast<const float2 *>(b + t * C::PK + i);
+                for (int i = 0; i < RK; i += VK) {
+                    if constexpr (VK == 4) *reinterpret_cast<float4 *>(fb + i) = *reinterpret_cast<const float4 *>(b + t * C::PK + 8 * i);
+                    else                   *reinterpret_cast<float2 *>(fb + i) = *reinterpret_cast<const float2 *>(b + t * C::PK + 8 * i);
+                }
 #pragma unroll
                 for (int i = 0; i < RL; ++i)
 #pragma unroll
@@ -625,9 +792,17 @@ __device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0,
 #pragma unroll
         for (int i = 0; i < RL; ++i)
 #pragma unroll
-            for (int k = 0; k < RK; ++k) {
-                float *d = dst + ((lane >> 3) * RL + i) * M + (lane & 7) * RK + k;
-                *d = add ? *d + acc[i][k][0] : acc[i][k][0];
+            for (int k = 0; k < RK; k += VK) {
+                float *d = dst + ((lane >> 3) * RL + i) * M + (lane & 7) * VK + 8 * k;
+                if constexpr (VK == 4) {
+                    float4 r = make_float4(acc[i][k][0], acc[i][k + 1][0], acc[i][k + 2][0], acc[i][k + 3][0]);
+                    if (add) { const float4 o = *reinterpret_cast<float4 *>(d); r.x += o.x; r.y += o.y; r.z += o.z; r.w += o.w; }
+                    *reinterpret_cast<float4 *>(d) = r;
+                } else {
+                    float2 r = make_float2(acc[i][k][0], acc[i][k + 1][0]);
+                    if (add) { const float2 o = *reinterpret_cast<float2 *>(d); r.x += o.x; r.y += o.y; }
+                    *reinterpret_cast<float2 *>(d) = r;
+                }
             }
     }
 }
@@ -742,7 +917,8 @@ __global__ void __launch_bounds__(C::kThreads, C::kCtas) units_kernel(const __gr
             const Op &op = p.op[o];
             if (op.kind == kStage) {
                 if (held_op != o) held_at = -1;
-                stage_units<C>(op, i0, i1, tiles, p.tokens, smem, held_at);
+                if constexpr (C::KC > 0) stage_units_chunked<C>(op, i0, i1, tiles, p.tokens, smem);
+                else                     stage_units<C>(op, i0, i1, tiles, p.tokens, smem, held_at);
                 held_op = o;
                 return true;
             }
@@ -762,7 +938,7 @@ __global__ void __launch_bounds__(C::kThreads, C::kCtas) units_kernel(const __gr
         });
         if (phase + 1 == p.n_phases) break;
         // the weights of the next phase do not depend on this one: fetched while the barrier is waited for
-        share(phase + 1, [&](int o, int i0, int) {
+        if constexpr (C::KC == 0) share(phase + 1, [&](int o, int i0, int) {
             if (p.op[o].kind == kStage) {
                 const int at = i0 / tiles;
                 if (held_op != o || held_at != at) {

@@ -939,7 +939,7 @@ def test_project_leading_pair(P, m, dtype, kind):
 
 
 @pytest.mark.parametrize("m,T,dtype", [(16, 2500, "bf16"), (16, 1100, "f32"), (32, 1185, "bf16"), (32, 1601, "bf16"),
-                                       (32, 833, "f32"), (32, 15, "bf16"), (32, 16 * 148, "bf16"), (32, 16 * 148 * 6 + 1, "bf16"), (64, 255, "bf16"), (64, 320, "bf16"), (64, 321, "bf16"), (64, 593, "f32"),
+                                       (32, 833, "f32"), (32, 1153, "f32"), (32, 15, "bf16"), (32, 16 * 148, "bf16"), (32, 16 * 148 * 6 + 1, "bf16"), (64, 255, "bf16"), (64, 320, "bf16"), (64, 321, "bf16"), (64, 593, "f32"),
                                        (64, 33, "bf16"), (64, 16 * 18, "bf16"), (64, 16 * 37 + 9, "bf16"), (64, 16 * 19 * 5 + 1, "bf16"),
                                        (128, 17, "bf16"), (128, 75, "f32")])
 def test_one_launch_over_units(P, m, T, dtype):
