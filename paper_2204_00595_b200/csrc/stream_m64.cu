@@ -36,7 +36,7 @@ constexpr int kBwdBlocks = 8, kBwdGroups = kM / kBwdBlocks, kBwdTile = kTok * kB
 // shared memory in tiles: slots of the input ring, then V tiles (du), then staging tiles of the results.  The last four tiles
 // hold the weights first.
 constexpr int kFwdSlots = 4, kFwdStages = 3, kFwdSmem = (kFwdSlots + kFwdStages) * kFwdTile + 1024;
-constexpr int kDuSlots = 9, kDuStages = 3, kDxSlots = 10, kDxStages = 4, kBwdSmem = 14 * kBwdTile + 1024;
+constexpr int kDuSlots = 8, kDuStages = 3, kDxSlots = 10, kDxStages = 4, kBwdSmem = 14 * kBwdTile + 1024;
 constexpr int kMaxRanks = 19;                            // CTAs of a group in the backward launches (148 / 8, rounded up)
 constexpr size_t kGradElems = (size_t)kM * kM * kM;
 
@@ -137,12 +137,37 @@ struct Sync {
     __device__ __forceinline__ void wait_staged(int i) const { wait(s.staged[i % stages], i / stages, kErrMmaWait); }
     __device__ __forceinline__ void across(int i) const { arrive(s.across[i % across_n]); }
     __device__ __forceinline__ void wait_across(int i) const { wait(s.across[i % across_n], i / across_n, kErrMmaWait); }
-    // the feeder, after store(i) is committed: store(i - 1) has left its staging tile
-    __device__ __forceinline__ void stored(int i) const
+    // Tiles are passed on by turns, each by three warps while the others go on: after its own tile k, warp k - 1 sends tile k - 1
+    // away, warp k + 7 has the tiles loaded whose slots that one's inputs leave free, and warp k - 2 frees the staging of tile
+    // k - 2 (all mod 16; by one warp for all tiles this took 400 to 1500 cycles of every tile, and the others waited).
+    template <typename Send, typename Load> __device__ __forceinline__ void pass_on(int k, Send send, Load load) const
     {
-        tma_store_wait_read<1>();
-        if (i > 0) mbar_arrive(smem_u32(&s.free_[(i - 1) % stages]));
+        if (k >= 1 && (turn(k - 1) || turn(k + 7))) {
+            wait_staged(k - 1);
+            if (turn(k - 1)) {
+                send(k - 1);
+                tma_store_commit();
+            } else {
+                load(k - 1);
+            }
+        }
+        if (k >= 2 && turn(k - 2)) {
+            tma_store_wait_read<0>();
+            mbar_arrive(smem_u32(&s.free_[(k - 2) % stages]));
+        }
+        __syncwarp();
     }
+    template <typename Send> __device__ __forceinline__ void pass_last(int count, Send send) const
+    {
+        if (count > 0 && turn(count - 1)) {
+            wait_staged(count - 1);
+            send(count - 1);
+            tma_store_commit();
+        }
+        tma_store_wait_all<0>();
+        __syncwarp();
+    }
+    __device__ __forceinline__ static bool turn(int k) { return threadIdx.x == (k & (kWarps - 1)) * 32; }
     // `blocks` blocks of W from block `first` on, as [row][64 columns] with 128-byte swizzle
     __device__ __forceinline__ void load_weights(uint32_t to, const CUtensorMap *tm_w, int first, int blocks) const
     {
@@ -205,12 +230,8 @@ stage1_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
         for (int i = 0; i < kFwdSlots - 1; ++i) load(i);
     }
-    auto feed = [&](int i) {
-        sync.wait_staged(i);
+    auto send = [&](int i) {
         tma_store_2d(&tm_u, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks * 8, tile(i) * (2 * kM));
-        tma_store_commit();
-        load(i + kFwdSlots);
-        sync.stored(i);
     };
     Weights<4> w;
     sync.take_weights(w, weights + ln.warp * (kM * 128), 0, false);
@@ -236,10 +257,9 @@ stage1_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                      pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3]));
             }
         sync.staged(i);
-        if (feeder && i > 0) feed(i - 1);
+        sync.pass_on(i, send, [&](int k) { load(k + kFwdSlots); });
     }
-    if (feeder && count > 0) feed(count - 1);
-    if (feeder) tma_store_wait_all<0>();
+    sync.pass_last(count, send);
     sync.leave();
 }
 
@@ -267,12 +287,8 @@ stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
         for (int i = 0; i < kFwdSlots - 1; ++i) load(i);
     }
-    auto feed = [&](int i) {
-        sync.wait_staged(i);
+    auto send = [&](int i) {
         tma_store_3d(&tm_y, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks, tile(i) * kTok, 0);
-        tma_store_commit();
-        load(i + kFwdSlots);
-        sync.stored(i);
     };
     Weights<4> w;
     sync.take_weights(w, weights + ln.warp * (kM * 128), 0, false);
@@ -323,10 +339,9 @@ stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 #pragma unroll
         for (int n = 0; n < 4; ++n) stm4(stage + (ln.warp * 4 + n) * (kTok * 32) + t * 32 + ((jg ^ (t >> 2 & 1)) << 4), v[n]);
         sync.staged(i);
-        if (feeder && i > 0) feed(i - 1);
+        sync.pass_on(i, send, [&](int k) { load(k + kFwdSlots); });
     }
-    if (feeder && count > 0) feed(count - 1);
-    if (feeder) tma_store_wait_all<0>();
+    sync.pass_last(count, send);
     sync.leave();
 }
 
@@ -382,35 +397,33 @@ bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, V0 = base + kDuSlots * kBwdTile, stage0 = V0 + 2 * kBwdTile;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, V0 = base + kDuSlots * kBwdTile, stage0 = V0 + 3 * kBwdTile;
     const uint32_t weights = base + 10 * kBwdTile;
     const Ring ring = {base, smem_u32(sh.full), kDuSlots, kBwdTile, p.status, &sh.dead};
-    const Sync sync = {sh, p.status, kDuStages, 2};
+    const Sync sync = {sh, p.status, kDuStages, 3};
     init(sh);
     const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     constexpr int kItems = DW ? 2 : 1;                       // per tile: dy, u
     const Lane ln;
-    int next = 0;
-    auto load_to = [&](int last) {
-        for (; next <= last && next < kItems * count; ++next) {
-            const int t = tile(next / kItems);
-            if (DW && (next & 1)) ring.load_linear(next, p.u + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
-            else                  ring.load(next, &tm_dy, t, 0, group * kBwdBlocks);
+    auto load = [&](int from, int to) {
+        for (int i = from; i <= to && i < kItems * count; ++i) {
+            const int t = tile(i / kItems);
+            if (DW && (i & 1)) ring.load_linear(i, p.u + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
+            else               ring.load(i, &tm_dy, t, 0, group * kBwdBlocks);
         }
     };
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
         sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks);
-        load_to(kDuSlots - 1);
+        load(0, kDuSlots - 1);
     }
-    auto feed = [&](int i) {
-        sync.wait_staged(i);
+    auto send = [&](int i) {
         tma_store_2d(&tm_du, stage0 + i % kDuStages * kBwdTile, group * kBwdBlocks * 8, tile(i) * (2 * kM));
-        tma_store_commit();
-        load_to((DW ? 2 * i + 2 : i + 1) + kDuSlots);                // dy(i + 1) and u(i) have been read
-        sync.stored(i);
+    };
+    auto refill = [&](int i) {                               // dy(i + 1) and u(i) have been read
+        load(i == 0 ? kDuSlots : kItems * i + 1 + kDuSlots, kItems * (i + 1) + kDuSlots);
     };
     const int blk = ln.warp >> 1, half = ln.warp & 1;
     Weights<2> w;
@@ -427,16 +440,16 @@ bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         for (int n = 0; n < 2; ++n) stm4(e_at(V, ln.r, h, ln.warp * 4 + n * 2 + lo), v[n]);
     };
     if (count > 0) {
-        sync.wait(sh.w_read, 0, kErrSlotWait);               // V(1) lies where the weights were
+        sync.wait(sh.w_read, 0, kErrSlotWait);               // V(2) lies where the weights were
         transpose(ring.wait(0), V0);
         sync.across(0);
     }
     for (int i = 0; i < count; ++i) {
-        const uint32_t V = V0 + (i & 1) * kBwdTile, stage = stage0 + i % kDuStages * kBwdTile;
+        const uint32_t V = V0 + i % 3 * kBwdTile, stage = stage0 + i % kDuStages * kBwdTile;
         if (i + 1 < count) {
             const uint32_t y = ring.wait(kItems * (i + 1));
-            if (i > 0) sync.wait_staged(i - 1);              // every warp is done with V(i - 1)
-            transpose(y, V0 + ((i + 1) & 1) * kBwdTile);
+            if (i > 1) sync.wait_staged(i - 2);              // every warp is done with V(i - 2)
+            transpose(y, V0 + (i + 1) % 3 * kBwdTile);
             sync.across(i + 1);
         }
         sync.wait_across(i);
@@ -455,12 +468,11 @@ bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         }
         if (DW) sums.add<false>(V, ring.wait(2 * i + 1), blk, half);
         sync.staged(i);
-        if (feeder && i > 0) feed(i - 1);
+        sync.pass_on(i, send, refill);
     }
-    if (feeder && count > 0) feed(count - 1);
+    sync.pass_last(count, send);
     if (DW && count > 0)
         sums.store(p.parts + (size_t)first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
-    if (feeder) tma_store_wait_all<0>();
     sync.leave();
 }
 
@@ -481,27 +493,20 @@ bwd_dx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     constexpr int kItems = DW ? 2 : 1;                       // per tile: du, x
     const Lane ln;
-    int next = 0;
-    auto load_to = [&](int last) {
-        for (; next <= last && next < kItems * count; ++next) {
-            const int t = tile(next / kItems);
-            if (DW && (next & 1)) ring.load(next, &tm_x, t, group * kBwdBlocks);
-            else                  ring.load_linear(next, p.e_in + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
+    auto load = [&](int from, int to) {
+        for (int i = from; i <= to && i < kItems * count; ++i) {
+            const int t = tile(i / kItems);
+            if (DW && (i & 1)) ring.load(i, &tm_x, t, group * kBwdBlocks);
+            else               ring.load_linear(i, p.e_in + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
         }
     };
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
         if (DX) sync.load_weights(stage0, &tm_w, group * kBwdBlocks, kBwdBlocks);
-        load_to(kDxSlots - 1);
+        load(0, kDxSlots - 1);
     }
-    auto feed = [&](int i) {
-        sync.wait_staged(i);
-        if (DX) {
-            tma_store_3d(&tm_dx, stage0 + i % kDxStages * kBwdTile, 0, tile(i) * kTok, group * kBwdBlocks);
-            tma_store_commit();
-        }
-        load_to(kItems * (i + 1) - 1 + kDxSlots);
-        if (DX) sync.stored(i);
+    auto send = [&](int i) {
+        if (DX) tma_store_3d(&tm_dx, stage0 + i % kDxStages * kBwdTile, 0, tile(i) * kTok, group * kBwdBlocks);
     };
     const int blk = ln.warp >> 1, half = ln.warp & 1;
     Weights<2> w;
@@ -526,12 +531,11 @@ bwd_dx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         }
         if (DW) sums.add<true>(du, ring.wait(2 * i + 1), blk, half);
         sync.staged(i);
-        if (feeder && i > 0) feed(i - 1);
+        sync.pass_on(i, send, [&](int k) { load(kItems * k + kDxSlots, kItems * (k + 1) - 1 + kDxSlots); });
     }
-    if (feeder && count > 0) feed(count - 1);
+    sync.pass_last(count, send);
     if (DW && count > 0)
         sums.store(p.parts + (size_t)first * kGradElems + (size_t)(group * kBwdBlocks + blk) * kM * kM, half);
-    if (feeder) tma_store_wait_all<0>();
     sync.leave();
 }
 
