@@ -547,6 +547,8 @@ int monarch_cplx_fwd(const void *x, const void *L, const void *R, void *y, int a
     const Range out[] = {{y, 2 * plane}};
     const size_t need = monarch_workspace_bytes(MONARCH_OP_CPLX, tokens, n, m, dtype);
     MONARCH_TRY(check_buffers(in, 3, out, 1, workspace, workspace_bytes, need));
+    if (m == 64 && dtype == MONARCH_BF16 && pick(MONARCH_OP_FWD, m, dtype) == kFused && !fused_fwd_m64_on_clusters())
+        return fused_cplx_m64(x, L, R, y, adjoint, tokens, workspace, (cudaStream_t)stream);
     const size_t res = round256(2 * plane);
     const size_t inner = need - 4 * res;
     char *ws = (char *)workspace;
@@ -647,7 +649,7 @@ const char *monarch_impl_name(int op, int32_t m, int dtype)
     if (op < MONARCH_OP_FWD || op > MONARCH_OP_CPLX) return "unsupported";
     if (check_shape(0, m * m, m, dtype) != MONARCH_OK) return "unsupported";
     if (op == MONARCH_OP_MLP_BWD) op = MONARCH_OP_BWD;      // its Monarch passes are monarch_bwd's
-    if (op == MONARCH_OP_CPLX) op = MONARCH_OP_FWD;         // four real forward (or dx) passes
+    if (op == MONARCH_OP_CPLX) op = MONARCH_OP_FWD;         // m = 64, bf16: kernels of its own; else four real forward (or dx) passes
     const int which = pick(op, m, dtype);
     if (which == kSimt && op == MONARCH_OP_FWD && m == 16 &&
         g_impl.load(std::memory_order_relaxed) == MONARCH_IMPL_AUTO)

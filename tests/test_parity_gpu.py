@@ -802,6 +802,13 @@ def test_cplx_fwd(P, impl, m, T, dtype, adjoint):
     _check_guard(yf, "complex y")
 
 
+@pytest.mark.parametrize("adjoint", [0, 1])
+@pytest.mark.parametrize("T", [1, 16, 33, 16 * 19, 16 * 19 * 5 + 1])
+def test_cplx_m64_tiles(P, T, adjoint):
+    """m = 64, bf16: part of a tile, one to six tiles per CTA (the permuted side keeps three in flight), a CTA with one more."""
+    test_cplx_fwd(P, "auto", 64, T, "bf16", adjoint)
+
+
 def test_cplx_dft_closed_form(P):
     """Section 3.2: with the Cooley-Tukey factors the multiply is the DFT of the permuted input; numpy.fft is
     the reference, independent of the oracle's loops."""
