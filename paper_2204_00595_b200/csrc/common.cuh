@@ -182,7 +182,7 @@ int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t 
 // where the forward keeps u inside its workspace (null: nowhere)
 const void *fused_fwd_m64_saved_u(const void *fwd_ws);
 // one pass y = act(M x + bias), act = GELU or identity; workspace of fused_fwd_m64 (u stays behind)
-int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws,
+int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws, void *status,
                        cudaStream_t s);
 size_t fused_mlp_fwd_m64_workspace_bytes(int64_t tokens);
 int fused_mlp_fwd_m64(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2, void *y,
@@ -259,7 +259,7 @@ int project_to_factors(const void *A, void *L, void *R, int m, int dtype, unsign
 
 // ---- elementwise steps of the feed-forward block's backward pass (mlp_bwd.cu) ----
 // h = GELU(a (+ b1)); b1 may be null when a already holds the bias
-int mlp_act(const void *a, const void *b1, void *h, int64_t tokens, int n, int dtype, cudaStream_t s);
+int mlp_act(const void *a, const void *b1, void *h, float *zero1, float *zero2, int64_t tokens, int n, int dtype, cudaStream_t s);
 // dh <- dh * GELU'(a (+ b1)) in place, db1 += column sums of the result, db2 += column sums of dy
 int mlp_dact(void *dh, const void *a, const void *b1, const void *dy, float *db1, float *db2, int64_t tokens, int n,
              int dtype, cudaStream_t s);

@@ -5,7 +5,7 @@
 //   mlp_act:   h = GELU(a)                                   (a recomputed by a forward pass of M1)
 //   mlp_dact:  da = dh * GELU'(a),  db1 += sum_t da,  db2 += sum_t dy
 // Both are pure streaming kernels (16-byte accesses, one pass over their operands).
-#include "common.cuh"
+#include "mma_tiles.cuh"
 
 namespace monarch {
 namespace {
@@ -61,13 +61,17 @@ template <> struct act_math<__nv_bfloat16> {
     static __device__ __forceinline__ float grad(float a) { return gelu_fast_grad(a); }
 };
 
-// h[t][q] = GELU(a[t][q] (+ b1[q])); n is a multiple of the vector width
+// h[t][q] = GELU(a[t][q] (+ b1[q])); n is a multiple of the vector width.  zero1, zero2 (or null): n sums to start from zero
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-mlp_act_kernel(const T *__restrict__ a, const T *__restrict__ b1, T *__restrict__ h, long long vecs, int n)
+mlp_act_kernel(const T *__restrict__ a, const T *__restrict__ b1, T *__restrict__ h, float *__restrict__ zero1, float *__restrict__ zero2,
+               long long vecs, int n)
 {
+    tc::depend_wait();
     constexpr int V = vec16<T>::kElems, U = 4;          // U independent 16-byte loads in flight per thread
     const long long stride = (long long)gridDim.x * kThreads;
+    if (zero1 != nullptr)
+        for (long long i = (long long)blockIdx.x * kThreads + threadIdx.x; i < n; i += stride) zero1[i] = zero2[i] = 0.0f;
     for (long long i0 = (long long)blockIdx.x * kThreads + threadIdx.x; i0 < vecs; i0 += U * stride) {
         float v[U][V];
 #pragma unroll
@@ -101,6 +105,7 @@ mlp_dact_kernel(T *__restrict__ dh, const T *__restrict__ a, const T *__restrict
 {
     constexpr int V = vec16<T>::kElems, kRows = kThreads / 32;
     __shared__ float red[kRows][2][32 * V];
+    tc::depend_wait();
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int col = (blockIdx.x * 32 + lane) * V;      // n is a multiple of 256, and of 32 V
     float bias[V], s1[V], s2[V];
@@ -109,20 +114,33 @@ mlp_dact_kernel(T *__restrict__ dh, const T *__restrict__ a, const T *__restrict
     if (b1 != nullptr) vec16<T>::load(b1 + col, bias);
     const long long t0 = (long long)blockIdx.y * tokens_per_slab;
     const long long t1 = t0 + tokens_per_slab < tokens ? t0 + tokens_per_slab : tokens;
-#pragma unroll 2
-    for (long long t = t0 + row; t < t1; t += kRows) {
-        const long long off = t * n + col;
-        float g[V], av[V], yv[V];
-        vec16<T>::load(dh + off, g);
-        vec16<T>::load(a + off, av);
-        vec16<T>::load(dy + off, yv);
+    // U tokens' loads before the first store: dh is written in place, so the compiler keeps later loads behind a store
+    constexpr int U = 4;
+    for (long long t = t0 + row; t < t1; t += U * kRows) {
+        uint4 g4[U], a4[U], y4[U];
 #pragma unroll
-        for (int e = 0; e < V; ++e) {
-            g[e] *= act_math<T>::grad(av[e] + bias[e]);
-            s1[e] += g[e];
-            s2[e] += yv[e];
+        for (int u = 0; u < U; ++u) {
+            if (t + u * kRows >= t1) break;
+            const long long off = (t + u * kRows) * n + col;
+            g4[u] = *reinterpret_cast<const uint4 *>(dh + off);
+            a4[u] = *reinterpret_cast<const uint4 *>(a + off);
+            y4[u] = *reinterpret_cast<const uint4 *>(dy + off);
         }
-        vec16<T>::store(dh + off, g);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (t + u * kRows >= t1) break;
+            float g[V], av[V], yv[V];
+            vec16<T>::load(reinterpret_cast<const T *>(&g4[u]), g);
+            vec16<T>::load(reinterpret_cast<const T *>(&a4[u]), av);
+            vec16<T>::load(reinterpret_cast<const T *>(&y4[u]), yv);
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                g[e] *= act_math<T>::grad(av[e] + bias[e]);
+                s1[e] += g[e];
+                s2[e] += yv[e];
+            }
+            vec16<T>::store(dh + (t + u * kRows) * n + col, g);
+        }
     }
 #pragma unroll
     for (int e = 0; e < V; ++e) {
@@ -176,16 +194,13 @@ __global__ void merge_status_kernel(unsigned *outer, unsigned *inner)
 }
 
 template <typename T>
-int act_t(const void *a, const void *b1, void *h, int64_t tokens, int n, cudaStream_t s)
+int act_t(const void *a, const void *b1, void *h, float *zero1, float *zero2, int64_t tokens, int n, cudaStream_t s)
 {
     const long long vecs = (long long)tokens * n / vec16<T>::kElems;
     if (vecs == 0) return MONARCH_OK;
     long long blocks = (vecs + kThreads - 1) / kThreads;
     if (blocks > 148 * 16) blocks = 148 * 16;
-    mlp_act_kernel<T><<<(unsigned)blocks, kThreads, 0, s>>>((const T *)a, (const T *)b1, (T *)h, vecs, n);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
-    return MONARCH_OK;
+    return tc::launch_serialized(mlp_act_kernel<T>, (unsigned)blocks, kThreads, 0, s, (const T *)a, (const T *)b1, (T *)h, zero1, zero2, vecs, n);
 }
 
 template <typename T>
@@ -199,18 +214,15 @@ int dact_t(void *dh, const void *a, const void *b1, const void *dy, float *db1, 
     if (slabs > (tokens + 31) / 32) slabs = (tokens + 31) / 32;
     const int per = (int)((tokens + slabs - 1) / slabs);
     slabs = (tokens + per - 1) / per;
-    mlp_dact_kernel<T><<<dim3((unsigned)bx, (unsigned)slabs), kThreads, 0, s>>>((T *)dh, (const T *)a, (const T *)b1,
-                                                                               (const T *)dy, db1, db2, tokens, n, per);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
-    return MONARCH_OK;
+    return tc::launch_serialized(mlp_dact_kernel<T>, dim3((unsigned)bx, (unsigned)slabs), kThreads, 0, s, (T *)dh, (const T *)a, (const T *)b1,
+                                 (const T *)dy, db1, db2, (long long)tokens, n, per);
 }
 
 }  // namespace
 
-int mlp_act(const void *a, const void *b1, void *h, int64_t tokens, int n, int dtype, cudaStream_t s)
+int mlp_act(const void *a, const void *b1, void *h, float *zero1, float *zero2, int64_t tokens, int n, int dtype, cudaStream_t s)
 {
-    return dtype == MONARCH_F32 ? act_t<float>(a, b1, h, tokens, n, s) : act_t<__nv_bfloat16>(a, b1, h, tokens, n, s);
+    return dtype == MONARCH_F32 ? act_t<float>(a, b1, h, zero1, zero2, tokens, n, s) : act_t<__nv_bfloat16>(a, b1, h, zero1, zero2, tokens, n, s);
 }
 
 int mlp_dact(void *dh, const void *a, const void *b1, const void *dy, float *db1, float *db2, int64_t tokens, int n,

@@ -69,10 +69,10 @@ __device__ __forceinline__ void depend_wait() { asm volatile("griddepcontrol.wai
 __device__ __forceinline__ void depend_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... Ts, typename... As>
-int launch_serialized(void (*kern)(Ts...), int grid, int threads, int smem, cudaStream_t s, As... args)
+int launch_serialized(void (*kern)(Ts...), dim3 grid, int threads, int smem, cudaStream_t s, As... args)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = s;

@@ -384,24 +384,25 @@ int monarch_mlp_bwd(const void *x, const void *dy, const void *L1, const void *R
     cudaStream_t s = (cudaStream_t)stream;
     if (use_units(MONARCH_OP_MLP_BWD, m, dtype, tokens))
         return units::mlp_bwd(x, dy, L1, R1, b1, L2, R2, dx, dL1, dR1, db1, dL2, dR2, db2, accumulate, tokens, m, dtype, workspace, s);
-    if (!accumulate) {
+    if (!accumulate && tokens == 0) {
         MONARCH_CUDA_TRY(cudaMemsetAsync(db1, 0, gbias, s));
         MONARCH_CUDA_TRY(cudaMemsetAsync(db2, 0, gbias, s));
     }
     char *ws = (char *)workspace;
     void *ws_b = ws, *ws_f = ws + lay.off_f;
     void *a = ws + lay.off_a, *h = ws + lay.off_h, *dh = ws + lay.off_dh;
-    // the inner forward workspace starts with its own status word and tile counters
-    MONARCH_TRY(monarch_workspace_init(ws_f, lay.ws_f, stream));
     // a = M1 x + b1: the fused m = 64 forward adds the bias in its epilogue, the others leave it to the
     // elementwise kernels (a then holds M1 x)
     const bool bias_in_a = pick(MONARCH_OP_FWD, m, dtype) == kFused && m == 64 && !use_units(MONARCH_OP_FWD, m, dtype, tokens);
     if (bias_in_a)
-        MONARCH_TRY(fused_fwd_bias_m64(x, L1, R1, b1, 0, a, tokens, ws_f, s));
-    else
+        MONARCH_TRY(fused_fwd_bias_m64(x, L1, R1, b1, 0, a, tokens, ws_f, ws_b, s));
+    else {
+        // the inner forward workspace starts with its own status word and tile counters
+        MONARCH_TRY(monarch_workspace_init(ws_f, lay.ws_f, stream));
         MONARCH_TRY(monarch_fwd(x, L1, R1, a, tokens, n, m, dtype, ws_f, lay.ws_f, stream));
+    }
     const void *b1_late = bias_in_a ? nullptr : b1;
-    MONARCH_TRY(mlp_act(a, b1_late, h, tokens, n, dtype, s));
+    MONARCH_TRY(mlp_act(a, b1_late, h, accumulate ? nullptr : db1, accumulate ? nullptr : db2, tokens, n, dtype, s));
     // second matrix: dh = M2^T dy and its block gradients, input h
     MONARCH_TRY(monarch_bwd(h, dy, L2, R2, nullptr, dh, dL2, dR2, accumulate, tokens, n, m, dtype, ws_b,
                             lay.ws_b, stream));
@@ -409,7 +410,7 @@ int monarch_mlp_bwd(const void *x, const void *dy, const void *L1, const void *R
     // first matrix: dx = M1^T da and its block gradients; u = P^T R1 x is still in the forward workspace
     MONARCH_TRY(monarch_bwd(x, dh, L1, R1, ws_f, dx, dL1, dR1, accumulate, tokens, n, m, dtype, ws_b, lay.ws_b,
                             stream));
-    return merge_status((unsigned *)ws_b, (unsigned *)ws_f, s);
+    return bias_in_a ? MONARCH_OK : merge_status((unsigned *)ws_b, (unsigned *)ws_f, s);
 }
 
 size_t monarch_rect_workspace_bytes(int64_t tokens, int32_t q, int32_t b1, int32_t b, int32_t r, int dtype)

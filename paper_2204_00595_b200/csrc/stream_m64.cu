@@ -895,9 +895,11 @@ int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t 
     }
     return stream_fwd(x, L, R, nullptr, 0, y, head(ws), tokens, (unsigned *)ws, s);
 }
-int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws, cudaStream_t s)
+// (the status word is the caller's: `ws` is not initialised)
+int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws, void *status,
+                       cudaStream_t s)
 {
-    return stream_fwd(x, L, R, bias, gelu, y, head(ws), tokens, (unsigned *)ws, s);
+    return stream_fwd(x, L, R, bias, gelu, y, head(ws), tokens, (unsigned *)status, s);
 }
 
 size_t fused_mlp_fwd_m64_workspace_bytes(int64_t tokens) { return kHead + 2 * tc::e_bytes(tokens); }
