@@ -41,27 +41,31 @@ template <typename T> Sizes sizes_t(int m, bool large)
 }
 Sizes sizes(int dtype, int m, bool large) { return dtype == MONARCH_F32 ? sizes_t<float>(m, large) : sizes_t<bf16>(m, large); }
 
-// the large tiles once a stage cut into them has a unit for every SM
+// The large tiles once a stage cut into them has a unit for every SM.  fp32: a unit of the large tiles is long (18 us at
+// m = 64), so what counts is how full its last wave is; measured, a full wave costs 0.8 of the same work in small tiles plus
+// 20 units (m = 64 forward, us, large / small: 500 tokens 37 / 47, 600 tokens 67 / 54, 1000 tokens 74 / 83).
 bool use_large(int dtype, int m, int64_t tokens)
 {
     const Sizes s = sizes(dtype, m, true);
-    return (m / 8) * (m / s.ES) * ceil_div(tokens, s.TT) >= kSms;
+    const long long units = (m / 8) * (m / s.ES) * ceil_div(tokens, s.TT), waves = ceil_div(units, kSms);
+    return dtype == MONARCH_F32 && m > 16 ? 5 * (units + 20) >= 4 * kSms * waves : units >= kSms;
 }
 
 constexpr int kMaxSplits = 16;
 // token ranges of a weight gradient: enough units for every SM, at least four steps in a range
-int wgrad_splits(int dtype, int m, int64_t tokens)
+int wgrad_splits(int dtype, int m, int64_t tokens, bool large)
 {
-    const Sizes s = sizes(dtype, m, use_large(dtype, m, tokens));
+    const Sizes s = sizes(dtype, m, large);
     const long long base = (long long)(m / 8) * (m / s.LS) * (m / s.KS), steps = ceil_div(tokens, s.TW);
     long long n = kSms / base;
     if (n > steps / 4) n = steps / 4;
     if (n > kMaxSplits) n = kMaxSplits;
     return n < 1 ? 1 : (int)n;
 }
+// (for either tiles: a workspace for a batch serves every smaller one)
 size_t parts_bytes(int dtype, int m, int64_t tokens)
 {
-    const int s = wgrad_splits(dtype, m, tokens);
+    const int a = wgrad_splits(dtype, m, tokens, false), b = wgrad_splits(dtype, m, tokens, true), s = a > b ? a : b;
     return s > 1 ? up256((size_t)s * m * m * m * sizeof(float)) : 0;
 }
 size_t act_bytes(int dtype, int m, int64_t tokens) { return up256((size_t)tokens * m * m * esize(dtype)); }
@@ -131,7 +135,7 @@ struct Builder {
     // the sums in `phase`; where the tokens are split, the parts are added in the next one
     void wgrad(int phase, int perm, View rows, View cols, float *sums, int accumulate, void *parts)
     {
-        const int n = wgrad_splits(dtype, m, p.tokens);
+        const int n = wgrad_splits(dtype, m, p.tokens, large);
         Op &o = add(kWgrad, phase, (long long)(m / 8) * (m / sz.LS) * (m / sz.KS) * n,
                     ceil_div(p.tokens, n) * (sz.LS + sz.KS) * 8);
         o.perm = perm;

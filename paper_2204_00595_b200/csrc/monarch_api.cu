@@ -116,7 +116,8 @@ int pick(int op, int m, int dtype)
 //                 the feed-forward block, eight launches otherwise, 45 / 48 at 64, 58 / 49 at 128 (with its forward)
 //   bf16 m = 64   forward 10.7 / 9.2 at 64; forward + backward 23 / 24.5 at 4, 26.7 / 26.3 at 64; block 18.6 / 19.5 at 64,
 //                 22.6 / 19.8 at 128, with its backward 76 / 80 at 96, 113 / 82 at 256
-//   bf16 m = 128  forward 10.7 / 12.1 at 16; block 25 / 25 at 32, with its backward 98 / 101 at 32, 142 / 102 at 64
+//   bf16 m = 128  forward 10.4 / 12.1 at 16, but the backward then has u to recompute: 34.9 / 32.4 together; block 25 / 25 at 32,
+//                 with its backward 98 / 101 at 32, 142 / 102 at 64
 //   fp32          the other family (one launch per stage) is slower at every size
 int64_t units_limit(int op, int m, int dtype)
 {
@@ -125,7 +126,7 @@ int64_t units_limit(int op, int m, int dtype)
     const bool fwd = op == MONARCH_OP_FWD, mlp = op == MONARCH_OP_MLP_FWD, mlp_bwd = op == MONARCH_OP_MLP_BWD;
     if (m == 32) return mlp_bwd ? 72 : 0;
     if (m == 64) return fwd ? 0 : mlp ? 64 : mlp_bwd ? 96 : 32;
-    return fwd ? 16 : mlp ? 24 : mlp_bwd ? 32 : 0;
+    return mlp ? 24 : mlp_bwd ? 32 : 0;
 }
 
 // (the switches that ask for a particular form of the other kernels keep their meaning at every size)
