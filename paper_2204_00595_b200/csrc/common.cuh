@@ -216,11 +216,13 @@ int rect_stage1_tc(const void *x, const void *R, void *u, int64_t tokens, int q,
                    cudaStream_t s);
 int rect_stage1_adjoint_tc(const void *du, const void *R, void *dx, int64_t tokens, int q, int b1, int b,
                            unsigned *status, cudaStream_t s);
-// du = L^T dy and dL += for blocks up to 4 x 4 in one TMA-fed streaming pass (rect_tc.cu): sizes as rect_stage2_stream_available
+// du = L^T dy and dL += for blocks up to 4 x 4 in one TMA-fed streaming pass (rect_tc.cu): sizes as rect_stage2_stream_available;
+// zero[0 .. zero_n) is zeroed beside
 int rect_bwd_stream(const void *dy, const void *u, const void *Lp, void *du, float *dL, int64_t tokens, int q, int b, int r,
-                    unsigned *status, cudaStream_t s);
+                    unsigned *status, float *zero, size_t zero_n, cudaStream_t s);
 bool rect_wgrad_R_tc_available(int q, int b1, int b, int dtype);
-// dR = (accumulate ? dR : 0) + ...
+// dR (+)= ...: _adds says whether the sums are added to what is in dR, so that the caller zeroes it first unless it accumulates
+int rect_wgrad_R_tc_adds(int64_t tokens, int q, int b1, int b, bool *adds);
 int rect_wgrad_R_tc(const void *du, const void *x, float *dR, int accumulate, int64_t tokens, int q, int b1, int b, unsigned *status,
                     cudaStream_t s);
 // stage 2 as a TMA-fed streaming pass (rect_tc.cu): bf16, q and r at most 4, b a multiple of 8 and at least 128

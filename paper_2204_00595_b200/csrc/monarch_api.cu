@@ -508,10 +508,11 @@ int monarch_rect_bwd(const void *x, const void *dy, const void *L, const void *R
     cudaStream_t s = (cudaStream_t)stream;
     const bool fast = g_impl.load(std::memory_order_relaxed) != MONARCH_IMPL_STAGED;
     const bool tc_dR = fast && rect_wgrad_R_tc_available(q, b1, b, dtype);
-    if (!accumulate) {
-        MONARCH_CUDA_TRY(cudaMemsetAsync(dL, 0, lb * sizeof(float), s));
-        if (!tc_dR || tokens == 0) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, rb * sizeof(float), s));
-    }
+    const bool streamed = fast && rect_stage2_stream_available(q, b, r, dtype);
+    bool zero_dR = !accumulate;
+    if (zero_dR && tc_dR && tokens > 0) MONARCH_TRY(rect_wgrad_R_tc_adds(tokens, q, b1, b, &zero_dR));
+    if (!accumulate) MONARCH_CUDA_TRY(cudaMemsetAsync(dL, 0, lb * sizeof(float), s));
+    if (zero_dR && !(streamed && tokens > 0)) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, rb * sizeof(float), s));
     if (tokens == 0) return MONARCH_OK;
     unsigned *status = (unsigned *)workspace;
     char *u_own = (char *)workspace + MONARCH_STATUS_BYTES;
@@ -525,9 +526,8 @@ int monarch_rect_bwd(const void *x, const void *dy, const void *L, const void *R
             MONARCH_TRY(rect_stage1_simt(x, R, u_own, tokens, q, b1, b, dtype, 0, s));
     }
     // du = L^T dy (stage 2 with the roles of q and r exchanged and the blocks read transposed), with dL where both stream
-    const bool streamed = fast && rect_stage2_stream_available(q, b, r, dtype);
     if (streamed)
-        MONARCH_TRY(rect_bwd_stream(dy, u, L, du, dL, tokens, q, b, r, status, s));
+        MONARCH_TRY(rect_bwd_stream(dy, u, L, du, dL, tokens, q, b, r, status, zero_dR ? dR : nullptr, zero_dR ? rb : 0, s));
     else
         MONARCH_TRY(rect_stage2_simt(dy, L, du, tokens, r, b, q, dtype, 1, s));
     // dx = blockdiag(R)^T du: stage 1 with the roles of b1 and b exchanged and the blocks read transposed

@@ -15,7 +15,10 @@
 // The same kernel with BT = true computes the adjoint  dx[t][k*b1 + i] = sum_j R[k][j][i] du[t][k*b + j]:  the
 // contraction then runs over the rows of R_k, so the B operand is MN-major (64 x 64 boxes of R_k, 128-byte swizzle,
 // atoms 8 KB apart along N, 16 rows of K = 2 KB).
-#include "tc_common.cuh"
+//
+// The launches of a call follow one another by programmatic serialization (mma_tiles.cuh): a kernel sets up its barriers and
+// tensor memory while the one before it drains.  It lets the next one in only once it has its own tensor memory.
+#include "mma_tiles.cuh"
 
 namespace monarch {
 namespace tc {
@@ -82,6 +85,8 @@ rect_stage1_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_s;
+    depend_launch();
+    depend_wait();
 
     const int ntiles = p.q * p.ntiles_per_block;
     const long long total = (long long)p.mtiles * ntiles;
@@ -256,6 +261,8 @@ rect_stage1_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_c
     cluster_wait_acquire();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_s;
+    depend_launch();
+    depend_wait();
 
     const int ntiles = p.q * p.ntiles_per_block;
     const int mpairs = (p.mtiles + 1) / 2;                                // token tiles come in pairs, one per CTA
@@ -423,11 +430,8 @@ int launch_pair(const void *in, const void *W, void *out, int64_t tokens, int q,
     p.ntiles_per_block = ndim / 256;
     const long long total = (long long)((p.mtiles + 1) / 2) * q * p.ntiles_per_block;
     const int pairs = (int)(total < max_pairs ? total : max_pairs);
-    rect_stage1_pair_kernel<BT><<<2 * pairs, kThreads, kPairSmem, s>>>(tm_x, tm_R, tm_u, p);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
     *used = true;
-    return MONARCH_OK;
+    return launch_serialized(rect_stage1_pair_kernel<BT>, 2 * pairs, kThreads, kPairSmem, s, tm_x, tm_R, tm_u, p);
 }
 
 // in: [tokens][q * kdim], W: [q][b][b1] (kdim = b1, ndim = b) or, with BT, contracted over its rows (kdim = b, ndim = b1)
@@ -447,11 +451,6 @@ int launch(const void *in, const void *W, void *out, int64_t tokens, int q, int 
     // cache would not be safe against two host threads
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
-    static bool attr = false;
-    if (!attr) {
-        MONARCH_CUDA_TRY(cudaFuncSetAttribute(rect_stage1_kernel<NT, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes));
-        attr = true;
-    }
     RectParams p;
     p.status = status;
     p.q = q; p.kdim = kdim; p.ndim = ndim;
@@ -459,10 +458,7 @@ int launch(const void *in, const void *W, void *out, int64_t tokens, int q, int 
     p.ntiles_per_block = ndim / NT;
     const long long total = (long long)p.mtiles * q * p.ntiles_per_block;
     const int grid = (int)(total < sms ? total : sms);
-    rect_stage1_kernel<NT, BT><<<grid, kThreads, S::kBytes, s>>>(tm_x, tm_R, tm_u, p);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
-    return MONARCH_OK;
+    return launch_serialized(rect_stage1_kernel<NT, BT>, grid, kThreads, S::kBytes, s, tm_x, tm_R, tm_u, p);
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -513,6 +509,8 @@ rect_stage2_stream_kernel(const __grid_constant__ CUtensorMap tm_u, const __nv_b
         dead_s = 0;
         tma_prefetch_desc(&tm_u);
     }
+    depend_launch();
+    depend_wait();
     for (int i = threadIdx.x; i < 16 * kS2Cols; i += kS2Threads) {
         const int jl = i >> 4, l = (i >> 2) & 3, k = i & 3;
         float v = 0.0f;
@@ -594,7 +592,8 @@ rect_stage2_stream_kernel(const __grid_constant__ CUtensorMap tm_u, const __nv_b
 __global__ void __launch_bounds__(kS2Threads, 1)
 rect_bwd_stream_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_constant__ CUtensorMap tm_u,
                        const __nv_bfloat16 *__restrict__ Lp, __nv_bfloat16 *__restrict__ du, float *__restrict__ dL,
-                       unsigned *status, long long tokens, int q, int b, int r, int tokens_per_slab)
+                       unsigned *status, long long tokens, int q, int b, int r, int tokens_per_slab, float4 *__restrict__ zero,
+                       long long zero_n)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ float4 ws[4][4][2][32];            // [l][k][half][lane]: columns 8 lane + 4 half + (0..3)
@@ -608,6 +607,8 @@ rect_bwd_stream_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_c
         fence_mbar_init();
         dead_s = 0;
     }
+    depend_launch();
+    depend_wait();
     __syncthreads();
     const long long t0 = (long long)blockIdx.y * tokens_per_slab;
     const long long t1 = t0 + tokens_per_slab < tokens ? t0 + tokens_per_slab : tokens;
@@ -630,6 +631,10 @@ rect_bwd_stream_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_c
         const float v = j0 + jl < b && l < r && k < q ? __bfloat162float(Lp[(size_t)(j0 + jl) * r * q + l * q + k]) : 0.0f;
         reinterpret_cast<float *>(&ws[l][k][(jl >> 2) & 1][jl >> 3])[jl & 3] = v;
     }
+    // the sums of a later launch start from zero (a memset of its own costs more than this at small sizes)
+    for (long long i = ((long long)blockIdx.y * gridDim.x + blockIdx.x) * kS2Threads + threadIdx.x; i < zero_n;
+         i += (long long)gridDim.x * gridDim.y * kS2Threads)
+        zero[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     __syncthreads();
 
     const int lane = threadIdx.x & 31, tr = threadIdx.x >> 5;
@@ -763,6 +768,8 @@ rect_wgrad_kernel(const __grid_constant__ CUtensorMap tm_du, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_s;
+    depend_launch();
+    depend_wait();
     const uint32_t full0 = smem_u32(bar_full), empty0 = smem_u32(bar_empty), acc = smem_u32(&bar_acc);
 
     if (first < p.chunks) {
@@ -870,6 +877,8 @@ rect_wgrad_pair_kernel(const __grid_constant__ CUtensorMap tm_du, const __grid_c
     cluster_wait_acquire();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_s;
+    depend_launch();
+    depend_wait();
     const uint32_t full0 = smem_u32(bars.full), empty0 = smem_u32(bars.empty), acc = smem_u32(&bars.acc_full[0]);
 
     if (warp == 4) {
@@ -933,7 +942,7 @@ rect_wgrad_pair_kernel(const __grid_constant__ CUtensorMap tm_du, const __grid_c
 
 // dR = (accumulate ? dR : 0) + ...; b and b1 multiples of 256; *used = false where no pair can be resident
 int launch_wgrad_pair(const void *du, const void *x, float *dR, int accumulate, int64_t tokens, int q, int b1, int b, unsigned *status,
-                      cudaStream_t s, bool *used)
+                      cudaStream_t s, bool *used, bool dry = false)
 {
     static PerDeviceCache cache;
     constexpr int smem = kPairStages * kPairStageBytes + 1024;
@@ -941,9 +950,6 @@ int launch_wgrad_pair(const void *du, const void *x, float *dR, int accumulate, 
     *used = false;
     MONARCH_TRY(max_pairs_of(rect_wgrad_pair_kernel, cache, smem, &pairs));
     if (pairs < 1) return MONARCH_OK;
-    CUtensorMap tm_du, tm_x;
-    MONARCH_TRY(encode_tmap_2d(&tm_du, du, (uint64_t)tokens, (uint64_t)q * b, (uint64_t)q * b * 2, 64, 64, 128));
-    MONARCH_TRY(encode_tmap_2d(&tm_x, x, (uint64_t)tokens, (uint64_t)q * b1, (uint64_t)q * b1 * 2, 64, 64, 128));
     WgParams p;
     p.out = dR;
     p.status = status;
@@ -957,12 +963,16 @@ int launch_wgrad_pair(const void *du, const void *x, float *dR, int accumulate, 
     if (slices > p.chunks) slices = p.chunks;
     if (tiles > 0x3fffffffLL || slices > 65535) return MONARCH_ERR_UNSUPPORTED;
     p.slices = (int)slices;
-    if (slices > 1 && !accumulate) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, (size_t)q * b * b1 * sizeof(float), s));
-    rect_wgrad_pair_kernel<<<dim3((unsigned)(2 * tiles), (unsigned)slices), kThreads, smem, s>>>(tm_du, tm_x, p, slices > 1 || accumulate);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
+    if (dry) {
+        *used = slices == 1;
+        return MONARCH_OK;
+    }
+    CUtensorMap tm_du, tm_x;
+    MONARCH_TRY(encode_tmap_2d(&tm_du, du, (uint64_t)tokens, (uint64_t)q * b, (uint64_t)q * b * 2, 64, 64, 128));
+    MONARCH_TRY(encode_tmap_2d(&tm_x, x, (uint64_t)tokens, (uint64_t)q * b1, (uint64_t)q * b1 * 2, 64, 64, 128));
     *used = true;
-    return MONARCH_OK;
+    return launch_serialized(rect_wgrad_pair_kernel, dim3((unsigned)(2 * tiles), (unsigned)slices), kThreads, smem, s, tm_du, tm_x, p,
+                             (int)(slices > 1 || accumulate));
 }
 
 template <int NT>
@@ -977,7 +987,6 @@ int launch_wgrad(const void *du, const void *x, float *dR, int64_t tokens, int q
     // cache would not be safe against two host threads
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
-    MONARCH_CUDA_TRY(cudaFuncSetAttribute(rect_wgrad_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     WgParams p;
     p.out = dR;
     p.status = status;
@@ -991,10 +1000,7 @@ int launch_wgrad(const void *du, const void *x, float *dR, int64_t tokens, int q
     if (slices > p.chunks) slices = p.chunks;
     if (tiles > 0x7fffffffLL || slices > 65535) return MONARCH_ERR_UNSUPPORTED;
     p.slices = (int)slices;
-    rect_wgrad_kernel<NT><<<dim3((unsigned)tiles, (unsigned)slices), kThreads, smem, s>>>(tm_du, tm_x, p);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
-    return MONARCH_OK;
+    return launch_serialized(rect_wgrad_kernel<NT>, dim3((unsigned)tiles, (unsigned)slices), kThreads, smem, s, tm_du, tm_x, p);
 }
 
 }  // namespace
@@ -1022,8 +1028,6 @@ int rect_stage2_stream(const void *u, const void *Lp, void *y, int64_t tokens, i
     // cache would not be safe against two host threads
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
-    MONARCH_CUDA_TRY(cudaFuncSetAttribute(rect_stage2_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          kS2SmemBytes));
     const int cx = (b + kS2Cols - 1) / kS2Cols;
     long long slabs = (2LL * sms + cx - 1) / cx;                     // two CTAs per SM, one wave
     if (slabs > (tokens + kS2Tok - 1) / kS2Tok) slabs = (tokens + kS2Tok - 1) / kS2Tok;
@@ -1031,11 +1035,8 @@ int rect_stage2_stream(const void *u, const void *Lp, void *y, int64_t tokens, i
     per = (per + kS2Tok - 1) / kS2Tok * kS2Tok;
     slabs = (tokens + per - 1) / per;
     if (slabs > 65535) return MONARCH_ERR_UNSUPPORTED;
-    rect_stage2_stream_kernel<<<dim3((unsigned)cx, (unsigned)slabs), kS2Threads, kS2SmemBytes, s>>>(
-        tm_u, (const __nv_bfloat16 *)Lp, (__nv_bfloat16 *)y, status, tokens, q, b, r, (int)per);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
-    return MONARCH_OK;
+    return launch_serialized(rect_stage2_stream_kernel, dim3((unsigned)cx, (unsigned)slabs), kS2Threads, kS2SmemBytes, s, tm_u,
+                             (const __nv_bfloat16 *)Lp, (__nv_bfloat16 *)y, status, (long long)tokens, q, b, r, (int)per);
 }
 
 int rect_stage1_tc(const void *x, const void *R, void *u, int64_t tokens, int q, int b1, int b, unsigned *status,
@@ -1053,9 +1054,9 @@ int rect_stage1_tc(const void *x, const void *R, void *u, int64_t tokens, int q,
                         : tc::launch<64, false>(x, R, u, tokens, q, b1, b, status, s);
 }
 
-// du and dL in one TMA-fed streaming pass: same sizes as the streaming stage 2
+// du and dL in one TMA-fed streaming pass: same sizes as the streaming stage 2; zeroes zero[0 .. zero_n) beside
 int rect_bwd_stream(const void *dy, const void *u, const void *Lp, void *du, float *dL, int64_t tokens, int q, int b, int r,
-                    unsigned *status, cudaStream_t s)
+                    unsigned *status, float *zero, size_t zero_n, cudaStream_t s)
 {
     using namespace tc;
     if (tokens == 0) return MONARCH_OK;
@@ -1067,7 +1068,6 @@ int rect_bwd_stream(const void *dy, const void *u, const void *Lp, void *du, flo
     // cache would not be safe against two host threads
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
-    MONARCH_CUDA_TRY(cudaFuncSetAttribute(rect_bwd_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int cx = (b + kS2Cols - 1) / kS2Cols;
     long long slabs = (sms + cx - 1) / cx;                            // one CTA per SM, one wave
     if (slabs > (tokens + kS2Tok - 1) / kS2Tok) slabs = (tokens + kS2Tok - 1) / kS2Tok;
@@ -1075,11 +1075,9 @@ int rect_bwd_stream(const void *dy, const void *u, const void *Lp, void *du, flo
     per = (per + kS2Tok - 1) / kS2Tok * kS2Tok;
     slabs = (tokens + per - 1) / per;
     if (slabs > 65535) return MONARCH_ERR_UNSUPPORTED;
-    rect_bwd_stream_kernel<<<dim3((unsigned)cx, (unsigned)slabs), kS2Threads, smem, s>>>(
-        tm_dy, tm_u, (const __nv_bfloat16 *)Lp, (__nv_bfloat16 *)du, dL, status, tokens, q, b, r, (int)per);
-    note_launch();
-    MONARCH_CUDA_TRY(cudaGetLastError());
-    return MONARCH_OK;
+    return launch_serialized(rect_bwd_stream_kernel, dim3((unsigned)cx, (unsigned)slabs), kS2Threads, smem, s, tm_dy, tm_u,
+                             (const __nv_bfloat16 *)Lp, (__nv_bfloat16 *)du, dL, status, (long long)tokens, q, b, r, (int)per, (float4 *)zero,
+                             (long long)(zero_n / 4));
 }
 
 // dR on the tensor cores: bf16, b and b1 multiples of 64 (the rows of a last half tile of 128 are not stored)
@@ -1087,6 +1085,16 @@ bool rect_wgrad_R_tc_available(int q, int b1, int b, int dtype)
 {
     (void)q;
     return dtype == MONARCH_BF16 && b % 64 == 0 && b1 % 64 == 0;
+}
+
+// Whether its sums start from what is in dR: the caller zeroes it (unless they are to be added)
+int rect_wgrad_R_tc_adds(int64_t tokens, int q, int b1, int b, bool *adds)
+{
+    bool stores = false;
+    if (tokens > 0 && b % 256 == 0 && b1 % 256 == 0)
+        MONARCH_TRY(tc::launch_wgrad_pair(nullptr, nullptr, nullptr, 0, tokens, q, b1, b, nullptr, nullptr, &stores, true));
+    *adds = !stores;
+    return MONARCH_OK;
 }
 
 int rect_wgrad_R_tc(const void *du, const void *x, float *dR, int accumulate, int64_t tokens, int q, int b1, int b, unsigned *status,
@@ -1097,7 +1105,6 @@ int rect_wgrad_R_tc(const void *du, const void *x, float *dR, int accumulate, in
         MONARCH_TRY(tc::launch_wgrad_pair(du, x, dR, accumulate, tokens, q, b1, b, status, s, &used));
         if (used) return MONARCH_OK;
     }
-    if (!accumulate) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, (size_t)q * b * b1 * sizeof(float), s));
     if (tokens == 0) return MONARCH_OK;
     if (b1 % 256 == 0) return tc::launch_wgrad<256>(du, x, dR, tokens, q, b1, b, status, s);
     return b1 % 128 == 0 ? tc::launch_wgrad<128>(du, x, dR, tokens, q, b1, b, status, s)

@@ -206,10 +206,10 @@ int rectw_bwd(const void *x, const void *dy, const void *Lw, const void *R, void
     const size_t es = dtype == MONARCH_F32 ? 4 : 2, bmax = b2 > b3 ? b2 : b3;
     const size_t lw = (size_t)r * q * bmax, rb = (size_t)q * b2 * b1;
     const bool tc_dR = fast && rect_wgrad_R_tc_available(q, b1, b2, dtype);
-    if (!accumulate) {
-        MONARCH_CUDA_TRY(cudaMemsetAsync(dLw, 0, lw * sizeof(float), s));
-        if (!tc_dR || tokens == 0) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, rb * sizeof(float), s));
-    }
+    bool zero_dR = !accumulate;
+    if (zero_dR && tc_dR && tokens > 0) MONARCH_TRY(rect_wgrad_R_tc_adds(tokens, q, b1, b2, &zero_dR));
+    if (!accumulate) MONARCH_CUDA_TRY(cudaMemsetAsync(dLw, 0, lw * sizeof(float), s));
+    if (zero_dR) MONARCH_CUDA_TRY(cudaMemsetAsync(dR, 0, rb * sizeof(float), s));
     if (tokens == 0) return MONARCH_OK;
     unsigned *status = (unsigned *)ws;
     char *u = (char *)ws + MONARCH_STATUS_BYTES;
@@ -229,7 +229,7 @@ int rectw_bwd(const void *x, const void *dy, const void *Lw, const void *R, void
         // dLp of the re-labelled problem goes into zeroed scratch.  du = L^T dy: stage 2 with the roles of q and r exchanged
         // and the blocks read transposed.
         MONARCH_CUDA_TRY(cudaMemsetAsync(dLp, 0, lw * sizeof(float), s));
-        if (stream) MONARCH_TRY(rect_bwd_stream(dy, u, Lp, du, dLp, tokens, m.q2, m.bb, m.r2, status, s));
+        if (stream) MONARCH_TRY(rect_bwd_stream(dy, u, Lp, du, dLp, tokens, m.q2, m.bb, m.r2, status, nullptr, 0, s));
         else MONARCH_TRY(rect_stage2_simt(dy, Lp, du, tokens, m.r2, m.bb, m.q2, dtype, 1, s));
     } else {
         const int g = grid_for(tokens * q * b2);
