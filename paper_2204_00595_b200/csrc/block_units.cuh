@@ -88,7 +88,7 @@ template <typename T_, int M_, int TT_, int ES_, int LS_, int KS_, int KC_ = 0> 
     static constexpr int kStepBytes = G * TW * (PL + PK) * (int)sizeof(T);
     // Two CTAs per SM work on different units while each waits for its own loads.  Within that share of shared memory: two
     // tiles (the next unit's input is on its way during this one's work), or one, or one that the results are staged over.
-    static constexpr int kChunkA = G * TT * PC * 4, kChunkW = cmax(G * ES * PC, G * KC * (ES + 4)) * 4, kChunk = kChunkA + kChunkW;
+    static constexpr int kBlockA = TT * PC + 4, kChunkA = G * kBlockA * 4, kChunkW = cmax(G * ES * PC, G * KC * (ES + 4)) * 4, kChunk = kChunkA + kChunkW;
     static constexpr int kHalf = KC ? 226 * 1024 : 113 * 1024 - 512;
     static constexpr int kBufs = 2 * kTileBytes + kWBytes + kStageBytes <= kHalf ? 2 : 1;
     static constexpr bool kAlias = KC == 0 && kTileBytes + kWBytes + kStageBytes > kHalf;
@@ -339,7 +339,7 @@ template <typename C> __device__ __forceinline__ void stage_results(Acc<C> &acc,
 }
 
 template <typename C>
-__device__ __forceinline__ void copy_out(const unsigned char *stage, const View &out, int perm, int b0, int e0, int t0, int left)
+__device__ __forceinline__ void copy_out(const unsigned char *stage, const View &out, int perm, int b0, int e0, int t0, int left, int part = 0, int parts = 1)
 {
     typedef typename C::T T;
     constexpr int H = (int)sizeof(T) / 2;
@@ -348,7 +348,7 @@ __device__ __forceinline__ void copy_out(const unsigned char *stage, const View 
     if (!perm) {
         const unsigned first = t0 * out.t_stride + b0 * out.b_stride + e0 / 8 * out.c_stride;
 #pragma unroll 4
-        for (int j = threadIdx.x; j < kVecs; j += C::kThreads) {
+        for (int j = part * kVecs / parts + threadIdx.x; j < (part + 1) * kVecs / parts; j += C::kThreads) {
             const int h = j % H, i = j / H;
             int b, c;
             if (out.mid) { b = i % 8; c = i / 8 % (C::ES / 8); }
@@ -362,7 +362,7 @@ __device__ __forceinline__ void copy_out(const unsigned char *stage, const View 
     }
     const unsigned first = t0 * out.t_stride + b0 / 8 * out.b_stride + e0 * out.c_stride;
 #pragma unroll 4
-    for (int j = threadIdx.x; j < kVecs; j += C::kThreads) {
+    for (int j = part * kVecs / parts + threadIdx.x; j < (part + 1) * kVecs / parts; j += C::kThreads) {
         const int h = j % H, e = j / H % C::ES, t = j / (H * C::ES);
         if (t >= left) break;
         constexpr int kPlane = C::TT * C::PS;
@@ -476,6 +476,34 @@ template <typename C> struct Chunks {
 #pragma unroll
             for (int q = 0; q < RE; ++q) s[i][q] = 0;
     }
+    // columns c0 .. c0 + KC of the input: permuted pieces (8 blocks, 32 bytes) go to the blocks' rows 4 bytes at a time
+    static __device__ __forceinline__ void load_a(float *tile, const View &v, int perm, int b0, int c0, int t0, int left)
+    {
+        if (!perm) {
+            const float4 *src = static_cast<const float4 *>(v.p);
+            const unsigned first = t0 * v.t_stride + b0 * v.b_stride + c0 / 8 * v.c_stride;
+#pragma unroll 4
+            for (int j = threadIdx.x; j < TT * KC * 2; j += C::kThreads) {
+                const int h = j % 2, i = j / 2, t = i / KC;
+                int b, c;
+                if (v.mid) { b = i % 8; c = i / 8 % (KC / 8); }
+                else       { c = i % (KC / 8); b = i / (KC / 8) % 8; }
+                const bool ok = t < left;
+                cp_async16(tile + b * C::kBlockA + t * PC + c * 8 + h * 4,
+                           src + (size_t)(first + (ok ? t : 0) * v.t_stride + b * v.b_stride + c * v.c_stride) * 2 + h, ok);
+            }
+            return;
+        }
+        const float *src = static_cast<const float *>(v.p);
+        const unsigned first = t0 * v.t_stride + b0 / 8 * v.b_stride + c0 * v.c_stride;
+#pragma unroll 4
+        for (int j = threadIdx.x; j < TT * KC * 8; j += C::kThreads) {
+            const int b = j % 8, c = j / 8 % KC, t = j / (8 * KC);
+            const bool ok = t < left;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_addr(tile + b * C::kBlockA + t * PC + c)),
+                         "l"(src + (size_t)(first + (ok ? t : 0) * v.t_stride + c * v.c_stride) * 8 + b), "r"(ok ? 4 : 0) : "memory");
+        }
+    }
     static __device__ __forceinline__ void load_w(float *wt, const void *w, int trans, int b0, int e0, int c0)
     {
         const float *src = static_cast<const float *>(w) + (size_t)b0 * M * M;
@@ -495,7 +523,7 @@ template <typename C> struct Chunks {
     {
         const int w = (threadIdx.x >> 5) / C::kWpb, e0 = (threadIdx.x >> 5) % C::kWpb * EW;
         const int tl = (threadIdx.x & 31) >> 3, el = threadIdx.x & 7;
-        const float *a = tile + (w * TT + tl) * PC;
+        const float *a = tile + w * C::kBlockA + tl * PC;
         if (!trans) {
             const float *b = wt + (w * ES + e0 + el) * PC;
 #pragma unroll
@@ -655,19 +683,21 @@ __device__ __forceinline__ void stage_units_chunked(const Op &op, int i0, int i1
 {
     constexpr int M = C::M, kSlices = M / C::ES, KC = C::KC, kChunks = M / KC;
     unsigned char *stage = smem + C::kStageAt;
-    TileLoad<C, C::TT, KC, C::PC> load;
     // where unit i, chunk k is loaded to and from
     auto tile = [&](int n) { return reinterpret_cast<float *>(smem + (n & 1) * C::kChunk); };
     auto wt = [&](int n) { return reinterpret_cast<float *>(smem + (n & 1) * C::kChunk + C::kChunkA); };
     auto begin = [&](int n, int i, int k) {
         const int at = i / tiles, tile_no = i % tiles, b0 = at / kSlices * 8, e0 = at % kSlices * C::ES;
-        load.begin(tile(n), op.in, op.perm, b0, k * KC / 8, tile_no * C::TT, tokens - tile_no * C::TT);
+        Chunks<C>::load_a(tile(n), op.in, op.perm, b0, k * KC, tile_no * C::TT, tokens - tile_no * C::TT);
         Chunks<C>::load_w(wt(n), op.w, op.trans, b0, e0, k * KC);
+    };
+    auto copy = [&](int i, int part, int parts) {
+        const int at = i / tiles, tile_no = i % tiles;
+        copy_out<C>(stage, op.out, op.perm, at / kSlices * 8, at % kSlices * C::ES, tile_no * C::TT, tokens - tile_no * C::TT, part, parts);
     };
     int n = 0;
     __syncthreads();                                   // what ran before has left shared memory
     begin(0, i0, 0);
-    load.end(tile(0), op.perm);
     for (int i = i0; i < i1; ++i) {
         Chunks<C> sums;
         sums.clear();
@@ -677,16 +707,17 @@ __device__ __forceinline__ void stage_units_chunked(const Op &op, int i0, int i1
             __syncthreads();                           // chunk n is here, chunk n - 1 has been read
             const bool more = k + 1 < kChunks || i + 1 < i1;
             if (more) begin(n + 1, k + 1 < kChunks ? i : i + 1, k + 1 < kChunks ? k + 1 : 0);
+            // the previous unit's results leave during this one's products, but for the last chunk: behind its barrier they
+            // may be staged over
+            if (i > i0 && k < kChunks - 1) copy(i - 1, k, kChunks - 1);
             sums.multiply(tile(n), wt(n), op.trans);
-            if (more) load.end(tile(n + 1), op.perm);
         }
         const int at = i / tiles, tile_no = i % tiles, b0 = at / kSlices * 8, e0 = at % kSlices * C::ES;
         Acc<C> acc;
         sums.finish(acc, op.trans);
         finish_unit<C>(op, acc, stage, b0, e0, tile_no, tokens);
-        copy_out<C>(stage, op.out, op.perm, b0, e0, tile_no * C::TT, tokens - tile_no * C::TT);
-        // (staged again only after the next unit's barriers)
     }
+    copy(i1 - 1, 0, 1);
 }
 
 // ---------------------------------------------------------------- a weight-gradient unit
