@@ -85,7 +85,9 @@ template <typename T_, int M_, int TT_, int ES_, int LS_, int KS_, int KC_ = 0> 
     static constexpr int kStageBytes = cmax(kPlanes * TT * PS * 4, TT * kNatT);
     static constexpr int kTileBytes = G * TT * PA * (int)sizeof(T);
     static constexpr int kWBytes = cmax(G * ES * PA, kBf ? G * M * PE : 0) * (int)sizeof(T);
-    static constexpr int kStepBytes = G * TW * (PL + PK) * (int)sizeof(T);
+    static constexpr int kPadB = KC ? 4 : 0;                  // between the blocks of a step: 4-byte copies of 8 blocks without conflicts
+    static constexpr int kBlockL = TW * PL + kPadB, kBlockK = TW * PK + kPadB;
+    static constexpr int kStepBytes = G * (kBlockL + kBlockK) * (int)sizeof(T);
     // Two CTAs per SM work on different units while each waits for its own loads.  Within that share of shared memory: two
     // tiles (the next unit's input is on its way during this one's work), or one, or one that the results are staged over.
     static constexpr int kBlockA = TT * PC + 4, kChunkA = G * kBlockA * 4, kChunkW = cmax(G * ES * PC, G * KC * (ES + 4)) * 4, kChunk = kChunkA + kChunkW;
@@ -339,7 +341,7 @@ template <typename C> __device__ __forceinline__ void stage_results(Acc<C> &acc,
 }
 
 template <typename C>
-__device__ __forceinline__ void copy_out(const unsigned char *stage, const View &out, int perm, int b0, int e0, int t0, int left, int part = 0, int parts = 1)
+__device__ __forceinline__ void copy_out(const unsigned char *stage, const View &out, int perm, int b0, int e0, int t0, int left)
 {
     typedef typename C::T T;
     constexpr int H = (int)sizeof(T) / 2;
@@ -348,7 +350,7 @@ __device__ __forceinline__ void copy_out(const unsigned char *stage, const View 
     if (!perm) {
         const unsigned first = t0 * out.t_stride + b0 * out.b_stride + e0 / 8 * out.c_stride;
 #pragma unroll 4
-        for (int j = part * kVecs / parts + threadIdx.x; j < (part + 1) * kVecs / parts; j += C::kThreads) {
+        for (int j = threadIdx.x; j < kVecs; j += C::kThreads) {
             const int h = j % H, i = j / H;
             int b, c;
             if (out.mid) { b = i % 8; c = i / 8 % (C::ES / 8); }
@@ -362,7 +364,7 @@ __device__ __forceinline__ void copy_out(const unsigned char *stage, const View 
     }
     const unsigned first = t0 * out.t_stride + b0 / 8 * out.b_stride + e0 * out.c_stride;
 #pragma unroll 4
-    for (int j = part * kVecs / parts + threadIdx.x; j < (part + 1) * kVecs / parts; j += C::kThreads) {
+    for (int j = threadIdx.x; j < kVecs; j += C::kThreads) {
         const int h = j % H, e = j / H % C::ES, t = j / (H * C::ES);
         if (t >= left) break;
         constexpr int kPlane = C::TT * C::PS;
@@ -459,6 +461,40 @@ __device__ __forceinline__ void multiply(Acc<C> &acc, const typename C::T *tile,
     }
 }
 
+// NC columns from c0 on of R tokens and 8 blocks to tile[block][token][column] (fp32, asynchronous; rows PITCH, blocks BLOCK
+// floats apart): permuted pieces (8 blocks, 32 bytes) go to the blocks' rows 4 bytes at a time.  A thread's pieces differ in
+// the token only: one address and an add per piece.
+template <typename C, int R, int NC, int PITCH, int BLOCK>
+__device__ __forceinline__ void load_async(float *tile, const View &v, int perm, int b0, int c0, int t0, int left)
+{
+    const unsigned j = threadIdx.x;
+    if (!perm) {
+        constexpr int kStep = C::kThreads / (2 * NC);
+        const unsigned h = j % 2, i = j / 2, t = i / NC;
+        const unsigned b = v.mid ? i % 8 : i / (NC / 8) % 8, c = v.mid ? i / 8 % (NC / 8) : i % (NC / 8);
+        const float4 *src = static_cast<const float4 *>(v.p) +
+                            (size_t)((t0 + t) * v.t_stride + (b0 + b) * v.b_stride + (c0 / 8 + c) * v.c_stride) * 2 + h;
+        float *dst = tile + b * BLOCK + t * PITCH + c * 8 + h * 4;
+#pragma unroll
+        for (int n = 0; n < R / kStep; ++n) {
+            const bool ok = (int)t + n * kStep < left;
+            cp_async16(dst + n * kStep * PITCH, ok ? src + (size_t)n * kStep * v.t_stride * 2 : static_cast<const float4 *>(v.p), ok);
+        }
+        return;
+    }
+    constexpr int kStep = C::kThreads / (8 * NC);
+    static_assert(kStep >= 1 && R % kStep == 0, "");
+    const unsigned b = j % 8, c = j / 8 % NC, t = j / (8 * NC);
+    const float *src = static_cast<const float *>(v.p) + (size_t)((t0 + t) * v.t_stride + b0 / 8 * v.b_stride + (c0 + c) * v.c_stride) * 8 + b;
+    const uint32_t dst = smem_addr(tile + b * BLOCK + t * PITCH + c);
+#pragma unroll
+    for (int n = 0; n < R / kStep; ++n) {
+        const bool ok = (int)t + n * kStep < left;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + n * kStep * PITCH * 4),
+                     "l"(ok ? src + (size_t)n * kStep * v.t_stride * 8 : static_cast<const float *>(v.p)), "r"(ok ? 4 : 0) : "memory");
+    }
+}
+
 // ---- the same with both operands streamed in chunks of KC columns (fp32, many tokens)
 // Bound by FMA issue once a lane has 8 x 4 results: 12 loads of 16 bytes from shared memory feed 64 packed FMAs, where the
 // 4 x 4 results that fit beside resident operands take 8 for 32 and wait for shared memory (m = 64, us: forward of 1500
@@ -476,48 +512,18 @@ template <typename C> struct Chunks {
 #pragma unroll
             for (int q = 0; q < RE; ++q) s[i][q] = 0;
     }
-    // columns c0 .. c0 + KC of the input: permuted pieces (8 blocks, 32 bytes) go to the blocks' rows 4 bytes at a time
-    static __device__ __forceinline__ void load_a(float *tile, const View &v, int perm, int b0, int c0, int t0, int left)
-    {
-        if (!perm) {
-            const float4 *src = static_cast<const float4 *>(v.p);
-            const unsigned first = t0 * v.t_stride + b0 * v.b_stride + c0 / 8 * v.c_stride;
-#pragma unroll 4
-            for (int j = threadIdx.x; j < TT * KC * 2; j += C::kThreads) {
-                const int h = j % 2, i = j / 2, t = i / KC;
-                int b, c;
-                if (v.mid) { b = i % 8; c = i / 8 % (KC / 8); }
-                else       { c = i % (KC / 8); b = i / (KC / 8) % 8; }
-                const bool ok = t < left;
-                cp_async16(tile + b * C::kBlockA + t * PC + c * 8 + h * 4,
-                           src + (size_t)(first + (ok ? t : 0) * v.t_stride + b * v.b_stride + c * v.c_stride) * 2 + h, ok);
-            }
-            return;
-        }
-        const float *src = static_cast<const float *>(v.p);
-        const unsigned first = t0 * v.t_stride + b0 / 8 * v.b_stride + c0 * v.c_stride;
-#pragma unroll 4
-        for (int j = threadIdx.x; j < TT * KC * 8; j += C::kThreads) {
-            const int b = j % 8, c = j / 8 % KC, t = j / (8 * KC);
-            const bool ok = t < left;
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_addr(tile + b * C::kBlockA + t * PC + c)),
-                         "l"(src + (size_t)(first + (ok ? t : 0) * v.t_stride + c * v.c_stride) * 8 + b), "r"(ok ? 4 : 0) : "memory");
-        }
-    }
     static __device__ __forceinline__ void load_w(float *wt, const void *w, int trans, int b0, int e0, int c0)
     {
         const float *src = static_cast<const float *>(w) + (size_t)b0 * M * M;
-        constexpr int kVecs = 8 * ES * KC / 4;
-#pragma unroll 4
-        for (int i = threadIdx.x; i < kVecs; i += C::kThreads) {
-            if (!trans) {
-                const int c = i % (KC / 4) * 4, e = i / (KC / 4) % ES, b = i / (KC / 4 * ES);
-                cp_async16(wt + (b * ES + e) * PC + c, src + (b * M + e0 + e) * M + c0 + c, true);
-            } else {
-                const int e = i % (ES / 4) * 4, c = i / (ES / 4) % KC, b = i / (ES / 4 * KC);
-                cp_async16(wt + (b * KC + c) * (ES + 4) + e, src + (b * M + c0 + c) * M + e0 + e, true);
-            }
-        }
+        const unsigned j = threadIdx.x;
+        constexpr int kPer = ES * KC / 4, kStep = C::kThreads / kPer;      // pieces of a block, blocks per step
+        const unsigned c = trans ? j / (ES / 4) % KC : j % (KC / 4) * 4, e = trans ? j % (ES / 4) * 4 : j / (KC / 4) % ES, b = j / kPer;
+        src += (b * M + (trans ? c0 + c : e0 + e)) * M + (trans ? e0 + e : c0 + c);
+        float *dst = wt + (trans ? (b * KC + c) * (ES + 4) + e : (b * ES + e) * PC + c);
+        const int step = trans ? kStep * KC * (ES + 4) : kStep * ES * PC;
+        static_assert(C::kThreads % kPer == 0 && 8 % kStep == 0, "");
+#pragma unroll
+        for (int n = 0; n < 8 / kStep; ++n) cp_async16(dst + n * step, src + (size_t)n * kStep * M * M, true);
     }
     __device__ __forceinline__ void multiply(const float *tile, const float *wt, int trans)
     {
@@ -678,6 +684,29 @@ __device__ __forceinline__ void stage_units(const Op &op, int i0, int i1, int ti
     }
 }
 
+// part of PARTS of copy_out
+template <typename C, int PARTS>
+__device__ __forceinline__ void copy_part(const unsigned char *stage, const View &out, int perm, int b0, int e0, int t0, int left, int part)
+{
+    constexpr int ES = C::ES, kTok = C::TT / PARTS, kStep = C::kThreads / (2 * ES), kPlane = C::TT * C::PS;
+    static_assert(C::kThreads % (2 * ES) == 0 && kTok % kStep == 0, "");
+    const unsigned j = threadIdx.x, h = j % 2, i = j / 2 % ES, t = part * kTok + j / (2 * ES);
+    const unsigned b = perm ? 0 : out.mid ? i % 8 : i / (ES / 8), c = perm ? i : out.mid ? i / 8 : i % (ES / 8);
+    uint4 *dst = static_cast<uint4 *>(out.p) +
+                 (size_t)((t0 + t) * out.t_stride + (perm ? b0 / 8 : b0 + b) * out.b_stride + ((perm ? e0 : e0 / 8) + c) * out.c_stride) * 2 + h;
+    const unsigned char *from = stage + (perm ? (h * 4 * kPlane + t * C::PS + c) * 4 : t * C::kNatT + b * C::kNatB + c * 32 + h * 16);
+#pragma unroll
+    for (int n = 0; n < kTok / kStep; ++n, dst += (size_t)kStep * out.t_stride * 2) {
+        if ((int)t + n * kStep >= left) break;
+        if (perm) {
+            const uint32_t *s = reinterpret_cast<const uint32_t *>(from) + n * kStep * C::PS;
+            *dst = make_uint4(s[0], s[kPlane], s[2 * kPlane], s[3 * kPlane]);
+        } else {
+            *dst = *reinterpret_cast<const uint4 *>(from + n * kStep * C::kNatT);
+        }
+    }
+}
+
 template <typename C>
 __device__ __forceinline__ void stage_units_chunked(const Op &op, int i0, int i1, int tiles, int tokens, unsigned char *smem)
 {
@@ -688,12 +717,13 @@ __device__ __forceinline__ void stage_units_chunked(const Op &op, int i0, int i1
     auto wt = [&](int n) { return reinterpret_cast<float *>(smem + (n & 1) * C::kChunk + C::kChunkA); };
     auto begin = [&](int n, int i, int k) {
         const int at = i / tiles, tile_no = i % tiles, b0 = at / kSlices * 8, e0 = at % kSlices * C::ES;
-        Chunks<C>::load_a(tile(n), op.in, op.perm, b0, k * KC, tile_no * C::TT, tokens - tile_no * C::TT);
+        load_async<C, C::TT, KC, C::PC, C::kBlockA>(tile(n), op.in, op.perm, b0, k * KC, tile_no * C::TT, tokens - tile_no * C::TT);
         Chunks<C>::load_w(wt(n), op.w, op.trans, b0, e0, k * KC);
     };
-    auto copy = [&](int i, int part, int parts) {
+    constexpr int kParts = kChunks / 2;
+    auto copy = [&](int i, int part) {
         const int at = i / tiles, tile_no = i % tiles;
-        copy_out<C>(stage, op.out, op.perm, at / kSlices * 8, at % kSlices * C::ES, tile_no * C::TT, tokens - tile_no * C::TT, part, parts);
+        copy_part<C, kParts>(stage, op.out, op.perm, at / kSlices * 8, at % kSlices * C::ES, tile_no * C::TT, tokens - tile_no * C::TT, part);
     };
     int n = 0;
     __syncthreads();                                   // what ran before has left shared memory
@@ -707,9 +737,8 @@ __device__ __forceinline__ void stage_units_chunked(const Op &op, int i0, int i1
             __syncthreads();                           // chunk n is here, chunk n - 1 has been read
             const bool more = k + 1 < kChunks || i + 1 < i1;
             if (more) begin(n + 1, k + 1 < kChunks ? i : i + 1, k + 1 < kChunks ? k + 1 : 0);
-            // the previous unit's results leave during this one's products, but for the last chunk: behind its barrier they
-            // may be staged over
-            if (i > i0 && k < kChunks - 1) copy(i - 1, k, kChunks - 1);
+            // the previous unit's results leave during the first half of this one's products
+            if (i > i0 && k < kParts) copy(i - 1, k);
             sums.multiply(tile(n), wt(n), op.trans);
         }
         const int at = i / tiles, tile_no = i % tiles, b0 = at / kSlices * 8, e0 = at % kSlices * C::ES;
@@ -717,7 +746,7 @@ __device__ __forceinline__ void stage_units_chunked(const Op &op, int i0, int i1
         sums.finish(acc, op.trans);
         finish_unit<C>(op, acc, stage, b0, e0, tile_no, tokens);
     }
-    copy(i1 - 1, 0, 1);
+    for (int part = 0; part < kParts; ++part) copy(i1 - 1, part);
 }
 
 // ---------------------------------------------------------------- a weight-gradient unit
@@ -736,9 +765,15 @@ __device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0,
     TileLoad<C, TW, LS, C::PL> load_a;
     TileLoad<C, TW, KS, C::PK> load_b;
     auto tile_a = [&](int buf) { return reinterpret_cast<T *>(smem + buf * C::kStepBytes); };
-    auto tile_b = [&](int buf) { return tile_a(buf) + C::G * TW * C::PL; };
-    // the operand of the natural role is asynchronous; the other goes through registers, one operand after the other
+    auto tile_b = [&](int buf) { return tile_a(buf) + C::G * C::kBlockL; };
+    // operands of the natural role are asynchronous; the others go through registers, one operand after the other, unless many
+    // fp32 tokens make the copies of 4 bytes worth their number
     auto load = [&](int s) {
+        if constexpr (C::KC > 0) {
+            load_async<C, TW, LS, C::PL, C::kBlockL>(tile_a(s & kMask), op.in, op.perm, b0, l0, s * TW, tokens - s * TW);
+            load_async<C, TW, KS, C::PK, C::kBlockK>(tile_b(s & kMask), op.in2, op.perm, b0, k0, s * TW, tokens - s * TW);
+            return;
+        }
         load_a.begin(tile_a(s & kMask), op.in, op.perm, b0, l0 / 8, s * TW, tokens - s * TW);
         load_a.end(tile_a(s & kMask), op.perm);
         load_b.begin(tile_b(s & kMask), op.in2, op.perm, b0, k0 / 8, s * TW, tokens - s * TW);
@@ -754,7 +789,7 @@ __device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0,
     for (int s = s0; s < s1; ++s) {
         cp_async_wait();
         __syncthreads();                               // the operands of s are here, those of s - 1 have been read
-        const bool early = C::kSteps == 2 && !op.perm;
+        const bool early = C::kSteps == 2 && (C::KC > 0 || !op.perm);
         if (early && s + 1 < s1) load(s + 1);
         if constexpr (C::kBf) {
             const bf16 *a = tile_a(s & kMask) + (bw * TW + (lane & 7) + (lane >> 4) * 8) * C::PL + (lane >> 3 & 1) * 8;
@@ -784,7 +819,7 @@ __device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0,
                 }
             }
         } else {
-            const float *a = tile_a(s & kMask) + bw * TW * C::PL + (lane >> 3) * RL, *b = tile_b(s & kMask) + bw * TW * C::PK + kw + (lane & 7) * VK;
+            const float *a = tile_a(s & kMask) + bw * C::kBlockL + (lane >> 3) * RL, *b = tile_b(s & kMask) + bw * C::kBlockK + kw + (lane & 7) * VK;
 #pragma unroll 4
             for (int t = 0; t < TW; ++t) {
                 float fa[RL], fb[RK];
