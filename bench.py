@@ -604,8 +604,7 @@ def main_cplx(args):
         "config": {"workload": workload, "l2": "each call streams > 1 GB of planes and partial results",
                    "device_status": status},
         "clocks": clocks, "gpu_launches": int(launches),
-        "roofline": {"bound": "hbm", "kernel": "per call: 4 x fused_fwd_m64_team_kernel (or fused_bwd_dx_m64_kernel) "
-                                               "on 2 x tokens rows + cplx_combine_kernel",
+        "roofline": {"bound": "hbm", "kernel": "cplx_kernel (2 launches per call)",
                      "achieved": nbytes / ms / 1e6, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": nbytes / ms / 1e6 / peaks["hbm_gbs"], "peak_source": peaks["source"], "traffic": None,
                      "algorithmic_mb": nbytes / 1e6},
