@@ -221,20 +221,18 @@ KERNELS_OF = {
     (128, "bf16", "bwd_dx"): "plane_transpose_kernel + chain_gemm_kernel x 2 (3 launches)",
     (128, "bf16", "bwd_dw"): "chain_gemm_kernel (stage 1) + plane_transpose_kernel + chain_gemm_kernel x 2 (4 launches)",
 }
-_W3 = "profiles/fused_m64_workload3_ncu.md, full size"
+_W3 = "profiles/stream_kernels_ncu.md, full size, cold L2 per launch (upper bound)"
 _W4 = "profiles/chain_m128_workload4_ncu.md, full size, cold L2 per launch (upper bound)"
 NCU_TRAFFIC_MB = {
     (1, "fwd"): (0.1, "profiles/fused_fwd_m16_workload1_ncu.md, full size; the 65 KB output is still in L2 at kernel end"),
-    (2, "fwd"): (33.9, "profiles/fused_fwd_m32_workload2_ncu.md, full size; the 33.6 MB output is still in L2 at kernel end"),
-    (3, "fwd"): (146.9, _W3),
-    (3, "bwd"): (364.0, _W3),
-    (3, "bwd_dx"): (139.8, _W3),
-    (3, "bwd_dw"): (408.3, _W3),
+    (2, "fwd"): (34.1, "profiles/stream_kernels_ncu.md, full size; the 33.6 MB output is still in L2 at kernel end"),
+    (3, "fwd"): (164.9, _W3),
+    (3, "bwd"): (387.7, _W3),
     (4, "fwd"): (460.8, _W4),
     (4, "bwd"): (924.8, _W4),
     (4, "bwd_dx"): (637.8, _W4),
     (4, "bwd_dw"): (1055.3, _W4),
-    (5, "mlp_fwd"): (1511.0, "profiles/mlp_fwd_workload5_ncu.md, full size, both passes"),
+    (5, "mlp_fwd"): (1933.0, _W3),
 }
 
 
