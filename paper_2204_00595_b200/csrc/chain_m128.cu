@@ -809,9 +809,11 @@ chain_fused_fwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_co
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) {
-                                const float a = __uint_as_float(v[q][e]) + bias;
-                                v[q][e] = __float_as_uint(p.gelu ? gelu_fast(a) : a);
+                            for (int e = 0; e < 16; e += 2) {
+                                float a = __uint_as_float(v[q][e]) + bias, b = __uint_as_float(v[q][e + 1]) + bias;
+                                if (p.gelu) gelu_fast2(a, b);
+                                v[q][e] = __float_as_uint(a);
+                                v[q][e + 1] = __float_as_uint(b);
                             }
                     }
                     // staging half h is free once the store of the previous item's half h has read it

@@ -113,6 +113,45 @@ static __device__ __forceinline__ float gelu_fast(float a)
     return a * r;
 }
 
+// The same for two values, bit for bit, with packed instructions where there are any: 12 to issue instead of 18 (block of 4000
+// tokens at m = 128: 247 -> 241 us; m = 32, 16000 tokens: 40.6 -> 40.0; the m = 64 kernel, which holds its weights in
+// registers, was slower with the pairs: 389 against 384).  One reciprocal for both, of the product of their denominators, takes
+// more instructions and cost 5 % at m = 64 and 18 % at m = 128.
+static __device__ __forceinline__ void gelu_fast2(float &a, float &b)
+{
+    asm("{\n\t"
+        ".reg .b64 x, q, t, c;\n\t"
+        ".reg .f32 u, v, one;\n\t"
+        "mov.b64 x, {%0, %1};\n\t"
+        "mul.rn.f32x2 q, x, x;\n\t"
+        "mov.b64 {u, v}, q;\n\t"
+        "min.f32 u, u, 0f42800000;\n\t"
+        "min.f32 v, v, 0f42800000;\n\t"
+        "mov.b64 q, {u, v};\n\t"
+        "mov.b64 t, {%2, %2};\n\t"
+        "mov.b64 c, {%3, %3};\n\t"
+        "fma.rn.f32x2 t, q, t, c;\n\t"
+        "mov.b64 c, {%4, %4};\n\t"
+        "fma.rn.f32x2 t, q, t, c;\n\t"
+        "mul.rn.f32x2 t, x, t;\n\t"
+        "mov.b64 {u, v}, t;\n\t"
+        "ex2.approx.ftz.f32 u, u;\n\t"
+        "ex2.approx.ftz.f32 v, v;\n\t"
+        "mov.b64 t, {u, v};\n\t"
+        "mov.f32 one, 0f3F800000;\n\t"
+        "mov.b64 c, {one, one};\n\t"
+        "add.rn.f32x2 t, t, c;\n\t"
+        "mov.b64 {u, v}, t;\n\t"
+        "rcp.approx.ftz.f32 u, u;\n\t"
+        "rcp.approx.ftz.f32 v, v;\n\t"
+        "mov.b64 t, {u, v};\n\t"
+        "mul.rn.f32x2 t, x, t;\n\t"
+        "mov.b64 {%0, %1}, t;\n\t"
+        "}"
+        : "+f"(a), "+f"(b)
+        : "f"(0.0010142630198970437f), "f"(-0.10677572339773178f), "f"(-2.301121234893799f));
+}
+
 // d/da GELU(a) = Phi(a) + a phi(a) with Phi from the same sigmoid (|Phi error| <= 5.1e-5) and the normal
 // density phi evaluated directly: |error| <= 5.1e-5, for results that are rounded to bf16.
 static __device__ __forceinline__ float gelu_fast_grad(float a)

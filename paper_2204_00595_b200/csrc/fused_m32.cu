@@ -221,9 +221,10 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             wl.times(v >> 1, in.b[v >> 1][v & 1], acc);
             if (ACT)
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const float a = acc[k >> 2][k & 3] + bias[v >> 1][k >> 1];
-                    acc[k >> 2][k & 3] = p.gelu ? gelu_fast(a) : a;
+                for (int k = 0; k < 8; k += 2) {
+                    acc[k >> 2][k & 3] += bias[v >> 1][k >> 1];
+                    acc[k >> 2][(k & 3) + 1] += bias[v >> 1][k >> 1];
+                    if (p.gelu) gelu_fast2(acc[k >> 2][k & 3], acc[k >> 2][(k & 3) + 1]);
                 }
             pack_rows(acc, o);
             stm4(e_at(e, warp * 2 + (v >> 1), v & 1, ln.m * 8 + ln.r), o);
