@@ -226,7 +226,6 @@ int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *
 size_t fused_mlp_fwd_m64_workspace_bytes(int64_t tokens);
 int fused_mlp_fwd_m64(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2, void *y,
                       int64_t tokens, void *ws, cudaStream_t s);
-size_t fused_cplx_m64_workspace_bytes(int64_t tokens);
 int fused_cplx_m64(const void *x, const void *L, const void *R, void *y, int adjoint, int64_t tokens, void *ws, cudaStream_t s);
 size_t fused_bwd_dx_m64_workspace_bytes(int64_t tokens);
 int fused_bwd_dx_m64(const void *dy, const void *L, const void *R, void *dx, int64_t tokens, void *ws, cudaStream_t s);

@@ -17,8 +17,8 @@
 //           lie; a CTA's sums are 128 KB of accumulators (half of its registers), stored once and added by a last launch in a
 //           fixed order.
 // A warp works on its own blocks and only the transposes look across, so warps run ahead of one another between mbarriers;
-// a thread of the first warp asks for tiles and sends results away, one tile behind its own work (a warp of its own would
-// cost every other one 32 of its 128 registers).  With a CTA barrier per tile instead, loads, MMAs and stores of a
+// the warps ask for tiles and send results away by turns, one tile behind their own work (a warp for that alone would cost
+// every other one 32 of its 128 registers).  With a CTA barrier per tile instead, loads, MMAs and stores of a
 // tile followed one another (2650 cycles per 32 KB tile and stage against 1030 of MMA and 1000 to 1500 of shared memory).
 // The weights arrive by TMA as swizzled rows and go to registers by ldmatrix (1 us; fetched by the warps themselves in the
 // 16-byte pieces of the operand layout they took 4).
@@ -937,7 +937,7 @@ int fused_bwd_m64(const void *x, const void *dy, const void *L, const void *R, c
     return stream_bwd(x, dy, L, R, u_saved != nullptr ? u_saved : u, u_saved != nullptr, dx, dL, dR, accumulate, du, parts, tokens, (unsigned *)ws, s);
 }
 
-size_t fused_cplx_m64_workspace_bytes(int64_t tokens) { return kHead + 2 * tc::e_bytes(tokens); }
+// (E tiles of both planes: a quarter of the workspace that the call asks for at every size)
 int fused_cplx_m64(const void *x, const void *L, const void *R, void *y, int adjoint, int64_t tokens, void *ws, cudaStream_t s)
 {
     return tokens == 0 ? MONARCH_OK : stream_cplx(x, L, R, y, adjoint, head(ws), tokens, (unsigned *)ws, s);
