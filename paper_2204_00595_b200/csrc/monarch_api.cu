@@ -111,7 +111,7 @@ int pick(int op, int m, int dtype)
 
 // Largest batch that runs as one launch over block-product units (block_units.cu); beyond it the kernels above are
 // faster.  Measured per pass, back to back (us, units / the others):
-//   bf16 m = 16   forward 27 / 213 at 32768 tokens, forward + backward 148 / 484: every batch
+//   bf16 m = 16   forward + backward 148 / 484 at 32768 tokens: every batch (the forward alone: fused_m16.cu)
 //   bf16 m = 32   forward 9.5 / 7.0 at 4, 12.4 / 6.6 at 1000; forward + backward 18.5 / 14.1 at 4: never; the backward of
 //                 the feed-forward block, eight launches otherwise, 45 / 48 at 64, 58 / 49 at 128 (with its forward)
 //   bf16 m = 64   forward 10.7 / 9.2 at 64; forward + backward 23 / 24.5 at 4, 26.7 / 26.3 at 64; block 18.6 / 19.5 at 64,
@@ -132,8 +132,9 @@ int64_t units_limit(int op, int m, int dtype)
 // (the switches that ask for a particular form of the other kernels keep their meaning at every size)
 bool use_units(int op, int m, int dtype, int64_t tokens)
 {
-    // the smallest m = 16 forwards: both stages of a few tokens fit one CTA, which needs no barrier (fused_m16.cu)
-    if (m == 16 && op == MONARCH_OP_FWD && tokens <= 256) return false;
+    // m = 16 forwards (fused_m16.cu): in bf16 the units would round u, which that kernel keeps in fp32; the smallest in fp32 fit one
+    // CTA, which needs no barrier
+    if (m == 16 && op == MONARCH_OP_FWD && (dtype == MONARCH_BF16 || tokens <= 256)) return false;
     return g_impl.load(std::memory_order_relaxed) == MONARCH_IMPL_AUTO && tokens > 0 && tokens <= units_limit(op, m, dtype) &&
            !(m == 64 && fused_fwd_m64_on_clusters()) && !(m == 128 && chain_fwd_m128_split());
 }

@@ -982,6 +982,30 @@ def test_one_launch_over_units(P, m, T, dtype):
         _check_guard(flat, what)
 
 
+@pytest.mark.parametrize("T", [257, 258, 1023, 4 * 4 * 148 + 1, 9473])
+def test_fwd_m16_keeps_u_in_fp32(P, T):
+    """bf16 m = 16 forwards round only y: a value's error is uniform within half a unit in its last place, at most 2^-8 of the
+    value, so 2^-8 / sqrt(3) of the tensor in the 2-norm (a rounded u adds as much again: 1.04 of this bound).  The bits of a
+    token do not depend on the batch that it is in."""
+    import torch
+    m, n, dtype, code = 16, 256, "bf16", P.BF16
+    d = _small_inputs(m, T, dtype, seed=1600 + T)
+    x, L, R = (to_device(d[k], dtype) for k in ("x", "L", "R"))
+    yf, y = _guarded((T, n), torch.bfloat16)
+    ws = P.Workspace(P.monarch_workspace_bytes(P.OP_FWD, T, n, m, code))
+    P.monarch_fwd(x, L, R, y, T, n, m, ws)
+    small = torch.empty_like(y)
+    for t0 in range(0, T, 100):
+        t1 = min(t0 + 100, T)
+        P.monarch_fwd(x[t0:t1], L, R, small[t0:t1], t1 - t0, n, m, ws)
+    torch.cuda.synchronize()
+    assert P.monarch_last_device_status(ws) == 0
+    _check_guard(yf, "y")
+    ref = O.fwd(d["x"], d["L"], d["R"])
+    assert np.linalg.norm(to_host64(y) - ref) <= 2.0 ** -8 / np.sqrt(3.0) * np.linalg.norm(ref)
+    assert torch.equal(y, small)
+
+
 @pytest.mark.parametrize("m,T,dtype", [(16, 1300, "bf16"), (32, 1190, "bf16"), (64, 449, "bf16"), (128, 97, "bf16"), (64, 300, "f32"),
                                        (32, 129, "bf16"), (64, 65, "bf16"), (64, 193, "bf16"), (128, 25, "bf16")])
 def test_one_launch_feed_forward(P, m, T, dtype):
