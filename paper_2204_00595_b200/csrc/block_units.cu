@@ -51,21 +51,34 @@ bool use_large(int dtype, int m, int64_t tokens)
     return dtype == MONARCH_F32 && m > 16 ? 5 * (units + 20) >= 4 * kSms * waves : units >= kSms;
 }
 
-constexpr int kMaxSplits = 16;
-// token ranges of a weight gradient: enough units for every SM, at least four steps in a range
-int wgrad_splits(int dtype, int m, int64_t tokens, bool large)
+constexpr int kMaxSplits = 40;
+// Most token ranges of a weight gradient: enough units for every SM, at least four steps in a range.  And a range is summed by one
+// accumulator, whose rounding error grows with its length: none is longer than 256 tokens, or tokens / (592 / m) if that is more,
+// which is what the staged family sums at a time (staged_simt.cu).  fp32, error of dL for the staged family / at most 16 ranges /
+// this: m = 16, 32768 tokens 5.5e-7 / 8.1e-7 / 5.4e-7 (forward + backward 309 -> 180 us), m = 32, 8192 tokens 4.0e-7 / 4.2e-7 /
+// 3.0e-7 (256 -> 235 us; 4999 tokens 174 -> 181).
+int max_splits(int dtype, int m, int64_t tokens, bool large)
 {
     const Sizes s = sizes(dtype, m, large);
     const long long base = (long long)(m / 8) * (m / s.LS) * (m / s.KS), steps = ceil_div(tokens, s.TW);
     long long n = kSms / base;
     if (n > steps / 4) n = steps / 4;
     if (n > kMaxSplits) n = kMaxSplits;
+    const long long runs = ceil_div(tokens, 256), most = ceil_div(4 * kSms, m), least = runs < most ? runs : most;
+    if (n < least) n = least;
     return n < 1 ? 1 : (int)n;
 }
-// (for either tiles: a workspace for a batch serves every smaller one)
+// without empty ranges
+int wgrad_splits(int dtype, int m, int64_t tokens, bool large)
+{
+    const long long steps = ceil_div(tokens, sizes(dtype, m, large).TW), per = ceil_div(steps, max_splits(dtype, m, tokens, large));
+    return (int)ceil_div(steps, per);
+}
+// (for either tiles, and growing with the tokens: a workspace for a batch serves every smaller one)
 size_t parts_bytes(int dtype, int m, int64_t tokens)
 {
-    const int a = wgrad_splits(dtype, m, tokens, false), b = wgrad_splits(dtype, m, tokens, true), s = a > b ? a : b;
+    if (tokens == 0) return 0;
+    const int a = max_splits(dtype, m, tokens, false), b = max_splits(dtype, m, tokens, true), s = a > b ? a : b;
     return s > 1 ? up256((size_t)s * m * m * m * sizeof(float)) : 0;
 }
 size_t act_bytes(int dtype, int m, int64_t tokens) { return up256((size_t)tokens * m * m * esize(dtype)); }

@@ -880,7 +880,7 @@ __device__ __forceinline__ void reduce_unit(const Op &op, int unit)
     const long long i = (long long)unit * kReducePer + threadIdx.x * 4;
     if (threadIdx.x * 4 >= kReducePer || i >= op.count) return;
     float4 s = op.accumulate ? *reinterpret_cast<const float4 *>(op.sums + i) : make_float4(0, 0, 0, 0);
-#pragma unroll 4
+#pragma unroll 8
     for (int p = 0; p < op.splits; ++p) {
         const float4 v = *reinterpret_cast<const float4 *>(op.parts + p * op.count + i);
         s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;

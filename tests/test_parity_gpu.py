@@ -1006,6 +1006,28 @@ def test_fwd_m16_keeps_u_in_fp32(P, T):
     assert torch.equal(y, small)
 
 
+@pytest.mark.parametrize("m,T", [(16, 32768), (32, 8192), (64, 4096), (128, 2048)])
+def test_fp32_weight_gradients_sum_short_runs(P, m, T):
+    """What one fp32 accumulator of a weight gradient adds up: with the identity in every block, x = 1 and dy = 1 but for a first
+    token of 2^24, every entry of dL and dR is 2^24 + T - 1, and the ones that share an accumulator with the large value are
+    lost, each below half a unit of its last place.  A run is at most 256 tokens or T / ceil(592 / m), whichever is more; adding
+    the runs rounds by at most one (of 2^24's units of 2) each."""
+    import torch
+    n = m * m
+    eye = torch.eye(m, device="cuda").repeat(m, 1, 1)
+    x = torch.ones(T, n, device="cuda")
+    dy = torch.ones(T, n, device="cuda")
+    dy[0] = 2.0 ** 24
+    dx, dL, dR = torch.empty_like(x), torch.empty(m, m, m, device="cuda"), torch.empty(m, m, m, device="cuda")
+    ws = P.Workspace(P.monarch_workspace_bytes(P.OP_BWD, T, n, m, P.F32))
+    P.monarch_bwd(x, dy, eye, eye.clone(), dx, dL, dR, 0, T, n, m, ws)
+    torch.cuda.synchronize()
+    assert P.monarch_last_device_status(ws) == 0
+    run = max(256, -(-T // -(-592 // m)))
+    for g in (dL, dR):
+        assert float((g.double() - (2.0 ** 24 + T - 1)).abs().max()) <= run + 40
+
+
 @pytest.mark.parametrize("m,T,dtype", [(16, 1300, "bf16"), (32, 1190, "bf16"), (64, 449, "bf16"), (128, 97, "bf16"), (64, 300, "f32"),
                                        (32, 129, "bf16"), (64, 65, "bf16"), (64, 193, "bf16"), (128, 25, "bf16")])
 def test_one_launch_feed_forward(P, m, T, dtype):
