@@ -906,12 +906,16 @@ template <typename C> __device__ __forceinline__ void colsum_unit(const Op &op, 
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < V; ++e) red[r * kColsumCols + cl * V + e] = s[e];
+    // pairwise: a chain over the rows would round a short sum more often than one over its tokens
+#pragma unroll 1
+    for (int half = kRows / 2; half > 0; half /= 2) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < half * kColsumCols; i += C::kThreads) red[i] += red[i + half * kColsumCols];
+    }
     __syncthreads();
     if (threadIdx.x < kColsumCols) {
-        float v = 0.0f;
-        for (int q = 0; q < kRows; ++q) v += red[q * kColsumCols + threadIdx.x];
         float *d = op.sums + unit * kColsumCols + threadIdx.x;
-        *d = op.accumulate ? *d + v : v;
+        *d = op.accumulate ? *d + red[threadIdx.x] : red[threadIdx.x];
     }
 }
 

@@ -150,10 +150,14 @@ mlp_dact_kernel(T *__restrict__ dh, const T *__restrict__ a, const T *__restrict
     __syncthreads();
     for (int i = threadIdx.x; i < 2 * 32 * V; i += kThreads) {
         const int which = i / (32 * V), c = i % (32 * V);
-        float v = 0.0f;
+        float v[kRows];
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) v += red[r][which][c];
-        atomicAdd((which == 0 ? db1 : db2) + blockIdx.x * 32 * V + c, v);
+        for (int r = 0; r < kRows; ++r) v[r] = red[r][which][c];
+#pragma unroll
+        for (int half = kRows / 2; half > 0; half /= 2)        // pairwise: the fewest roundings
+#pragma unroll
+            for (int r = 0; r < half; ++r) v[r] += v[r + half];
+        atomicAdd((which == 0 ? db1 : db2) + blockIdx.x * 32 * V + c, v[0]);
     }
 }
 

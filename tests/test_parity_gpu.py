@@ -1028,6 +1028,27 @@ def test_fp32_weight_gradients_sum_short_runs(P, m, T):
         assert float((g.double() - (2.0 ** 24 + T - 1)).abs().max()) <= run + 40
 
 
+@pytest.mark.parametrize("m,T,dtype", [(16, 16, "f32"), (16, 24, "bf16"), (32, 32, "f32"), (32, 73, "bf16"), (64, 31, "f32"), (64, 97, "bf16"),
+                                       (128, 8, "f32"), (128, 100, "f32"), (128, 33, "bf16")])
+def test_bias_gradients_of_few_tokens(P, m, T, dtype):
+    """db2 = sum_t dy[t] over 2^24 in the first token and 1 in the others: a one that is added to the large value is lost.  Eight
+    tokens at a time and then pairs lose at most one of them per step, 8 + log2(T / 8) rounded up; a chain over all tokens loses
+    T - 1."""
+    import torch
+    n, code = m * m, _code(P, dtype)
+    d = _small_inputs(m, T, dtype, seed=41 * m + T)
+    t = {k: to_device(d[k], dtype) for k in ("x", "L", "R", "b1", "L2", "R2")}
+    t["dy"] = torch.ones(T, n, dtype=_tdtype(dtype), device="cuda")
+    t["dy"][0] = 2.0 ** 24
+    bufs = _mlp_bwd_buffers(m, T, dtype)
+    ws = P.Workspace(P.monarch_workspace_bytes(P.OP_MLP_BWD, T, n, m, code))
+    _call_mlp_bwd(P, t, bufs, 0, T, n, m, ws)
+    torch.cuda.synchronize()
+    assert P.monarch_last_device_status(ws) == 0
+    lost = (bufs["db2"][1].double() - (2.0 ** 24 + T - 1)).abs().max()
+    assert float(lost) <= 8 + np.ceil(np.log2(max(T / 8, 1)))
+
+
 @pytest.mark.parametrize("m,T,dtype", [(16, 1300, "bf16"), (32, 1190, "bf16"), (64, 449, "bf16"), (128, 97, "bf16"), (64, 300, "f32"),
                                        (32, 129, "bf16"), (64, 65, "bf16"), (64, 193, "bf16"), (128, 25, "bf16")])
 def test_one_launch_feed_forward(P, m, T, dtype):
