@@ -72,7 +72,7 @@ template <typename T_, int M_, int TT_, int ES_, int LS_, int KS_, int KC_ = 0> 
     static constexpr int kWpb = KC_ > 0 ? 2 : 1, kThreads = 32 * G * kWpb;   // warps per block
     static constexpr int EW = ES / kWpb, KW = KS / kWpb;      // outputs / gradient columns of one warp
     static constexpr int kPad = kBf ? 8 : 4;                  // rows 16 bytes longer: conflict-free ldmatrix / 16-byte reads
-    static constexpr int PA = M + kPad, PE = ES + kPad, PL = LS + kPad, PK = KS + kPad;
+    static constexpr int PA = M + kPad, PE = kBf ? ES + kPad : ES, PL = LS + kPad, PK = KS + kPad;
     // KC > 0 (fp32, many tokens): both operands of a stage stream through shared memory, KC columns at a time, which
     // leaves room for 8 x 8 results per lane; one CTA per SM
     static constexpr int KC = KC_, PC = KC + 4;
@@ -84,7 +84,7 @@ template <typename T_, int M_, int TT_, int ES_, int LS_, int KS_, int KC_ = 0> 
     static constexpr int kNatB = ES * (int)sizeof(T) + 16, kNatT = G * kNatB + 16;
     static constexpr int kStageBytes = cmax(kPlanes * TT * PS * 4, TT * kNatT);
     static constexpr int kTileBytes = G * TT * PA * (int)sizeof(T);
-    static constexpr int kWBytes = cmax(G * ES * PA, kBf ? G * M * PE : 0) * (int)sizeof(T);
+    static constexpr int kWBytes = cmax(G * ES * PA, G * M * PE) * (int)sizeof(T);
     static constexpr int kPadB = KC ? 4 : 0;                  // between the blocks of a step: 4-byte copies of 8 blocks without conflicts
     static constexpr int kBlockL = TW * PL + kPadB, kBlockK = TW * PK + kPadB;
     static constexpr int kStepBytes = G * (kBlockL + kBlockK) * (int)sizeof(T);
@@ -215,8 +215,8 @@ template <typename C, int R, int NC, int PITCH> struct TileLoad {
     }
 };
 
-// rows e0 .. e0 + ES of the result of 8 blocks: bf16 keeps the storage order (ldmatrix transposes), fp32 is stored
-// [b][e][c] either way
+// rows e0 .. e0 + ES of the result of 8 blocks in storage order, [b][e][c], of transposed blocks [b][c][e].  fp32: the ES / 8
+// neighbouring rows of a lane are kept 8 rows apart, so that the lanes' reads fall on different banks.
 template <typename C>
 __device__ __forceinline__ void load_weights(typename C::T *wt, const void *w, int trans, int b0, int e0)
 {
@@ -228,23 +228,15 @@ __device__ __forceinline__ void load_weights(typename C::T *wt, const void *w, i
 #pragma unroll 4
         for (int i = threadIdx.x; i < kVecs; i += C::kThreads) {
             const int c = i % (M / V) * V, e = i / (M / V) % ES, b = i / (M / V * ES);
-            cp_async16(wt + (b * ES + e) * C::PA + c, src + ((size_t)b * M + e0 + e) * M + c, true);
-        }
-    } else if constexpr (C::kBf) {
-        constexpr int kVecs = 8 * M * (ES / V);
-#pragma unroll 4
-        for (int i = threadIdx.x; i < kVecs; i += C::kThreads) {
-            const int e = i % (ES / V) * V, c = i / (ES / V) % M, b = i / (ES / V * M);
-            cp_async16(wt + (b * M + c) * C::PE + e, src + ((size_t)b * M + c) * M + e0 + e, true);
+            const int row = C::kBf ? e : e % (ES / 8) * 8 + e / (ES / 8);
+            cp_async16(wt + (b * ES + row) * C::PA + c, src + ((size_t)b * M + e0 + e) * M + c, true);
         }
     } else {
         constexpr int kVecs = 8 * M * (ES / V);
 #pragma unroll 4
         for (int i = threadIdx.x; i < kVecs; i += C::kThreads) {
-            const int c = i % M, e = i / M % (ES / V) * V, b = i / (ES / V * M);
-            const float4 f = *reinterpret_cast<const float4 *>(src + ((size_t)b * M + c) * M + e0 + e);
-            float *d = reinterpret_cast<float *>(wt) + (b * ES + e) * C::PA + c;
-            d[0] = f.x; d[C::PA] = f.y; d[2 * C::PA] = f.z; d[3 * C::PA] = f.w;
+            const int e = i % (ES / V) * V, c = i / (ES / V) % M, b = i / (ES / V * M);
+            cp_async16(wt + (b * M + c) * C::PE + e, src + ((size_t)b * M + c) * M + e0 + e, true);
         }
     }
 }
@@ -284,8 +276,8 @@ template <typename C> struct Acc<C, true> {
 template <typename C> struct Acc<C, false> {
     float v[C::TT / 4][C::EW / 8];
     static constexpr int V = C::EW / 8 < 4 ? C::EW / 8 : 4;
-    int packed;                                        // outputs of a lane: V neighbours at a time, else every eighth
-    __device__ __forceinline__ int output(int el, int q) const { return packed ? V * el + 8 * V * (q / V) + q % V : el + 8 * q; }
+    int packed;                                        // KC > 0: outputs of a lane are V neighbours at a time, else every eighth
+    __device__ __forceinline__ int output(int el, int q) const { return C::KC == 0 || packed ? V * el + 8 * V * (q / V) + q % V : el + 8 * q; }
     template <typename F> __device__ __forceinline__ void each(F f)
     {
         const int tl = (threadIdx.x & 31) >> 3, el = threadIdx.x & 7;
@@ -317,6 +309,19 @@ __device__ __forceinline__ uint32_t f2w(float x) { return __float_as_uint(x); }
 template <typename C> __device__ __forceinline__ void stage_results(Acc<C> &acc, unsigned char *stage, int perm)
 {
     const int w = threadIdx.x >> 5, b = w / C::kWpb, e0 = w % C::kWpb * C::EW;
+    if constexpr (!C::kBf && C::KC == 0) {             // a lane's outputs are neighbours
+        constexpr int V = C::ES / 8;
+        static_assert(V == 2 || V == 4, "");
+        const int tl = (threadIdx.x & 31) >> 3, el = threadIdx.x & 7;
+#pragma unroll
+        for (int i = 0; i < C::TT / 4; ++i) {
+            const int t = tl + 4 * i;
+            unsigned char *to = perm ? stage + ((b * C::TT + t) * C::PS + V * el) * 4 : stage + t * C::kNatT + b * C::kNatB + V * el * 4;
+            if constexpr (V == 4) *reinterpret_cast<float4 *>(to) = make_float4(acc.v[i][0], acc.v[i][1], acc.v[i][2], acc.v[i][3]);
+            else                  *reinterpret_cast<float2 *>(to) = make_float2(acc.v[i][0], acc.v[i][1]);
+        }
+        return;
+    }
     if (!perm) {
         if constexpr (C::kBf) {
             const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
@@ -374,6 +379,56 @@ __device__ __forceinline__ void copy_out(const unsigned char *stage, const View 
 }
 
 // ---------------------------------------------------------------- a stage unit
+// fp32, transposed blocks, whose columns are rows of shared memory: fma.rn.f32x2 takes two neighbouring outputs; partial sums over
+// even and odd columns as below.  (Transposed on their way into shared memory, through registers, dx of 200 tokens at m = 64
+// took 36 us, of 24 tokens at m = 128 37; now 31 and 29.)
+template <typename C> __device__ __forceinline__ Acc<C> multiply_transposed(const float *tile, const float *wt)
+{
+    constexpr int M = C::M, TT = C::TT, RE = C::EW / 8;
+    const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    Acc<C> acc;
+    const float *a = tile + (b * TT + (lane >> 3)) * C::PA, *bw = wt + b * M * C::PE + RE * (lane & 7);
+    f32x2 s[2][TT / 4][RE / 2];
+#pragma unroll
+    for (int i = 0; i < TT / 4; ++i)
+#pragma unroll
+        for (int q = 0; q < RE / 2; ++q) s[0][i][q] = s[1][i][q] = 0;
+#pragma unroll 1
+    for (int c = 0; c < M; c += 4) {
+        f32x2 fb[4][RE / 2];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if constexpr (RE == 4) {
+                const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(bw + (c + k) * C::PE);
+                fb[k][0] = t.x;
+                fb[k][1] = t.y;
+            } else {
+                fb[k][0] = *reinterpret_cast<const f32x2 *>(bw + (c + k) * C::PE);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < TT / 4; ++i) {
+            const float4 fa = *reinterpret_cast<const float4 *>(a + 4 * i * C::PA + c);
+            const float av[4] = {fa.x, fa.y, fa.z, fa.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int q = 0; q < RE / 2; ++q) s[k & 1][i][q] = fma2(pack2(av[k], av[k]), fb[k][q], s[k & 1][i][q]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < TT / 4; ++i)
+#pragma unroll
+        for (int q = 0; q < RE / 2; ++q) {
+            const float2 even = unpack2(s[0][i][q]), odd = unpack2(s[1][i][q]);
+            acc.v[i][2 * q] = even.x + odd.x;
+            acc.v[i][2 * q + 1] = even.y + odd.y;
+        }
+    return acc;
+}
+// out of line: inlined beside the other product it costs m = 128 registers (dx of 24 tokens 31 us, forward 26.6; so 28.8 and 24.7)
+template <typename C> __device__ __noinline__ Acc<C> multiply_transposed_far(const float *tile, const float *wt) { return multiply_transposed<C>(tile, wt); }
+
 template <typename C>
 __device__ __forceinline__ void multiply(Acc<C> &acc, const typename C::T *tile, const typename C::T *wt, int trans)
 {
@@ -432,7 +487,15 @@ __device__ __forceinline__ void multiply(Acc<C> &acc, const typename C::T *tile,
         }
     } else {
         // two partial sums per result (even and odd columns), packed for fma.rn.f32x2
-        const float *a = tile + (b * TT + (lane >> 3)) * C::PA, *bw = wt + (b * ES + e0 + (lane & 7)) * C::PA;
+        if (trans) {
+            const Acc<C> t = M == 128 ? multiply_transposed_far<C>(tile, wt) : multiply_transposed<C>(tile, wt);
+#pragma unroll
+            for (int i = 0; i < TT / 4; ++i)
+#pragma unroll
+                for (int q = 0; q < EW / 8; ++q) acc.v[i][q] = t.v[i][q];
+            return;
+        }
+        const float *a = tile + (b * TT + (lane >> 3)) * C::PA, *bw = wt + (b * ES + (lane & 7)) * C::PA;
         f32x2 s[TT / 4][EW / 8];
 #pragma unroll
         for (int i = 0; i < TT / 4; ++i)
@@ -457,7 +520,6 @@ __device__ __forceinline__ void multiply(Acc<C> &acc, const typename C::T *tile,
                 const float2 t = unpack2(s[i][q]);
                 acc.v[i][q] = t.x + t.y;
             }
-        acc.packed = 0;
     }
 }
 
@@ -919,6 +981,10 @@ template <typename C> __device__ __forceinline__ void colsum_unit(const Op &op, 
     }
 }
 
+// Out of line beside products that need every register (fp32 m = 64, 2048 tokens: backward 283 -> 264 us).
+template <typename C> __device__ __noinline__ void reduce_far(const Op &op, int unit) { reduce_unit(op, unit); }
+template <typename C> __device__ __noinline__ void colsum_far(const Op &op, int unit, int tokens, unsigned char *smem) { colsum_unit<C>(op, unit, tokens, smem); }
+
 // ---------------------------------------------------------------- the launch
 struct Plan {                                          // shares of the CTAs, worked out on the host
     int units[kMaxOps], shift[kMaxOps];                // of an operation: units, and log2 of the weight of one
@@ -998,9 +1064,11 @@ __global__ void __launch_bounds__(C::kThreads, C::kCtas) units_kernel(const __gr
                     wgrad_unit<C>(op, i / (kL * kK) % (M / 8) * 8, i / kK % kL * C::LS, i % kK * C::KS, i / (kL * kK * (M / 8)), p.tokens, smem);
                     held_op = -1;
                 } else if (op.kind == kReduce) {
-                    reduce_unit(op, i);
+                    if constexpr (M > 16) reduce_far<C>(op, i);
+                    else                  reduce_unit(op, i);
                 } else {
-                    colsum_unit<C>(op, i, p.tokens, smem);
+                    if constexpr (M > 16) colsum_far<C>(op, i, p.tokens, smem);
+                    else                  colsum_unit<C>(op, i, p.tokens, smem);
                     held_op = -1;
                 }
             }
