@@ -688,7 +688,7 @@ __device__ __forceinline__ void finish_unit(const Op &op, Acc<C> &acc, unsigned 
     } else if (op.act == kGeluGrad) {
         const T *a = static_cast<const T *>(op.in2.p);
         acc.each([&](float &v, int t, int e) {
-            if (t < left) v *= Math<T>::grad(elem<T>::load(a + (size_t)(t0 + t) * N + b * M + ew + e));
+            v = t < left ? v * Math<T>::grad(elem<T>::load(a + (size_t)(t0 + t) * N + b * M + ew + e)) : 0.0f;   // (0 x Inf of padding)
         });
         acc.column_sums([&](float s, int e) { op.sums[(size_t)tile_no * N + b * M + ew + e] = s; });
     }

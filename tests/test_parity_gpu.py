@@ -1049,6 +1049,25 @@ def test_bias_gradients_of_few_tokens(P, m, T, dtype):
     assert float(lost) <= 8 + np.ceil(np.log2(max(T / 8, 1)))
 
 
+@pytest.mark.parametrize("m,T,dtype", [(16, 3, "f32"), (16, 17, "bf16"), (32, 5, "f32"), (64, 7, "bf16"), (64, 33, "f32"), (128, 3, "f32"), (128, 5, "bf16")])
+def test_padding_stays_out_of_the_bias_gradients(P, m, T, dtype):
+    """One infinite entry of R2 makes one column of dh and of da infinite in every token; the rows that pad the last token tile are
+    zero times infinity there, and must not turn db1 into NaN."""
+    import torch
+    n, code, k, j, i = m * m, _code(P, dtype), 3, 5, 2
+    t = {"x": torch.zeros(T, n), "dy": torch.ones(T, n), "L": torch.zeros(m, m, m), "R": torch.zeros(m, m, m), "b1": torch.ones(n),
+         "L2": torch.ones(m, m, m), "R2": torch.ones(m, m, m)}
+    t["R2"][k, j, i] = float("inf")
+    t = {name: v.to("cuda", _tdtype(dtype)) for name, v in t.items()}
+    bufs = _mlp_bwd_buffers(m, T, dtype)
+    ws = P.Workspace(P.monarch_workspace_bytes(P.OP_MLP_BWD, T, n, m, code))
+    _call_mlp_bwd(P, t, bufs, 0, T, n, m, ws)
+    torch.cuda.synchronize()
+    assert P.monarch_last_device_status(ws) == 0
+    db1 = to_host64(bufs["db1"][1])
+    assert db1[k * m + i] == np.inf and np.isfinite(np.delete(db1, k * m + i)).all()
+
+
 @pytest.mark.parametrize("m,T,dtype", [(16, 1300, "bf16"), (32, 1190, "bf16"), (64, 449, "bf16"), (128, 97, "bf16"), (64, 300, "f32"),
                                        (32, 129, "bf16"), (64, 65, "bf16"), (64, 193, "bf16"), (128, 25, "bf16")])
 def test_one_launch_feed_forward(P, m, T, dtype):
