@@ -208,10 +208,13 @@ int launch_jacobi(const void *A, void *L, void *R, unsigned long long *rotations
 
 // ---- leading singular pair of a slice ------------------------------------------------------------------------------
 //  1. Power iteration on S^T S from TWO fixed unrelated start vectors.  It has converged when the two agree and have
-//     stopped moving, to kPowerTol: neither alone would show a start vector that happens to be orthogonal to v_1.
+//     stopped moving, to kPowerTol: neither alone would show a start vector that happens to be orthogonal to v_1.  Two that
+//     stand still and differ are eigenvectors both: singular values that are equal to rounding, or one vector that is
+//     orthogonal to v_1; the one with the larger singular value is taken.
 //     At most kPowerSteps steps are spent on it, enough for (sigma_2 / sigma_1)^2 up to about 0.7.
 //  2. Otherwise (a small gap) H = S^T S is squared and scaled to trace 1 until it has rank 1 - doubling the exponent
-//     each time, so the cost grows with the logarithm of 1 / gap and is bounded - and any column of H is v_1.
+//     each time, so the cost grows with the logarithm of 1 / gap and is bounded - and any column of H is v_1.  Orthogonal
+//     columns make H diagonal at once.
 // Both end in vectors accurate to rounding / gap.
 // One warp per slice (four for m = 128), a 4 x 8 grid of lanes, each lane holding an (m/4) x (m/8) patch of S in
 // registers for the whole iteration.  A product then needs m/8 (or m/4) values of the vector per lane from shared
@@ -463,7 +466,7 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
 
     for (int round = 0; round < 2; ++round) {
         bool done = round == 1;
-        float before[C::kZC] = {};
+        float before[C::kZC] = {}, before_b[C::kZC] = {};
         const int steps = round == 0 ? kPowerSteps : kPolishSteps;
 #pragma unroll 1
         for (int step = 0; step < steps; ++step) {
@@ -478,7 +481,7 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
             slice_sync<NT>();
             back(y, y + M, a, b);
             if ((step & 3) == 3) {
-                float v[3] = {0.0f, 0.0f, 0.0f}, d[2] = {0.0f, 0.0f};
+                float v[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
                 for (int i = 0; i < C::kZC; ++i) {
                     v[0] = fmaf(a[i], a[i], v[0]);
@@ -493,10 +496,20 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
                     b[i] *= nb;
                     d[0] = fmaf(a[i] - b[i], a[i] - b[i], d[0]);
                     d[1] = fmaf(a[i] - before[i], a[i] - before[i], d[1]);
+                    d[2] = fmaf(b[i] - before_b[i], b[i] - before_b[i], d[2]);
                     before[i] = a[i];
+                    before_b[i] = b[i];
                 }
                 slice_sum<NT>(d, red, phase);
-                if (fmaxf(d[0], d[1]) * kOnce < kPowerTol * kPowerTol) done = true;
+                constexpr float kStill = kPowerTol * kPowerTol / kOnce;
+                if (!(d[1] >= kStill) && !(d[0] >= kStill)) done = true;     // (NaN: nothing to wait for)
+                else if (d[1] < kStill && d[2] < kStill) {
+                    // both stand still and differ: eigenvectors, of the same singular value or not; the one with the larger is kept
+                    done = true;
+                    if (v[1] > v[0])
+#pragma unroll
+                        for (int i = 0; i < C::kZC; ++i) a[i] = b[i];
+                }
             }
 #pragma unroll
             for (int i = 0; i < C::kZC; ++i) {
@@ -527,6 +540,17 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
 #pragma unroll
                     for (int c = 0; c < C::kCQ * 4; ++c)
                         if (4 * (tr + r / 4 * C::kTR) + r % 4 == 4 * (tc + c / 4 * C::kTC) + c % 4) trace[0] += acc[r][c];
+            if (sq == 0) {                                // all products of different columns zero: the longest column is the answer
+                float off[1] = {0.0f};
+                if (on)
+#pragma unroll
+                    for (int r = 0; r < C::kRQ * 4; ++r)
+#pragma unroll
+                        for (int c = 0; c < C::kCQ * 4; ++c)
+                            if (4 * (tr + r / 4 * C::kTR) + r % 4 != 4 * (tc + c / 4 * C::kTC) + c % 4 && acc[r][c] != 0.0f) off[0] = 1.0f;
+                slice_sum<NT>(off, red, phase);
+                last = off[0] == 0.0f;
+            }
             slice_sum<NT>(trace, red, phase);
             slice_sync<NT>();                             // the reads of H are over
             const float scale = 1.0f / trace[0];

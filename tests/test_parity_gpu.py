@@ -911,11 +911,12 @@ def test_project_m128_sampled_slices(P):
 
 
 @pytest.mark.parametrize("m,dtype", [(16, "f32"), (32, "f32"), (64, "f32"), (128, "f32"), (16, "bf16"), (64, "bf16")])
-@pytest.mark.parametrize("kind", ["planted", "gauss", "near", "equal", "zero"])
+@pytest.mark.parametrize("kind", ["planted", "gauss", "near", "equal", "zero", "lengths", "tie", "rank1"])
 def test_project_leading_pair(P, m, dtype, kind):
     """The projection without a rotation count (power iteration, then repeated squaring where the gap is small): every
     slice's residual is the discarded spectrum to fp32 (bf16: rounding of both factors, 2 * 2^-9 of the slice) -
-    independent of the gap, from a clear one (planted) through sigma_2 = 0.999 sigma_1 (near) to none (equal)."""
+    independent of the gap, from a clear one (planted) through sigma_2 = 0.999 sigma_1 (near) to none (equal, tie); with
+    orthogonal columns of different lengths, and of matrices that are Monarch already (rank1)."""
     import torch
     n, rng = m * m, np.random.default_rng(760 + m)
     if kind in ("near", "equal"):
@@ -923,6 +924,14 @@ def test_project_leading_pair(P, m, dtype, kind):
         A4[np.arange(m), :, :, np.arange(m)] = 1.0                     # every slice the identity
         if kind == "near":
             A4[m // 2, :, :, m // 2] = 1.001 if dtype == "f32" else 1.0078125
+    elif kind in ("lengths", "tie"):                                   # signed permutations with scaled columns, no two slices alike
+        A4 = np.zeros((m, m, m, m), np.float32)
+        for j in range(m):
+            for k in range(m):
+                scale = 1.0 + 0.125 * rng.integers(0, 5, m) if kind == "lengths" else np.where(np.arange(m) < 2, 1.0, 0.25)
+                A4[rng.permutation(m), j, k, rng.permutation(m)] = scale * rng.choice([-1.0, 1.0], m)
+    elif kind == "rank1":
+        A4 = np.einsum("jlk,kji->ljki", rng.standard_normal((m, m, m)), rng.standard_normal((m, m, m))).astype(np.float32)
     else:
         A4 = rng.standard_normal((m, m, m, m), dtype=np.float32) * np.float32({"planted": 0.5, "gauss": 1.0, "zero": 0.0}[kind])
         if kind == "planted":
