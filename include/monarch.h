@@ -277,7 +277,8 @@ int monarch_last_device_status(void *workspace, void *stream);
  * one operand load of its last step (item = tile * 128 + output row block; -1 cancels), so the
  * thread block that owns the item waits for data that never arrives, gives up after the wait
  * limit, records MONARCH_ERR_TIMEOUT in the status word and returns; its outputs are undefined.
- * Nothing faults and no wait is unbounded. */
+ * An item of 2^40 + k, k = 0, 1 or 2, is the k-th tile that the first thread block loads in the next
+ * bf16 call on the m = 32 or m = 64 kernels.  Nothing faults and no wait is unbounded. */
 int monarch_debug_set_wait_limit(void *workspace, unsigned int microseconds, void *stream);
 int monarch_debug_skip_load(int64_t item);
 

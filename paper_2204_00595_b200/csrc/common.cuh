@@ -195,6 +195,8 @@ int chain_bwd_m128(const void *x, const void *dy, const void *L, const void *R, 
 const void *chain_fwd_m128_saved_u(const void *fwd_ws, int64_t tokens);
 // test aid: the next plane-transpose launch (last step of the m = 128 forward) leaves out the load of this item
 void debug_skip_next_plane_load(long long item);
+// test aid: the item that the first launch of the next m = 32 or m = 64 call leaves out, once; -1: none
+int take_skipped_tile();
 // true when the next forward call has to run as three launches: the switch for comparison runs, or a load to leave out
 bool chain_fwd_m128_split();
 

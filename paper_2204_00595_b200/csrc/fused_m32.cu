@@ -128,14 +128,17 @@ struct Params {
     const __nv_bfloat16 *L, *R, *bias;
     float *parts;                // backward: [kDL, kDR][ranks][32][32][32]
     int tiles, gelu, ranks;
+    int skip;                    // test aid: one of CTA 0's first tiles, never loaded; -1: none
+    __device__ __forceinline__ bool skips(int item) const { return blockIdx.x == 0 && item == skip; }
     int first[kKinds + 1];       // backward: CTAs of a kind start here
 };
 
-// Ring of T tiles filled by one thread
+// Ring of T tiles filled by one thread, which waits for every tile like the others
 struct Ring {
     uint32_t base, bars;
     unsigned *status;
     volatile int *dead;
+    int loads;                                           // tiles to load: none any more once a wait of this thread has run out
     __device__ __forceinline__ uint32_t slot(int item) const { return base + (item % kSlots) * kTile; }
     __device__ __forceinline__ void load(int item, const CUtensorMap *m, int tile) const
     {
@@ -143,11 +146,12 @@ struct Ring {
         mbar_expect_tx(bar, kTile);
         tma_load_3d(slot(item), m, 0, tile * kTok, 0, bar);
     }
-    // a wait that runs out leaves `dead` set and garbage in the tile; the loops still run to their end, every later wait
-    // returns at once
-    __device__ __forceinline__ uint32_t wait(int item) const
+    // A wait that runs out leaves `dead` set and garbage in the tile; the loops still run to their end, every later wait returns at
+    // once.  The slot may be asked for again although its copy is still under way, and arming a barrier in the middle of its phase
+    // is undefined: nothing is loaded any more.
+    __device__ __forceinline__ uint32_t wait(int item)
     {
-        mbar_wait(bars + (item % kSlots) * 8, (item / kSlots) & 1, status, dead, kErrTmaWait);
+        if (!mbar_wait(bars + (item % kSlots) * 8, (item / kSlots) & 1, status, dead, kErrTmaWait)) loads = 0;
         return slot(item);
     }
 };
@@ -176,15 +180,17 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const Ring ring = {base, smem_u32(sh.bars), p.status, &sh.dead};
+    Ring ring = {base, smem_u32(sh.bars), p.status, &sh.dead, 0};
     const uint32_t E[2] = {base + kSlots * kTile, base + (kSlots + 1) * kTile};
     init(sh);
     const int first = blockIdx.x, step = gridDim.x, count = (p.tiles - first + step - 1) / step;
+    ring.loads = count;
     const int warp = threadIdx.x >> 5;
     Weights wr, wl;
     depend_wait();
     if (threadIdx.x == 0)
-        for (int i = 0; i < 3 && i < count; ++i) ring.load(i, &tm_x, first + i * step);
+        for (int i = 0; i < 3 && i < count; ++i)
+            if (!p.skips(i)) ring.load(i, &tm_x, first + i * step);
     wr.load(p.R, warp, false);
     wl.load(p.L, warp, false);
     float bias[2][4];
@@ -205,7 +211,7 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
                 tma_store_3d(&tm_y, ring.slot(i - 1), 0, (first + (i - 1) * step) * kTok, 0);
                 tma_store_commit();
             }
-            if (i + 3 < count) {
+            if (i + 3 < ring.loads) {
                 tma_store_wait_read<1>();                // y(i - 2) has left its slot
                 ring.load(i + 3, &tm_x, first + (i + 3) * step);
             }
@@ -240,6 +246,7 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         tma_store_commit();
         tma_store_wait_all<0>();
     }
+    let_copies_land(&sh.dead);
 }
 
 // ---------------------------------------------------------------- backward
@@ -298,11 +305,12 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const Ring ring = {base, smem_u32(sh.bars), p.status, &sh.dead};
+    Ring ring = {base, smem_u32(sh.bars), p.status, &sh.dead, 0};
     const uint32_t V = base + kSlots * kTile, U = V + kTile;
     init(sh);
     const int b = blockIdx.x, kind = b < p.first[1] ? kDL : b < p.first[2] ? kDR : kDX;
     const int first = b - p.first[kind], step = p.first[kind + 1] - p.first[kind], count = (p.tiles - first + step - 1) / step;
+    ring.loads = kind == kDX ? count : 2 * count;
     const int warp = threadIdx.x >> 5;
 
     if (kind == kDX) {
@@ -310,7 +318,8 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         Weights wl, wr;
         depend_wait();
         if (threadIdx.x == 0)
-            for (int i = 0; i < 3 && i < count; ++i) ring.load(i, &tm_dy, first + i * step);
+            for (int i = 0; i < 3 && i < count; ++i)
+                if (!p.skips(i)) ring.load(i, &tm_dy, first + i * step);
         wl.load(p.L, warp, true);
         wr.load(p.R, warp, true);
         const Lane ln;
@@ -323,7 +332,7 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
                     tma_store_3d(&tm_dx, ring.slot(i - 1), 0, (first + (i - 1) * step) * kTok, 0);
                     tma_store_commit();
                 }
-                if (i + 3 < count) {
+                if (i + 3 < ring.loads) {
                     tma_store_wait_read<1>();
                     ring.load(i + 3, &tm_dy, first + (i + 3) * step);
                 }
@@ -349,12 +358,14 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
             tma_store_commit();
             tma_store_wait_all<0>();
         }
+        let_copies_land(&sh.dead);
         return;
     }
     // items of the ring: dy(i) = 2 i, x(i) = 2 i + 1
     int next = 0;
     auto load_to = [&](int last) {
-        for (; next <= last && next < 2 * count; ++next) ring.load(next, next & 1 ? &tm_x : &tm_dy, first + (next >> 1) * step);
+        for (; next <= last && next < ring.loads; ++next)
+            if (!p.skips(next)) ring.load(next, next & 1 ? &tm_x : &tm_dy, first + (next >> 1) * step);
     };
     Weights w;
     Operands in;
@@ -395,6 +406,7 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         }
     }
     sums.store(p.parts + ((size_t)kind * p.ranks + first) * kM * kM * kM);
+    let_copies_land(&sh.dead);
 }
 
 // grads = (accumulate ? grads : 0) + the parts, in order; 32 groups of 4 elements and 8 ranges of parts per CTA
@@ -452,6 +464,7 @@ int launch_fwd_m32(const void *x, const void *L, const void *R, const void *bias
     MONARCH_TRY(current_device_sms(&sms));
     auto kern = bias != nullptr ? fused_fwd_m32_kernel<true> : fused_fwd_m32_kernel<false>;
     Params p = {};
+    p.skip = take_skipped_tile();
     p.status = (unsigned *)ws;
     p.L = (const __nv_bfloat16 *)L;
     p.R = (const __nv_bfloat16 *)R;
@@ -509,6 +522,7 @@ int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, v
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
     Params p = {};
+    p.skip = take_skipped_tile();
     p.status = (unsigned *)ws;
     p.L = (const __nv_bfloat16 *)L;
     p.R = (const __nv_bfloat16 *)R;

@@ -63,6 +63,14 @@ struct Lane {                                            // rows of the four mat
     __device__ __forceinline__ Lane() : warp(threadIdx.x >> 5), m((threadIdx.x & 31) >> 3), r(threadIdx.x & 7) {}
 };
 
+// After a wait that ran out: no copy into this CTA's shared memory may outlive the CTA.  Nothing is loaded any more (Ring::load),
+// and what is under way lands within a millisecond.
+__device__ __forceinline__ void let_copies_land(volatile int *dead)
+{
+    if (*dead)
+        for (int i = 0; i < 4096; ++i) __nanosleep(256);
+}
+
 // Launched with programmatic serialization: a kernel may begin while the one before it drains; nothing is read or written
 // before the wait.
 __device__ __forceinline__ void depend_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

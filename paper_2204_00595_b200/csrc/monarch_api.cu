@@ -10,6 +10,9 @@ static std::atomic<uint64_t> g_launches{0};
 static std::atomic<int> g_impl{MONARCH_IMPL_AUTO};
 static std::atomic<int> g_fixed_order{0};     // monarch_set_deterministic
 
+static std::atomic<int> g_skip_tile{-1};      // monarch_debug_skip_load
+int take_skipped_tile() { return g_skip_tile.load(std::memory_order_relaxed) < 0 ? -1 : g_skip_tile.exchange(-1); }
+
 void note_launch(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order_relaxed); }
 
 int current_device_sms(int *sms)
@@ -632,7 +635,9 @@ int monarch_debug_set_wait_limit(void *workspace, unsigned int microseconds, voi
 
 int monarch_debug_skip_load(int64_t item)
 {
-    debug_skip_next_plane_load(item);
+    constexpr int64_t kTiles = (int64_t)1 << 40;
+    g_skip_tile.store(item >= kTiles && item < kTiles + (1 << 30) ? (int)(item - kTiles) : -1);
+    debug_skip_next_plane_load(item >= kTiles ? -1 : item);
     return MONARCH_OK;
 }
 

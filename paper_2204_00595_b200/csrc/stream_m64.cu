@@ -50,6 +50,8 @@ struct Params {
     float *parts;                // [rank][64][64][64]
     int tiles, gelu;
     int last;                    // tiles - 1: from the last tile to the first; 0: from the first to the last
+    int skip;                    // test aid: one of CTA 0's first tiles, never loaded; -1: none
+    __device__ __forceinline__ bool skips(int item) const { return blockIdx.x == 0 && item == skip; }
 };
 
 // Rows r0 .. r0 + 16 MT of one block, as operand A, from its 64 rows of 128 bytes in shared memory
@@ -80,6 +82,7 @@ struct Ring {
     int slots, bytes;
     unsigned *status;
     volatile int *dead;
+    int loads;                   // items to load: none any more once a wait of this thread has run out
     __device__ __forceinline__ uint32_t slot(int item) const { return base + (item % slots) * bytes; }
     __device__ __forceinline__ uint32_t expect(int item) const
     {
@@ -95,11 +98,12 @@ struct Ring {
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(slot(item)), "l"(from),
                      "r"(bytes), "r"(expect(item)) : "memory");
     }
-    // a wait that runs out leaves `dead` set and garbage in the tile; the loops still run to their end, every later wait
-    // returns at once
-    __device__ __forceinline__ uint32_t wait(int item) const
+    // A wait that runs out leaves `dead` set and garbage in the tile; the loops still run to their end, every later wait returns at
+    // once.  The slot may be asked for again although its copy is still under way, and arming a barrier in the middle of its phase
+    // is undefined: the thread loads nothing more (one whose own wait succeeded may: that phase is complete).
+    __device__ __forceinline__ uint32_t wait(int item)
     {
-        mbar_wait(bars + (item % slots) * 8, (item / slots) & 1, status, dead, kErrTmaWait);
+        if (!mbar_wait(bars + (item % slots) * 8, (item / slots) & 1, status, dead, kErrTmaWait)) loads = 0;
         return slot(item);
     }
 };
@@ -186,12 +190,7 @@ struct Sync {
         w.load(block, r0, trans);
         arrive(s.w_read);
     }
-    // after a wait that ran out: copies that are still under way land before the CTA leaves
-    __device__ __forceinline__ void leave() const
-    {
-        if (*(volatile int *)&s.dead)
-            for (int i = 0; i < 4096; ++i) __nanosleep(256);
-    }
+    __device__ __forceinline__ void leave() const { let_copies_land(&s.dead); }
 };
 __device__ __forceinline__ void init(Shared &s)
 {
@@ -220,20 +219,22 @@ stage1_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
-    const Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead};
+    Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, kFwdStages, kFwdSlots};
     init(sh);
     const int group = blockIdx.x % kFwdGroups, first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    ring.loads = count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     const Lane ln;
     auto load = [&](int i) {
-        if (i < count) ring.load(i, &tm_x, tile(i), group * kFwdBlocks);
+        if (i < ring.loads) ring.load(i, &tm_x, tile(i), group * kFwdBlocks);
     };
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
         sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
-        for (int i = 0; i < kFwdSlots - 1; ++i) load(i);
+        for (int i = 0; i < kFwdSlots - 1; ++i)
+            if (!p.skips(i)) load(i);
     }
     auto send = [&](int i) {
         tma_store_2d(&tm_u, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks * 8, tile(i) * (2 * kM));
@@ -288,15 +289,16 @@ stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
-    const Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead};
+    Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, kFwdStages, kFwdSlots};
     init(sh);
     const int group = blockIdx.x % kFwdGroups, first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    ring.loads = count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     const Lane ln;
     auto load = [&](int i) {
-        if (i < count) ring.load_linear(i, p.e_in + ((size_t)tile(i) * kM + group * kFwdBlocks) * kBlockBytes);
+        if (i < ring.loads) ring.load_linear(i, p.e_in + ((size_t)tile(i) * kM + group * kFwdBlocks) * kBlockBytes);
     };
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
@@ -415,16 +417,17 @@ bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     __shared__ Shared sh;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, V0 = base + kDuSlots * kBwdTile, stage0 = V0 + 3 * kBwdTile;
     const uint32_t weights = base + 10 * kBwdTile;
-    const Ring ring = {base, smem_u32(sh.full), kDuSlots, kBwdTile, p.status, &sh.dead};
+    Ring ring = {base, smem_u32(sh.full), kDuSlots, kBwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, kDuStages, 3};
     init(sh);
     const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    ring.loads = (DW ? 2 : 1) * count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     constexpr int kItems = DW ? 2 : 1;                       // per tile: dy, u
     const Lane ln;
     auto load = [&](int from, int to) {
-        for (int i = from; i <= to && i < kItems * count; ++i) {
+        for (int i = from; i <= to && i < ring.loads; ++i) {
             const int t = tile(i / kItems);
             if (DW && (i & 1)) ring.load_linear(i, p.u + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
             else               ring.load(i, &tm_dy, t, 0, group * kBwdBlocks);
@@ -433,7 +436,8 @@ bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
         sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks);
-        load(0, kDuSlots - 1);
+        for (int i = 0; i < kDuSlots; ++i)
+            if (!p.skips(i)) load(i, i);
     }
     auto send = [&](int i) {
         tma_store_2d(&tm_du, stage0 + i % kDuStages * kBwdTile, group * kBwdBlocks * 8, tile(i) * (2 * kM));
@@ -501,16 +505,17 @@ bwd_dx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kDxSlots * kBwdTile;
-    const Ring ring = {base, smem_u32(sh.full), kDxSlots, kBwdTile, p.status, &sh.dead};
+    Ring ring = {base, smem_u32(sh.full), kDxSlots, kBwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, DX ? kDxStages : kMaxStages, 1};   // without staging, warps are up to five tiles apart
     init(sh);
     const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    ring.loads = (DW ? 2 : 1) * count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     constexpr int kItems = DW ? 2 : 1;                       // per tile: du, x
     const Lane ln;
     auto load = [&](int from, int to) {
-        for (int i = from; i <= to && i < kItems * count; ++i) {
+        for (int i = from; i <= to && i < ring.loads; ++i) {
             const int t = tile(i / kItems);
             if (DW && (i & 1)) ring.load(i, &tm_x, t, group * kBwdBlocks);
             else               ring.load_linear(i, p.e_in + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
@@ -608,16 +613,17 @@ cplx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CU
     constexpr int kPair = 2 * kBwdTile, kTiles = PERM ? 3 : 4, kStages = PERM ? 2 : 3;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, V0 = base + kTiles * kPair, stage0 = V0 + (PERM ? 2 * kPair : 0);
     const uint32_t weights = base + 3 * kPair;
-    const Ring ring = {base, smem_u32(sh.full), 2 * kTiles, kBwdTile, p.status, &sh.dead};
+    Ring ring = {base, smem_u32(sh.full), 2 * kTiles, kBwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, kStages, 2};
     init(sh);
     const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    ring.loads = 2 * count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     const Lane ln;
     const int blk = ln.warp >> 1, half = ln.warp & 1;
     auto load = [&](int i) {
-        if (i >= count) return;
+        if (2 * i >= ring.loads) return;
         const int t = tile(i);
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
@@ -629,7 +635,8 @@ cplx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CU
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
         sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks, 2);
-        for (int i = 0; i < 3; ++i) load(i);
+        for (int i = 0; i < 3; ++i)
+            if (!p.skips(i)) load(i);
     }
     Weights<2> wr, wi;
     sync.wait(sh.w_full, 0, kErrTmaWait);
@@ -786,6 +793,7 @@ int stage1(const void *x, const void *R, char *u, int64_t tokens, int sms, unsig
     MONARCH_TRY(map_t(&tm_x, x, tokens, kFwdBlocks));
     MONARCH_TRY(map_e(&tm_u, u, (int)tiles_of(tokens), kFwdBlocks));
     Params p = {};
+    p.skip = take_skipped_tile();
     p.status = status;
     p.tiles = (int)tiles_of(tokens);
     return launch_serialized(stage1_kernel, grid_of(kFwdGroups, sms, tokens), kThreads, kFwdSmem, s, tm_w, tm_x, tm_u, p);
@@ -807,6 +815,7 @@ static int stream_fwd(const void *x, const void *L, const void *R, const void *b
     MONARCH_TRY(map_w(&tm_w, L));
     MONARCH_TRY(map_y(&tm_y, y, tokens, kFwdBlocks));
     Params p = {};
+    p.skip = -1;
     p.status = status;
     p.bias = (const __nv_bfloat16 *)bias;
     p.gelu = gelu;
@@ -844,11 +853,13 @@ static int stream_bwd(const void *x, const void *dy, const void *L, const void *
     MONARCH_TRY(map_t(&tm_x, dL != nullptr ? x : dy, tokens, kBwdBlocks));
     MONARCH_TRY(map_t(&tm_dx, dx != nullptr ? dx : dy, tokens, kBwdBlocks));
     Params p = {};
+    p.skip = take_skipped_tile();
     p.status = status;
     p.u = (const char *)u;
     p.parts = parts_l;
     p.tiles = tiles;
     MONARCH_TRY(launch_serialized(dL != nullptr ? bwd_du_kernel<true> : bwd_du_kernel<false>, grid, kThreads, kBwdSmem, s, tm_L, tm_dy, tm_du, p));
+    p.skip = -1;
     p.e_in = (const char *)du;
     p.parts = parts_r;
     p.last = tiles - 1;
@@ -877,10 +888,12 @@ static int stream_cplx(const void *x, const void *L, const void *R, void *y, int
         MONARCH_TRY(adjoint ? map_t(&tm_y[c], yc, tokens, kBwdBlocks) : map_y(&tm_y[c], yc, tokens, kBwdBlocks));
     }
     Params p = {};
+    p.skip = take_skipped_tile();
     p.status = status;
     p.e_in = (const char *)e;
     p.tiles = tiles;
     MONARCH_TRY(launch_serialized(adjoint ? cplx_kernel<true, true> : cplx_kernel<true, false>, grid, kThreads, kBwdSmem, s, tm_w[0], tm_e, tm_x[0], tm_x[1], p));
+    p.skip = -1;
     p.last = tiles - 1;
     return launch_serialized(adjoint ? cplx_kernel<false, false> : cplx_kernel<false, true>, grid, kThreads, kBwdSmem, s, tm_w[1], tm_e, tm_y[0], tm_y[1], p);
 }

@@ -1279,6 +1279,56 @@ def test_bounded_wait_runs_out_and_the_workspace_recovers(P):
     assert_close(to_host64(y), O.fwd(d["x"], d["L"], d["R"]), dtype, "y after recovery")
 
 
+@pytest.mark.parametrize("item", [0, 2])
+@pytest.mark.parametrize("call", ["fwd", "bwd", "bwd_dx", "cplx", "cplx adjoint", "mlp"])
+@pytest.mark.parametrize("m,T", [(32, 16 * 148 * 8), (64, 16 * 37 * 8)])
+def test_tile_that_never_arrives(P, m, T, call, item):
+    """m = 32 and m = 64: a thread block whose tile is left out gives up after its 2 ms, loads nothing more (its slots' barriers may
+    be in the middle of a phase), lets the copies under way land and returns; the call reports the time-out, and after
+    monarch_workspace_init the same workspace gives the same bits as before."""
+    import time
+    import torch
+    if call.startswith("cplx") and m == 32:
+        pytest.skip("four real calls")
+    n, code = m * m, P.BF16
+    gen = torch.Generator("cuda").manual_seed(m + item)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").mul_(m ** -0.5 if shape[-1] == m else 1.0).bfloat16()
+    planes = (2,) if call.startswith("cplx") else ()
+    if planes:
+        T //= 2
+    x, dy, L, R, b1 = draw(*planes, T, n), draw(T, n), draw(*planes, m, m, m), draw(*planes, m, m, m), draw(n)
+    y, dL, dR = torch.empty_like(x), torch.empty(m, m, m, device="cuda"), torch.empty(m, m, m, device="cuda")
+    op = {"fwd": P.OP_FWD, "bwd": P.OP_BWD, "bwd_dx": P.OP_BWD_DX, "mlp": P.OP_MLP_FWD}.get(call, P.OP_CPLX)
+    ws = P.Workspace(P.monarch_workspace_bytes(op, T, n, m, code))
+
+    def run():
+        if call == "fwd":
+            P.monarch_fwd(x, L, R, y, T, n, m, ws)
+        elif call == "bwd":
+            P.monarch_bwd(x, dy, L, R, y, dL, dR, 0, T, n, m, ws)
+        elif call == "bwd_dx":
+            P.monarch_bwd_dx(dy, L, R, y, T, n, m, ws)
+        elif call == "mlp":
+            P.monarch_mlp_fwd(x, L, R, b1, L, R, b1, y, T, n, m, ws)
+        else:
+            P.monarch_cplx_fwd(x, L, R, y, int(call == "cplx adjoint"), T, n, m, ws)
+        torch.cuda.synchronize()
+        return [t.clone() for t in ((y, dL, dR) if call == "bwd" else (y,))]
+
+    want = run()
+    assert P.monarch_last_device_status(ws) == 0
+    P.monarch_debug_set_wait_limit(ws, 2000)
+    P.monarch_debug_skip_load((1 << 40) + item)
+    t0 = time.perf_counter()
+    run()
+    assert time.perf_counter() - t0 < 5.0
+    assert P.monarch_last_device_status(ws) == 5   # MONARCH_ERR_TIMEOUT
+    P.monarch_workspace_init(ws)
+    y.fill_(float("nan"))
+    assert all(torch.equal(a, b) for a, b in zip(run(), want))
+    assert P.monarch_last_device_status(ws) == 0
+
+
 # ----------------------------------------------------------------- the m = 64 forward on clusters of four CTAs
 
 @pytest.mark.parametrize("T", [1, 63, 130, 257, 2500])
