@@ -214,7 +214,7 @@ KERNELS_OF = {
     (64, "bf16", "bwd_dx"): "bwd_du_kernel + bwd_dx_kernel (2 launches)",
     (64, "bf16", "bwd_dw"): "stage1_kernel + bwd_du_kernel + bwd_dx_kernel without dx + add_parts_m64_kernel (4 launches)",
     (64, "bf16", "mlp_fwd"): "2 x (stage1_kernel + stage2_kernel) (4 launches)",
-    (64, "bf16", "mlp_bwd"): "2 x forward + mlp_act_kernel + stage1_kernel + 2 x backward + mlp_dact_kernel + merge_status_kernel",
+    (64, "bf16", "mlp_bwd"): "stage1_kernel + stage2_kernel + mlp_act_kernel + stage1_kernel + 2 x (bwd_du_kernel + bwd_dx_kernel + add_parts_m64_kernel) + mlp_dact_kernel (11 launches)",
     (128, "bf16", "fwd"): "chain_fused_fwd_kernel (1 persistent launch; chain_gemm_kernel x 2 + plane_transpose_kernel "
                           "beyond 8192 tiles)",
     (128, "bf16", "bwd"): "plane_transpose_kernel + chain_gemm_kernel x 2 with the token reductions (3 launches)",
@@ -385,7 +385,7 @@ def main_rect(args):
                                                   + ("relabel_kernel + " if wrapped else "") +
                                                   "rect_stage2_stream_kernel (%d launches)" % (3 if wrapped else 2)
                                                   + ("; rect_bwd: stage 1, adjoint stage 2, adjoint stage 1 (tcgen05), "
-                                                     "rect_wgrad_kernel (tcgen05), dl_small4_kernel" if with_bwd else ""),
+                                                     "rect_wgrad_pair_kernel (tcgen05), rect_bwd_stream_kernel" if with_bwd else ""),
                      "achieved": tfl, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
                      "frac": tfl / peaks["bf16_tflops"], "peak_source": peaks["source"], "traffic": None,
                      "algorithmic_mb": nbytes / 1e6,
@@ -488,7 +488,7 @@ def main_project(args):
         "calls": {"project": {"ms": t_proj, "rotations": int(rot.item()) // args.steps,
                               "tflops": flops / t_proj / 1e9},
                   "dense": {"ms": t_dense, "gbs": n * n * 4 / t_dense / 1e6}},
-        "roofline": {"bound": "alu", "kernel": "project_kernel<float, 64>", "achieved": flops / t_proj / 1e9,
+        "roofline": {"bound": "alu", "kernel": "jacobi_kernel<float, 64>", "achieved": flops / t_proj / 1e9,
                      "peak": alu_peak, "unit": "TFLOP/s", "frac": flops / t_proj / 1e9 / alu_peak,
                      "peak_source": "148 SMs x 128 fp32 FMA lanes x 2 FLOP x max SM clock", "traffic": None},
         "e2e": None,

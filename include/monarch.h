@@ -72,9 +72,9 @@ typedef enum {
 
 /* Which kernel family serves a call (process-wide; default AUTO). */
 typedef enum {
-    MONARCH_IMPL_AUTO = 0,   /* fused tensor-core kernels where built, else staged */
+    MONARCH_IMPL_AUTO = 0,   /* the fastest for the size */
     MONARCH_IMPL_STAGED = 1, /* one block-diagonal stage per launch, CUDA-core FMA, any m */
-    MONARCH_IMPL_FUSED = 2   /* fused tcgen05 kernels only; UNSUPPORTED where none exists */
+    MONARCH_IMPL_FUSED = 2   /* bf16 m = 64 and the m = 32 forward only; UNSUPPORTED elsewhere */
 } monarch_impl_t;
 
 #define MONARCH_STATUS_BYTES 256
@@ -223,10 +223,12 @@ size_t monarch_rectw_bwd_workspace_bytes(int64_t tokens, int32_t q, int32_t b1, 
  * M = P L P^T R with complex blocks, M^H = R^H P L^H P.  An MM* product
  * M1 M2^H x is two calls.  Complex tensors are PLANAR in the storage dtype:
  * x, y: [2][tokens][n] (real plane, then imaginary plane); L, R: [2][m][m][m].
- * The call runs four real Monarch multiplies over both planes at once
- * (M(Lr,Rr), M(Li,Ri), M(Lr,Ri), M(Li,Rr) applied to [xr; xi]) and combines
- * them:  Re M = M(Lr,Rr) - M(Li,Ri),  Im M = M(Lr,Ri) + M(Li,Rr); each of the
- * four results is rounded to the storage dtype before the combination.
+ * bf16 with m = 64: the four real products of a stage add up in fp32 and the
+ * intermediate is rounded to bfloat16 once.  Other sizes and fp32: four real
+ * Monarch multiplies over both planes at once (M(Lr,Rr), M(Li,Ri), M(Lr,Ri),
+ * M(Li,Rr) applied to [xr; xi]) are combined,  Re M = M(Lr,Rr) - M(Li,Ri),
+ * Im M = M(Lr,Ri) + M(Li,Rr); each of the four results is rounded to the
+ * storage dtype before the combination.
  * Workspace: monarch_workspace_bytes with MONARCH_OP_CPLX. */
 int monarch_cplx_fwd(const void *x, const void *L, const void *R, void *y, int adjoint,
                      int64_t tokens, int32_t n, int32_t m, int dtype,
@@ -299,8 +301,15 @@ int monarch_set_impl(int impl);
  * calls.  Returns the previous setting. */
 int monarch_set_deterministic(int on);
 
-/* Name of the kernel family the next call with these arguments would use
- * ("staged-simt", "fused-simt", "staged-tcgen05", "fused-tcgen05"; "unsupported").  Static storage. */
+/* Name of the kernel family that a large batch with these arguments would use: a fixed label, which
+ * callers compare, not a list of instructions.  Static storage.
+ *   "staged-simt"    one launch per block-diagonal stage on the CUDA cores
+ *   "units"          the whole call as one launch over block products (fp32 and m = 16 under AUTO)
+ *   "fused-simt"     the m = 16 forward under AUTO
+ *   "fused-tcgen05"  bf16 m = 64, and the m = 32 forward: weights in registers, warp-level MMAs
+ *   "staged-tcgen05" the other bf16 calls of m = 32 (warp-level MMAs) and m = 128 (tcgen05)
+ *   "unsupported"
+ * Small bf16 batches of m >= 32 may run as "units" whatever the label. */
 const char *monarch_impl_name(int op, int32_t m, int dtype);
 
 /* Number of kernel launches the library has enqueued since load (for

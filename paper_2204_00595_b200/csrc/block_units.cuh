@@ -11,7 +11,7 @@
 // What bounds them: at a few tokens the chain of latencies of a phase (barrier, input from L2, product, result: 4 us
 // per phase with the cold instruction fetches), which is why a phase's weights are fetched before its barrier; at many
 // tokens the warps' issue of shared-memory accesses and legacy-shaped MMAs (ncu at 4096 tokens, m = 64: LSU data pipe
-// 52 %, issue 29 %), which is why the tcgen05 kernels take over there.  One CTA of 16 warps with a two-deep pipeline was
+// 52 %, issue 29 %), which is why the kernels with weights in registers and the tcgen05 kernels take over there.  One CTA of 16 warps with a two-deep pipeline was
 // no faster at any size than two CTAs of 8 warps whose loads overlap the other's work (23 against 27 us at 1000 tokens),
 // and starting the permuted loads early cost spills (31 us).
 #pragma once

@@ -196,8 +196,7 @@ size_t large_workspace_bytes(int op, int64_t tokens, int32_t n, int32_t m, int d
     }
     const int which = pick(op, m, dtype);
     if (which < 0) return 0;
-    // the fused m = 64 kernels keep one dependency counter per 64-token tile in 64 KB: beyond 2^20 tokens the calls
-    // refuse, and so does this query (shard the tokens)
+    // a limit that m = 64 calls have always had (shard the tokens): the E tiles of 2^20 tokens are 8 GB
     if (which == kFused && m == 64 && tokens > ((int64_t)1 << 20)) return 0;
     if (which == kTcStaged && m == 32 && op == MONARCH_OP_MLP_FWD) return fused_mlp_fwd_m32_workspace_bytes(tokens);
     if (which == kTcStaged && m == 32 && op != MONARCH_OP_FWD)
@@ -659,9 +658,8 @@ const char *monarch_impl_name(int op, int32_t m, int dtype)
     if (op == MONARCH_OP_MLP_BWD) op = MONARCH_OP_BWD;      // its Monarch passes are monarch_bwd's
     if (op == MONARCH_OP_CPLX) op = MONARCH_OP_FWD;         // m = 64, bf16: kernels of its own; else four real forward (or dx) passes
     const int which = pick(op, m, dtype);
-    if (which == kSimt && op == MONARCH_OP_FWD && m == 16 &&
-        g_impl.load(std::memory_order_relaxed) == MONARCH_IMPL_AUTO)
-        return "fused-simt";
+    if (which == kSimt && g_impl.load(std::memory_order_relaxed) == MONARCH_IMPL_AUTO)
+        return op == MONARCH_OP_FWD && m == 16 ? "fused-simt" : "units";
     return which < 0 ? "unsupported" : which == kFused ? "fused-tcgen05"
          : which == kTcStaged ? "staged-tcgen05" : "staged-simt";
 }

@@ -200,9 +200,8 @@ def test_bwd_m64_fixed_summation_order(P, T):
 
 
 def test_m32_backward_runs_on_the_tensor_cores(P):
-    """bf16 m = 32: dL and dR come from the tcgen05 token-reduction kernel (128-column windows whose diagonal 32 x 32
-    sub-blocks are the blocks' sums), not from the CUDA-core kernel - by name and against the oracle, on a token count
-    with a ragged last tile."""
+    """bf16 m = 32: dL and dR come from the warp-MMA kernels of that size, not from the CUDA-core kernel - by the family's label
+    and against the oracle, on a token count with a ragged last tile."""
     import torch
     m, T, dtype, code = 32, 64 * 9 + 5, "bf16", P.BF16
     n = m * m
@@ -1102,6 +1101,43 @@ def test_one_launch_feed_forward(P, m, T, dtype):
         _check_guard(flat, f"mlp {k}")
 
 
+@pytest.mark.parametrize("m,T,dtype", [(m, T, dtype) for dtype in ("f32", "bf16") for m, T in
+                                       ((16, 1), (16, 257), (32, 1), (32, 17), (32, 72), (64, 1), (64, 16), (64, 24), (64, 64), (128, 1), (128, 16), (128, 24))] +
+                         [(64, 125, "f32"), (64, 500, "f32"), (128, 125, "f32")])
+def test_units_feed_forward(P, m, T, dtype):
+    """The feed-forward block and its gradients as one launch, on as many tokens as that serves (fp32: small tiles and large ones),
+    overwriting and accumulating."""
+    import torch
+    n, code = m * m, _code(P, dtype)
+    d = _small_inputs(m, T, dtype, seed=53 * m + T)
+    t = {k: to_device(d[k], dtype) for k in ("x", "dy", "L", "R", "b1", "L2", "R2", "b2")}
+    yf, y = _guarded((T, n), _tdtype(dtype))
+    ws = P.Workspace(max(P.monarch_workspace_bytes(op, T, n, m, code) for op in (P.OP_MLP_FWD, P.OP_MLP_BWD)))
+    bufs = _mlp_bwd_buffers(m, T, dtype)
+    P.monarch_mlp_fwd(t["x"], t["L"], t["R"], t["b1"], t["L2"], t["R2"], t["b2"], y, T, n, m, ws)
+    ref = O.mlp_bwd(d["x"], d["dy"], d["L"], d["R"], d["b1"], d["L2"], d["R2"])
+    for accumulate in (0, 1):
+        _call_mlp_bwd(P, t, bufs, accumulate, T, n, m, ws)
+        torch.cuda.synchronize()
+        assert P.monarch_last_device_status(ws) == 0
+        assert_close(to_host64(bufs["dx"][1]), ref["dx"], dtype, "mlp dx")
+        _assert_mlp_grads(bufs, ref, dtype, "mlp", factor=1.0 + accumulate)
+    assert_close(to_host64(y), O.mlp_fwd(d["x"], d["L"], d["R"], d["b1"], d["L2"], d["R2"], d["b2"]), dtype, "mlp y")
+    _check_guard(yf, "mlp y")
+    for k, (flat, _) in bufs.items():
+        _check_guard(flat, f"mlp {k}")
+
+
+@pytest.mark.parametrize("m,T", [(32, 2047), (64, 400), (64, 500), (64, 1000), (64, 2047), (128, 125), (128, 257), (128, 400)])
+def test_large_fp32_tiles(P, m, T):
+    """The streamed fp32 tiles of m = 64 and m = 128 (the rule: a unit of 32 tokens x 8 blocks x 64 outputs for every SM, last wave
+    full enough), with part of a last tile: every call of test_one_launch_over_units."""
+    es = 32 if m == 32 else 64
+    units = (m // 8) * (m // es) * -(-T // 32)
+    assert 5 * (units + 20) >= 4 * 148 * -(-units // 148)
+    test_one_launch_over_units(P, m, T, "f32")
+
+
 # ----------------------------------------------------------------- the five workloads
 
 def _sample_tokens(T, count, seed):
@@ -1487,7 +1523,7 @@ def test_bwd_m32_fixed_summation_order(P, T):
 
 @pytest.mark.parametrize("m", [16, 32, 64])
 def test_fp32_weight_gradients_have_the_same_bits_every_run(P, m):
-    """fp32 runs on the CUDA-core family, whose token sums are taken slab by slab and added in slab order: dL and dR
+    """fp32 sums the tokens in fixed ranges, which a last phase adds in order: dL and dR
     from different initial contents (overwrite mode) agree bit for bit, through monarch_bwd and monarch_bwd_dw."""
     import torch
     T, dtype = 333, "f32"
