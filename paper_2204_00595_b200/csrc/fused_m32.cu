@@ -17,8 +17,8 @@
 //   backward:  z = P dy     T tile -> E tile [j][l];   du = L_j^T z_j -> E tile [k][j];   dx = R_k^T du_k -> T tile
 //              dL_j = sum_t z_j u_j^T, dR_k = sum_t du_k x_k^T: tokens are the contraction, both operands as they lie
 // Shared memory moves 16 to 18 KB per token at 128 bytes per clock, no access has a bank conflict.
-// Measured, back to back: forward 16384 tokens 29.2 -> 18.9 us (6.0 TB/s beyond a fixed 7 us of launch, first tile and
-// weights), 1000 tokens 14.5 -> 6.6; forward + backward 4999 tokens 103 -> 31, 16384 tokens 62 (the staged chain of nine
+// Measured, back to back: forward 16384 tokens 29.2 -> 15.6 us (3.4 of it when the weights came to be loaded by TMA), 1000 tokens
+// 14.5 -> 6.6; forward + backward 4999 tokens 103 -> 31, 16384 tokens 62 (the staged chain of nine
 // launches took 219 as units and more as tcgen05 stages); feed-forward block 16384 tokens 167 -> 40.
 //
 // Backward CTAs are of three kinds, dL, dR and dx: the sums of one gradient are 128 KB of accumulators, half the
@@ -41,18 +41,30 @@ constexpr int kMaxParts = 50;                            // CTAs of a kind: a th
 __device__ __forceinline__ uint32_t t_at(uint32_t base, int box, int t, int c) { return base + box * (kTok * 128) + t * 128 + ((c ^ (t & 7)) << 4); }
 __device__ __forceinline__ uint32_t e_at(uint32_t base, int b, int h, int c) { return base + b * 1024 + (((h * 32 + c) ^ (b & 7)) << 4); }
 
+// chunk c of row r of block b of the weights
+__device__ __forceinline__ uint32_t w_at(uint32_t base, int b, int r, int c)
+{
+    const int pair = b * (kM / 2) + (r >> 1);
+    return base + pair * 128 + ((((r & 1) * 4 + c) ^ (pair & 7)) << 4);
+}
+
 // Operand A of a warp's two blocks: rows = outputs, [block][16 rows][16 columns of the contraction]
 struct Weights {
     uint32_t a[2][2][2][4];
-    __device__ __forceinline__ void load(const __nv_bfloat16 *W, int warp, bool trans)
+    // from the 32 blocks in shared memory, two rows of a block in 128 swizzled bytes
+    __device__ __forceinline__ void load(uint32_t W, bool trans)
     {
+        const Lane ln;
 #pragma unroll
         for (int blk = 0; blk < 2; ++blk)
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                for (int ks = 0; ks < 2; ++ks)
-                    load_operand(a[blk][mt][ks], W + (size_t)(warp * 2 + blk) * kM * kM, kM, mt * 16, ks * 16, trans);
+                for (int ks = 0; ks < 2; ++ks) {
+                    const int row = mt * 16 + (ln.m & 1) * 8, col = ks * 16 + (ln.m >> 1) * 8;       // of the 8 x 8 piece
+                    if (trans) ldm4t(a[blk][mt][ks], w_at(W, ln.warp * 2 + blk, col + ln.r, row >> 3));
+                    else       ldm4(a[blk][mt][ks], w_at(W, ln.warp * 2 + blk, row + ln.r, col >> 3));
+                }
     }
     // acc = blk's rows times the operand b (both 16-column steps)
     __device__ __forceinline__ void times(int blk, const uint32_t (&b)[4], float (&acc)[2][4]) const
@@ -125,9 +137,10 @@ __device__ __forceinline__ void t_to_e(uint32_t T, uint32_t E)
 
 struct Params {
     unsigned *status;
-    const __nv_bfloat16 *L, *R, *bias;
+    const __nv_bfloat16 *bias;
     float *parts;                // backward: [kDL, kDR][ranks][32][32][32]
     int tiles, gelu, ranks;
+    int follows;                 // forward: behind another launch of the same call
     int skip;                    // test aid: one of CTA 0's first tiles, never loaded; -1: none
     __device__ __forceinline__ bool skips(int item) const { return blockIdx.x == 0 && item == skip; }
     int first[kKinds + 1];       // backward: CTAs of a kind start here
@@ -157,14 +170,21 @@ struct Ring {
 };
 
 struct Shared {
-    uint64_t bars[kSlots];
+    uint64_t bars[kSlots], w_full;
     int dead;
 };
+constexpr int kWeightBytes = kM * kM * kM * 2;           // of one factor: two tiles
+// The weights of a CTA come by TMA through shared memory that the first tiles do not need yet, and go to registers by ldmatrix.
+// (Fetched by the warps in 4-byte pieces of the operand layout they took 4 us: eight lines per load.)
+__device__ __forceinline__ void load_weights(uint32_t to, const CUtensorMap *m, Shared &s)
+{
+    for (int i = 0; i < 2; ++i) tma_load_2d(to + i * (kWeightBytes / 2), m, 0, i * 256, smem_u32(&s.w_full));
+}
 __device__ __forceinline__ void init(Shared &s)
 {
-    depend_launch();
     if (threadIdx.x == 0) {
         for (int i = 0; i < kSlots; ++i) mbar_init(smem_u32(&s.bars[i]), 1);
+        mbar_init(smem_u32(&s.w_full), 1);
         fence_mbar_init();
         s.dead = 0;
     }
@@ -175,7 +195,8 @@ __device__ __forceinline__ void init(Shared &s)
 // Per tile two barriers: [w(i) from u(i), u(i + 1) from x] [y(i)].  ACT: y = GELU(M x + bias), or without the GELU.
 template <bool ACT>
 __global__ void __launch_bounds__(kThreads, 1)
-fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_y, const Params p)
+fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_L,
+                     const __grid_constant__ CUtensorMap tm_R, const Params p)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
@@ -187,12 +208,21 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     ring.loads = count;
     const int warp = threadIdx.x >> 5;
     Weights wr, wl;
+    auto weights = [&] {
+        mbar_expect_tx(smem_u32(&sh.w_full), 2 * kWeightBytes);
+        load_weights(ring.slot(3), &tm_R, sh);
+        load_weights(E[0], &tm_L, sh);
+    };
+    // The second pass of a feed-forward block asks for its weights before it waits for the first one: that one lets its followers
+    // begin only after its own wait, so what ran before the call has finished.
+    if (p.follows && threadIdx.x == 0) weights();
     depend_wait();
-    if (threadIdx.x == 0)
+    depend_launch();
+    if (threadIdx.x == 0) {
+        if (!p.follows) weights();
         for (int i = 0; i < 3 && i < count; ++i)
             if (!p.skips(i)) ring.load(i, &tm_x, first + i * step);
-    wr.load(p.R, warp, false);
-    wl.load(p.L, warp, false);
+    }
     float bias[2][4];
     if (ACT)
 #pragma unroll
@@ -201,7 +231,11 @@ fused_fwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
 
     const Lane ln;
     Operands in;
+    mbar_wait(smem_u32(&sh.w_full), 0, p.status, &sh.dead, kErrTmaWait);
+    wr.load(ring.slot(3), false);
+    wl.load(E[0], false);
     in.from_t(ring.wait(0));
+    __syncthreads();                                     // every warp has its weights
     stage_to_e(wr, in, E[0]);
     for (int i = 0; i < count; ++i) {
         const uint32_t e = E[i & 1];
@@ -300,7 +334,8 @@ struct Sums {
 
 __global__ void __launch_bounds__(kThreads, 1)
 fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_dy,
-                     const __grid_constant__ CUtensorMap tm_dx, const Params p)
+                     const __grid_constant__ CUtensorMap tm_dx, const __grid_constant__ CUtensorMap tm_L, const __grid_constant__ CUtensorMap tm_R,
+                     const Params p)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ Shared sh;
@@ -317,11 +352,18 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
         // per tile [du(i) from z(i)] [dx(i), z(i + 1)]
         Weights wl, wr;
         depend_wait();
-        if (threadIdx.x == 0)
+        depend_launch();
+        if (threadIdx.x == 0) {
+            mbar_expect_tx(smem_u32(&sh.w_full), 2 * kWeightBytes);
+            load_weights(ring.slot(3), &tm_L, sh);
+            load_weights(V, &tm_R, sh);
             for (int i = 0; i < 3 && i < count; ++i)
                 if (!p.skips(i)) ring.load(i, &tm_dy, first + i * step);
-        wl.load(p.L, warp, true);
-        wr.load(p.R, warp, true);
+        }
+        mbar_wait(smem_u32(&sh.w_full), 0, p.status, &sh.dead, kErrTmaWait);
+        wl.load(ring.slot(3), true);
+        wr.load(V, true);
+        __syncthreads();                                 // every warp has its weights
         const Lane ln;
         Operands in;
         t_to_e(ring.wait(0), V);
@@ -372,9 +414,15 @@ fused_bwd_m32_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_cons
     Sums sums;
     sums.clear();
     depend_wait();
-    if (threadIdx.x == 0) load_to(kSlots - 1);
-    if (kind == kDL) w.load(p.R, warp, false);
-    else             w.load(p.L, warp, true);
+    depend_launch();
+    if (threadIdx.x == 0) {
+        mbar_expect_tx(smem_u32(&sh.w_full), kWeightBytes);
+        load_weights(V, kind == kDL ? &tm_R : &tm_L, sh);
+        load_to(kSlots - 1);
+    }
+    mbar_wait(smem_u32(&sh.w_full), 0, p.status, &sh.dead, kErrTmaWait);
+    w.load(V, kind != kDL);
+    __syncthreads();                                     // every warp has its weights
     if (kind == kDL) {
         // per tile [sums from z(i), u(i)] [z(i + 1), u(i + 1)]
         t_to_e(ring.wait(0), V);
@@ -451,27 +499,31 @@ int map_tile(CUtensorMap *m, const void *p, int64_t tokens)
     return encode_tmap_nd(m, p, 2, 3, dims, strides, box, 128);
 }
 
+// the blocks of a factor as rows of 128 bytes
+int map_weights(CUtensorMap *m, const void *W) { return encode_tmap_2d(m, W, kM * kM * kM / 64, 64, 128, 256, 64, 128); }
+
 // bias null: y = M x
 int launch_fwd_m32(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws,
-                   cudaStream_t s)
+                   int follows, cudaStream_t s)
 {
     if (tokens == 0) return MONARCH_OK;
     if (tokens > 0x7fffffffLL - kTok) return MONARCH_ERR_UNSUPPORTED;
-    CUtensorMap tm_x, tm_y;
+    CUtensorMap tm_x, tm_y, tm_L, tm_R;
     MONARCH_TRY(map_tile(&tm_x, x, tokens));
     MONARCH_TRY(map_tile(&tm_y, y, tokens));
+    MONARCH_TRY(map_weights(&tm_L, L));
+    MONARCH_TRY(map_weights(&tm_R, R));
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
     auto kern = bias != nullptr ? fused_fwd_m32_kernel<true> : fused_fwd_m32_kernel<false>;
     Params p = {};
     p.skip = take_skipped_tile();
     p.status = (unsigned *)ws;
-    p.L = (const __nv_bfloat16 *)L;
-    p.R = (const __nv_bfloat16 *)R;
     p.bias = (const __nv_bfloat16 *)bias;
     p.gelu = gelu;
+    p.follows = follows;
     p.tiles = (int)((tokens + kTok - 1) / kTok);
-    return launch_serialized(kern, p.tiles < sms ? p.tiles : sms, kThreads, kSmemBytes, s, tm_x, tm_y, p);
+    return launch_serialized(kern, p.tiles < sms ? p.tiles : sms, kThreads, kSmemBytes, s, tm_x, tm_y, tm_L, tm_R, p);
 }
 
 }  // namespace
@@ -480,7 +532,7 @@ int launch_fwd_m32(const void *x, const void *L, const void *R, const void *bias
 // Workspace: only the status word is used.
 int fused_fwd_m32(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s)
 {
-    return tc::launch_fwd_m32(x, L, R, nullptr, 0, y, tokens, ws, s);
+    return tc::launch_fwd_m32(x, L, R, nullptr, 0, y, tokens, ws, 0, s);
 }
 
 // The feed-forward block as two passes; workspace: status word, then h.
@@ -492,8 +544,8 @@ int fused_mlp_fwd_m32(const void *x, const void *L1, const void *R1, const void 
                       void *y, int64_t tokens, void *ws, cudaStream_t s)
 {
     void *h = (char *)ws + MONARCH_STATUS_BYTES;
-    MONARCH_TRY(tc::launch_fwd_m32(x, L1, R1, b1, 1, h, tokens, ws, s));
-    return tc::launch_fwd_m32(h, L2, R2, b2, 0, y, tokens, ws, s);
+    MONARCH_TRY(tc::launch_fwd_m32(x, L1, R1, b1, 1, h, tokens, ws, 0, s));
+    return tc::launch_fwd_m32(h, L2, R2, b2, 0, y, tokens, ws, 1, s);
 }
 
 // Workspace: status word, then the sums of every CTA (64 KB are left out for the counters of the kernels that share it).
@@ -515,7 +567,9 @@ int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, v
         return MONARCH_OK;
     }
     if (tokens > 0x7fffffffLL - kTok) return MONARCH_ERR_UNSUPPORTED;
-    CUtensorMap tm_x, tm_dy, tm_dx;
+    CUtensorMap tm_x, tm_dy, tm_dx, tm_L, tm_R;
+    MONARCH_TRY(map_weights(&tm_L, L));
+    MONARCH_TRY(map_weights(&tm_R, R));
     MONARCH_TRY(map_tile(&tm_dy, dy, tokens));
     MONARCH_TRY(map_tile(&tm_x, dL != nullptr ? x : dy, tokens));
     MONARCH_TRY(map_tile(&tm_dx, dx != nullptr ? dx : dy, tokens));
@@ -524,8 +578,6 @@ int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, v
     Params p = {};
     p.skip = take_skipped_tile();
     p.status = (unsigned *)ws;
-    p.L = (const __nv_bfloat16 *)L;
-    p.R = (const __nv_bfloat16 *)R;
     p.parts = (float *)((char *)ws + MONARCH_STATUS_BYTES + 65536);
     p.tiles = (int)((tokens + kTok - 1) / kTok);
     // The kinds cost the same per tile (256 KB of shared-memory traffic): equal shares, and the same share of a gradient
@@ -538,7 +590,7 @@ int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, v
         p.first[k + 1] = p.first[k] + n[k];
     }
     p.ranks = n[kDL];
-    MONARCH_TRY(launch_serialized(fused_bwd_m32_kernel, p.first[kKinds], kThreads, kSmemBytes, s, tm_x, tm_dy, tm_dx, p));
+    MONARCH_TRY(launch_serialized(fused_bwd_m32_kernel, p.first[kKinds], kThreads, kSmemBytes, s, tm_x, tm_dy, tm_dx, tm_L, tm_R, p));
     if (dL == nullptr) return MONARCH_OK;
     return launch_serialized(add_parts_m32_kernel, 2 * kM * kM * kM / 128, 256, 0, s, (const float *)p.parts, dL, dR, p.ranks, accumulate);
 }

@@ -43,21 +43,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *m, uint32_t src,
     asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(m), "r"(src), "r"(x), "r"(y), "r"(z) : "memory");
 }
 
-// A operand of mma for 16 rows x 16 columns of a row-major m x m block at (row, col); trans: of the transposed block (8 x 8
-// pieces transposed in registers)
-__device__ __forceinline__ void load_operand(uint32_t (&a)[4], const __nv_bfloat16 *block, int m, int row, int col, bool trans)
-{
-    const int g = (threadIdx.x & 31) >> 2, q = threadIdx.x & 3;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int pr = row + (r & 1) * 8, pc = col + (r >> 1) * 8;       // of the 8 x 8 piece
-        a[r] = *reinterpret_cast<const uint32_t *>(block + (trans ? (pc + g) * m + pr : (pr + g) * m + pc) + 2 * q);
-    }
-    if (trans)
-#pragma unroll
-        for (int r = 0; r < 4; ++r) asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(a[r]) : "r"(a[r]));
-}
-
 struct Lane {                                            // rows of the four matrices of an x4 instruction
     int warp, m, r;
     __device__ __forceinline__ Lane() : warp(threadIdx.x >> 5), m((threadIdx.x & 31) >> 3), r(threadIdx.x & 7) {}
