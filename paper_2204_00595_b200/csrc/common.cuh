@@ -222,8 +222,8 @@ size_t fused_fwd_m64_workspace_bytes(int64_t tokens);
 int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s);
 // where the forward keeps u inside its workspace (null: nowhere)
 const void *fused_fwd_m64_saved_u(const void *fwd_ws);
-// one pass y = act(M x + bias), act = GELU or identity; workspace of fused_fwd_m64 (u stays behind)
-int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws, void *status,
+// one pass y = M x + bias; workspace of fused_fwd_m64 (u stays behind)
+int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, void *y, int64_t tokens, void *ws, void *status,
                        cudaStream_t s);
 size_t fused_mlp_fwd_m64_workspace_bytes(int64_t tokens);
 int fused_mlp_fwd_m64(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2, void *y,

@@ -399,7 +399,7 @@ int monarch_mlp_bwd(const void *x, const void *dy, const void *L1, const void *R
     // elementwise kernels (a then holds M1 x)
     const bool bias_in_a = pick(MONARCH_OP_FWD, m, dtype) == kFused && m == 64 && !use_units(MONARCH_OP_FWD, m, dtype, tokens);
     if (bias_in_a)
-        MONARCH_TRY(fused_fwd_bias_m64(x, L1, R1, b1, 0, a, tokens, ws_f, ws_b, s));
+        MONARCH_TRY(fused_fwd_bias_m64(x, L1, R1, b1, a, tokens, ws_f, ws_b, s));
     else {
         // the inner forward workspace starts with its own status word and tile counters
         MONARCH_TRY(monarch_workspace_init(ws_f, lay.ws_f, stream));

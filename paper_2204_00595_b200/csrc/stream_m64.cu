@@ -7,8 +7,9 @@
 // of the one before it: what that one wrote last is still in L2.  (Chunks of tokens whose intermediate stays there cost more in
 // launches and last waves than they save: 4096 tokens a chunk, 194 us forward and backward at 8192 tokens, none 164.)
 // The intermediates are stored as the next stage's operands lie in shared memory:
-//   E tile  [tile of 16 tokens][consumer block c][8-token half][producer block p] chunks of 8 tokens, XORed with c % 8:
-//           2 KB per (tile, c); a consumer's blocks are one linear copy, a producer's 16 (8) blocks 256- (128-) byte pieces
+//   E tile  [tile of 16 tokens][8 consumer blocks][producer block p][8-token half][consumer c % 8] chunks of 8 tokens, the last
+//           XORed with p % 8: 16 KB per 8 consumers; a consumer's blocks are one linear copy, a producer's 16 (8) blocks eight
+//           of 4 (2) KB
 //   T tile  natural rows of 64 columns, 128 bytes per token, 16-byte chunks XORed with t % 8 (TMA's 128-byte swizzle)
 //   Y tile  [l][token][16 neighbouring columns j]: the 32-byte pieces of a permuted row (TMA's 32-byte swizzle)
 // forward   x --T--> u_k = R_k x_k --E--> w_j = L_j u_j, in place in the E tile, transposed 8 x 8 to Y --> y
@@ -29,8 +30,9 @@ namespace tc {
 namespace {
 
 constexpr int kM = 64, kN = kM * kM, kTok = 16, kWarps = 16, kThreads = kWarps * 32;
-constexpr int kBlockBytes = 2 * kM * 16;                 // a block of an E tile
-constexpr int kTileBytes = kM * kBlockBytes;             // an E tile: 128 KB
+constexpr int kRowBytes = 2 * 8 * 16;                    // a producer's 16 tokens for 8 consumers
+constexpr int kGroupBytes = kM * kRowBytes;              // 8 consumers of an E tile: 16 KB
+constexpr int kTileBytes = kM / 8 * kGroupBytes;         // an E tile: 128 KB
 constexpr int kFwdBlocks = 16, kFwdGroups = kM / kFwdBlocks, kFwdTile = kTok * kFwdBlocks * kM * 2;   // 32 KB of any kind
 constexpr int kBwdBlocks = 8, kBwdGroups = kM / kBwdBlocks, kBwdTile = kTok * kBwdBlocks * kM * 2;    // 16 KB
 // shared memory in tiles: slots of the input ring, then V tiles (du), then staging tiles of the results.  The last four tiles
@@ -41,15 +43,23 @@ constexpr int kMaxRanks = 19;                            // CTAs of a group in t
 constexpr size_t kGradElems = (size_t)kM * kM * kM;
 
 __device__ __forceinline__ uint32_t t_at(uint32_t base, int box, int t, int c) { return base + box * (kTok * 128) + t * 128 + ((c ^ (t & 7)) << 4); }
-__device__ __forceinline__ uint32_t e_at(uint32_t base, int b, int h, int c) { return base + b * kBlockBytes + (((h * kM + c) ^ (b & 7)) << 4); }
+__device__ __forceinline__ uint32_t e_at(uint32_t base, int b, int h, int c) { return base + (b >> 3) * kGroupBytes + c * kRowBytes + h * 128 + (((b ^ c) & 7) << 4); }
+// results for consumer block b from the CTA's block c of `blocks`, in a staging tile that leaves as eight linear pieces
+__device__ __forceinline__ uint32_t out_at(uint32_t base, int blocks, int b, int h, int c) { return base + ((b >> 3) * blocks + c) * kRowBytes + h * 128 + (((b ^ c) & 7) << 4); }
+// (of map_e) by the CTA's group of `blocks` producers
+__device__ __forceinline__ void store_e(const CUtensorMap *m, int64_t tile, uint32_t from, int group, int blocks)
+{
+    tma_store_3d(m, from, 0, group * (blocks / 8), (int)tile * (kM / 8));
+}
 
 struct Params {
     unsigned *status;
     const __nv_bfloat16 *bias;
     const char *e_in, *u;        // E tiles that linear copies read
     float *parts;                // [rank][64][64][64]
-    int tiles, gelu;
+    int tiles;
     int last;                    // tiles - 1: from the last tile to the first; 0: from the first to the last
+    int follows;                 // behind another launch of the same call: init()
     int skip;                    // test aid: one of CTA 0's first tiles, never loaded; -1: none
     __device__ __forceinline__ bool skips(int item) const { return blockIdx.x == 0 && item == skip; }
 };
@@ -192,9 +202,17 @@ struct Sync {
     }
     __device__ __forceinline__ void leave() const { let_copies_land(&s.dead); }
 };
-__device__ __forceinline__ void init(Shared &s)
+// weights(): by one thread.  A launch behind another one of its call asks for them before it waits for that one, which lets its
+// followers begin only after its own wait: what ran before the call has finished.
+template <typename F> __device__ __forceinline__ void begin(int follows, F weights)
 {
+    if (follows && threadIdx.x == 0) weights();
+    depend_wait();
     depend_launch();
+    if (!follows && threadIdx.x == 0) weights();
+}
+template <typename F> __device__ __forceinline__ void init(Shared &s, int follows, F weights)
+{
     if (threadIdx.x == 0) {
         for (uint64_t &b : s.full) mbar_init(smem_u32(&b), 1);
         for (uint64_t &b : s.staged) mbar_init(smem_u32(&b), kWarps);
@@ -206,12 +224,36 @@ __device__ __forceinline__ void init(Shared &s)
         s.dead = 0;
     }
     __syncthreads();
-    depend_wait();
+    begin(follows, weights);
 }
 // CTA -> (group of blocks, rank among the CTAs of that group)
 __device__ __forceinline__ int ranks_of(int groups, int group) { return ((int)gridDim.x - group + groups - 1) / groups; }
 
+// Biases of the rows of a warp's block `own` that a lane has results of: 16 mt + lane / 4 and + 8, as bf16 pairs
+struct Bias {
+    uint32_t v[4];
+    __device__ __forceinline__ void load(const __nv_bfloat16 *bias, int own)
+    {
+#pragma unroll
+        for (int mt = 0; mt < 4; ++mt) {
+            const unsigned short *at = reinterpret_cast<const unsigned short *>(bias) + (mt * 16 + ((threadIdx.x & 31) >> 2)) * kM + own;
+            v[mt] = __ldg(at) | (uint32_t)__ldg(at + 8 * kM) << 16;
+        }
+    }
+    __device__ __forceinline__ void add(int mt, float (&acc)[4]) const
+    {
+        const float lo = __uint_as_float(v[mt] << 16), hi = __uint_as_float(v[mt] & 0xFFFF0000u);
+        acc[0] += lo;
+        acc[1] += lo;
+        acc[2] += hi;
+        acc[3] += hi;
+    }
+};
 // ---------------------------------------------------------------- forward, stage 1: x -> u (E tiles)
+// E_IN: from E tiles; ACT: u = GELU(. + bias).  The middle of a feed-forward block is E tiles on both sides: stage 2 of the first
+// matrix and stage 1 of the second are this kernel too, and h needs no transposes (8192 tokens 103 -> 100 us, 32768 383 -> 375; the
+// GELU alone is 20 of that: without one the same launch takes what its transfers take).
+template <bool E_IN, bool ACT>
 __global__ void __launch_bounds__(kThreads, 1)
 stage1_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_u,
               const Params p)
@@ -221,24 +263,28 @@ stage1_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
     Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, kFwdStages, kFwdSlots};
-    init(sh);
-    const int group = blockIdx.x % kFwdGroups, first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
+    const int group = blockIdx.x % kFwdGroups;
+    init(sh, p.follows, [&] { sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks); });
+    const int first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
     ring.loads = count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     const Lane ln;
     auto load = [&](int i) {
-        if (i < ring.loads) ring.load(i, &tm_x, tile(i), group * kFwdBlocks);
+        if (i >= ring.loads) return;
+        if (E_IN) ring.load_linear(i, p.e_in + (size_t)tile(i) * kTileBytes + group * (kFwdBlocks / 8 * kGroupBytes));
+        else      ring.load(i, &tm_x, tile(i), group * kFwdBlocks);
     };
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
-        sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
         for (int i = 0; i < kFwdSlots - 1; ++i)
             if (!p.skips(i)) load(i);
     }
     auto send = [&](int i) {
-        tma_store_2d(&tm_u, stage0 + i % kFwdStages * kFwdTile, group * kFwdBlocks * 8, tile(i) * (2 * kM));
+        store_e(&tm_u, tile(i), stage0 + i % kFwdStages * kFwdTile, group, kFwdBlocks);
     };
+    Bias bias;
+    if (ACT) bias.load(p.bias, group * kFwdBlocks + ln.warp);
     Weights<4> w;
     sync.take_weights(w, weights + ln.warp * (kM * 128), 0, false);
     if (feeder) {
@@ -253,20 +299,33 @@ stage1_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         const uint32_t x = ring.wait(i), stage = stage0 + i % kFwdStages * kFwdTile;
         uint32_t b[2][2][4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) ldm4(b[v >> 1][v & 1], t_at(x, ln.warp, (v >> 1) * 8 + ln.r, (v & 1) * 4 + ln.m));
+        for (int v = 0; v < 4; ++v) {
+            if (E_IN) ldm4t(b[v >> 1][v & 1], e_at(x, ln.warp, v >> 1, (v & 1) * 32 + ln.m * 8 + ln.r));
+            else      ldm4(b[v >> 1][v & 1], t_at(x, ln.warp, (v >> 1) * 8 + ln.r, (v & 1) * 4 + ln.m));
+        }
         if (early) sync.across(i);
         sync.wait_staging(i);
+        // a step is 32 rows of 8 tokens; the MMAs of the next one run beside what follows this one's
+        float acc[2][2][4];
+        auto products = [&](int step) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+            for (int k = 0; k < 2; ++k) w.times(2 * (step & 1) + k, b[step >> 1], acc[step & 1][k]);
+        };
+        products(0);
 #pragma unroll
-            for (int n = 0; n < 2; ++n) {
-                float a0[4], a1[4];
-                w.times(2 * n, b[h], a0);
-                w.times(2 * n + 1, b[h], a1);
-                const int j = n * 32 + ln.m * 8 + ln.r;      // row j of this block goes to block j
-                stm4(stage + (j * 2 + h) * (kFwdBlocks * 16) + ((ln.warp ^ (j & 7)) << 4), pack_bf16(a0[0], a0[1]), pack_bf16(a0[2], a0[3]),
-                     pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3]));
+        for (int step = 0; step < 4; ++step) {
+            if (step < 3) products(step + 1);
+            float (&a)[2][4] = acc[step & 1];
+            if (ACT) {
+                bias.add(2 * (step & 1), a[0]);
+                bias.add(2 * (step & 1) + 1, a[1]);
+#pragma unroll
+                for (int k = 0; k < 8; k += 2) gelu_fast2(a[k >> 2][k & 3], a[k >> 2][(k & 3) + 1]);
             }
+            const int j = (step & 1) * 32 + ln.m * 8 + ln.r;     // row j of this block goes to block j
+            stm4(out_at(stage, kFwdBlocks, j, step >> 1, ln.warp), pack_bf16(a[0][0], a[0][1]), pack_bf16(a[0][2], a[0][3]), pack_bf16(a[1][0], a[1][1]),
+                 pack_bf16(a[1][2], a[1][3]));
+        }
         sync.staged(i);
         if (early && sync.turn(i + 4)) {
             sync.wait_across(i);
@@ -281,8 +340,8 @@ stage1_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 }
 
 // ---------------------------------------------------------------- forward, stage 2: u -> y
-// ACT: y = GELU(M x + bias), or without the GELU.  Iteration i multiplies tile i + 1 and transposes tile i.
-template <bool ACT>
+// BIAS: y = M x + bias.  Iteration i multiplies tile i + 1 and transposes tile i.
+template <bool BIAS>
 __global__ void __launch_bounds__(kThreads, 1)
 stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_y, const Params p)
 {
@@ -291,18 +350,18 @@ stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kFwdSlots * kFwdTile, weights = base + 3 * kFwdTile;
     Ring ring = {base, smem_u32(sh.full), kFwdSlots, kFwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, kFwdStages, kFwdSlots};
-    init(sh);
-    const int group = blockIdx.x % kFwdGroups, first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
+    const int group = blockIdx.x % kFwdGroups;
+    init(sh, p.follows, [&] { sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks); });
+    const int first = blockIdx.x / kFwdGroups, step = ranks_of(kFwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
     ring.loads = count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
     const Lane ln;
     auto load = [&](int i) {
-        if (i < ring.loads) ring.load_linear(i, p.e_in + ((size_t)tile(i) * kM + group * kFwdBlocks) * kBlockBytes);
+        if (i < ring.loads) ring.load_linear(i, p.e_in + (size_t)tile(i) * kTileBytes + group * (kFwdBlocks / 8 * kGroupBytes));
     };
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
-        sync.load_weights(weights, &tm_w, group * kFwdBlocks, kFwdBlocks);
         for (int i = 0; i < kFwdSlots - 1; ++i) load(i);
     }
     auto send = [&](int i) {
@@ -314,7 +373,8 @@ stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         sync.wait(sh.w_read, 0, kErrSlotWait);
         load(kFwdSlots - 1);
     }
-    const __nv_bfloat16 *bias = ACT ? p.bias + ((threadIdx.x & 31) >> 2) * kM + group * kFwdBlocks + ln.warp : nullptr;
+    Bias bias;
+    if (BIAS) bias.load(p.bias, group * kFwdBlocks + ln.warp);
     auto multiply = [&](uint32_t e) {                        // in place: a warp's own block
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -325,12 +385,7 @@ stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             for (int mt = 0; mt < 4; ++mt) {
                 float acc[4];
                 w.times(mt, b, acc);
-                if (ACT)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {            // row l = 16 mt + 8 (k / 2) + lane / 4 of block j
-                        const float a = acc[k] + __bfloat162float(__ldg(bias + (mt * 16 + (k >> 1) * 8) * kM));
-                        acc[k] = p.gelu ? gelu_fast(a) : a;
-                    }
+                if (BIAS) bias.add(mt, acc);
                 o[2 * mt] = pack_bf16(acc[0], acc[1]);
                 o[2 * mt + 1] = pack_bf16(acc[2], acc[3]);
             }
@@ -419,8 +474,9 @@ bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const uint32_t weights = base + 10 * kBwdTile;
     Ring ring = {base, smem_u32(sh.full), kDuSlots, kBwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, kDuStages, 3};
-    init(sh);
-    const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
+    const int group = blockIdx.x % kBwdGroups;
+    init(sh, p.follows, [&] { sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks); });
+    const int first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
     ring.loads = (DW ? 2 : 1) * count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
@@ -429,18 +485,17 @@ bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     auto load = [&](int from, int to) {
         for (int i = from; i <= to && i < ring.loads; ++i) {
             const int t = tile(i / kItems);
-            if (DW && (i & 1)) ring.load_linear(i, p.u + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
+            if (DW && (i & 1)) ring.load_linear(i, p.u + (size_t)t * kTileBytes + group * kGroupBytes);
             else               ring.load(i, &tm_dy, t, 0, group * kBwdBlocks);
         }
     };
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
-        sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks);
         for (int i = 0; i < kDuSlots; ++i)
             if (!p.skips(i)) load(i, i);
     }
     auto send = [&](int i) {
-        tma_store_2d(&tm_du, stage0 + i % kDuStages * kBwdTile, group * kBwdBlocks * 8, tile(i) * (2 * kM));
+        store_e(&tm_du, tile(i), stage0 + i % kDuStages * kBwdTile, group, kBwdBlocks);
     };
     auto refill = [&](int i) {                               // dy(i + 1) and u(i) have been read
         load(i == 0 ? kDuSlots : kItems * i + 1 + kDuSlots, kItems * (i + 1) + kDuSlots);
@@ -483,7 +538,7 @@ bwd_du_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             w.times(0, b[h], a0);
             w.times(1, b[h], a1);
             const int k = half * 32 + ln.m * 8 + ln.r;       // row k of this block goes to block k
-            stm4(stage + (k * 2 + h) * (kBwdBlocks * 16) + ((blk ^ (k & 7)) << 4), pack_bf16(a0[0], a0[1]), pack_bf16(a0[2], a0[3]),
+            stm4(out_at(stage, kBwdBlocks, k, h, blk), pack_bf16(a0[0], a0[1]), pack_bf16(a0[2], a0[3]),
                  pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3]));
         }
         if (DW) sums.add<false>(V, ring.wait(2 * i + 1), blk, half);
@@ -507,8 +562,11 @@ bwd_dx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, stage0 = base + kDxSlots * kBwdTile;
     Ring ring = {base, smem_u32(sh.full), kDxSlots, kBwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, DX ? kDxStages : kMaxStages, 1};   // without staging, warps are up to five tiles apart
-    init(sh);
-    const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
+    const int group = blockIdx.x % kBwdGroups;
+    init(sh, p.follows, [&] {
+        if (DX) sync.load_weights(stage0, &tm_w, group * kBwdBlocks, kBwdBlocks);
+    });
+    const int first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
     ring.loads = (DW ? 2 : 1) * count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
@@ -518,14 +576,11 @@ bwd_dx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         for (int i = from; i <= to && i < ring.loads; ++i) {
             const int t = tile(i / kItems);
             if (DW && (i & 1)) ring.load(i, &tm_x, t, group * kBwdBlocks);
-            else               ring.load_linear(i, p.e_in + ((size_t)t * kM + group * kBwdBlocks) * kBlockBytes);
+            else               ring.load_linear(i, p.e_in + (size_t)t * kTileBytes + group * kGroupBytes);
         }
     };
     const bool feeder = threadIdx.x == 0;
-    if (feeder) {
-        if (DX) sync.load_weights(stage0, &tm_w, group * kBwdBlocks, kBwdBlocks);
-        load(0, kDxSlots - 1);
-    }
+    if (feeder) load(0, kDxSlots - 1);
     auto send = [&](int i) {
         if (DX) tma_store_3d(&tm_dx, stage0 + i % kDxStages * kBwdTile, 0, tile(i) * kTok, group * kBwdBlocks);
     };
@@ -615,8 +670,9 @@ cplx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CU
     const uint32_t weights = base + 3 * kPair;
     Ring ring = {base, smem_u32(sh.full), 2 * kTiles, kBwdTile, p.status, &sh.dead, 0};
     const Sync sync = {sh, p.status, kStages, 2};
-    init(sh);
-    const int group = blockIdx.x % kBwdGroups, first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
+    const int group = blockIdx.x % kBwdGroups;
+    init(sh, p.follows, [&] { sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks, 2); });
+    const int first = blockIdx.x / kBwdGroups, step = ranks_of(kBwdGroups, group);
     const int count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
     ring.loads = 2 * count;
     auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
@@ -627,14 +683,13 @@ cplx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CU
         const int t = tile(i);
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            if (!FIRST)    ring.load_linear(2 * i + c, p.e_in + ((size_t)(c * p.tiles + t) * kM + group * kBwdBlocks) * kBlockBytes);
+            if (!FIRST)    ring.load_linear(2 * i + c, p.e_in + (size_t)(c * p.tiles + t) * kTileBytes + group * kGroupBytes);
             else if (PERM) ring.load(2 * i + c, c ? &tm_im : &tm_re, t, 0, group * kBwdBlocks);
             else           ring.load(2 * i + c, c ? &tm_im : &tm_re, t, group * kBwdBlocks);
         }
     };
     const bool feeder = threadIdx.x == 0;
     if (feeder) {
-        sync.load_weights(weights, &tm_w, group * kBwdBlocks, kBwdBlocks, 2);
         for (int i = 0; i < 3; ++i)
             if (!p.skips(i)) load(i);
     }
@@ -708,7 +763,7 @@ cplx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CU
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const uint32_t from = stage0 + k % kStages * kPair + c * kBwdTile;
-            if (FIRST)     tma_store_2d(&tm_e, from, group * kBwdBlocks * 8, (c * p.tiles + t) * (2 * kM));
+            if (FIRST)     store_e(&tm_e, c * p.tiles + t, from, group, kBwdBlocks);
             else if (PERM) tma_store_3d(c ? &tm_im : &tm_re, from, group * kBwdBlocks, t * kTok, 0);
             else           tma_store_3d(c ? &tm_im : &tm_re, from, 0, t * kTok, group * kBwdBlocks);
         }
@@ -738,7 +793,7 @@ cplx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CU
         } else {
             product(re, im, [&](int h, int c, const uint32_t (&o)[4]) {
                 const int k = half * 32 + ln.m * 8 + ln.r;
-                if (FIRST) stm4(stage + c * kBwdTile + (k * 2 + h) * (kBwdBlocks * 16) + ((blk ^ (k & 7)) << 4), o);
+                if (FIRST) stm4(out_at(stage + c * kBwdTile, kBwdBlocks, k, h, blk), o);
                 else       stm4t(t_at(stage + c * kBwdTile, blk, h * 8 + ln.r, half * 4 + ln.m), o);
             });
         }
@@ -767,12 +822,16 @@ int map_y(CUtensorMap *m, const void *p, int64_t tokens, int columns)
     const uint32_t box[3] = {(uint32_t)columns, kTok, kM};
     return encode_tmap_nd(m, p, 2, 3, dims, strides, box, columns == 16 ? 32 : 0);
 }
-// E tiles as rows (tile, consumer, half) of 64 chunks: the chunks of `blocks` producers in all rows of a tile
+// E tiles as (tile, 8 consumers) x 8 producers x 2 KB: the pieces of `blocks` producers in all groups of a tile.  (As eight linear
+// copies of a thread per tile the complex multiply of 8192 tokens took 306 us, as one tensor
+// copy 288; as 256-byte pieces, in the order [consumer][half][producer], 295.)
 int map_e(CUtensorMap *m, const void *p, int tiles, int blocks)
 {
-    return encode_tmap_2d(m, p, (uint64_t)tiles * 2 * kM, kM * 8, kM * 16, 2 * kM, (uint32_t)blocks * 8, 0);
+    constexpr uint32_t kPiece = 8 * kRowBytes;
+    const uint64_t dims[3] = {kPiece / 8, 8, (uint64_t)tiles * (kM / 8)}, strides[2] = {kPiece, kGroupBytes};
+    const uint32_t box[3] = {kPiece / 8, (uint32_t)blocks / 8, kM / 8};
+    return encode_tmap_nd(m, p, 8, 3, dims, strides, box);
 }
-
 // blocks as rows of 64 columns, four blocks a copy
 int map_w(CUtensorMap *m, const void *W, int planes = 1) { return encode_tmap_2d(m, W, planes * kN, kM, kM * 2, 4 * kM, kM, 128); }
 
@@ -786,44 +845,53 @@ int grid_of(int groups, int sms, int64_t tokens)
     return (int)(all < sms ? all : sms);
 }
 
-int stage1(const void *x, const void *R, char *u, int64_t tokens, int sms, unsigned *status, cudaStream_t s)
+// x: token rows or E tiles; u: E tiles
+template <bool E_IN, bool ACT>
+int stage1(const void *x, const void *W, const void *bias, void *u, int64_t tokens, int follows, bool backwards, int sms, unsigned *status, cudaStream_t s)
 {
-    CUtensorMap tm_w, tm_x, tm_u;
-    MONARCH_TRY(map_w(&tm_w, R));
-    MONARCH_TRY(map_t(&tm_x, x, tokens, kFwdBlocks));
+    CUtensorMap tm_w, tm_x = {}, tm_u;
+    MONARCH_TRY(map_w(&tm_w, W));
     MONARCH_TRY(map_e(&tm_u, u, (int)tiles_of(tokens), kFwdBlocks));
+    if (!E_IN) MONARCH_TRY(map_t(&tm_x, x, tokens, kFwdBlocks));
     Params p = {};
-    p.skip = take_skipped_tile();
+    p.skip = follows ? -1 : take_skipped_tile();
+    p.follows = follows;
     p.status = status;
+    p.bias = (const __nv_bfloat16 *)bias;
+    p.e_in = (const char *)x;
     p.tiles = (int)tiles_of(tokens);
-    return launch_serialized(stage1_kernel, grid_of(kFwdGroups, sms, tokens), kThreads, kFwdSmem, s, tm_w, tm_x, tm_u, p);
+    p.last = backwards ? p.tiles - 1 : 0;
+    return launch_serialized(stage1_kernel<E_IN, ACT>, grid_of(kFwdGroups, sms, tokens), kThreads, kFwdSmem, s, tm_w, tm_x, tm_u, p);
 }
-
-}  // namespace
-}  // namespace tc
-
-// y = act(M x + bias) (bias null: y = M x); u: E tiles of all tokens, kept for the backward call
-static int stream_fwd(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, void *u, int64_t tokens,
-                      unsigned *status, cudaStream_t s)
+int stage2(const void *u, const void *W, const void *bias, void *y, int64_t tokens, int sms, unsigned *status, cudaStream_t s)
 {
-    using namespace tc;
-    if (tokens == 0) return MONARCH_OK;
-    int sms = 0;
-    MONARCH_TRY(current_device_sms(&sms));
-    MONARCH_TRY(stage1(x, R, (char *)u, tokens, sms, status, s));
     CUtensorMap tm_w, tm_y;
-    MONARCH_TRY(map_w(&tm_w, L));
+    MONARCH_TRY(map_w(&tm_w, W));
     MONARCH_TRY(map_y(&tm_y, y, tokens, kFwdBlocks));
     Params p = {};
     p.skip = -1;
+    p.follows = 1;
     p.status = status;
     p.bias = (const __nv_bfloat16 *)bias;
-    p.gelu = gelu;
     p.e_in = (const char *)u;
     p.tiles = (int)tiles_of(tokens);
     p.last = p.tiles - 1;
     return launch_serialized(bias != nullptr ? stage2_kernel<true> : stage2_kernel<false>, grid_of(kFwdGroups, sms, tokens), kThreads, kFwdSmem, s,
                              tm_w, tm_y, p);
+}
+
+}  // namespace
+}  // namespace tc
+
+// y = M x + bias (bias null: y = M x); u: E tiles of all tokens, kept for the backward call
+static int stream_fwd(const void *x, const void *L, const void *R, const void *bias, void *y, void *u, int64_t tokens, unsigned *status, cudaStream_t s)
+{
+    using namespace tc;
+    if (tokens == 0) return MONARCH_OK;
+    int sms = 0;
+    MONARCH_TRY(current_device_sms(&sms));
+    MONARCH_TRY((stage1<false, false>(x, R, nullptr, u, tokens, 0, false, sms, status, s)));
+    return stage2(u, L, bias, y, tokens, sms, status, s);
 }
 
 // dx null: gradients only; dL null: dx only.  u: what the forward call left (u_saved), or scratch for E tiles of all tokens;
@@ -844,7 +912,7 @@ static int stream_bwd(const void *x, const void *dy, const void *L, const void *
     if (sms > kMaxRanks * kBwdGroups) sms = kMaxRanks * kBwdGroups;
     float *parts_l = (float *)parts, *parts_r = parts_l + max_ranks(tokens) * kGradElems;
     const int grid = grid_of(kBwdGroups, sms, tokens), tiles = (int)tiles_of(tokens);
-    if (dL != nullptr && !u_saved) MONARCH_TRY(stage1(x, R, (char *)u, tokens, sms, status, s));
+    if (dL != nullptr && !u_saved) MONARCH_TRY((stage1<false, false>(x, R, nullptr, (void *)u, tokens, 0, false, sms, status, s)));
     CUtensorMap tm_L, tm_R, tm_dy, tm_du, tm_x, tm_dx;
     MONARCH_TRY(map_w(&tm_L, L));
     MONARCH_TRY(map_w(&tm_R, R));
@@ -860,6 +928,7 @@ static int stream_bwd(const void *x, const void *dy, const void *L, const void *
     p.tiles = tiles;
     MONARCH_TRY(launch_serialized(dL != nullptr ? bwd_du_kernel<true> : bwd_du_kernel<false>, grid, kThreads, kBwdSmem, s, tm_L, tm_dy, tm_du, p));
     p.skip = -1;
+    p.follows = 1;
     p.e_in = (const char *)du;
     p.parts = parts_r;
     p.last = tiles - 1;
@@ -879,9 +948,9 @@ static int stream_cplx(const void *x, const void *L, const void *R, void *y, int
     const int tiles = (int)tiles_of(tokens), grid = grid_of(kBwdGroups, sms, tokens);
     const size_t plane = (size_t)tokens * kN * 2;
     CUtensorMap tm_w[2], tm_e, tm_x[2], tm_y[2];
+    MONARCH_TRY(map_e(&tm_e, e, 2 * tiles, kBwdBlocks));
     MONARCH_TRY(map_w(&tm_w[0], adjoint ? L : R, 2));
     MONARCH_TRY(map_w(&tm_w[1], adjoint ? R : L, 2));
-    MONARCH_TRY(map_e(&tm_e, e, 2 * tiles, kBwdBlocks));
     for (int c = 0; c < 2; ++c) {
         const char *xc = (const char *)x + c * plane, *yc = (const char *)y + c * plane;
         MONARCH_TRY(adjoint ? map_y(&tm_x[c], xc, tokens, kBwdBlocks) : map_t(&tm_x[c], xc, tokens, kBwdBlocks));
@@ -894,6 +963,7 @@ static int stream_cplx(const void *x, const void *L, const void *R, void *y, int
     p.tiles = tiles;
     MONARCH_TRY(launch_serialized(adjoint ? cplx_kernel<true, true> : cplx_kernel<true, false>, grid, kThreads, kBwdSmem, s, tm_w[0], tm_e, tm_x[0], tm_x[1], p));
     p.skip = -1;
+    p.follows = 1;
     p.last = tiles - 1;
     return launch_serialized(adjoint ? cplx_kernel<false, false> : cplx_kernel<false, true>, grid, kThreads, kBwdSmem, s, tm_w[1], tm_e, tm_y[0], tm_y[1], p);
 }
@@ -918,22 +988,29 @@ int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t 
         const int st = fused_fwd_m64_cluster(x, L, R, y, tokens, ws, s);
         if (st != MONARCH_ERR_UNSUPPORTED) return st;
     }
-    return stream_fwd(x, L, R, nullptr, 0, y, head(ws), tokens, (unsigned *)ws, s);
+    return stream_fwd(x, L, R, nullptr, y, head(ws), tokens, (unsigned *)ws, s);
 }
 // (the status word is the caller's: `ws` is not initialised)
-int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws, void *status,
+int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, void *y, int64_t tokens, void *ws, void *status,
                        cudaStream_t s)
 {
-    return stream_fwd(x, L, R, bias, gelu, y, head(ws), tokens, (unsigned *)status, s);
+    return stream_fwd(x, L, R, bias, y, head(ws), tokens, (unsigned *)status, s);
 }
 
 size_t fused_mlp_fwd_m64_workspace_bytes(int64_t tokens) { return kHead + 2 * tc::e_bytes(tokens); }
 int fused_mlp_fwd_m64(const void *x, const void *L1, const void *R1, const void *b1, const void *L2, const void *R2, const void *b2, void *y,
                       int64_t tokens, void *ws, cudaStream_t s)
 {
-    char *u = head(ws), *h = u + tc::e_bytes(tokens);
-    MONARCH_TRY(stream_fwd(x, L1, R1, b1, 1, h, u, tokens, (unsigned *)ws, s));
-    return stream_fwd(h, L2, R2, b2, 0, y, u, tokens, (unsigned *)ws, s);
+    using namespace tc;
+    if (tokens == 0) return MONARCH_OK;
+    char *u = head(ws), *h = u + e_bytes(tokens);
+    unsigned *status = (unsigned *)ws;
+    int sms = 0;
+    MONARCH_TRY(current_device_sms(&sms));
+    MONARCH_TRY((stage1<false, false>(x, R1, nullptr, u, tokens, 0, false, sms, status, s)));
+    MONARCH_TRY((stage1<true, true>(u, L1, b1, h, tokens, 1, true, sms, status, s)));
+    MONARCH_TRY((stage1<true, false>(h, R2, nullptr, u, tokens, 1, false, sms, status, s)));
+    return stage2(u, L2, b2, y, tokens, sms, status, s);
 }
 
 size_t fused_bwd_dx_m64_workspace_bytes(int64_t tokens) { return kHead + tc::e_bytes(tokens); }
