@@ -56,6 +56,7 @@ struct Params {
     unsigned *status;
     const __nv_bfloat16 *bias;
     const char *e_in, *u;        // E tiles that linear copies read
+    char *e_out, *u_out;         // E tiles that linear copies write
     float *parts;                // [rank][64][64][64]
     int tiles;
     int last;                    // tiles - 1: from the last tile to the first; 0: from the first to the last
@@ -416,6 +417,259 @@ stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     }
     sync.pass_last(count, send);
     sync.leave();
+}
+
+// ---------------------------------------------------------------- forward on clusters of eight CTAs
+// Both stages in one launch: CTA c of a cluster keeps blocks 8 c .. 8 c + 8 of R and of L in registers, a block per warp (warps 0 to
+// 7: R, the others: L), and u crosses through distributed shared memory: each warp of stage 1 sends a consumer CTA 256 bytes per
+// tile, asynchronously and counted on its barrier, which land as the CTA's 16 KB of an E tile.  So x and y make their one trip and
+// u, where the backward call wants it, one more as linear copies.  For small batches, which the two launches of the streams cost
+// most (forward of 64 tokens 9.1 -> 6.7 us, block 18.6 -> 12.5 where it was four phases of one launch over units).
+// What bounds it, cycles per 16-token tile: MMAs 1030, the exchange 1020 (1860 where the 16-byte pieces of a warp lie 2 KB apart: what
+// the order of an E tile is for), y in 16-byte pieces 1200; but a tile takes 2600, most of it the chain of one warp: loads, MMAs,
+// transposes, sends and the barriers between.  Taken back, none faster beyond 1500 tokens: half a block of both factors per warp
+// (3300 cycles), four more warps that transpose and send (2500), loads of the next tile under the sends (2700).
+// Fifteen clusters fit the device (120 of 148 SMs).
+//   E_IN    x is E tiles, not token rows          E_OUT  results are E tiles (of the next matrix), not token rows
+//   BIAS, GELU                                     SAVE   u is left in p.e_out's place p.u_out
+constexpr int kCl = 8, kHalfWarps = kWarps / 2;
+constexpr int kClX = 3, kClE = 4, kClV = 3, kClY = 3;        // tiles of 16 KB: input slots, exchange slots, w, results
+constexpr int kClSmem = (kClX + kClE + 1 + kClV + kClY) * kBwdTile + 1024;
+struct ClusterShared {
+    uint64_t x_full[kClX], x_read[kClX], e_full[kClE], e_free[kClE], across[kClV], staged[8], sent[kClV + kClY], w_full;
+    int dead;
+};
+
+__device__ __forceinline__ void st_async_16(uint32_t to, uint4 v, uint32_t bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(to), "r"(v.x), "r"(v.y),
+                 "r"(v.z), "r"(v.w), "r"(bar) : "memory");
+}
+
+template <bool E_IN, bool E_OUT, bool BIAS, bool GELU, bool SAVE>
+__global__ void __launch_bounds__(kThreads, 1)
+fwd_cluster_kernel(const __grid_constant__ CUtensorMap tm_R, const __grid_constant__ CUtensorMap tm_L, const __grid_constant__ CUtensorMap tm_x,
+                   const __grid_constant__ CUtensorMap tm_y, const Params p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ ClusterShared s;
+    const uint32_t X0 = (smem_u32(smem_raw) + 1023u) & ~1023u, E0 = X0 + kClX * kBwdTile, U0 = E0 + kClE * kBwdTile, V0 = U0 + kBwdTile;
+    constexpr int kOut = E_OUT ? kClV + kClY : kClY;         // result tiles
+    const uint32_t Y0 = E_OUT ? V0 : V0 + kClV * kBwdTile;
+    const Lane ln;
+    const int rank = (int)cluster_ctarank(), lane = threadIdx.x & 31, w = ln.warp & (kHalfWarps - 1), own = rank * kBwdBlocks + w;
+    const int first = blockIdx.x / kCl, step = gridDim.x / kCl, count = first < p.tiles ? (p.tiles - first + step - 1) / step : 0;
+    auto tile = [&](int i) { return p.last != 0 ? p.last - first - i * step : first + i * step; };
+    // by one lane, or by a warp, whose lanes all learn if one ran out: the warp then does nothing more
+    auto wait1 = [&](const uint64_t &bar, int phase, unsigned code) { return mbar_wait(smem_u32(&bar), phase & 1, p.status, &s.dead, code); };
+    auto wait = [&](const uint64_t &bar, int phase, unsigned code) { return __all_sync(0xffffffffu, wait1(bar, phase, code)) != 0; };
+    auto turn = [&](int k) { return lane == 0 && (k & (kHalfWarps - 1)) == w; };
+    auto arrive = [&](uint64_t &bar) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bar));
+    };
+    auto load = [&](int i) {
+        const uint32_t bar = smem_u32(&s.x_full[i % kClX]), to = X0 + i % kClX * kBwdTile;
+        mbar_expect_tx(bar, kBwdTile);
+        if (E_IN)
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(to),
+                         "l"(p.e_in + (size_t)tile(i) * kTileBytes + rank * kGroupBytes), "r"(kBwdTile), "r"(bar) : "memory");
+        else
+            tma_load_3d(to, &tm_x, 0, tile(i) * kTok, rank * kBwdBlocks, bar);
+    };
+    if (threadIdx.x == 0) {
+        for (uint64_t &b : s.x_full) mbar_init(smem_u32(&b), 1);
+        for (uint64_t &b : s.x_read) mbar_init(smem_u32(&b), kHalfWarps);
+        for (uint64_t &b : s.e_full) mbar_init(smem_u32(&b), 1);
+        for (uint64_t &b : s.e_free) mbar_init(smem_u32(&b), kCl * kHalfWarps);
+        for (uint64_t &b : s.across) mbar_init(smem_u32(&b), kHalfWarps);
+        for (uint64_t &b : s.staged) mbar_init(smem_u32(&b), kHalfWarps);
+        for (uint64_t &b : s.sent) mbar_init(smem_u32(&b), 1);
+        mbar_init(smem_u32(&s.w_full), 1);
+        fence_mbar_init();
+        s.dead = 0;
+    }
+    __syncthreads();
+    begin(p.follows, [&] {                                   // into the exchange slots and where the results go
+        const uint32_t bar = smem_u32(&s.w_full);
+        mbar_expect_tx(bar, 2 * kBwdBlocks * kM * 128);
+        for (int b = 0; b < kBwdBlocks; b += 4) {
+            tma_load_2d(V0 + b * kM * 128, &tm_R, 0, (rank * kBwdBlocks + b) * kM, bar);
+            tma_load_2d(E0 + b * kM * 128, &tm_L, 0, (rank * kBwdBlocks + b) * kM, bar);
+        }
+    });
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kClX && i < count; ++i)
+            if (!p.skips(i)) load(i);
+        for (int i = 0; i < kClE && i < count; ++i) mbar_expect_tx(smem_u32(&s.e_full[i]), kBwdTile);
+    }
+    Weights<4> wt;
+    bool ok = wait(s.w_full, 0, kErrTmaWait);
+    wt.load((ln.warp < kHalfWarps ? V0 : E0) + w * (kM * 128), 0, false);
+    cluster_arrive_release();                                // every CTA of the cluster takes the exchange's bytes from here on
+    cluster_wait_acquire();
+
+    if (ln.warp < kHalfWarps) {
+        // ---- stage 1: u_k = R_k x_k; row j goes to block j, in CTA j / 8
+        const uint32_t mine = U0 + w * 2048;
+        uint32_t to[2], bar[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int j = q * 32 + lane;
+            to[q] = map_to_cta(e_at(E0, j & 7, 0, own), j >> 3);
+            bar[q] = map_to_cta(smem_u32(s.e_full), j >> 3);
+        }
+        for (int i = 0; ok && i < count; ++i) {
+            const uint32_t x = X0 + i % kClX * kBwdTile;
+            uint32_t b[2][2][4];
+            if (!wait(s.x_full[i % kClX], i / kClX, kErrTmaWait)) break;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                if (E_IN) ldm4t(b[v >> 1][v & 1], e_at(x, w, v >> 1, (v & 1) * 32 + ln.m * 8 + ln.r));
+                else      ldm4(b[v >> 1][v & 1], t_at(x, w, (v >> 1) * 8 + ln.r, (v & 1) * 4 + ln.m));
+            }
+            arrive(s.x_read[i % kClX]);
+            if (i > 0 && turn(i) && i - 1 + kClX < count && wait1(s.x_read[(i - 1) % kClX], (i - 1) / kClX, kErrSlotWait)) load(i - 1 + kClX);
+            __syncwarp();
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int n = 0; n < 2; ++n) {
+                    float a0[4], a1[4];
+                    wt.times(2 * n, b[h], a0);
+                    wt.times(2 * n + 1, b[h], a1);
+                    stm4(mine + h * 1024 + (n * 32 + ln.m * 8 + ln.r) * 16, pack_bf16(a0[0], a0[1]), pack_bf16(a0[2], a0[3]),
+                         pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3]));
+                }
+            if (i >= kClE && !wait(s.e_free[i % kClE], i / kClE - 1, kErrPeerWait)) break;
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint4 v;
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(mine + q * 512 + lane * 16) : "memory");
+                st_async_16(to[q & 1] + i % kClE * kBwdTile + (q >> 1) * 128, v, bar[q & 1] + i % kClE * 8);
+            }
+            __syncwarp();                                    // `mine` has been read
+        }
+    } else {
+        // ---- stage 2: w_j = L_j u_j
+        const uint32_t peer_free = map_to_cta(smem_u32(s.e_free), lane & (kCl - 1));
+        auto release = [&](int i) { mbar_arrive_remote(peer_free + i % kClE * 8); };         // by eight lanes, one per CTA
+        Bias bias;
+        if (BIAS) bias.load(p.bias, own);
+        // put(h, four words of rows 0 .. 31 or 32 .. 63 x 8 tokens, n)
+        auto multiply = [&](int i, auto put) {
+            const uint32_t e = E0 + i % kClE * kBwdTile;
+            if (!__all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&s.e_full[i % kClE]), i / kClE & 1, p.status, &s.dead, kErrPeerWait))) return false;
+            if (threadIdx.x == kHalfWarps * 32 && i + kClE < count) mbar_expect_tx(smem_u32(&s.e_full[i % kClE]), kBwdTile);
+            const bool saves = SAVE && turn(i + 4);
+            if (saves) {
+                fence_proxy_async_smem();
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(p.u_out + (size_t)tile(i) * kTileBytes + rank * kGroupBytes),
+                             "r"(e), "r"(kBwdTile) : "memory");
+                tma_store_commit();
+            }
+            __syncwarp();
+            uint32_t b[2][2][4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) ldm4t(b[v >> 1][v & 1], e_at(e, w, v >> 1, (v & 1) * 32 + ln.m * 8 + ln.r));
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t o[8];
+#pragma unroll
+                for (int mt = 0; mt < 4; ++mt) {
+                    float acc[4];
+                    wt.times(mt, b[h], acc);
+                    if (BIAS) bias.add(mt, acc);
+                    if (GELU) {
+                        gelu_fast2(acc[0], acc[1]);
+                        gelu_fast2(acc[2], acc[3]);
+                    }
+                    o[2 * mt] = pack_bf16(acc[0], acc[1]);
+                    o[2 * mt + 1] = pack_bf16(acc[2], acc[3]);
+                }
+                if (!put(h, o)) return false;
+            }
+            // (after the products: the tile is in registers.)  A saved tile is released once its copy has read it, a tile later.
+            if (SAVE && i > 0 && w == ((i + 3) & (kHalfWarps - 1))) {
+                if (lane == 0) tma_store_wait_read<0>();
+                __syncwarp();
+                if (lane < kCl) release(i - 1);
+            }
+            if ((!SAVE || w != ((i + 4) & (kHalfWarps - 1))) && lane < kCl) release(i);
+            return true;
+        };
+        auto send = [&](int i) {
+            const uint32_t from = Y0 + i % kOut * kBwdTile;
+            if (E_OUT)                                       // (one tensor copy instead: block of 512 tokens 20.1 against 19.4 us)
+#pragma unroll
+                for (int g = 0; g < kM / 8; ++g)
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(p.e_out + (size_t)tile(i) * kTileBytes + g * kGroupBytes + rank * (kBwdBlocks * kRowBytes)),
+                                 "r"(from + g * (kBwdBlocks * kRowBytes)), "r"(kBwdBlocks * kRowBytes) : "memory");
+            else
+                tma_store_3d(&tm_y, from, rank * kBwdBlocks, tile(i) * kTok, 0);
+            tma_store_commit();
+        };
+        // results of tile i are in their tile; the ones before leave, by turns
+        auto pass_on = [&](int i) {
+            fence_proxy_async_smem();
+            arrive(s.staged[i & 7]);
+            if (i >= 2 && turn(i - 2)) {
+                tma_store_wait_read<0>();
+                mbar_arrive(smem_u32(&s.sent[(i - 2) % kOut]));
+            }
+            if (i >= 1 && turn(i - 1) && wait1(s.staged[(i - 1) & 7], (i - 1) >> 3, kErrMmaWait)) send(i - 1);
+            __syncwarp();
+        };
+        auto wait_sent = [&](int i) { return i < kOut || wait(s.sent[i % kOut], i / kOut - 1, kErrSlotWait); };
+        int i = 0;
+        if (E_OUT) {
+            for (; ok && i < count; ++i) {
+                const uint32_t out = Y0 + i % kOut * kBwdTile;
+                if (!multiply(i, [&](int h, const uint32_t (&o)[8]) {
+                        if (h == 0 && !wait_sent(i)) return false;
+#pragma unroll
+                        for (int n = 0; n < 2; ++n) stm4(out_at(out, kBwdBlocks, n * 32 + ln.m * 8 + ln.r, h, w), o[4 * n], o[4 * n + 1], o[4 * n + 2], o[4 * n + 3]);
+                        return true;
+                    }))
+                    break;
+                pass_on(i);
+            }
+        } else {
+            auto ahead = [&](int k) {                        // w, as an E tile: transposed below
+                const uint32_t V = V0 + k % kClV * kBwdTile;
+                if (!multiply(k, [&](int h, const uint32_t (&o)[8]) {
+                        if (h == 0 && k >= kClV && !wait(s.staged[(k - kClV) & 7], (k - kClV) >> 3, kErrMmaWait)) return false;
+#pragma unroll
+                        for (int n = 0; n < 2; ++n) stm4(e_at(V, w, h, n * 32 + ln.m * 8 + ln.r), o[4 * n], o[4 * n + 1], o[4 * n + 2], o[4 * n + 3]);
+                        return true;
+                    }))
+                    return false;
+                arrive(s.across[k % kClV]);
+                return true;
+            };
+            ok = ok && (count == 0 || ahead(0));
+            for (; ok && i < count; ++i) {
+                if (i + 1 < count && !ahead(i + 1)) break;
+                const uint32_t V = V0 + i % kClV * kBwdTile, out = Y0 + i % kOut * kBwdTile;
+                if (!wait(s.across[i % kClV], i / kClV, kErrMmaWait)) break;
+                uint32_t v[4][4];
+                const int h = ln.m & 1, lo = ln.m >> 1;
+#pragma unroll
+                for (int n = 0; n < 4; ++n) ldm4t(v[n], e_at(V, ln.r, h, w * 8 + n * 2 + lo));
+                if (!wait_sent(i)) break;
+#pragma unroll
+                for (int n = 0; n < 4; ++n) stm4(out + (w * 8 + n * 2 + lo) * (kTok * 16) + (h * 8 + ln.r) * 16, v[n]);
+                pass_on(i);
+            }
+        }
+        if (i == count && count > 0 && turn(count - 1) && wait1(s.staged[(count - 1) & 7], (count - 1) >> 3, kErrMmaWait)) send(count - 1);
+        tma_store_wait_all<0>();
+    }
+    let_copies_land(&s.dead);
+    __syncthreads();
+    cluster_arrive_release();                                // nobody leaves while others may still write here
+    cluster_wait_acquire();
 }
 
 // ---------------------------------------------------------------- backward
@@ -880,8 +1134,91 @@ int stage2(const void *u, const void *W, const void *bias, void *y, int64_t toke
                              tm_w, tm_y, p);
 }
 
+// Launch attributes of a cluster kernel, and how many clusters fit the device at once (0: none do)
+struct ClusterLaunch {
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg;
+    explicit ClusterLaunch(cudaStream_t s) : cfg()
+    {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kCl;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.blockDim = dim3(kThreads);
+        cfg.gridDim = dim3(kCl);
+        cfg.dynamicSmemBytes = kClSmem;
+        cfg.stream = s;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+};
+template <bool E_IN, bool E_OUT, bool BIAS, bool GELU, bool SAVE> int clusters()
+{
+    static PerDeviceCache fit;
+    auto kern = fwd_cluster_kernel<E_IN, E_OUT, BIAS, GELU, SAVE>;
+    int n = fit.get();
+    if (n < 0) {
+        const ClusterLaunch launch(nullptr);
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kClSmem) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, kern, &launch.cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        fit.set(n);
+    }
+    return n;
+}
+
+// One multiply on clusters; x, y: token rows or E tiles
+template <bool E_IN, bool E_OUT, bool BIAS, bool GELU, bool SAVE>
+int fwd_on_clusters(const void *x, const void *L, const void *R, const void *bias, void *y, void *u, int64_t tokens, bool follows, unsigned *status,
+                    cudaStream_t s)
+{
+    const int64_t fit = clusters<E_IN, E_OUT, BIAS, GELU, SAVE>();
+    if (fit <= 0) return MONARCH_ERR_UNSUPPORTED;
+    ClusterLaunch launch(s);
+    launch.cfg.numAttrs = 2;
+    launch.cfg.gridDim = dim3((unsigned)(kCl * (tiles_of(tokens) < fit ? tiles_of(tokens) : fit)));
+    CUtensorMap tm_R, tm_L, tm_x = {}, tm_y = {};
+    MONARCH_TRY(map_w(&tm_R, R));
+    MONARCH_TRY(map_w(&tm_L, L));
+    if (!E_IN) MONARCH_TRY(map_t(&tm_x, x, tokens, kBwdBlocks));
+    if (!E_OUT) MONARCH_TRY(map_y(&tm_y, y, tokens, kBwdBlocks));
+    Params p = {};
+    p.skip = take_skipped_tile();
+    p.status = status;
+    p.bias = (const __nv_bfloat16 *)bias;
+    p.e_in = (const char *)x;
+    p.e_out = (char *)y;
+    p.u_out = (char *)u;
+    p.tiles = (int)tiles_of(tokens);
+    p.follows = follows;
+    p.last = follows ? p.tiles - 1 : 0;
+    MONARCH_CUDA_TRY(cudaLaunchKernelEx(&launch.cfg, fwd_cluster_kernel<E_IN, E_OUT, BIAS, GELU, SAVE>, tm_R, tm_L, tm_x, tm_y, p));
+    note_launch();
+    return MONARCH_OK;
+}
+
 }  // namespace
 }  // namespace tc
+
+// Where the forward runs on clusters.  They take 5.6 us and 1.45 for every round of tiles, of which there are as many as clusters
+// fit (15); the streams, in which a tile takes four CTAs, 8 us as long as each CTA has one.  So: one round, or more tiles than
+// the streams' CTAs, up to five rounds (us, clusters / streams: 240 tokens 7.1 / 8.3, 300 8.6 / 8.4, 600 10.5 / 11.7, 960
+// 12.4 / 13.1, 1500 16.2 / 15.8).  Under the feed-forward backward, whose next launch reads y, one round (1000 tokens 122.8 / 121.7).
+static bool fwd_prefers_clusters(int64_t tokens, bool bias, int sms)
+{
+    const int64_t tiles = tc::tiles_of(tokens), fit = bias ? tc::clusters<false, false, true, false, true>() : tc::clusters<false, false, false, false, true>();
+    return fit > 0 && (tiles <= fit || (!bias && tiles * tc::kFwdGroups > sms && tiles <= 5 * fit));
+}
+// The feed-forward block, whose streams are four launches, up to ten rounds (16 tokens 11.7 / 17.4, 1000 25.3 / 28.9, 2400 40.4 /
+// 42.5, 2700 45.5 / 44.3)
+static bool mlp_prefers_clusters(int64_t tokens)
+{
+    const int64_t fit = tc::clusters<false, true, true, true, false>(), last = tc::clusters<true, false, true, false, false>();
+    return fit > 0 && last > 0 && tc::tiles_of(tokens) <= 10 * fit;
+}
 
 // y = M x + bias (bias null: y = M x); u: E tiles of all tokens, kept for the backward call
 static int stream_fwd(const void *x, const void *L, const void *R, const void *bias, void *y, void *u, int64_t tokens, unsigned *status, cudaStream_t s)
@@ -890,6 +1227,9 @@ static int stream_fwd(const void *x, const void *L, const void *R, const void *b
     if (tokens == 0) return MONARCH_OK;
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
+    if (fwd_prefers_clusters(tokens, bias != nullptr, sms))
+        return bias != nullptr ? fwd_on_clusters<false, false, true, false, true>(x, L, R, bias, y, u, tokens, false, status, s)
+                               : fwd_on_clusters<false, false, false, false, true>(x, L, R, nullptr, y, u, tokens, false, status, s);
     MONARCH_TRY((stage1<false, false>(x, R, nullptr, u, tokens, 0, false, sms, status, s)));
     return stage2(u, L, bias, y, tokens, sms, status, s);
 }
@@ -1005,6 +1345,10 @@ int fused_mlp_fwd_m64(const void *x, const void *L1, const void *R1, const void 
     if (tokens == 0) return MONARCH_OK;
     char *u = head(ws), *h = u + e_bytes(tokens);
     unsigned *status = (unsigned *)ws;
+    if (mlp_prefers_clusters(tokens)) {
+        MONARCH_TRY((fwd_on_clusters<false, true, true, true, false>(x, L1, R1, b1, h, nullptr, tokens, false, status, s)));
+        return fwd_on_clusters<true, false, true, false, false>(h, L2, R2, b2, y, nullptr, tokens, true, status, s);
+    }
     int sms = 0;
     MONARCH_TRY(current_device_sms(&sms));
     MONARCH_TRY((stage1<false, false>(x, R1, nullptr, u, tokens, 0, false, sms, status, s)));

@@ -1400,6 +1400,49 @@ print("ok")
     assert out.returncode == 0 and "ok" in out.stdout, out.stderr[-2000:]
 
 
+# ----------------------------------------------------------------- the m = 64 forward on clusters of eight CTAs
+
+# around its tiles of 16 tokens and its rounds of 15 tiles, and on both sides of every size at which a call changes kernels
+@pytest.mark.parametrize("T", [1, 16, 17, 239, 241, 592, 593, 960, 961, 1200, 1201, 2400, 2401])
+def test_fwd_m64_rounds_of_clusters(P, T):
+    """Forward and feed-forward block against the oracle; the u left for the backward gives the bits of the u it works out itself."""
+    import torch
+    m, n, code = 64, 4096, P.BF16
+    d = _small_inputs(m, T, "bf16", seed=8800 + T)
+    x, dy, L, R, L2, R2, b1, b2 = (to_device(d[k], "bf16") for k in ("x", "dy", "L", "R", "L2", "R2", "b1", "b2"))
+    rows = np.unique(np.concatenate([_sample_tokens(T, 48, 5), np.arange(T - 40, T)])) if T > 96 else np.arange(T)
+    yf, y = _guarded((T, n), torch.bfloat16)
+    ws = P.Workspace(P.monarch_workspace_bytes(P.OP_FWD, T, n, m, code))
+    ws_b = P.Workspace(P.monarch_workspace_bytes(P.OP_BWD, T, n, m, code))
+    ws_m = P.Workspace(P.monarch_workspace_bytes(P.OP_MLP_FWD, T, n, m, code))
+    P.monarch_fwd(x, L, R, y, T, n, m, ws)
+    torch.cuda.synchronize()
+    assert P.monarch_last_device_status(ws) == 0
+    assert_close(to_host64(y)[rows], O.fwd(d["x"][rows], d["L"], d["R"]), "bf16", "y")
+    _check_guard(yf, "y")
+    out = []
+    for saved in (ws, None):
+        dx, dL, dR = torch.empty_like(x), torch.empty(m, m, m, device="cuda"), torch.empty(m, m, m, device="cuda")
+        P.monarch_bwd(x, dy, L, R, dx, dL, dR, 0, T, n, m, ws_b, fwd_workspace=saved)
+        out.append((dx, dL, dR))
+    torch.cuda.synchronize()
+    assert P.monarch_last_device_status(ws_b) == 0
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+    y.fill_(float("nan"))
+    P.monarch_mlp_fwd(x, L, R, b1, L2, R2, b2, y, T, n, m, ws_m)
+    torch.cuda.synchronize()
+    assert P.monarch_last_device_status(ws_m) == 0
+    assert_close(to_host64(y)[rows], O.mlp_fwd(d["x"][rows], d["L"], d["R"], d["b1"], d["L2"], d["R2"], d["b2"]), "bf16", "mlp y")
+    _check_guard(yf, "mlp y")
+
+
+@pytest.mark.parametrize("item", [0, 2])
+@pytest.mark.parametrize("call", ["fwd", "mlp"])
+def test_tile_that_never_arrives_on_clusters(P, call, item):
+    """The same as above where the calls run on clusters: the CTAs that the missing rows would have gone to give up as well."""
+    test_tile_that_never_arrives(P, 64, 16 * 15 * 4, call, item)
+
+
 # ----------------------------------------------------------------- m = 128: the three-launch forward, and run-to-run bits
 
 @pytest.mark.parametrize("T", [1, 130, 700])
