@@ -537,7 +537,12 @@ __device__ __forceinline__ void load_async(float *tile, const View &v, int perm,
         const float4 *src = static_cast<const float4 *>(v.p) +
                             (size_t)((t0 + t) * v.t_stride + (b0 + b) * v.b_stride + (c0 / 8 + c) * v.c_stride) * 2 + h;
         float *dst = tile + b * BLOCK + t * PITCH + c * 8 + h * 4;
+        if (left >= R) {                                   // (most tiles are whole)
 #pragma unroll
+            for (int n = 0; n < R / kStep; ++n, src += (size_t)kStep * v.t_stride * 2) cp_async16(dst + n * kStep * PITCH, src, true);
+            return;
+        }
+#pragma unroll 1
         for (int n = 0; n < R / kStep; ++n) {
             const bool ok = (int)t + n * kStep < left;
             cp_async16(dst + n * kStep * PITCH, ok ? src + (size_t)n * kStep * v.t_stride * 2 : static_cast<const float4 *>(v.p), ok);
@@ -549,7 +554,13 @@ __device__ __forceinline__ void load_async(float *tile, const View &v, int perm,
     const unsigned b = j % 8, c = j / 8 % NC, t = j / (8 * NC);
     const float *src = static_cast<const float *>(v.p) + (size_t)((t0 + t) * v.t_stride + b0 / 8 * v.b_stride + (c0 + c) * v.c_stride) * 8 + b;
     const uint32_t dst = smem_addr(tile + b * BLOCK + t * PITCH + c);
+    if (left >= R) {
 #pragma unroll
+        for (int n = 0; n < R / kStep; ++n, src += (size_t)kStep * v.t_stride * 8)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + n * kStep * PITCH * 4), "l"(src) : "memory");
+        return;
+    }
+#pragma unroll 1
     for (int n = 0; n < R / kStep; ++n) {
         const bool ok = (int)t + n * kStep < left;
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + n * kStep * PITCH * 4),
@@ -587,15 +598,16 @@ template <typename C> struct Chunks {
 #pragma unroll
         for (int n = 0; n < 8 / kStep; ++n) cp_async16(dst + n * step, src + (size_t)n * kStep * M * M, true);
     }
-    __device__ __forceinline__ void multiply(const float *tile, const float *wt, int trans)
+    // the columns of one half of a chunk
+    __device__ __forceinline__ void multiply(const float *tile, const float *wt, int trans, int half)
     {
         const int w = (threadIdx.x >> 5) / C::kWpb, e0 = (threadIdx.x >> 5) % C::kWpb * EW;
         const int tl = (threadIdx.x & 31) >> 3, el = threadIdx.x & 7;
-        const float *a = tile + w * C::kBlockA + tl * PC;
+        const float *a = tile + w * C::kBlockA + tl * PC + half * (KC / 2);
         if (!trans) {
-            const float *b = wt + (w * ES + e0 + el) * PC;
+            const float *b = wt + (w * ES + e0 + el) * PC + half * (KC / 2);
 #pragma unroll
-            for (int c = 0; c < KC; c += 4) {
+            for (int c = 0; c < KC / 2; c += 4) {
                 ulonglong2 fb[RE];
 #pragma unroll
                 for (int q = 0; q < RE; ++q) fb[q] = *reinterpret_cast<const ulonglong2 *>(b + 8 * q * PC + c);
@@ -608,9 +620,9 @@ template <typename C> struct Chunks {
             }
         } else {
             constexpr int V = RE < 4 ? RE : 4;             // neighbouring outputs of a lane
-            const float *b = wt + w * KC * (ES + 4) + e0 + V * el;
+            const float *b = wt + (w * KC + half * (KC / 2)) * (ES + 4) + e0 + V * el;
 #pragma unroll
-            for (int c = 0; c < KC; c += 4) {
+            for (int c = 0; c < KC / 2; c += 4) {
                 f32x2 fb[4][RE / 2];
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
@@ -774,41 +786,58 @@ __device__ __forceinline__ void stage_units_chunked(const Op &op, int i0, int i1
 {
     constexpr int M = C::M, kSlices = M / C::ES, KC = C::KC, kChunks = M / KC;
     unsigned char *stage = smem + C::kStageAt;
-    // where unit i, chunk k is loaded to and from
+    struct Unit {
+        int at, tile_no;
+        __device__ __forceinline__ int b0() const { return at / kSlices * 8; }
+        __device__ __forceinline__ int e0() const { return at % kSlices * C::ES; }
+        __device__ __forceinline__ int t0() const { return tile_no * C::TT; }
+    };
+    auto after = [&](Unit u) { return u.tile_no + 1 == tiles ? Unit{u.at + 1, 0} : Unit{u.at, u.tile_no + 1}; };
     auto tile = [&](int n) { return reinterpret_cast<float *>(smem + (n & 1) * C::kChunk); };
     auto wt = [&](int n) { return reinterpret_cast<float *>(smem + (n & 1) * C::kChunk + C::kChunkA); };
-    auto begin = [&](int n, int i, int k) {
-        const int at = i / tiles, tile_no = i % tiles, b0 = at / kSlices * 8, e0 = at % kSlices * C::ES;
-        load_async<C, C::TT, KC, C::PC, C::kBlockA>(tile(n), op.in, op.perm, b0, k * KC, tile_no * C::TT, tokens - tile_no * C::TT);
-        Chunks<C>::load_w(wt(n), op.w, op.trans, b0, e0, k * KC);
+    auto begin = [&](int n, Unit u, int k) {
+        load_async<C, C::TT, KC, C::PC, C::kBlockA>(tile(n), op.in, op.perm, u.b0(), k * KC, u.t0(), tokens - u.t0());
+        Chunks<C>::load_w(wt(n), op.w, op.trans, u.b0(), u.e0(), k * KC);
     };
     constexpr int kParts = kChunks / 2;
-    auto copy = [&](int i, int part) {
-        const int at = i / tiles, tile_no = i % tiles;
-        copy_part<C, kParts>(stage, op.out, op.perm, at / kSlices * 8, at % kSlices * C::ES, tile_no * C::TT, tokens - tile_no * C::TT, part);
+    auto copy = [&](Unit u, int part) {
+        copy_part<C, kParts>(stage, op.out, op.perm, u.b0(), u.e0(), u.t0(), tokens - u.t0(), part);
     };
+    // Of the four warps of a scheduler two start the next loads before their products and two between the halves of theirs: with
+    // all of them in step the FMAs of a chunk and the address arithmetic of the next one followed one another (forward of 2048
+    // tokens at m = 64 113 -> 106 us, forward + backward at m = 32, 8000 tokens, 226 -> 208; a quarter each: 107 and 209, and at
+    // m = 128, 500 tokens, forward + backward 741 where halves take 711).
+    const int mine = threadIdx.x >> 7 & 1;
     int n = 0;
+    Unit u = {i0 / tiles, i0 % tiles}, last = u;
     __syncthreads();                                   // what ran before has left shared memory
-    begin(0, i0, 0);
+    begin(0, u, 0);
     for (int i = i0; i < i1; ++i) {
         Chunks<C> sums;
         sums.clear();
+        const Unit next = after(u);
 #pragma unroll 1
         for (int k = 0; k < kChunks; ++k, ++n) {
             cp_async_wait();
             __syncthreads();                           // chunk n is here, chunk n - 1 has been read
-            const bool more = k + 1 < kChunks || i + 1 < i1;
-            if (more) begin(n + 1, k + 1 < kChunks ? i : i + 1, k + 1 < kChunks ? k + 1 : 0);
-            // the previous unit's results leave during the first half of this one's products
-            if (i > i0 && k < kParts) copy(i - 1, k);
-            sums.multiply(tile(n), wt(n), op.trans);
+#pragma unroll 1
+            for (int half = 0; half < 2; ++half) {
+                if (half == mine) {
+                    if (k + 1 < kChunks)  begin(n + 1, u, k + 1);
+                    else if (i + 1 < i1)  begin(n + 1, next, 0);
+                    // the previous unit's results leave during the first half of this one's products
+                    if (i > i0 && k < kParts) copy(last, k);
+                }
+                sums.multiply(tile(n), wt(n), op.trans, half);
+            }
         }
-        const int at = i / tiles, tile_no = i % tiles, b0 = at / kSlices * 8, e0 = at % kSlices * C::ES;
         Acc<C> acc;
         sums.finish(acc, op.trans);
-        finish_unit<C>(op, acc, stage, b0, e0, tile_no, tokens);
+        finish_unit<C>(op, acc, stage, u.b0(), u.e0(), u.tile_no, tokens);
+        last = u;
+        u = next;
     }
-    for (int part = 0; part < kParts; ++part) copy(i1 - 1, part);
+    for (int part = 0; part < kParts; ++part) copy(last, part);
 }
 
 // ---------------------------------------------------------------- a weight-gradient unit
@@ -852,7 +881,8 @@ __device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0,
         cp_async_wait();
         __syncthreads();                               // the operands of s are here, those of s - 1 have been read
         const bool early = C::kSteps == 2 && (C::KC > 0 || !op.perm);
-        if (early && s + 1 < s1) load(s + 1);
+        const int mine = C::KC > 0 ? threadIdx.x >> 7 & 1 : 0;    // (as in stage_units_chunked)
+        if (early && s + 1 < s1 && mine == 0) load(s + 1);
         if constexpr (C::kBf) {
             const bf16 *a = tile_a(s & kMask) + (bw * TW + (lane & 7) + (lane >> 4) * 8) * C::PL + (lane >> 3 & 1) * 8;
             // with 8 columns per warp one ldmatrix brings both 16-token steps
@@ -884,6 +914,7 @@ __device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0,
             const float *a = tile_a(s & kMask) + bw * C::kBlockL + (lane >> 3) * RL, *b = tile_b(s & kMask) + bw * C::kBlockK + kw + (lane & 7) * VK;
 #pragma unroll 4
             for (int t = 0; t < TW; ++t) {
+                if (C::KC > 0 && t == TW / 2 && mine == 1 && s + 1 < s1) load(s + 1);
                 float fa[RL], fb[RK];
 #pragma unroll
                 for (int i = 0; i < RL; i += 4) *reinterpret_cast<float4 *>(fa + i) = *reinterpret_cast<const float4 *>(a + t * C::PL + i);
