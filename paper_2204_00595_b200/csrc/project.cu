@@ -216,7 +216,8 @@ int launch_jacobi(const void *A, void *L, void *R, unsigned long long *rotations
 //        their way to the same vector and one of them goes on alone, with S^T S - shift I: the shift is half of what the rate says
 //        of sigma_2^2, which brings the other eigenvalues to both sides of zero.  It has converged when its last move times the
 //        rate at which the moves shrink is below kPowerTol (m = 64 with a clear leading value 128 -> 107 us with the matrix
-//        written out again, 4096 slices; the error against 64 bits stays 1.2e-7).
+//        written out again, 4096 slices; the error against 64 bits stays 1.2e-7).  Not at m = 16, whose 256 slices are one wave
+//        that takes as long as its slowest (noise as large as the leading value: 31.3 us, so 32.9).
 //  2. Otherwise (a small gap) H = S^T S is squared and scaled to trace 1 until it has rank 1 - doubling the exponent
 //     each time, so the cost grows with the logarithm of 1 / gap and is bounded - and any column of H is v_1.  Orthogonal
 //     columns make H diagonal at once.
@@ -345,6 +346,7 @@ template <typename T, int M>
 __global__ void __launch_bounds__(LeadCfg<M>::kThreads)
 leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ R)
 {
+    constexpr bool kAlone = M > 16;                          // step 1a
     using C = LeadCfg<M>;
     constexpr int N = M * M, NT = C::kThreads, W = C::kWarps, P = C::kPitch, RH = C::kRows, CW = C::kCols;
     constexpr float kOnce = (float)M / (NT * C::kZC);     // columns are held 1 / kOnce times over the CTA
@@ -489,7 +491,7 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
             }
             slice_sync<NT>();
             back(std::true_type(), y, y + M, a, b);
-            if ((step & 3) == 3 || step == 1) {
+            if ((step & 3) == 3 || (kAlone && step == 1)) {
                 float v[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
                 for (int i = 0; i < C::kZC; ++i) {
@@ -511,7 +513,7 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
                 }
                 slice_sum<NT>(d, red, phase);
                 constexpr float kStill = kPowerTol * kPowerTol / kOnce;
-                if (step == 1) {
+                if (kAlone && step == 1) {
                     apart = d[0];
                 } else if (!(d[1] >= kStill) && !(d[0] >= kStill)) {
                     done = true;                          // (NaN: nothing to wait for)
@@ -521,7 +523,7 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
                     if (v[1] > v[0])
 #pragma unroll
                         for (int i = 0; i < C::kZC; ++i) a[i] = b[i];
-                } else if (step == 3 && round == 0 && d[0] * kOnce < kNear * kNear && d[0] < kFast * kFast * kFast * kFast * apart) {
+                } else if (kAlone && step == 3 && round == 0 && d[0] * kOnce < kNear * kNear && d[0] < kFast * kFast * kFast * kFast * apart) {
                     shift = 0.5f * sqrtf(sqrtf(v[0] * kOnce * (d[0] / apart)));
                 }
             }
@@ -531,9 +533,9 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
                 x[M + my_col + i] = b[i];
             }
             slice_sync<NT>();
-            if ((done && (step & 3) == 3) || shift >= 0.0f) break;
+            if ((done && (step & 3) == 3) || (kAlone && shift >= 0.0f)) break;
         }
-        if (shift >= 0.0f) {
+        if (kAlone && shift >= 0.0f) {
             float moved = 1.0f / kOnce;
 #pragma unroll 1
             for (++step; step < steps; ++step) {
