@@ -213,7 +213,7 @@ KERNELS_OF = {
     (64, "bf16", "bwd"): "bwd_du_kernel + bwd_dx_kernel + add_parts_m64_kernel (3 launches)",
     (64, "bf16", "bwd_dx"): "bwd_du_kernel + bwd_dx_kernel (2 launches)",
     (64, "bf16", "bwd_dw"): "stage1_kernel + bwd_du_kernel + bwd_dx_kernel without dx + add_parts_m64_kernel (4 launches)",
-    (64, "bf16", "mlp_fwd"): "2 x (stage1_kernel + stage2_kernel) (4 launches)",
+    (64, "bf16", "mlp_fwd"): "3 x stage1_kernel + stage2_kernel (4 launches)",
     (64, "bf16", "mlp_bwd"): "stage1_kernel + stage2_kernel + mlp_act_kernel + stage1_kernel + 2 x (bwd_du_kernel + bwd_dx_kernel + add_parts_m64_kernel) + mlp_dact_kernel (11 launches)",
     (128, "bf16", "fwd"): "chain_fused_fwd_kernel (1 persistent launch; chain_gemm_kernel x 2 + plane_transpose_kernel "
                           "beyond 8192 tiles)",

@@ -1,4 +1,5 @@
 // m = 64 (n = 4096), bf16: forward, backward and feed-forward block as streaming launches, one per block-diagonal stage.
+// Small forwards and blocks run on clusters of eight CTAs instead, one launch per multiply (further down).
 //
 // The weights of a stage are 512 KB, so an SM cannot hold both stages and every block of stage 2 needs a row of every block
 // of stage 1: the intermediate has to cross SMs.  Each launch is one stage for all tokens: a CTA keeps the weights of its 16
