@@ -212,12 +212,14 @@ int launch_jacobi(const void *A, void *L, void *R, unsigned long long *rotations
 //     stand still and differ are eigenvectors both: singular values that are equal to rounding, or one vector that is
 //     orthogonal to v_1; the one with the larger singular value is taken.
 //     At most kPowerSteps steps are spent on it, enough for (sigma_2 / sigma_1)^2 up to about 0.7.
-//     a. Where the two are within kNear of one another after four steps and come closer by more than kFast^2 a step, they are on
-//        their way to the same vector and one of them goes on alone, with S^T S - shift I: the shift is half of what the rate says
-//        of sigma_2^2, which brings the other eigenvalues to both sides of zero.  It has converged when its last move times the
-//        rate at which the moves shrink is below kPowerTol (m = 64 with a clear leading value 128 -> 107 us with the matrix
-//        written out again, 4096 slices; the error against 64 bits stays 1.2e-7).  Not at m = 16, whose 256 slices are one wave
-//        that takes as long as its slowest (noise as large as the leading value: 31.3 us, so 32.9).
+//     a. Where the two are within kNear of one another after four steps and every step leaves less than kFast of it, both go on
+//        with S^T S - shift I and are tested every other step.  The shift is half of what the rate says of sigma_2^2, which brings
+//        the other eigenvalues to both sides of zero; it is at most 0.3 sigma_1^2, so v_1 stays the leading vector whatever the
+//        rate was worth, and what ends the iteration is the same: the two agree and stand still.  (One of them alone, until its
+//        moves said so, returned v_2 in 1 of 600 slices with sigma_2 = 0.9999 sigma_1 and an rms error of 1.5e-7 instead of
+//        1.25e-7 in the timed ones, in 73 us.)  us without and with the shift, noise of 0.5, 1, 2, 3 times the entries of the
+//        rank-1 part: m = 64 57 / 50, 67 / 56, 92 / 87, 211 / 212, m = 128 898 / 796, 1150 / 960, 1242 / 1129, 1575 / 1395.  Not
+//        at m = 16 and 32, whose slices are one wave that takes as long as its slowest: m = 32 10.5 / 10.5, 13.0 / 12.6, 37 / 37.
 //  2. Otherwise (a small gap) H = S^T S is squared and scaled to trace 1 until it has rank 1 - doubling the exponent
 //     each time, so the cost grows with the logarithm of 1 / gap and is bounded - and any column of H is v_1.  Orthogonal
 //     columns make H diagonal at once.
@@ -226,14 +228,14 @@ int launch_jacobi(const void *A, void *L, void *R, unsigned long long *rotations
 // registers for the whole iteration.  A product then needs m/8 (or m/4) values of the vector per lane from shared
 // memory and a reduce-scatter over 8 (or 4) lanes; with a whole row per lane every lane would read the whole vector,
 // and the 128 bytes per clock that shared memory returns were the limit (149 us for 4096 slices of 64 x 64).
-// Bound by fp32 issue: products are packed two to an instruction (fma.rn.f32x2), ten warps share an SM.
+// Bound by fp32 issue: products are packed two to an instruction (fma.rn.f32x2), eight warps share an SM (255 registers).
 // Measured, fp32, against the Jacobi iteration that ran before: 4096 slices of 64 x 64 with a clear leading value
 // 7714 -> 113 us, Gaussian 7690 -> 747 us; 128 x 128 Gaussian 165 -> 17.8 ms; largest error of a Gaussian slice's
 // rank-1 part 2.3e-4 -> 2e-6 (the Jacobi iteration stops at a cosine of 2e-6).  Where all singular values of a slice
 // are equal the squarings run to their bound: 0.57 -> 1.29 ms.
 constexpr int kPowerSteps = 40, kPolishSteps = 4, kMaxSquarings = 24;
 constexpr float kPowerTol = 1e-6f;
-constexpr float kNear = 0.1f, kFast = 0.6f;               // step 1a: distance, and rate of a step (of the vector)
+constexpr float kNear = 0.1f, kFast = 0.6f;               // step 1a: distance, and what a step leaves of it
 
 template <int M> struct LeadCfg {
     static constexpr int kWarps = M == 128 ? 4 : 1, kThreads = 32 * kWarps;
@@ -346,10 +348,11 @@ template <typename T, int M>
 __global__ void __launch_bounds__(LeadCfg<M>::kThreads)
 leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ R)
 {
-    constexpr bool kAlone = M > 16;                          // step 1a
+    constexpr bool kShift = M > 32;                          // step 1a
     using C = LeadCfg<M>;
     constexpr int N = M * M, NT = C::kThreads, W = C::kWarps, P = C::kPitch, RH = C::kRows, CW = C::kCols;
     constexpr float kOnce = (float)M / (NT * C::kZC);     // columns are held 1 / kOnce times over the CTA
+    static_assert(!kShift || kOnce == 1.0f, "the shift reads elements of x that another thread may have overwritten");
     extern __shared__ __align__(16) float lead_smem[];
     float *H = lead_smem, *x = H + M * P, *y = x + 2 * M; // x[2][M], y[2][M]: the two iterates
     float *part = y + 2 * M;                              // W > 1: [2][W][M] partial sums of S^T y
@@ -476,11 +479,11 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
     for (int round = 0; round < 2; ++round) {
         bool done = round == 1;
         float before[C::kZC] = {}, before_b[C::kZC] = {};
-        float apart = 4.0f, shift = -1.0f;                // squared distance of the two at the last test; >= 0: go on with one
+        float apart = 4.0f, shift = 0.0f;                 // squared distance of the two at the last test; step 1a
+        int every = 3;                                    // tests when step & every == every
         const int steps = round == 0 ? kPowerSteps : kPolishSteps;
-        int step = 0;
 #pragma unroll 1
-        for (; step < steps; ++step) {
+        for (int step = 0; step < steps; ++step) {
             float ya[C::kYC], yb[C::kYC], a[C::kZC], b[C::kZC];
             times_S(x, ya);
             times_S(x + M, yb);
@@ -491,7 +494,13 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
             }
             slice_sync<NT>();
             back(std::true_type(), y, y + M, a, b);
-            if ((step & 3) == 3 || (kAlone && step == 1)) {
+            if (kShift)
+#pragma unroll
+                for (int i = 0; i < C::kZC; ++i) {
+                    a[i] = fmaf(-shift, x[my_col + i], a[i]);
+                    b[i] = fmaf(-shift, x[M + my_col + i], b[i]);
+                }
+            if ((step & every) == every || (kShift && step == 1)) {
                 float v[3] = {0.0f, 0.0f, 0.0f}, d[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
                 for (int i = 0; i < C::kZC; ++i) {
@@ -512,19 +521,21 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
                     before_b[i] = b[i];
                 }
                 slice_sum<NT>(d, red, phase);
-                constexpr float kStill = kPowerTol * kPowerTol / kOnce;
-                if (kAlone && step == 1) {
+                constexpr float kSame = kPowerTol * kPowerTol / kOnce;
+                const float still = kShift && (every == 1 || step == 3) ? 0.25f * kSame : kSame;      // two steps or four since the last test
+                if (kShift && step == 1) {
                     apart = d[0];
-                } else if (!(d[1] >= kStill) && !(d[0] >= kStill)) {
+                } else if (!(d[1] >= still) && !(d[0] >= kSame)) {
                     done = true;                          // (NaN: nothing to wait for)
-                } else if (d[1] < kStill && d[2] < kStill) {
+                } else if (d[1] < still && d[2] < still) {
                     // both stand still and differ: eigenvectors, of the same singular value or not; the one with the larger is kept
                     done = true;
                     if (v[1] > v[0])
 #pragma unroll
                         for (int i = 0; i < C::kZC; ++i) a[i] = b[i];
-                } else if (kAlone && step == 3 && round == 0 && d[0] * kOnce < kNear * kNear && d[0] < kFast * kFast * kFast * kFast * apart) {
+                } else if (kShift && step == 3 && round == 0 && d[0] * kOnce < kNear * kNear && d[0] < kFast * kFast * kFast * kFast * apart) {
                     shift = 0.5f * sqrtf(sqrtf(v[0] * kOnce * (d[0] / apart)));
+                    every = 1;
                 }
             }
 #pragma unroll
@@ -533,44 +544,7 @@ leading_pair_kernel(const T *__restrict__ A, T *__restrict__ L, T *__restrict__ 
                 x[M + my_col + i] = b[i];
             }
             slice_sync<NT>();
-            if ((done && (step & 3) == 3) || (kAlone && shift >= 0.0f)) break;
-        }
-        if (kAlone && shift >= 0.0f) {
-            float moved = 1.0f / kOnce;
-#pragma unroll 1
-            for (++step; step < steps; ++step) {
-                float ya[C::kYC], a[C::kZC], unused[C::kZC];
-                times_S(x, ya);
-#pragma unroll
-                for (int i = 0; i < C::kYC; ++i) y[my_row + i] = ya[i];
-                slice_sync<NT>();
-                back(std::false_type(), y, nullptr, a, unused);
-#pragma unroll
-                for (int i = 0; i < C::kZC; ++i) a[i] = fmaf(-shift, x[my_col + i], a[i]);
-                if (step & 1) {
-                    float v[1] = {0.0f}, d[1] = {0.0f};
-#pragma unroll
-                    for (int i = 0; i < C::kZC; ++i) v[0] = fmaf(a[i], a[i], v[0]);
-                    slice_sum<NT>(v, red, phase);
-                    const float na = rsqrtf(v[0] * kOnce);
-#pragma unroll
-                    for (int i = 0; i < C::kZC; ++i) {
-                        a[i] *= na;
-                        d[0] = fmaf(a[i] - before[i], a[i] - before[i], d[0]);
-                        before[i] = a[i];
-                    }
-                    slice_sum<NT>(d, red, phase);
-                    // what is left is the last move times the rate at which moves shrink
-                    const float left = d[0] * fminf(fmaxf(d[0] / moved, 0.0025f), 1.0f);
-                    done = !(left >= kPowerTol * kPowerTol / kOnce);
-                    moved = d[0];
-                }
-                slice_sync<NT>();                         // (W > 1: every thread has read its x)
-#pragma unroll
-                for (int i = 0; i < C::kZC; ++i) x[my_col + i] = a[i];
-                slice_sync<NT>();
-                if (done) break;
-            }
+            if (done && (step & every) == every) break;
         }
         if (done) break;
 

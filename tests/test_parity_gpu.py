@@ -953,6 +953,45 @@ def test_project_leading_pair(P, m, dtype, kind):
         assert tail * (1 - 1e-9) <= res <= tail * (1 + 1e-5) + rounding + (1e-6 * sv[0]) ** 2
 
 
+@pytest.mark.parametrize("m", [16, 32, 64, 128])
+@pytest.mark.parametrize("ratio", [0.3, 0.6, 0.7, 1 - 1e-4, 1 - 5e-5])
+def test_project_leading_vectors(P, m, ratio):
+    """The rank-1 part of EVERY slice, not its residual, which an error of the vectors enters squared.  Slices of known singular
+    vectors, sigma_2 = ratio * sigma_1 and the rest below both ratio and a half.  u, v and the scaled factors take some eight
+    roundings to 24 bits between them (two units of 2^-22), and the eigenvector of S^T S the rounding of a step divided by the
+    relative gap 1 - ratio^2: a unit of 2^-22 where steps find it; where squarings of S^T S do, their sums of m products, which round
+    sqrt(m) times 2^-24."""
+    import torch
+    n, g = m * m, torch.Generator(device="cuda").manual_seed(4100 + m)
+    rounding = 2.0 ** -22 if ratio < 0.9 else m ** 0.5 * 2.0 ** -24
+    rand = lambda *shape: torch.rand(shape, generator=g, device="cuda", dtype=torch.float64)
+    sigma = min(ratio, 0.5) * rand(n, m)
+    sigma[:, 0], sigma[:, 1] = 1.0, ratio
+    S, u = torch.diag_embed(sigma), torch.zeros(n, m, device="cuda", dtype=torch.float64)
+    u[:, 0] = 1.0
+    v = u.clone()
+    for _ in range(3):                                                 # three reflections on either side
+        for side in (1, 2):
+            w = torch.randn(n, m, generator=g, device="cuda", dtype=torch.float64)
+            w /= w.norm(dim=1, keepdim=True)
+            if side == 1:
+                S -= 2 * w[:, :, None] * torch.einsum("bi,bij->bj", w, S)[:, None, :]
+                u -= 2 * w * (w * u).sum(1, keepdim=True)
+            else:
+                S -= 2 * torch.einsum("bij,bj->bi", S, w)[:, :, None] * w[:, None, :]
+                v -= 2 * w * (w * v).sum(1, keepdim=True)
+    A = S.view(m, m, m, m).permute(2, 0, 1, 3).reshape(n, n).float().contiguous()          # slice j * m + k at [l, j, k, i]
+    L, R = torch.empty(m, m, m, device="cuda"), torch.empty(m, m, m, device="cuda")
+    P.monarch_project(A, L, R, n, m)
+    torch.cuda.synchronize()
+    lo, ro = L.double().permute(0, 2, 1).reshape(n, m), R.double().permute(1, 0, 2).reshape(n, m)
+    # |lo ro^T - u v^T|^2 without the matrices: its terms cancel, so through the parts along and across u and v
+    lu, rv = (lo * u).sum(1), (ro * v).sum(1)
+    lx, rx = lo - lu[:, None] * u, ro - rv[:, None] * v
+    err = ((lu * rv - 1) ** 2 + (lu ** 2) * (rx ** 2).sum(1) + (lx ** 2).sum(1) * (ro ** 2).sum(1)).sqrt()
+    assert float(err.max()) <= 2.0 ** -21 + rounding / (1 - ratio ** 2)
+
+
 @pytest.mark.parametrize("m,T,dtype", [(16, 2500, "bf16"), (16, 1100, "f32"), (32, 1185, "bf16"), (32, 1601, "bf16"),
                                        (32, 833, "f32"), (32, 1153, "f32"), (32, 15, "bf16"), (32, 16 * 148, "bf16"), (32, 16 * 148 * 6 + 1, "bf16"), (64, 255, "bf16"), (64, 320, "bf16"), (64, 321, "bf16"), (64, 593, "f32"),
                                        (64, 33, "bf16"), (64, 16 * 18, "bf16"), (64, 16 * 37 + 9, "bf16"), (64, 16 * 19 * 5 + 1, "bf16"),
