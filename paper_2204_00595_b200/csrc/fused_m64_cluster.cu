@@ -226,7 +226,7 @@ fused_fwd_m64_cluster_kernel(const __grid_constant__ CUtensorMap tm_x, const __g
             for (int it = 0; it < nt; ++it) {
                 mbar_expect_tx(ufull, kRemoteBytes);
                 if (!mbar_wait(udone, it & 1, p.status, dead, kErrMmaWait)) break;
-                for (uint32_t d = 0; d < kCluster; ++d) mbar_arrive_remote(map_to_cta(ufree, d));
+                for (uint32_t d = 0; d < kCluster; ++d) mbar_arrive_cluster(map_to_cta(ufree, d));
             }
         }
     } else {

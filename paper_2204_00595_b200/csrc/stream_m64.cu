@@ -437,7 +437,7 @@ constexpr int kCl = 8, kHalfWarps = kWarps / 2;
 constexpr int kClX = 3, kClE = 4, kClV = 3, kClY = 3;        // tiles of 16 KB: input slots, exchange slots, w, results
 constexpr int kClSmem = (kClX + kClE + 1 + kClV + kClY) * kBwdTile + 1024;
 struct ClusterShared {
-    uint64_t x_full[kClX], x_read[kClX], e_full[kClE], e_free[kClE], across[kClV], staged[8], sent[kClV + kClY], w_full;
+    uint64_t x_full[kClX], x_read[kClX], e_full[kClE], e_read[kClE], e_free[kClE], across[kClV], staged[8], sent[kClV + kClY], w_full;
     int dead;
 };
 
@@ -464,6 +464,10 @@ fwd_cluster_kernel(const __grid_constant__ CUtensorMap tm_R, const __grid_consta
     // by one lane, or by a warp, whose lanes all learn if one ran out: the warp then does nothing more
     auto wait1 = [&](const uint64_t &bar, int phase, unsigned code) { return mbar_wait(smem_u32(&bar), phase & 1, p.status, &s.dead, code); };
     auto wait = [&](const uint64_t &bar, int phase, unsigned code) { return __all_sync(0xffffffffu, wait1(bar, phase, code)) != 0; };
+    // the same on what the other CTAs of the cluster arrive at
+    auto wait_cluster = [&](const uint64_t &bar, int phase) {
+        return __all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&bar), phase & 1, p.status, &s.dead, kErrPeerWait)) != 0;
+    };
     auto turn = [&](int k) { return lane == 0 && (k & (kHalfWarps - 1)) == w; };
     auto arrive = [&](uint64_t &bar) {
         __syncwarp();
@@ -482,7 +486,8 @@ fwd_cluster_kernel(const __grid_constant__ CUtensorMap tm_R, const __grid_consta
         for (uint64_t &b : s.x_full) mbar_init(smem_u32(&b), 1);
         for (uint64_t &b : s.x_read) mbar_init(smem_u32(&b), kHalfWarps);
         for (uint64_t &b : s.e_full) mbar_init(smem_u32(&b), 1);
-        for (uint64_t &b : s.e_free) mbar_init(smem_u32(&b), kCl * kHalfWarps);
+        for (uint64_t &b : s.e_read) mbar_init(smem_u32(&b), kHalfWarps);
+        for (uint64_t &b : s.e_free) mbar_init(smem_u32(&b), kCl);
         for (uint64_t &b : s.across) mbar_init(smem_u32(&b), kHalfWarps);
         for (uint64_t &b : s.staged) mbar_init(smem_u32(&b), kHalfWarps);
         for (uint64_t &b : s.sent) mbar_init(smem_u32(&b), 1);
@@ -542,7 +547,7 @@ fwd_cluster_kernel(const __grid_constant__ CUtensorMap tm_R, const __grid_consta
                     stm4(mine + h * 1024 + (n * 32 + ln.m * 8 + ln.r) * 16, pack_bf16(a0[0], a0[1]), pack_bf16(a0[2], a0[3]),
                          pack_bf16(a1[0], a1[1]), pack_bf16(a1[2], a1[3]));
                 }
-            if (i >= kClE && !wait(s.e_free[i % kClE], i / kClE - 1, kErrPeerWait)) break;
+            if (i >= kClE && !wait_cluster(s.e_free[i % kClE], i / kClE - 1)) break;
             __syncwarp();
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -555,13 +560,20 @@ fwd_cluster_kernel(const __grid_constant__ CUtensorMap tm_R, const __grid_consta
     } else {
         // ---- stage 2: w_j = L_j u_j
         const uint32_t peer_free = map_to_cta(smem_u32(s.e_free), lane & (kCl - 1));
-        auto release = [&](int i) { mbar_arrive_remote(peer_free + i % kClE * 8); };         // by eight lanes, one per CTA
+        // Hands tile i's slot back to the eight CTAs, which overwrite it: a release at cluster scope of what this CTA's warps have
+        // read, by eight lanes of one warp once they all have.  It costs that warp some 0.5 us, so not by every warp (forward of 1200
+        // tokens 16.2 us, 12.9 so), and only where the slot is filled again.
+        auto release = [&](int i) {
+            if (!wait(s.e_read[i % kClE], i / kClE, kErrMmaWait)) return false;
+            if (lane < kCl) mbar_arrive_cluster(peer_free + i % kClE * 8);
+            return true;
+        };
         Bias bias;
         if (BIAS) bias.load(p.bias, own);
         // put(h, four words of rows 0 .. 31 or 32 .. 63 x 8 tokens, n)
         auto multiply = [&](int i, auto put) {
             const uint32_t e = E0 + i % kClE * kBwdTile;
-            if (!__all_sync(0xffffffffu, mbar_wait<true>(smem_u32(&s.e_full[i % kClE]), i / kClE & 1, p.status, &s.dead, kErrPeerWait))) return false;
+            if (!wait_cluster(s.e_full[i % kClE], i / kClE)) return false;
             if (threadIdx.x == kHalfWarps * 32 && i + kClE < count) mbar_expect_tx(smem_u32(&s.e_full[i % kClE]), kBwdTile);
             const bool saves = SAVE && turn(i + 4);
             if (saves) {
@@ -591,13 +603,13 @@ fwd_cluster_kernel(const __grid_constant__ CUtensorMap tm_R, const __grid_consta
                 }
                 if (!put(h, o)) return false;
             }
-            // (after the products: the tile is in registers.)  A saved tile is released once its copy has read it, a tile later.
-            if (SAVE && i > 0 && w == ((i + 3) & (kHalfWarps - 1))) {
-                if (lane == 0) tma_store_wait_read<0>();
+            // (after the products: the tile is in registers)  By turns, a tile later: the others have read it, and so has its copy.
+            arrive(s.e_read[i % kClE]);
+            if (i > 0 && w == ((i + 3) & (kHalfWarps - 1))) {
+                if (SAVE && lane == 0) tma_store_wait_read<0>();
                 __syncwarp();
-                if (lane < kCl) release(i - 1);
+                if (i - 1 + kClE < count && !release(i - 1)) return false;
             }
-            if ((!SAVE || w != ((i + 4) & (kHalfWarps - 1))) && lane < kCl) release(i);
             return true;
         };
         auto send = [&](int i) {

@@ -68,7 +68,8 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar)
                  : "memory");
 }
 // The same with the default (CTA-scope release) semantics: what a handshake needs that carries no data through
-// shared or global memory (e.g. "I have finished reading my TMEM"); the cluster-scope release costs about 1 us.
+// shared or global memory (e.g. "I have finished reading my TMEM"); the cluster-scope release costs about 1 us.  Not for shared
+// memory that the other CTA overwrites next.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_bar)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");

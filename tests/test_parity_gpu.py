@@ -1475,6 +1475,40 @@ def test_fwd_m64_rounds_of_clusters(P, T):
     _check_guard(yf, "mlp y")
 
 
+# CTAs with one tile more than they have exchange slots, up to ten tiles; the block also where the forward takes the streams
+@pytest.mark.parametrize("T", [961, 1200, 2399])
+def test_clusters_reuse_their_exchange_slots(P, T):
+    """A slot that is handed back and filled again holds what a call whose CTAs use each slot once holds: the same bits of y, u (as
+    the weight gradients see it) and the block's y."""
+    import torch
+    m, n, code, part = 64, 4096, P.BF16, 240
+    d = _small_inputs(m, T, "bf16", seed=8900 + T)
+    x, dy, L, R, L2, R2, b1, b2 = (to_device(d[k], "bf16") for k in ("x", "dy", "L", "R", "L2", "R2", "b1", "b2"))
+    ws, ws_b, ws_m = (P.Workspace(P.monarch_workspace_bytes(op, T, n, m, code)) for op in (P.OP_FWD, P.OP_BWD, P.OP_MLP_FWD))
+    y, want, dx = (torch.empty_like(x) for _ in range(3))
+    for t0 in range(0, T, part):
+        t = min(part, T - t0)
+        P.monarch_fwd(x[t0:t0 + t], L, R, want[t0:t0 + t], t, n, m, ws)
+    for _ in range(4):
+        y.fill_(float("nan"))
+        P.monarch_fwd(x, L, R, y, T, n, m, ws)
+        grads = []
+        for saved in (ws, None):
+            grads.append([torch.empty(m, m, m, device="cuda") for _ in range(2)])
+            P.monarch_bwd(x, dy, L, R, dx, *grads[-1], 0, T, n, m, ws_b, fwd_workspace=saved)
+        torch.cuda.synchronize()
+        assert torch.equal(y, want) and all(torch.equal(a, b) for a, b in zip(*grads))
+    for t0 in range(0, T, part):
+        t = min(part, T - t0)
+        P.monarch_mlp_fwd(x[t0:t0 + t], L, R, b1, L2, R2, b2, want[t0:t0 + t], t, n, m, ws_m)
+    for _ in range(4):
+        y.fill_(float("nan"))
+        P.monarch_mlp_fwd(x, L, R, b1, L2, R2, b2, y, T, n, m, ws_m)
+        torch.cuda.synchronize()
+        assert torch.equal(y, want)
+    assert all(P.monarch_last_device_status(w) == 0 for w in (ws, ws_b, ws_m))
+
+
 @pytest.mark.parametrize("item", [0, 2])
 @pytest.mark.parametrize("call", ["fwd", "mlp"])
 def test_tile_that_never_arrives_on_clusters(P, call, item):
