@@ -576,6 +576,7 @@ __device__ __forceinline__ void load_async(float *tile, const View &v, int perm,
 // it packs two outputs.
 template <typename C> struct Chunks {
     static constexpr int TT = C::TT, ES = C::ES, KC = C::KC, PC = C::PC, M = C::M, EW = C::EW, RT = TT / 4, RE = EW / 8;
+    static_assert(KC % 8 == 0, "a half of a chunk is multiplied four columns at a time");
     f32x2 s[RT][RE];                                   // [out][in]: sums over even and odd columns; else [RT][RE / 2] used
 
     __device__ __forceinline__ void clear()
@@ -853,6 +854,7 @@ __device__ __forceinline__ void wgrad_unit(const Op &op, int b0, int l0, int k0,
     float *dst = op.sums + (op.splits > 1 ? (size_t)split * M * M * M : 0) + (size_t)(b0 + bw) * M * M + (size_t)l0 * M + k0 + kw;
     const bool add = op.splits == 1 && op.accumulate;
     constexpr int kMask = C::kSteps - 1;
+    static_assert(C::KC == 0 || (C::kSteps == 2 && !C::kBf && C::TW > 1), "half of the warps load in the middle of a step, into the other buffer");
     TileLoad<C, TW, LS, C::PL> load_a;
     TileLoad<C, TW, KS, C::PK> load_b;
     auto tile_a = [&](int buf) { return reinterpret_cast<T *>(smem + buf * C::kStepBytes); };
