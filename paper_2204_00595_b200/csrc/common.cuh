@@ -220,7 +220,7 @@ int fused_bwd_m32(const void *x, const void *dy, const void *L, const void *R, v
 // ---- m = 64, bf16: one streaming launch per stage (stream_m64.cu) ----
 size_t fused_fwd_m64_workspace_bytes(int64_t tokens);
 int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s);
-// where the forward keeps u inside its workspace (null: nowhere)
+// where the forward keeps u inside its workspace
 const void *fused_fwd_m64_saved_u(const void *fwd_ws);
 // one pass y = M x + bias; workspace of fused_fwd_m64 (u stays behind)
 int fused_fwd_bias_m64(const void *x, const void *L, const void *R, const void *bias, void *y, int64_t tokens, void *ws, void *status,
@@ -235,10 +235,6 @@ int fused_bwd_dx_m64(const void *dy, const void *L, const void *R, void *dx, int
 size_t fused_bwd_m64_workspace_bytes(int64_t tokens);
 int fused_bwd_m64(const void *x, const void *dy, const void *L, const void *R, const void *u_saved, void *dx, float *dL, float *dR,
                   int accumulate, int64_t tokens, void *ws, cudaStream_t s);
-// the forward on clusters of four CTAs with the intermediate in distributed shared memory (fused_m64_cluster.cu), selected by
-// MONARCH_M64_CLUSTER; MONARCH_ERR_UNSUPPORTED when the device cannot host such a cluster
-int fused_fwd_m64_cluster(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s);
-bool fused_fwd_m64_on_clusters();
 
 // ---- general (rectangular) Monarch multiply on the CUDA cores (rect_simt.cu); workspace = [status][u] ----
 size_t rect_workspace_bytes(int64_t tokens, int q, int b, int dtype);

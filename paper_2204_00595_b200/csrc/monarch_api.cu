@@ -132,14 +132,14 @@ int64_t units_limit(int op, int m, int dtype)
     return mlp ? 24 : mlp_bwd ? 32 : 0;
 }
 
-// (the switches that ask for a particular form of the other kernels keep their meaning at every size)
+// (a switch that asks for a particular form of the other kernels keeps its meaning at every size)
 bool use_units(int op, int m, int dtype, int64_t tokens)
 {
     // m = 16 forwards (fused_m16.cu): in bf16 the units would round u, which that kernel keeps in fp32; the smallest in fp32 fit one
     // CTA, which needs no barrier
     if (m == 16 && op == MONARCH_OP_FWD && (dtype == MONARCH_BF16 || tokens <= 256)) return false;
     return g_impl.load(std::memory_order_relaxed) == MONARCH_IMPL_AUTO && tokens > 0 && tokens <= units_limit(op, m, dtype) &&
-           !(m == 64 && fused_fwd_m64_on_clusters()) && !(m == 128 && chain_fwd_m128_split());
+           !(m == 128 && chain_fwd_m128_split());
 }
 
 // grows with the tokens: a workspace sized for a batch serves every smaller one, whichever kernels run it
@@ -552,7 +552,7 @@ int monarch_cplx_fwd(const void *x, const void *L, const void *R, void *y, int a
     const Range out[] = {{y, 2 * plane}};
     const size_t need = monarch_workspace_bytes(MONARCH_OP_CPLX, tokens, n, m, dtype);
     MONARCH_TRY(check_buffers(in, 3, out, 1, workspace, workspace_bytes, need));
-    if (m == 64 && dtype == MONARCH_BF16 && pick(MONARCH_OP_FWD, m, dtype) == kFused && !fused_fwd_m64_on_clusters())
+    if (m == 64 && dtype == MONARCH_BF16 && pick(MONARCH_OP_FWD, m, dtype) == kFused)
         return fused_cplx_m64(x, L, R, y, adjoint, tokens, workspace, (cudaStream_t)stream);
     const size_t res = round256(2 * plane);
     const size_t inner = need - 4 * res;

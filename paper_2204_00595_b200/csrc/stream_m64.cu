@@ -1330,20 +1330,11 @@ constexpr size_t kHead = MONARCH_STATUS_BYTES + 65536;
 char *head(const void *ws) { return (char *)ws + kHead; }
 }  // namespace
 
-size_t fused_fwd_m64_workspace_bytes(int64_t tokens)
-{
-    // at least 1 MB: the forward on clusters keeps its weight images where the E tiles start
-    return kHead + tc::e_bytes(tokens < 128 ? 128 : tokens);
-}
-const void *fused_fwd_m64_saved_u(const void *fwd_ws) { return fused_fwd_m64_on_clusters() ? nullptr : head(fwd_ws); }
+size_t fused_fwd_m64_workspace_bytes(int64_t tokens) { return kHead + tc::e_bytes(tokens); }
+const void *fused_fwd_m64_saved_u(const void *fwd_ws) { return head(fwd_ws); }
 
 int fused_fwd_m64(const void *x, const void *L, const void *R, void *y, int64_t tokens, void *ws, cudaStream_t s)
 {
-    if (tokens == 0) return MONARCH_OK;
-    if (fused_fwd_m64_on_clusters()) {
-        const int st = fused_fwd_m64_cluster(x, L, R, y, tokens, ws, s);
-        if (st != MONARCH_ERR_UNSUPPORTED) return st;
-    }
     return stream_fwd(x, L, R, nullptr, y, head(ws), tokens, (unsigned *)ws, s);
 }
 // (the status word is the caller's: `ws` is not initialised)
