@@ -225,14 +225,14 @@ _W3 = "profiles/stream_kernels_ncu.md, full size, cold L2 per launch (upper boun
 _W4 = "profiles/chain_m128_workload4_ncu.md, full size, cold L2 per launch (upper bound)"
 NCU_TRAFFIC_MB = {
     (1, "fwd"): (0.1, "profiles/fused_fwd_m16_workload1_ncu.md, full size; the 65 KB output is still in L2 at kernel end"),
-    (2, "fwd"): (34.1, "profiles/stream_kernels_ncu.md, full size; the 33.6 MB output is still in L2 at kernel end"),
-    (3, "fwd"): (164.9, _W3),
-    (3, "bwd"): (387.7, _W3),
+    (2, "fwd"): (33.8, "profiles/stream_kernels_ncu.md, full size; the 33.6 MB output is still in L2 at kernel end"),
+    (3, "fwd"): (164.8, _W3),
+    (3, "bwd"): (388.0, _W3),
     (4, "fwd"): (460.8, _W4),
     (4, "bwd"): (924.8, _W4),
     (4, "bwd_dx"): (637.8, _W4),
     (4, "bwd_dw"): (1055.3, _W4),
-    (5, "mlp_fwd"): (1933.0, _W3),
+    (5, "mlp_fwd"): (1926.2, _W3),
 }
 
 

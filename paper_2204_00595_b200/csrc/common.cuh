@@ -114,9 +114,9 @@ static __device__ __forceinline__ float gelu_fast(float a)
 }
 
 // The same for two values, bit for bit, with packed instructions where there are any: 12 to issue instead of 18 (block of 4000
-// tokens at m = 128: 247 -> 241 us; m = 32, 16000 tokens: 40.6 -> 40.0; the m = 64 kernel, which holds its weights in
-// registers, was slower with the pairs: 389 against 384).  One reciprocal for both, of the product of their denominators, takes
-// more instructions and cost 5 % at m = 64 and 18 % at m = 128.
+// tokens at m = 128: 247 -> 241 us; m = 32, 16000 tokens: 40.6 -> 40.0; m = 64, where the GELU stands between the products of the
+// middle launch, 32768 tokens: 391 -> 381).  One reciprocal for both, of the product of their denominators, takes more
+// instructions: nothing gained at m = 64 (391), 18 % lost at m = 128.
 static __device__ __forceinline__ void gelu_fast2(float &a, float &b)
 {
     asm("{\n\t"

@@ -17,9 +17,9 @@
 //   backward:  z = P dy     T tile -> E tile [j][l];   du = L_j^T z_j -> E tile [k][j];   dx = R_k^T du_k -> T tile
 //              dL_j = sum_t z_j u_j^T, dR_k = sum_t du_k x_k^T: tokens are the contraction, both operands as they lie
 // Shared memory moves 16 to 18 KB per token at 128 bytes per clock, no access has a bank conflict.
-// Measured, back to back: forward 16384 tokens 29.2 -> 15.6 us (3.4 of it when the weights came to be loaded by TMA), 1000 tokens
-// 14.5 -> 6.6; forward + backward 4999 tokens 103 -> 31, 16384 tokens 62 (the staged chain of nine
-// launches took 219 as units and more as tcgen05 stages); feed-forward block 16384 tokens 167 -> 40.
+// Measured, back to back: forward 16384 tokens 29.2 -> 15.5 us (3.4 of it when the weights came to be loaded by TMA), 1000 tokens
+// 14.5 -> 4.9; forward + backward 4999 tokens 103 -> 30.5, 16384 tokens 61 (the staged chain of nine
+// launches took 219 as units and more as tcgen05 stages); feed-forward block 16384 tokens 167 -> 36.
 //
 // Backward CTAs are of three kinds, dL, dR and dx: the sums of one gradient are 128 KB of accumulators, half the
 // registers of an SM, and a kind needs one or two sets of weights beside them.  u and du are recomputed by the kind that

@@ -229,10 +229,10 @@ int launch_jacobi(const void *A, void *L, void *R, unsigned long long *rotations
 // memory and a reduce-scatter over 8 (or 4) lanes; with a whole row per lane every lane would read the whole vector,
 // and the 128 bytes per clock that shared memory returns were the limit (149 us for 4096 slices of 64 x 64).
 // Bound by fp32 issue: products are packed two to an instruction (fma.rn.f32x2), eight warps share an SM (255 registers).
-// Measured, fp32, against the Jacobi iteration that ran before: 4096 slices of 64 x 64 with a clear leading value
-// 7714 -> 113 us, Gaussian 7690 -> 747 us; 128 x 128 Gaussian 165 -> 17.8 ms; largest error of a Gaussian slice's
-// rank-1 part 2.3e-4 -> 2e-6 (the Jacobi iteration stops at a cosine of 2e-6).  Where all singular values of a slice
-// are equal the squarings run to their bound: 0.57 -> 1.29 ms.
+// Measured, fp32, against the Jacobi iteration: 4096 slices of 64 x 64 with a clear leading value 7714 -> 87 us, Gaussian
+// 7690 -> 731 us; 128 x 128 Gaussian 165 -> 18.1 ms; largest error of a Gaussian slice's rank-1 part 2.3e-4 -> 2e-6 (the Jacobi
+// iteration stops at a cosine of 2e-6).  Where the columns of a slice are orthogonal up to rounding the squarings run to their
+// bound: 0.57 -> 1.29 ms (exactly orthogonal ones of equal length 35 us).
 constexpr int kPowerSteps = 40, kPolishSteps = 4, kMaxSquarings = 24;
 constexpr float kPowerTol = 1e-6f;
 constexpr float kNear = 0.1f, kFast = 0.6f;               // step 1a: distance, and what a step leaves of it

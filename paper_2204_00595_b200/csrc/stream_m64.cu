@@ -425,14 +425,14 @@ stage2_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 // 7: R, the others: L), and u crosses through distributed shared memory: each warp of stage 1 sends a consumer CTA 256 bytes per
 // tile, asynchronously and counted on its barrier, which land as the CTA's 16 KB of an E tile.  So x and y make their one trip and
 // u, where the backward call wants it, one more as linear copies.  For small batches, which the two launches of the streams cost
-// most (forward of 64 tokens 9.1 -> 6.7 us, block 18.6 -> 12.5 where it was four phases of one launch over units).
+// most (forward of 64 tokens 9.1 -> 6.9 us, block 18.6 -> 12.3 where it was four phases of one launch over units).
 // What bounds it, cycles per 16-token tile: MMAs 1030, the exchange 1020 (1860 where the 16-byte pieces of a warp lie 2 KB apart: what
 // the order of an E tile is for), y in 16-byte pieces 1200; but a tile takes 2600, most of it the chain of one warp: loads, MMAs,
 // transposes, sends and the barriers between.  Taken back, none faster beyond 1500 tokens: half a block of both factors per warp
 // (3300 cycles), four more warps that transpose and send (2500), loads of the next tile under the sends (2700).
 // Fifteen clusters fit the device (120 of 148 SMs).
 //   E_IN    x is E tiles, not token rows          E_OUT  results are E tiles (of the next matrix), not token rows
-//   BIAS, GELU                                     SAVE   u is left in p.e_out's place p.u_out
+//   BIAS, GELU                                     SAVE   u is left at p.u_out, as E tiles, for the backward call
 constexpr int kCl = 8, kHalfWarps = kWarps / 2;
 constexpr int kClX = 3, kClE = 4, kClV = 3, kClY = 3;        // tiles of 16 KB: input slots, exchange slots, w, results
 constexpr int kClSmem = (kClX + kClE + 1 + kClV + kClY) * kBwdTile + 1024;
@@ -896,8 +896,9 @@ add_parts_m64_kernel(const float *__restrict__ parts_l, const float *__restrict_
     float *dst = (kind == 0 ? dL : dR) + at;
     float4 s = make_float4(0, 0, 0, 0);
     depend_wait();
-    // What follows takes the SMs over as they empty (forward + backward of 2000 tokens 61.0 -> 56.2 us); with fewer parts to add its
-    // blocks are only in the way (64 tokens 23.5 -> 23.8).
+    // What follows takes the SMs over as they empty (forward + backward of 500 tokens 36 -> 34 us, 2000 60.1 -> 56.7, 8192 142 -> 137;
+    // the feed-forward block's 500 tokens 92 -> 89, 3000 210.5 -> 208.5, 6000 333 -> 334.5, 8192 426 -> 429); with fewer parts to add
+    // its blocks are only in the way (64 tokens 23.5 -> 23.8).
     if (n >= 8) depend_launch();
 #pragma unroll 5
     for (int i = range * per; i < (range + 1) * per && i < n; ++i) {
@@ -925,7 +926,7 @@ add_parts_m64_kernel(const float *__restrict__ parts_l, const float *__restrict_
 // leaves E tiles, the other way round otherwise; PERM: the token rows are the permuted side (the forward's output, the
 // adjoint's input).  A CTA keeps both planes of 8 blocks, so the four real products of a stage add up in the accumulators and
 // the intermediate is rounded once; as four real calls on the stacked planes and a combining pass this took twice the MMAs and
-// 5 x the memory traffic (2048 tokens, M^H (M x): 293 us, now 95; 64 tokens 72, now 23).
+// 5 x the memory traffic (2048 tokens, M^H (M x): 293 us, now 87; 64 tokens 72, now 21.6).
 template <bool FIRST, bool PERM>
 __global__ void __launch_bounds__(kThreads, 1)
 cplx_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_e, const __grid_constant__ CUtensorMap tm_re,
@@ -1221,14 +1222,14 @@ int fwd_on_clusters(const void *x, const void *L, const void *R, const void *bia
 
 // Where the forward runs on clusters.  They take 5.6 us and 1.45 for every round of tiles, of which there are as many as clusters
 // fit (15); the streams, in which a tile takes four CTAs, 8 us as long as each CTA has one.  So: one round, or more tiles than
-// the streams' CTAs, up to five rounds (us, clusters / streams: 240 tokens 7.1 / 8.3, 300 8.6 / 8.4, 600 10.5 / 11.7, 960
-// 12.4 / 13.1, 1500 16.2 / 15.8).  Under the feed-forward backward, whose next launch reads y, one round (1000 tokens 122.8 / 121.7).
+// the streams' CTAs, up to five rounds (us, clusters / streams: 240 tokens 6.9 / 8.3, 300 8.6 / 8.4, 600 9.8 / 11.7, 960
+// 11.6 / 13.1, 1500 16.2 / 15.8).  Under the feed-forward backward, whose next launch reads y, one round (1000 tokens 122.8 / 121.7).
 static bool fwd_prefers_clusters(int64_t tokens, bool bias, int sms)
 {
     const int64_t tiles = tc::tiles_of(tokens), fit = bias ? tc::clusters<false, false, true, false, true>() : tc::clusters<false, false, false, false, true>();
     return fit > 0 && (tiles <= fit || (!bias && tiles * tc::kFwdGroups > sms && tiles <= 5 * fit));
 }
-// The feed-forward block, whose streams are four launches, up to ten rounds (16 tokens 11.7 / 17.4, 1000 25.3 / 28.9, 2400 40.4 /
+// The feed-forward block, whose streams are four launches, up to ten rounds (16 tokens 11.5 / 17.4, 1000 24.9 / 28.9, 2400 40.5 /
 // 42.5, 2700 45.5 / 44.3)
 static bool mlp_prefers_clusters(int64_t tokens)
 {
