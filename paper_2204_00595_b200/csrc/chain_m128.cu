@@ -72,6 +72,7 @@ struct ChainParams {
     int reverse;                             // walk the tiles from the last to the first: what the previous launch of
                                              // the chain wrote last is still in L2
     int discard_t0;                          // the T0 slabs are dead once read (dw', du'; not u', which the backward call reads)
+    int follows;                             // behind another launch of the same call
 };
 
 struct ChainBars {
@@ -83,7 +84,9 @@ struct ChainBars {
 
 // Programmatic dependent launch: a kernel of the chain lets its successor start as SMs become free (barrier set-up, TMEM
 // allocation and the weight load overlap this kernel's tail); the successor waits here, once per thread, before it
-// touches anything the chain wrote.  Both are no-ops in a launch without the attribute.
+// touches anything the chain wrote.  A thread signals after its own wait, so what ran before the call has finished when a launch
+// that `follows` begins, and only such a launch may ask for its weights before it waits: a call's first launch may begin while the
+// kernel that writes them still runs.  Both are no-ops in a launch without the attribute.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -241,12 +244,14 @@ chain_gemm_kernel(const __grid_constant__ CUtensorMap tm_t0, const __grid_consta
         tmem_alloc(smem_u32(&tmem_base_s), 512);
         tmem_relinquish();
     }
-    pdl_launch_dependents();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_s;
-    if (!(warp == 4 && lane == 0)) pdl_wait();          // the loader waits after it has asked for its first weight block
+    if (!(p.follows && warp == 4 && lane == 0)) {       // that loader waits after it has asked for its first weight block
+        pdl_wait();
+        pdl_launch_dependents();
+    }
 
     // items = (block, tile), block-major.  With a token reduction a CTA owns whole blocks (its accumulator lives in
     // TMEM across the tiles of a block); otherwise the items are cut into equal contiguous runs.
@@ -485,9 +490,9 @@ plane_transpose_kernel(const __grid_constant__ CUtensorMap tm_in, const __grid_c
         dead_s = 0;
         tma_prefetch_desc(&tm_in); tma_prefetch_desc(&tm_out);
     }
-    pdl_launch_dependents();
     __syncthreads();
     pdl_wait();
+    pdl_launch_dependents();
     // items (tile, plane), tile-major, dealt out round robin: the whole grid moves through the tiles together, so the
     // next launch of the chain can start with the tiles written last (still in L2)
     const long long total = (long long)p.ntiles * p.nplanes;
@@ -603,6 +608,7 @@ struct FusedParams {
     const char *x;                           // input, for the L2 prefetch hints only (the data path goes through TMA)
     const __nv_bfloat16 *bias;               // ACT: added to y, [n]
     int gelu;                                // ACT: y = GELU(M x + bias)
+    int follows;                             // behind another launch of the same call
     long long tokens;
     int ntiles;
     long long *trace;                        // debug builds: per-CTA cycle sums of the waits, else null
@@ -697,12 +703,14 @@ chain_fused_fwd_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_co
         tmem_alloc(smem_u32(&tmem_base_s), 256);
         tmem_relinquish();
     }
-    pdl_launch_dependents();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_s;
-    if (!(warp == 8 && lane == 0)) pdl_wait();          // the loader waits after it has asked for the weights
+    if (!(p.follows && warp == 8 && lane == 0)) {       // that loader waits after it has asked for the weights
+        pdl_wait();
+        pdl_launch_dependents();
+    }
 
     const int nt = p.ntiles, nsteps = nt + 2 * kFusedLag;
     const uint32_t full0 = smem_u32(bars.full), empty0 = smem_u32(bars.empty);
@@ -1027,7 +1035,7 @@ struct Src {
 
 template <int T0_LD, bool W_IS_A, bool W_MN, bool T0_MN, int ST, bool WG, int T1_LD, bool T1_MN, bool MAIN>
 int launch_gemm(Src t0, Src t1, const CUtensorMap &w, const CUtensorMap &out, float *dW, int ntiles, unsigned *status, cudaStream_t s,
-                int overwrite = 0, int reverse = 0, int discard_t0 = 0)
+                int follows, int overwrite = 0, int reverse = 0, int discard_t0 = 0)
 {
     constexpr int SLOTS = WG ? 2 : 3;
     constexpr int smem = 2 * kOpBytes + SLOTS * (WG ? 2 : 1) * kOpBytes + kStagingBytes + 1024;
@@ -1041,6 +1049,7 @@ int launch_gemm(Src t0, Src t1, const CUtensorMap &w, const CUtensorMap &out, fl
     p.overwrite = overwrite;
     p.reverse = reverse;
     p.discard_t0 = discard_t0;
+    p.follows = follows;
     p.t0_base = t0.base;
     p.t1_base = t1.base;
     p.ntiles = ntiles;
@@ -1121,7 +1130,7 @@ namespace tc {
 namespace {
 // one persistent launch; every CTA must be resident at once (one per SM).  bias (optional): y = act(M x + bias)
 int launch_fused_fwd(const void *x, const void *L, const void *R, const void *bias, int gelu, void *y, int64_t tokens, void *ws,
-                     cudaStream_t s)
+                     int follows, cudaStream_t s)
 {
     char *up = (char *)ws + MONARCH_STATUS_BYTES + kChainCounterBytes;
     CUtensorMap mx, mR, mL;
@@ -1139,6 +1148,7 @@ int launch_fused_fwd(const void *x, const void *L, const void *R, const void *bi
     fp.x = (const char *)x;
     fp.bias = (const __nv_bfloat16 *)bias;
     fp.gelu = gelu;
+    fp.follows = follows;
     fp.tokens = tokens;
     fp.trace = nullptr;
 #ifdef MONARCH_TRACE
@@ -1165,8 +1175,8 @@ int chain_mlp_fwd_m128(const void *x, const void *L1, const void *R1, const void
 {
     if (tokens == 0) return MONARCH_OK;
     void *h = (char *)ws + chain_fwd_m128_workspace_bytes(tokens);
-    MONARCH_TRY(tc::launch_fused_fwd(x, L1, R1, b1, 1, h, tokens, ws, s));
-    return tc::launch_fused_fwd(h, L2, R2, b2, 0, y, tokens, ws, s);
+    MONARCH_TRY(tc::launch_fused_fwd(x, L1, R1, b1, 1, h, tokens, ws, 0, s));
+    return tc::launch_fused_fwd(h, L2, R2, b2, 0, y, tokens, ws, 1, s);
 }
 
 // y = P L P^T R x (Def. 3.1; Section 3.3 steps 1-3): one persistent launch, or three launches.
@@ -1176,7 +1186,7 @@ int chain_fwd_m128(const void *x, const void *L, const void *R, void *y, int64_t
     if (tokens == 0) return MONARCH_OK;
     if (tokens > (int64_t)1 << 30) return MONARCH_ERR_UNSUPPORTED;
     if (fwd_runs_fused(tokens) && g_skip_load.load(std::memory_order_relaxed) < 0)
-        return launch_fused_fwd(x, L, R, nullptr, 0, y, tokens, ws, s);
+        return launch_fused_fwd(x, L, R, nullptr, 0, y, tokens, ws, 0, s);
     const int ntiles = (int)((tokens + 127) / 128);
     unsigned *status = (unsigned *)ws;
     char *up = (char *)ws + MONARCH_STATUS_BYTES + kChainCounterBytes, *wp = up + planes_bytes(tokens);
@@ -1189,10 +1199,10 @@ int chain_fwd_m128(const void *x, const void *L, const void *R, void *y, int64_t
     MONARCH_TRY(map_pieces(&mw_st, wp, ntiles));
     // step 1 + inner permutation: D_k[j][t] = sum_i R[k][j][i] x[t][k*128+i]  ->  pieces of u' (row j to consumer j)
     MONARCH_TRY((launch_gemm<kLdX, true, false, false, kStP, false, kLdX, false, true>({&mx, nullptr}, {nullptr, nullptr}, mR, mu_st, nullptr,
-                                                                                          ntiles, status, s)));
+                                                                                          ntiles, status, s, 0)));
     // step 2: D_j[l][t] = sum_k L[j][l][k] u'_j[k][t]  ->  pieces of w' (row l to consumer l)
     MONARCH_TRY((launch_gemm<kLdC, true, false, true, kStP, false, kLdX, false, true>({nullptr, up}, {nullptr, nullptr}, mL, mw_st, nullptr,
-                                                                                         ntiles, status, s, 0, 1)));
+                                                                                         ntiles, status, s, 1, 0, 1)));
     // step 3 (outer permutation): y[t][l*128+j] = w'_l[j][t]
     return launch_transpose<false>({nullptr, wp}, my, ntiles, status, s);
 }
@@ -1229,7 +1239,7 @@ int chain_bwd_m128(const void *x, const void *dy, const void *L, const void *R, 
         if (up == nullptr) {
             MONARCH_TRY(map_pieces(&mu_st, up_own, ntiles));
             MONARCH_TRY((launch_gemm<kLdX, true, false, false, kStP, false, kLdX, false, true>({&mx, nullptr}, {nullptr, nullptr}, mR, mu_st,
-                                                                                                  nullptr, ntiles, status, s)));
+                                                                                                  nullptr, ntiles, status, s, 0)));
             up = up_own;
         }
     }
@@ -1240,18 +1250,18 @@ int chain_bwd_m128(const void *x, const void *dy, const void *L, const void *R, 
     // du'_k[j][t] = sum_l L[j][l][k] dw'_j[l][t] -> pieces of du' (row k to consumer k)   (+ dL[j][l][k] += sum_t dw'_j[l][t] u'_j[k][t])
     if (want_dw)
         MONARCH_TRY((launch_gemm<kLdC, true, true, true, kStP, true, kLdC, false, true>({nullptr, dwp}, {nullptr, up}, mL, mdu_st, dL, ntiles,
-                                                                                          status, s, !accumulate, 1, 1)));
+                                                                                          status, s, 1, !accumulate, 1, 1)));
     else
         MONARCH_TRY((launch_gemm<kLdC, true, true, true, kStP, false, kLdC, false, true>({nullptr, dwp}, {nullptr, nullptr}, mL, mdu_st, nullptr,
-                                                                                           ntiles, status, s, 0, 1, 1)));
+                                                                                           ntiles, status, s, 1, 0, 1, 1)));
     // dx[t][k*128+i] = sum_j du'_k[j][t] R[k][j][i]        (+ dR[k][j][i] += sum_t du'_k[j][t] x[t][k*128+i])
     if (want_dw && want_dx)
-        return launch_gemm<kLdC, false, true, true, kStX, true, kLdX, true, true>({nullptr, dup}, {&mx, nullptr}, mR, mdx, dR, ntiles, status, s,
+        return launch_gemm<kLdC, false, true, true, kStX, true, kLdX, true, true>({nullptr, dup}, {&mx, nullptr}, mR, mdx, dR, ntiles, status, s, 1,
                                                                                   !accumulate, 0, 1);
     if (want_dw)
-        return launch_gemm<kLdC, false, true, true, kStX, true, kLdX, true, false>({nullptr, dup}, {&mx, nullptr}, mR, mdx, dR, ntiles, status, s,
+        return launch_gemm<kLdC, false, true, true, kStX, true, kLdX, true, false>({nullptr, dup}, {&mx, nullptr}, mR, mdx, dR, ntiles, status, s, 1,
                                                                                    !accumulate, 0, 1);
-    return launch_gemm<kLdC, false, true, true, kStX, false, kLdX, true, true>({nullptr, dup}, {nullptr, nullptr}, mR, mdx, nullptr, ntiles, status, s,
+    return launch_gemm<kLdC, false, true, true, kStX, false, kLdX, true, true>({nullptr, dup}, {nullptr, nullptr}, mR, mdx, nullptr, ntiles, status, s, 1,
                                                                                0, 0, 1);
 }
 

@@ -59,7 +59,7 @@ __device__ __forceinline__ void let_copies_land(volatile int *dead)
 // Launched with programmatic serialization: a kernel may begin while the one before it drains.  Before its wait it may read only
 // what no kernel of its own call writes (the weights), and only behind a kernel of that call that signals after its own wait: what
 // ran before the call has then finished.  Everything else, and all writes, come after the wait.  The kernels of rect_tc.cu
-// and chain_m128.cu signal before they wait, so a launch behind one of them reads nothing early.
+// signal before they wait, so a launch behind one of them reads nothing early.
 __device__ __forceinline__ void depend_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void depend_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -1515,6 +1515,54 @@ def test_tile_that_never_arrives_on_clusters(P, call, item):
     test_tile_that_never_arrives(P, 64, 16 * 15 * 4, call, item)
 
 
+# ----------------------------------------------------------------- weights that the launch before the call still writes
+
+@pytest.mark.parametrize("m", [32, 64, 128])
+@pytest.mark.parametrize("call", ["fwd", "bwd", "bwd_dx", "bwd_dw", "mlp"])
+def test_weights_written_by_the_launch_before(P, m, call):
+    """Launches may begin while the one before them drains (monarch_rect_fwd lets its followers begin at once): a call whose weights
+    that one writes, in the rows it writes last, gives the bits that it gives once everything has finished."""
+    import torch
+    n, T, code, g = m * m, 300, P.BF16, torch.Generator(device="cuda").manual_seed(1200 + m)
+    draw = lambda *shape, std=1.0: (torch.randn(*shape, generator=g, device="cuda") * std).bfloat16()
+    q, b, t = 4, 1024, 8192
+    rx, rR, rL, ry = draw(t, q * b), draw(q, b, b, std=b ** -0.5), draw(b, q, q, std=(q * m) ** -0.5), torch.empty(t, q * b, device="cuda", dtype=torch.bfloat16)
+    tail = ry.view(-1)[-4 * m ** 3:].view(4, m, m, m)
+    x, dy, b1, b2 = draw(T, n), draw(T, n), draw(n, std=0.1), draw(n, std=0.1)
+    outs = [torch.empty_like(x), torch.empty(m, m, m, device="cuda"), torch.empty(m, m, m, device="cuda")]
+    op = {"fwd": P.OP_FWD, "bwd": P.OP_BWD, "bwd_dx": P.OP_BWD_DX, "bwd_dw": P.OP_BWD_DW, "mlp": P.OP_MLP_FWD}[call]
+    ws, ws_r = P.Workspace(P.monarch_workspace_bytes(op, T, n, m, code)), P.Workspace(P.monarch_rect_workspace_bytes(t, q, b, b, q, code))
+
+    def run(weights):
+        L, R, L2, R2 = weights
+        if call == "fwd":
+            P.monarch_fwd(x, L, R, outs[0], T, n, m, ws)
+        elif call == "bwd":
+            P.monarch_bwd(x, dy, L, R, *outs, 0, T, n, m, ws)
+        elif call == "bwd_dx":
+            P.monarch_bwd_dx(dy, L, R, outs[0], T, n, m, ws)
+        elif call == "bwd_dw":
+            P.monarch_bwd_dw(x, dy, L, R, *outs[1:], 0, T, n, m, ws)
+        else:
+            P.monarch_mlp_fwd(x, L, R, b1, L2, R2, b2, outs[0], T, n, m, ws)
+
+    for o in outs:
+        o.zero_()
+    P.monarch_rect_fwd(rx, rL, rR, ry, t, q, b, b, q, ws_r)
+    torch.cuda.synchronize()
+    run(tail.clone())
+    torch.cuda.synchronize()
+    want = [o.clone() for o in outs]
+    for _ in range(6):
+        ry.fill_(float("nan"))
+        torch.cuda.synchronize()
+        P.monarch_rect_fwd(rx, rL, rR, ry, t, q, b, b, q, ws_r)
+        run(tail)
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, w) for o, w in zip(outs, want))
+    assert P.monarch_last_device_status(ws) == 0
+
+
 # ----------------------------------------------------------------- m = 128: the three-launch forward, and run-to-run bits
 
 @pytest.mark.parametrize("T", [1, 130, 700])
