@@ -1404,12 +1404,12 @@ def test_tile_that_never_arrives(P, m, T, call, item):
     assert P.monarch_last_device_status(ws) == 0
 
 
-# ----------------------------------------------------------------- the m = 64 forward in a process of its own
+# ----------------------------------------------------------------- the m = 64 forward on clusters, in a process of its own
 
 @pytest.mark.parametrize("T", [1, 63, 130, 257, 2500])
 def test_fwd_m64_on_clusters(T):
     """The first calls of a process, which find out how many clusters fit the device (T <= 240: on clusters), against the
-    oracle."""
+    oracle.  The environment is one that asked for a variant of earlier versions: it changes nothing."""
     import os
     import subprocess
     import sys
@@ -1431,10 +1431,11 @@ for _ in range(2):
     P.monarch_fwd(x, L, R, y, T, n, m, ws)
 torch.cuda.synchronize()
 assert P.monarch_last_device_status(ws) == 0
-assert_close(to_host64(y), O.fwd(hx, hL, hR), "bf16", "y")
+assert_close(to_host64(y), O.fwd(hx, hL, hR), "bf16", "y on clusters")
 print("ok")
 """
-    out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=600)
+    env = dict(os.environ, MONARCH_M64_CLUSTER="1")
+    out = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=600)
     assert out.returncode == 0 and "ok" in out.stdout, out.stderr[-2000:]
 
 
