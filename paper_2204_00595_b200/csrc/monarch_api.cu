@@ -117,7 +117,7 @@ int pick(int op, int m, int dtype)
 //   bf16 m = 16   forward + backward 148 / 484 at 32768 tokens: every batch (the forward alone: fused_m16.cu)
 //   bf16 m = 32   forward 9.5 / 7.0 at 4, 12.4 / 6.6 at 1000; forward + backward 18.5 / 14.1 at 4: never; the backward of
 //                 the feed-forward block, eight launches otherwise, 45 / 48 at 64, 58 / 49 at 128 (with its forward)
-//   bf16 m = 64   forward 10.7 / 6.7 at 64; forward + backward 23 / 24.5 at 4, 26.7 / 26.3 at 64; block 18.6 / 12.5 at 64,
+//   bf16 m = 64   forward 10.7 / 6.9 at 64; forward + backward 23 / 24.5 at 4, 26.7 / 26.3 at 64; block 18.6 / 12.3 at 64,
 //                 with its backward 76 / 80 at 96, 113 / 82 at 256
 //   bf16 m = 128  forward 10.4 / 12.1 at 16, but the backward then has u to recompute: 34.9 / 32.4 together; block 25 / 25 at 32,
 //                 with its backward 98 / 101 at 32, 142 / 102 at 64
